@@ -11,7 +11,7 @@ from ._binding import (  # noqa: F401
     MODE_NONE, MODE_BSPARQ, MODE_VSPARQ,
     ROUND_TRUNCATE, ROUND_NEAREST,
     SET_5OPT, SET_3OPT, SET_2OPT, SET_6OPT, SET_7OPT,
-    library_path, load_library,
+    library_path, load_library, load_native,
     sparq_quantize, sparq_gemm_s8, sparq_conv2d_nhwc_s8,
     sparq_quantize_host, sparq_gemm_s8_host, sparq_conv2d_nhwc_s8_host,
     sparq_gemm_s8_static, STATIC_SCRATCH_BYTES,

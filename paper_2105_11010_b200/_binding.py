@@ -1,8 +1,10 @@
-"""ctypes binding with the same names as the C ABI in ``include/sparq.h``.
+"""Binding with the same names as the C ABI in ``include/sparq.h``.
 
 Argument marshalling only.  Tensors must already live on the CUDA device (the
 raw ``data_ptr`` is handed to the library) and work is enqueued on torch's
-current stream unless a stream is given.
+current stream unless a stream is given.  The calls of a forward pass go through the
+native module ``_native`` (``csrc/sparq_py.cpp``), which takes their arguments by position;
+diagnostics and set-up calls use ctypes.
 """
 from __future__ import annotations
 
@@ -121,6 +123,29 @@ def load_library() -> ctypes.CDLL:
     return _lib
 
 
+def load_native():
+    """The native call module; raises if it has not been built."""
+    load_library()
+    try:
+        from . import _native
+    except ImportError as e:
+        raise ImportError("the native call module of this package is missing or does not load: build it with "
+                          "`python -m paper_2105_11010_b200.build`") from e
+    return _native
+
+
+class _LazyNative:
+    """Stands for the native module until the first call, so that the package imports unbuilt."""
+
+    def __getattr__(self, name):
+        global _native
+        _native = load_native()
+        return getattr(_native, name)
+
+
+_native = _LazyNative()
+
+
 def _stream_ptr(stream) -> Optional[int]:
     if stream is None:
         stream = torch.cuda.current_stream()
@@ -181,31 +206,9 @@ def sparq_shutdown() -> None:
 def sparq_quantize(inp: torch.Tensor, out: torch.Tensor, rows: int, row_len: int,
                    params: SparqParams, stream=None) -> None:
     """``out = T(inp)`` for ``rows`` rows of ``row_len`` uint8 activations."""
-    if inp.numel() < rows * row_len or out.numel() < rows * row_len:
-        raise ValueError("tensor smaller than rows * row_len")
-    p = params._c()
-    _raise(load_library().sparq_quantize(_dev(inp, torch.uint8, "inp"), _dev(out, torch.uint8, "out"),
-                                         rows, row_len, ctypes.byref(p), _stream_ptr(stream)))
-
-
-def _next(next_transform):
-    """(pointer for the struct, object that keeps the pointee alive)"""
-    if next_transform is None:
-        return None, None
-    c = next_transform._c()
-    return ctypes.pointer(c), c
-
-
-def _epilogue(n_cols: int, scale, bias, relu, inv_out_scale, acc_out, f32_out, u8_out, next_transform=None,
-              residual=None, residual_scale=0.0) -> _CEpilogue:
-    for name, t in (("scale", scale), ("bias", bias)):
-        if t is not None and t.numel() < n_cols:
-            raise ValueError(f"{name} has fewer than N elements")
-    return _CEpilogue(_dev(scale, torch.float32, "scale"), _dev(bias, torch.float32, "bias"),
-                      int(bool(relu)), float(inv_out_scale),
-                      _dev(acc_out, torch.int32, "acc_out"), _dev(f32_out, torch.float32, "f32_out"),
-                      _dev(u8_out, torch.uint8, "u8_out"), _next(next_transform)[0],
-                      _dev(residual, torch.uint8, "residual"), float(residual_scale))
+    rc = _native.quantize(inp, out, rows, row_len, params, stream)
+    if rc:
+        _raise(rc)
 
 
 def sparq_gemm_s8(A: torch.Tensor, B: torch.Tensor, params: SparqParams, *,
@@ -216,18 +219,10 @@ def sparq_gemm_s8(A: torch.Tensor, B: torch.Tensor, params: SparqParams, *,
                   next_transform: Optional[SparqParams] = None,
                   residual: Optional[torch.Tensor] = None, residual_scale: float = 0.0, stream=None) -> None:
     """``acc = T(A) @ B^T`` with A (M, K) uint8 and B (N, K) int8, then the epilogue."""
-    M, K = A.shape
-    N, K2 = B.shape
-    if K != K2:
-        raise ValueError("A and B disagree on K")
-    for name, t in (("acc_out", acc_out), ("f32_out", f32_out), ("u8_out", u8_out), ("residual", residual)):
-        if t is not None and t.numel() < M * N:
-            raise ValueError(f"{name} has fewer than M*N elements")
-    p = params._c()
-    e = _epilogue(N, scale, bias, relu, inv_out_scale, acc_out, f32_out, u8_out, next_transform,
-                  residual, residual_scale)
-    _raise(load_library().sparq_gemm_s8(_dev(A, torch.uint8, "A"), K, _dev(B, torch.int8, "B"), K,
-                                        M, N, K, ctypes.byref(p), ctypes.byref(e), _stream_ptr(stream)))
+    rc = _native.gemm(A, B, params, scale, bias, relu, inv_out_scale, acc_out, f32_out, u8_out,
+                      next_transform, residual, residual_scale, stream)
+    if rc:
+        _raise(rc)
 
 
 def sparq_conv2d_nhwc_s8(x: torch.Tensor, w: torch.Tensor, stride, pad, params: SparqParams, *,
@@ -238,23 +233,10 @@ def sparq_conv2d_nhwc_s8(x: torch.Tensor, w: torch.Tensor, stride, pad, params: 
                   next_transform: Optional[SparqParams] = None,
                   residual: Optional[torch.Tensor] = None, residual_scale: float = 0.0, stream=None) -> None:
     """Fused convolution of NHWC uint8 ``x`` with [cout][r][s][c] int8 ``w``."""
-    nb, h, wd, c = x.shape
-    cout, r, s, c2 = w.shape
-    if c != c2:
-        raise ValueError("x and w disagree on the channel count")
-    ho = (h + 2 * pad[0] - r) // stride[0] + 1
-    wo = (wd + 2 * pad[1] - s) // stride[1] + 1
-    m = nb * ho * wo
-    for name, t in (("acc_out", acc_out), ("f32_out", f32_out), ("u8_out", u8_out), ("residual", residual)):
-        if t is not None and t.numel() < m * cout:
-            raise ValueError(f"{name} has fewer than N*Ho*Wo*Cout elements")
-    p = params._c()
-    e = _epilogue(cout, scale, bias, relu, inv_out_scale, acc_out, f32_out, u8_out, next_transform,
-                  residual, residual_scale)
-    _raise(load_library().sparq_conv2d_nhwc_s8(_dev(x, torch.uint8, "x"), nb, h, wd, c,
-                                               _dev(w, torch.int8, "w"), cout, r, s,
-                                               stride[0], stride[1], pad[0], pad[1],
-                                               ctypes.byref(p), ctypes.byref(e), _stream_ptr(stream)))
+    rc = _native.conv2d(x, w, stride, pad, params, scale, bias, relu, inv_out_scale, acc_out, f32_out, u8_out,
+                        next_transform, residual, residual_scale, stream)
+    if rc:
+        _raise(rc)
 
 
 # ---- packed stream ------------------------------------------------------------------------
@@ -268,34 +250,19 @@ def sparq_packed_ctrl_bits(params: SparqParams) -> int:
     return rc
 
 
-def _rows(t: torch.Tensor):
-    row_len = t.shape[-1] if t.dim() else 1
-    return (t.numel() // row_len if row_len else 0), row_len
-
-
 def sparq_pack(inp: torch.Tensor, params: SparqParams, data: torch.Tensor, ctrl: torch.Tensor, stream=None) -> None:
     """Packed stream of ``inp`` (rows along the last axis) into the caller's ``data``
     (numel / 16 * 2 * window_bits bytes) and ``ctrl`` (numel / 16 * ctrl_bits bytes) planes."""
-    rows, row_len = _rows(inp)
-    cb = sparq_packed_ctrl_bits(params)
-    if data.numel() < inp.numel() // 16 * 2 * params.window_bits or ctrl.numel() < inp.numel() // 16 * cb:
-        raise ValueError("data / ctrl plane too small")
-    p = params._c()
-    _raise(load_library().sparq_pack(_dev(inp, torch.uint8, "inp"), rows, row_len, ctypes.byref(p),
-                                     _dev(data, torch.uint8, "data"), _dev(ctrl, torch.uint8, "ctrl"),
-                                     _stream_ptr(stream)))
+    rc = _native.pack(inp, params, data, ctrl, stream)
+    if rc:
+        _raise(rc)
 
 
 def sparq_unpack(data: torch.Tensor, ctrl: torch.Tensor, params: SparqParams, out: torch.Tensor, stream=None) -> None:
     """``out`` (rows along the last axis) = T(x) of the packed stream."""
-    rows, row_len = _rows(out)
-    cb = sparq_packed_ctrl_bits(params)
-    if data.numel() < out.numel() // 16 * 2 * params.window_bits or ctrl.numel() < out.numel() // 16 * cb:
-        raise ValueError("data / ctrl plane too small")
-    p = params._c()
-    _raise(load_library().sparq_unpack(_dev(data, torch.uint8, "data"), _dev(ctrl, torch.uint8, "ctrl"),
-                                       rows, row_len, ctypes.byref(p), _dev(out, torch.uint8, "out"),
-                                       _stream_ptr(stream)))
+    rc = _native.unpack(out, params, data, ctrl, stream)
+    if rc:
+        _raise(rc)
 
 
 # ---- uniform min-max quantization front end -----------------------------------------------
@@ -303,36 +270,25 @@ def sparq_unpack(data: torch.Tensor, ctrl: torch.Tensor, params: SparqParams, ou
 DTYPE_F32, DTYPE_BF16 = 0, 1
 
 
-def _float_ptr(x: torch.Tensor, name: str):
-    if x is None or not x.is_cuda or not x.is_contiguous() or x.dtype not in (torch.float32, torch.bfloat16):
-        raise ValueError(f"{name} must be a contiguous CUDA tensor of float32 or bfloat16")
-    return x.data_ptr(), (DTYPE_BF16 if x.dtype == torch.bfloat16 else DTYPE_F32)
-
-
 def sparq_absmax(x: torch.Tensor, max_inout: torch.Tensor, stream=None) -> None:
     """``max_inout[0] = max(max_inout[0], max |x|)`` on the device (float32, 1 element)."""
-    ptr, dt = _float_ptr(x, "x")
-    _raise(load_library().sparq_absmax(ptr, dt, x.numel(), _dev(max_inout, torch.float32, "max_inout"),
-                                       _stream_ptr(stream)))
+    rc = _native.absmax(x, max_inout, stream)
+    if rc:
+        _raise(rc)
 
 
 def sparq_quantize_act_u8(x: torch.Tensor, max_dev: torch.Tensor, out: torch.Tensor, stream=None) -> None:
     """Unsigned symmetric per-layer quantization of ``x`` onto [0, max] in 255 steps."""
-    ptr, dt = _float_ptr(x, "x")
-    if out.numel() < x.numel():
-        raise ValueError("out is smaller than x")
-    _raise(load_library().sparq_quantize_act_u8(ptr, dt, x.numel(), _dev(max_dev, torch.float32, "max_dev"),
-                                                _dev(out, torch.uint8, "out"), _stream_ptr(stream)))
+    rc = _native.quantize_act(x, max_dev, out, stream)
+    if rc:
+        _raise(rc)
 
 
 def sparq_quantize_weight_s8(w: torch.Tensor, out: torch.Tensor, scale_out: torch.Tensor, stream=None) -> None:
     """Signed symmetric per-kernel quantization of float32 ``w`` (kernels along axis 0)."""
-    cout = w.shape[0]
-    k = w.numel() // cout if cout else 0
-    if out.numel() < w.numel() or scale_out.numel() < cout:
-        raise ValueError("out / scale_out too small")
-    _raise(load_library().sparq_quantize_weight_s8(_dev(w, torch.float32, "w"), cout, k, _dev(out, torch.int8, "out"),
-                                                   _dev(scale_out, torch.float32, "scale_out"), _stream_ptr(stream)))
+    rc = _native.quantize_weight(w, out, scale_out, stream)
+    if rc:
+        _raise(rc)
 
 
 # ---- 2:4 sparse weights ---------------------------------------------------------------------
@@ -360,12 +316,9 @@ def sparq_sparse24_expand_weights(vals: torch.Tensor, pos: torch.Tensor, params:
 
 def sparq_sparse24_expand_activations(A: torch.Tensor, params: SparqParams, a_exp: torch.Tensor, stream=None) -> None:
     """Activations (rows along the last axis, K) -> ``a_exp`` with K' per row."""
-    rows, K = _rows(A)
-    if a_exp.numel() < rows * sparq_sparse24_expanded_k(K, params):
-        raise ValueError("a_exp too small")
-    p = params._c()
-    _raise(load_library().sparq_sparse24_expand_activations(_dev(A, torch.uint8, "A"), rows, K, ctypes.byref(p),
-                                                            _dev(a_exp, torch.uint8, "a_exp"), _stream_ptr(stream)))
+    rc = _native.expand_activations(A, params, a_exp, stream)
+    if rc:
+        _raise(rc)
 
 
 def sparq_gemm_s8_sparse24(A: torch.Tensor, w_exp: torch.Tensor, params: SparqParams, *,
@@ -376,40 +329,20 @@ def sparq_gemm_s8_sparse24(A: torch.Tensor, w_exp: torch.Tensor, params: SparqPa
                            u8_out: Optional[torch.Tensor] = None, stream=None) -> None:
     """``acc[m][j] = sum_g T2(selected pair) . (v0, v1)`` for 2:4 weights expanded by
     :func:`sparq_sparse24_expand_weights`, then the epilogue."""
-    M, K = A.shape
-    N = w_exp.shape[0]
-    kx = sparq_sparse24_expanded_k(K, params)
-    if w_exp.numel() != N * kx:
-        raise ValueError("w_exp does not have N * K' elements")
-    if workspace is not None and workspace.numel() < M * kx:
-        raise ValueError("workspace smaller than M * K'")
-    p = params._c()
-    e = _epilogue(N, scale, bias, relu, inv_out_scale, acc_out, f32_out, u8_out)
-    _raise(load_library().sparq_gemm_s8_sparse24(_dev(A, torch.uint8, "A"), _dev(w_exp, torch.int8, "w_exp"), M, N, K,
-                                                 ctypes.byref(p), ctypes.byref(e),
-                                                 _dev(workspace, torch.uint8, "workspace"), _stream_ptr(stream)))
+    rc = _native.gemm_sparse24(A, w_exp, params, workspace, scale, bias, relu, inv_out_scale, acc_out, f32_out, u8_out,
+                               None, None, 0.0, stream)
+    if rc:
+        _raise(rc)
 
 
 # ---- host-buffer forms ------------------------------------------------------------------
 
-def _host(t: Optional[torch.Tensor], dtype, name: str) -> Optional[int]:
-    if t is None:
-        return None
-    if t.is_cuda:
-        raise ValueError(f"{name} must be a CPU tensor (pinned for asynchronous copies)")
-    if t.dtype != dtype or not t.is_contiguous():
-        raise ValueError(f"{name} must be a contiguous {dtype} tensor")
-    return t.data_ptr() or None
-
-
 def sparq_quantize_host(inp: torch.Tensor, out: torch.Tensor, rows: int, row_len: int,
                         params: SparqParams, stream=None) -> None:
     """Host-buffer form of :func:`sparq_quantize`; returns after the result is in ``out``."""
-    if inp.numel() < rows * row_len or out.numel() < rows * row_len:
-        raise ValueError("tensor smaller than rows * row_len")
-    p = params._c()
-    _raise(load_library().sparq_quantize_host(_host(inp, torch.uint8, "inp"), _host(out, torch.uint8, "out"),
-                                              rows, row_len, ctypes.byref(p), _stream_ptr(stream)))
+    rc = _native.quantize_host(inp, out, rows, row_len, params, stream)
+    if rc:
+        _raise(rc)
 
 
 def sparq_gemm_s8_host(A: torch.Tensor, B: torch.Tensor, params: SparqParams, *,
@@ -419,21 +352,10 @@ def sparq_gemm_s8_host(A: torch.Tensor, B: torch.Tensor, params: SparqParams, *,
                        u8_out: Optional[torch.Tensor] = None,
                   residual: Optional[torch.Tensor] = None, residual_scale: float = 0.0, stream=None) -> None:
     """Host-buffer form of :func:`sparq_gemm_s8`: ``A`` and the outputs are CPU tensors."""
-    M, K = A.shape
-    N, K2 = B.shape
-    if K != K2:
-        raise ValueError("A and B disagree on K")
-    for name, t in (("acc_out", acc_out), ("f32_out", f32_out), ("u8_out", u8_out), ("residual", residual)):
-        if t is not None and t.numel() < M * N:
-            raise ValueError(f"{name} has fewer than M*N elements")
-    p = params._c()
-    e = _CEpilogue(_dev(scale, torch.float32, "scale"), _dev(bias, torch.float32, "bias"),
-                   int(bool(relu)), float(inv_out_scale),
-                   _host(acc_out, torch.int32, "acc_out"), _host(f32_out, torch.float32, "f32_out"),
-                   _host(u8_out, torch.uint8, "u8_out"), None,
-                   _host(residual, torch.uint8, "residual"), float(residual_scale))
-    _raise(load_library().sparq_gemm_s8_host(_host(A, torch.uint8, "A"), K, _dev(B, torch.int8, "B"), K,
-                                             M, N, K, ctypes.byref(p), ctypes.byref(e), _stream_ptr(stream)))
+    rc = _native.gemm_host(A, B, params, scale, bias, relu, inv_out_scale, acc_out, f32_out, u8_out,
+                           None, residual, residual_scale, stream)
+    if rc:
+        _raise(rc)
 
 
 def sparq_conv2d_nhwc_s8_host(x: torch.Tensor, w: torch.Tensor, stride, pad, params: SparqParams, *,
@@ -443,26 +365,10 @@ def sparq_conv2d_nhwc_s8_host(x: torch.Tensor, w: torch.Tensor, stride, pad, par
                               u8_out: Optional[torch.Tensor] = None,
                   residual: Optional[torch.Tensor] = None, residual_scale: float = 0.0, stream=None) -> None:
     """Host-buffer form of :func:`sparq_conv2d_nhwc_s8`: ``x`` and the outputs are CPU tensors."""
-    nb, h, wd, c = x.shape
-    cout, r, s, c2 = w.shape
-    if c != c2:
-        raise ValueError("x and w disagree on the channel count")
-    ho = (h + 2 * pad[0] - r) // stride[0] + 1
-    wo = (wd + 2 * pad[1] - s) // stride[1] + 1
-    m = nb * ho * wo
-    for name, t in (("acc_out", acc_out), ("f32_out", f32_out), ("u8_out", u8_out), ("residual", residual)):
-        if t is not None and t.numel() < m * cout:
-            raise ValueError(f"{name} has fewer than N*Ho*Wo*Cout elements")
-    p = params._c()
-    e = _CEpilogue(_dev(scale, torch.float32, "scale"), _dev(bias, torch.float32, "bias"),
-                   int(bool(relu)), float(inv_out_scale),
-                   _host(acc_out, torch.int32, "acc_out"), _host(f32_out, torch.float32, "f32_out"),
-                   _host(u8_out, torch.uint8, "u8_out"), None,
-                   _host(residual, torch.uint8, "residual"), float(residual_scale))
-    _raise(load_library().sparq_conv2d_nhwc_s8_host(_host(x, torch.uint8, "x"), nb, h, wd, c,
-                                                    _dev(w, torch.int8, "w"), cout, r, s,
-                                                    stride[0], stride[1], pad[0], pad[1],
-                                                    ctypes.byref(p), ctypes.byref(e), _stream_ptr(stream)))
+    rc = _native.conv2d_host(x, w, stride, pad, params, scale, bias, relu, inv_out_scale, acc_out, f32_out, u8_out,
+                             None, residual, residual_scale, stream)
+    if rc:
+        _raise(rc)
 
 
 STATIC_SCRATCH_BYTES = 8 << 20
@@ -482,15 +388,7 @@ def sparq_gemm_s8_static(A: torch.Tensor, B: torch.Tensor, params: SparqParams, 
     the library (``M * K <= STATIC_SCRATCH_BYTES``).  Synchronous; one call at a time per
     device.  The first call on a device performs the address look-up: make it before any
     stream capture."""
-    M, K = A.shape
-    N, K2 = B.shape
-    if K != K2:
-        raise ValueError("A and B disagree on K")
-    for name, t in (("acc_out", acc_out), ("f32_out", f32_out), ("u8_out", u8_out), ("residual", residual)):
-        if t is not None and t.numel() < M * N:
-            raise ValueError(f"{name} has fewer than M*N elements")
-    p = params._c()
-    e = _epilogue(N, scale, bias, relu, inv_out_scale, acc_out, f32_out, u8_out, next_transform,
-                  residual, residual_scale)
-    _raise(load_library().sparq_gemm_s8_static(_dev(A, torch.uint8, "A"), K, _dev(B, torch.int8, "B"), K,
-                                               M, N, K, ctypes.byref(p), ctypes.byref(e), _stream_ptr(stream)))
+    rc = _native.gemm_static(A, B, params, scale, bias, relu, inv_out_scale, acc_out, f32_out, u8_out,
+                             next_transform, residual, residual_scale, stream)
+    if rc:
+        _raise(rc)

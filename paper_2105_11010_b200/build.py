@@ -1,10 +1,12 @@
-"""Builds ``libsparq_b200.so`` (the C-ABI library) in-tree with nvcc for sm_100a."""
+"""Builds ``libsparq_b200.so`` (the C-ABI library) in-tree with nvcc for sm_100a, and ``_native``
+(the CPython call module over it, ``csrc/sparq_py.cpp``) with the host compiler."""
 from __future__ import annotations
 
 import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -19,6 +21,9 @@ NVCC_FLAGS = [
     "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
     "-I", os.path.join(ROOT, "include"), "-I", CSRC,
 ]
+
+
+NATIVE = os.path.join(PKG, "_native" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 
 
 def _nvcc() -> str:
@@ -70,5 +75,33 @@ def build_library(force: bool = False, verbose: bool = False) -> str:
     return LIB
 
 
+def build_native(force: bool = False, verbose: bool = False) -> str:
+    """The call module: torch's headers, linked to the C-ABI library beside it."""
+    src = os.path.join(CSRC, "sparq_py.cpp")
+    lib = build_library(verbose=verbose)
+    if not (force or _stale(NATIVE, [src, os.path.join(ROOT, "include", "sparq.h")])):
+        return NATIVE
+    import torch
+    troot = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(os.path.realpath(_nvcc())))
+    tmp = NATIVE + f".tmp{os.getpid()}"
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}",
+           "-I", os.path.join(ROOT, "include"), "-I", sysconfig.get_paths()["include"],
+           "-isystem", os.path.join(troot, "include"),
+           "-isystem", os.path.join(troot, "include", "torch", "csrc", "api", "include"),
+           "-isystem", os.path.join(cuda, "include"), src, "-o", tmp,
+           "-L", os.path.join(troot, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda",
+           "-L", os.path.dirname(lib), "-l:" + os.path.basename(lib), "-Wl,-rpath,$ORIGIN"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if verbose or r.returncode:
+        sys.stderr.write(r.stdout + r.stderr)
+    if r.returncode:
+        raise RuntimeError("building the native call module failed: " + " ".join(cmd))
+    os.replace(tmp, NATIVE)
+    return NATIVE
+
+
 if __name__ == "__main__":
     print(build_library(force="--force" in sys.argv, verbose="-v" in sys.argv))
+    print(build_native(force="--force" in sys.argv, verbose="-v" in sys.argv))
