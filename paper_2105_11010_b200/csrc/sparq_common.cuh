@@ -32,6 +32,43 @@ int validate_params(const sparq_params *p, XformArgs *x);
 // Bit 0: a bounded wait expired.  Allocated on first use, freed by sparq_shutdown().
 int get_status_word(unsigned int **dptr);
 
+// Memory that a launch writes (ptr == nullptr: nothing).
+struct OutRange {
+    const void *ptr;
+    size_t bytes;
+};
+
+// Records what the launch about to be enqueued on `st` writes; returns whether the weights (may
+// be null) are known to be clear of what the previous launch on the stream writes.
+bool note_outputs(cudaStream_t st, const OutRange (&outs)[3], const void *wgt = nullptr, size_t wgt_bytes = 0);
+
+// ---- overlapped launches ----------------------------------------------------------------
+// The library's kernels are launched with programmatic stream serialization: a kernel may start,
+// and set itself up, while its predecessor on the stream is finishing.  dep_wait() blocks until
+// every earlier kernel has completed and its writes are visible; no thread touches the caller's
+// memory before it (the fused kernels' early weights aside, see note_outputs).  dep_launch()
+// lets the next kernel start.
+#ifdef __CUDACC__
+__device__ __forceinline__ void dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class Kernel, class... Args>
+cudaError_t launch_overlapped(Kernel kernel, int grid, int threads, int smem_bytes, cudaStream_t st, const Args &...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = (size_t)smem_bytes;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+#endif
+
 // ---- device side -------------------------------------------------------------------
 
 #define SPARQ_HD __host__ __device__ __forceinline__

@@ -261,8 +261,8 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
         issue_resident_weights();
         b_issued = true;
     }
-    dep_launch();
     dep_wait();
+    dep_launch();
 
 
     if (warp == 0) {
@@ -737,7 +737,7 @@ cudaError_t launch_window_shape(const CUtensorMap &mx0, const CUtensorMap &mx1, 
             if (e_ != cudaSuccess) return e_;                                                          \
             if (dev_ >= 0 && dev_ < 64) attr_set[dev_] = true;                                         \
         }                                                                                              \
-        return launch_pdl<kWindowThreads>(kfn, grid, smem_bytes, st, mx0, mx1, mw, g);                                       \
+        return launch_overlapped(kfn, grid, kWindowThreads, smem_bytes, st, mx0, mx1, mw, g);         \
     } while (0)
 
 #define SPARQ_DEFINE_WINDOW_SHAPE(BN_, CB_, RES_)                                                      \

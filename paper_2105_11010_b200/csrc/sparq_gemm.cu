@@ -205,13 +205,15 @@ static int pick_bn(int64_t M, int64_t N, int sms, bool transform)
     return best;
 }
 
-// ---- what the previous fused launch on a stream wrote ---------------------------------------------
-// The fused kernels are launched with programmatic stream serialization and let their successor
-// start early; a successor may fetch its WEIGHTS before it waits for them -- provided the weights
-// are not among their outputs.  Every fused launch records its output ranges per (device,
-// stream) here and learns whether its own weights are clear of the previous launch's.  Kernels
-// of other libraries never release their successor early, so only these launches matter.  A
-// stream that is not in the table (first launch, or evicted) counts as "not clear".
+// ---- what the previous launch on a stream wrote ----------------------------------------------------
+// The library's kernels are launched with programmatic stream serialization and let their
+// successor start once they themselves may run; a fused successor may fetch its WEIGHTS before it
+// waits for them -- provided the weights are not among their outputs.  Every launch that lets
+// its successor start early records its output ranges per (device, stream) here, and a fused one
+// learns whether its own weights are clear of the previous launch's.  (Launches before that one
+// have completed: a kernel releases its successor after its own wait.)  Kernels of other libraries
+// never release their successor early.  A stream that is not in the table (first launch, or
+// evicted) counts as "not clear".
 struct LastLaunch {
     bool used;
     int dev;
@@ -224,7 +226,7 @@ static LastLaunch g_last[kLastSlots];
 static uint64_t g_last_age = 0;
 static std::mutex g_last_mutex;
 
-static bool record_launch_weights_clear(cudaStream_t st, const sparq_epilogue *e, size_t out_elems, const void *wgt, size_t wgt_bytes)
+bool note_outputs(cudaStream_t st, const OutRange (&outs)[3], const void *wgt, size_t wgt_bytes)
 {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return false; }
@@ -232,7 +234,7 @@ static bool record_launch_weights_clear(cudaStream_t st, const sparq_epilogue *e
     LastLaunch *slot = nullptr, *oldest = &g_last[0];
     for (LastLaunch &l : g_last) {
         if (l.used && l.dev == dev && l.stream == st) { slot = &l; break; }
-        if (!l.used || l.age < oldest->age || oldest->used && !l.used) oldest = &l;
+        if (!l.used || l.age < oldest->age || (oldest->used && !l.used)) oldest = &l;
     }
     bool clear = false;
     if (slot) {
@@ -243,14 +245,17 @@ static bool record_launch_weights_clear(cudaStream_t st, const sparq_epilogue *e
     } else {
         slot = oldest;
     }
-    const void *outs[3] = {e->acc_out, e->f32_out, e->u8_out};
-    const size_t width[3] = {4, 4, 1};
     slot->used = true; slot->dev = dev; slot->stream = st; slot->age = ++g_last_age;
     for (int i = 0; i < 3; ++i) {
-        slot->lo[i] = (uintptr_t)outs[i];
-        slot->hi[i] = outs[i] ? (uintptr_t)outs[i] + out_elems * width[i] : 0;
+        slot->lo[i] = (uintptr_t)outs[i].ptr;
+        slot->hi[i] = outs[i].ptr ? (uintptr_t)outs[i].ptr + outs[i].bytes : 0;
     }
     return clear;
+}
+
+static bool record_launch_weights_clear(cudaStream_t st, const sparq_epilogue *e, size_t out_elems, const void *wgt, size_t wgt_bytes)
+{
+    return note_outputs(st, {{e->acc_out, 4 * out_elems}, {e->f32_out, 4 * out_elems}, {e->u8_out, out_elems}}, wgt, wgt_bytes);
 }
 
 // Variant argument of the launchers: 4 = n = 4 with all five placements, 8 = another full

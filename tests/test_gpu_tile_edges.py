@@ -1,0 +1,35 @@
+"""Kernels at the sizes where their tilings can go wrong, byte for byte against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import sparq_synth as synth
+import paper_2105_11010_b200 as sparq
+
+pytestmark = pytest.mark.gpu
+
+# a warp encodes chunks of 128 units of 16 activations, two blocks of 16 warps per SM
+CHUNKS_RESIDENT = 148 * 2 * 16
+
+
+@pytest.mark.parametrize("n,mask", [(4, 0x1F), (4, 0x15), (4, 0x11), (3, 0x3F), (3, 0x35), (3, 0x29), (2, 0x7F), (2, 0x55)])
+@pytest.mark.parametrize("mode,units", [(m, u) for m in (sparq.MODE_BSPARQ, sparq.MODE_VSPARQ) for u in (1, 127, 129)] +
+                         [(sparq.MODE_VSPARQ, CHUNKS_RESIDENT * 128 + 131)])
+def test_codec_chunks(n, mask, mode, units):
+    x = synth.activations(units % 97, (units, 16), 0.5)
+    p = sparq.SparqParams(mode, n, mask, 1)
+    cb = sparq.sparq_packed_ctrl_bits(p)
+    xg = torch.from_numpy(x).cuda()
+    # guard bytes behind every plane: nothing may be written past its end
+    data = torch.full((units * 2 * n + 16,), 0xA5, dtype=torch.uint8, device="cuda")
+    ctrl = torch.full((units * cb + 16,), 0xA5, dtype=torch.uint8, device="cuda")
+    out = torch.full((units * 16 + 16,), 0xA5, dtype=torch.uint8, device="cuda")
+    sparq.sparq_pack(xg, p, data, ctrl)
+    sparq.sparq_unpack(data, ctrl, p, out[:units * 16].view(units, 16))
+    sparq.sparq_check()
+    wd, wc = oracle.pack_n(x, mode, n, mask, 1)
+    for got, want in ((data, wd), (ctrl, wc), (out, oracle.transform(x, mode, n, mask, 1).reshape(-1))):
+        got = got.cpu().numpy()
+        assert np.array_equal(got[:-16], want.reshape(-1))
+        assert (got[-16:] == 0xA5).all()
