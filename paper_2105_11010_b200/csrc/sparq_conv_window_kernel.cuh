@@ -75,8 +75,10 @@ struct WindowArgs {
     float residual_scale;
 };
 
-// dynamic shared memory the kernel may ask for: 227 KB minus room for its static variables
+// dynamic shared memory the kernel may ask for: 227 KB minus room for its static variables (with
+// streamed weights the epilogue teams keep scale and bias of their own column tiles)
 constexpr int kWindowMaxDynSmem = 232448 - 4096;
+constexpr int kWindowMaxDynSmemStreamed = kWindowMaxDynSmem - 3072;
 constexpr int kMaxWinBufs = 4;
 constexpr int kMaxG = 8;
 constexpr int kMaxBStages = 12;
@@ -161,17 +163,22 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
     __shared__ __align__(8) uint64_t bar_win_full[kMaxWinBufs * kMaxG], bar_win_xf[kMaxWinBufs * kMaxG];
     __shared__ __align__(8) uint64_t bar_win_empty[kMaxWinBufs];
     __shared__ __align__(8) uint64_t bar_b_full[kMaxBStages], bar_b_empty[kMaxBStages];
-    // Accumulator stages in tensor memory; tile number t uses stage t % kAcc.  (Four stages were
-    // measured and changed nothing for tiles that run one after the other: the epilogue hands a
-    // stage back well within one tile.)  Streamed weights on 128-wide tiles: the tiles of a group
-    // are accumulated TOGETHER during one pass over the weights (kBatched), so a group holds up
-    // to two stages and four let the next group start while the previous one is in its epilogue.
+    // Accumulator stages in tensor memory; tile number t uses stage t % kAcc.  Streamed weights on
+    // 128-wide tiles: the tiles of a group are accumulated TOGETHER during one pass over the
+    // weights (kBatched), so a group holds up to two stages and four let the next group start
+    // while the previous one is in its epilogue.
     constexpr bool kBatched = !B_RESIDENT && BN == 128;
-    constexpr int kAcc = kBatched ? 4 : 2;
+    constexpr int kAcc = BN == 256 ? 2 : 4;
+    // epilogue teams: as in sparq_gemm_kernel
+    constexpr int kGroups = epi_warps(MODE) / 4;
+    constexpr int kMaxTeams = kGroups < kAcc ? kGroups : kAcc;
+    const int teams = g.units > gridDim.x ? kMaxTeams : 1;
     __shared__ __align__(8) uint64_t bar_acc_full[kAcc], bar_acc_empty[kAcc], bar_done;
     __shared__ uint32_t tmem_base_slot;
     __shared__ uint32_t abort_word;
-    __shared__ __align__(16) float s_scale[BN], s_bias[BN];
+    // one column tile (resident weights): the teams share one copy, all writing the same values
+    constexpr int kCopies = B_RESIDENT ? 1 : kMaxTeams;
+    __shared__ __align__(16) float s_scale_all[kCopies][BN], s_bias_all[kCopies][BN];
 
     constexpr int kBBlock = BN * CB;                   // one (tap, channel block) of weights
     constexpr int kTmemCols = kAcc * BN;
@@ -190,17 +197,6 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
 
     const int taps = g.R * g.S;
     const int kb_count = taps * g.c_blocks;            // weight blocks per tile
-    // A tile's epilogue is mostly latency (barrier read, tensor-memory loads, stores), not
-    // arithmetic.  When only requantized bytes are wanted and there is one column tile, the epilogue
-    // warps split into two teams, one per accumulator stage, each warp taking twice the columns of
-    // its lane quarter, so that the epilogues of two consecutive tiles overlap.
-    // (Measured: a gain on 64-wide tiles and on 128-wide tiles with a transform, whose eight epilogue
-    // warps are latency-bound; a loss where sixteen warps are already bound by instruction issue or
-    // where a warp would hold a 256-column accumulator for eight loads.)
-    constexpr bool kTeamsPay = BN == 64 || (BN == 128 && MODE != SPARQ_MODE_NONE);
-    const bool epi_teams = kTeamsPay && g.u8_out && !g.acc_out && !g.f32_out && !g.residual && g.next_mode == SPARQ_MODE_NONE &&
-                           g.n_tiles == 1 && (g.N % 32) == 0 && (!g.relu || g.inv_out_scale > 0.0f) &&
-                           (reinterpret_cast<uintptr_t>(g.u8_out) & 31u) == 0;
     if (threadIdx.x == 0) {
         prefetch_tensormap(&map_x0);
         prefetch_tensormap(&map_x1);
@@ -219,7 +215,7 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
         }
         if (lane < kAcc) {
             mbar_init(smem_u32(&bar_acc_full[lane]), 1);
-            mbar_init(smem_u32(&bar_acc_empty[lane]), epi_teams ? epi_warps(MODE) / 2 : epi_warps(MODE));
+            mbar_init(smem_u32(&bar_acc_empty[lane]), 4 * epi_parts(kGroups, teams, BN));
         }
         if (lane == 0) {
             mbar_init(smem_u32(&bar_done), 2);
@@ -530,11 +526,13 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
         __syncwarp();
     } else if (warp < kFirstEpiWarp + epi_warps(MODE)) {
         // ================= epilogue =================
-        constexpr int kEpi = epi_warps(MODE);
-        constexpr int kColsPerWarp = BN / (kEpi / 4);     // the tile's columns are split over the warps of a quarter
         const int quarter = warp & 3;
-        const int part = (warp - kFirstEpiWarp) >> 2;
-        const int et = threadIdx.x - kFirstEpiWarp * 32;
+        const int group = (warp - kFirstEpiWarp) >> 2;
+        const uint32_t team = (uint32_t)(group % teams);     // tiles whose number is team modulo teams
+        const int parts = epi_parts(kGroups, teams, BN), part = group / teams;
+        const int cols = BN / parts, cbase = part * cols;
+        const int team_thread = (part * 4 + quarter) * 32 + lane, team_threads = parts * 128;
+        float *s_scale = s_scale_all[B_RESIDENT ? 0 : team], *s_bias = s_bias_all[B_RESIDENT ? 0 : team];
         const EpiView ev = make_epi_view(g);
         uint32_t wt = 0;
         int64_t staged_nt = -1;
@@ -543,121 +541,25 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
         const int tr = slot / g.Wp;
         const int ow = slot - tr * g.Wp;
         const bool slot_ok = (tr < g.TR) && (ow < g.Wo);
-        // 64-wide tiles have one column tile and 16 or 32 columns per warp.  When only the
-        // requantized bytes are wanted (the form every layer of a network uses), the warp keeps
-        // the scale and bias of its columns in registers for the whole launch -- shared-memory
-        // reads queue behind the tensor core's operand fetches -- and takes the accumulator in
-        // 16-column pieces so that those registers fit beside it.
-        if (epi_teams) {
-            constexpr int kTeamWarps = kEpi / 2;
-            constexpr int kTeamCols = BN / (kTeamWarps / 4);      // columns per warp
-            epi_stage_scale_bias<kEpi>(g, 0, BN, et, s_scale, s_bias);
-            const uint32_t team = (uint32_t)(warp - kFirstEpiWarp) / kTeamWarps;     // team t takes the tiles of parity t (kAcc is even)
-            const int cbase = (((warp - kFirstEpiWarp) % kTeamWarps) >> 2) * kTeamCols;
-            for (; have; have = walk.next()) {
-                for (int j = 0; j < (int)walk.cnt; ++j, ++wt) {
-                    if ((wt & 1u) != team) continue;
-                    const int oh = ((int)walk.tin + j) * g.TR + tr;
-                    const bool row_ok = slot_ok && (oh < g.Ho);
-                    const int64_t row = ((int64_t)walk.img * g.Ho + oh) * g.Wo + ow;
-                    const uint32_t acc = wt & (uint32_t)(kAcc - 1);
-                    const uint32_t taddr0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + (uint32_t)cbase;
-                    mbar_wait(smem_u32(&bar_acc_full[acc]), (wt / (uint32_t)kAcc) & 1u, abort_flag, g.status, g.wait_limit);
-                    tc_fence_after();
-#pragma unroll 1
-                    for (int ch = 0; ch < kTeamCols / 32; ++ch) {
-                        uint32_t v[32];
-                        tmem_ld_32x32_issue(taddr0 + (uint32_t)(ch * 32), v);
-                        tmem_ld_wait();
-                        if (ch + 1 == kTeamCols / 32) {
-                            tc_fence_before();
-                            __syncwarp();
-                            if (lane == 0) mbar_arrive(smem_u32(&bar_acc_empty[acc]));
-                        }
-                        const int ct = cbase + ch * 32;
-                        if (!row_ok || ct >= (int)g.N) continue;       // N is a multiple of 32 here
-                        if (ev.small_acc) epi_chunk_u8<true>(ev, v, row, ct, ct, s_scale, s_bias);
-                        else epi_chunk_u8<false>(ev, v, row, ct, ct, s_scale, s_bias);
-                    }
+        for (; have && part < parts; have = walk.next()) {
+            for (int j = 0; j < (int)walk.cnt; ++j, ++wt) {
+                if (wt % (uint32_t)teams != team) continue;
+                const int64_t nt = (int64_t)walk.nt;
+                const uint32_t acc = wt % (uint32_t)kAcc, acc_use = wt / (uint32_t)kAcc;
+                if (ev.need_f && nt != staged_nt) {
+                    staged_nt = nt;
+                    epi_stage_scale_bias(g, nt * BN, BN, team_thread, team_threads, 1 + (int)team, s_scale, s_bias);
                 }
-            }
-        } else
-        if (BN == 64 && ev.need_f && !g.acc_out && !g.f32_out && !g.residual && g.N == 64) {
-            epi_stage_scale_bias<kEpi>(g, 0, BN, et, s_scale, s_bias);
-            const int cbase = part * kColsPerWarp;
-            float rs[kColsPerWarp], rb[kColsPerWarp];
-#pragma unroll
-            for (int i = 0; i < kColsPerWarp; ++i) {
-                rs[i] = s_scale[cbase + i];
-                rb[i] = s_bias[cbase + i];
-            }
-            uint32_t pre_full = 0;     // the next tile's accumulator was seen complete
-            for (; have; have = walk.next()) {
-              for (int j = 0; j < (int)walk.cnt; ++j, ++wt) {
-                const uint32_t acc = wt & (uint32_t)(kAcc - 1);
-                // coordinates first: they do not depend on the accumulator
                 const int oh = ((int)walk.tin + j) * g.TR + tr;
                 const bool row_ok = slot_ok && (oh < g.Ho);
-                uint8_t *dst = g.u8_out + (((int64_t)walk.img * g.Ho + oh) * g.Wo + ow) * 64 + cbase;
+                const int64_t row = ((int64_t)walk.img * g.Ho + oh) * g.Wo + ow;
                 const uint32_t taddr0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + (uint32_t)cbase;
-                if (!pre_full) mbar_wait(smem_u32(&bar_acc_full[acc]), (wt / (uint32_t)kAcc) & 1u, abort_flag, g.status, g.wait_limit);
-                tc_fence_after();
-                pre_full = 0;
-#pragma unroll
-                for (int hh = 0; hh < kColsPerWarp / 16; ++hh) {
-                    uint32_t v[16];
-                    tmem_ld_32x16_issue(taddr0 + (uint32_t)(hh * 16), v);
-                    // While the load is in flight: has the next tile of the group been accumulated
-                    // already?  A barrier read takes hundreds of cycles behind the tensor core's
-                    // shared-memory traffic; here it overlaps the tensor-memory load, and a "yes"
-                    // lets the next tile start without one.
-                    if (hh == 0 && j + 1 < (int)walk.cnt)
-                        pre_full = mbar_test(smem_u32(&bar_acc_full[(wt + 1u) & (uint32_t)(kAcc - 1)]), ((wt + 1u) / (uint32_t)kAcc) & 1u);
-                    tmem_ld_wait();
-                    if (hh + 1 == kColsPerWarp / 16) {
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(smem_u32(&bar_acc_empty[acc]));
-                    }
-                    if (!row_ok) continue;
-                    uint32_t w[4];
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        float z[4];
-#pragma unroll
-                        for (int jj = 0; jj < 4; ++jj) {
-                            const int c = hh * 16 + 4 * q + jj;
-                            const float y = ev.small_acc ? dequant<true>((int32_t)v[4 * q + jj], rs[c], rb[c], ev.relu_op)
-                                                         : dequant<false>((int32_t)v[4 * q + jj], rs[c], rb[c], ev.relu_op);
-                            z[jj] = __fmul_rn(y, ev.inv_out_scale);
-                        }
-                        w[q] = requant_pack4(z[0], z[1], z[2], z[3]);
-                    }
-                    if (ev.next_mode != SPARQ_MODE_NONE) next_xform_words(w, 4, ev.next_mode, ev.next_rnd, ev.next_xf);
-                    *reinterpret_cast<uint4 *>(dst + hh * 16) = make_uint4(w[0], w[1], w[2], w[3]);
-                }
-              }
+                epi_warp_columns(ev, taddr0, cbase, cols, row, row_ok, nt * BN, s_scale, s_bias,
+                                 smem_u32(&bar_acc_empty[acc]), lane, [&]() {
+                                     mbar_wait(smem_u32(&bar_acc_full[acc]), acc_use & 1u, abort_flag, g.status, g.wait_limit);
+                                     tc_fence_after();
+                                 });
             }
-        } else
-        for (; have; have = walk.next()) {
-          for (int j = 0; j < (int)walk.cnt; ++j, ++wt) {
-            const int64_t nt = (int64_t)walk.nt;
-            const int acc = (int)(wt & (uint32_t)(kAcc - 1));
-            const uint32_t acc_use = wt / (uint32_t)kAcc;
-            if (ev.need_f && nt != staged_nt) {
-                staged_nt = nt;
-                epi_stage_scale_bias<kEpi>(g, nt * BN, BN, et, s_scale, s_bias);
-            }
-            mbar_wait(smem_u32(&bar_acc_full[acc]), acc_use & 1, abort_flag, g.status, g.wait_limit);
-            tc_fence_after();
-            const int oh = ((int)walk.tin + j) * g.TR + tr;
-            const bool row_ok = slot_ok && (oh < g.Ho);
-            const int64_t row = ((int64_t)walk.img * g.Ho + oh) * g.Wo + ow;
-            const int cbase = part * kColsPerWarp;
-            const uint32_t taddr0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * BN + cbase);
-            epi_warp_columns<kColsPerWarp>(ev, taddr0, cbase, row, row_ok, nt * BN, s_scale, s_bias,
-                                      smem_u32(&bar_acc_empty[acc]), lane);
-          }
         }
     } else if (MODE != SPARQ_MODE_NONE) {
         // ================= transform: once per piece =================
@@ -733,7 +635,7 @@ cudaError_t launch_window_shape(const CUtensorMap &mx0, const CUtensorMap &mx1, 
         if (e_ != cudaSuccess) return e_;                                                              \
         if (dev_ < 0 || dev_ >= 64 || !attr_set[dev_]) {                                               \
             e_ = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize,                \
-                                      kWindowMaxDynSmem);                                              \
+                                      RES ? kWindowMaxDynSmem : kWindowMaxDynSmemStreamed);            \
             if (e_ != cudaSuccess) return e_;                                                          \
             if (dev_ >= 0 && dev_ < 64) attr_set[dev_] = true;                                         \
         }                                                                                              \

@@ -270,15 +270,14 @@ static XformDev xform_dev(const XformArgs &x)
     return d;
 }
 
-static cudaError_t launch(int bn, int bk, const CUtensorMap &ma, const CUtensorMap &mb, const GemmArgs &g,
-                          const XformArgs &x, int grid, cudaStream_t st)
+static cudaError_t launch(int bn, int bk, const GemmMaps &m, GemmArgs &g, const XformArgs &x, int grid, cudaStream_t st)
 {
-    if (bn == 64 && bk == 64) return launch_gemm_shape<64, 64>(ma, mb, g, x.mode, variant_n(x), x.rnd, grid, st);
-    if (bn == 64) return launch_gemm_shape<64, 128>(ma, mb, g, x.mode, variant_n(x), x.rnd, grid, st);
-    if (bn == 128 && bk == 64) return launch_gemm_shape<128, 64>(ma, mb, g, x.mode, variant_n(x), x.rnd, grid, st);
-    if (bn == 128) return launch_gemm_shape<128, 128>(ma, mb, g, x.mode, variant_n(x), x.rnd, grid, st);
-    if (bk == 64) return launch_gemm_shape<256, 64>(ma, mb, g, x.mode, variant_n(x), x.rnd, grid, st);
-    return launch_gemm_shape<256, 128>(ma, mb, g, x.mode, variant_n(x), x.rnd, grid, st);
+    if (bn == 64 && bk == 64) return launch_gemm_shape<64, 64>(m, g, x.mode, variant_n(x), x.rnd, grid, st);
+    if (bn == 64) return launch_gemm_shape<64, 128>(m, g, x.mode, variant_n(x), x.rnd, grid, st);
+    if (bn == 128 && bk == 64) return launch_gemm_shape<128, 64>(m, g, x.mode, variant_n(x), x.rnd, grid, st);
+    if (bn == 128) return launch_gemm_shape<128, 128>(m, g, x.mode, variant_n(x), x.rnd, grid, st);
+    if (bk == 64) return launch_gemm_shape<256, 64>(m, g, x.mode, variant_n(x), x.rnd, grid, st);
+    return launch_gemm_shape<256, 128>(m, g, x.mode, variant_n(x), x.rnd, grid, st);
 }
 
 static int fill_common(GemmArgs *g, const XformArgs &x, const sparq_epilogue *e, unsigned int *status)
@@ -296,6 +295,29 @@ static int fill_common(GemmArgs *g, const XformArgs &x, const sparq_epilogue *e,
     g->residual = e->residual;
     g->residual_scale = e->residual_scale;
     return next_transform_args(e, g->N, &g->next_mode, &g->next_rnd, &g->next_xf);
+}
+
+// Chooses the staged output (epi_staged_box) and encodes its tensor maps: for requantized bytes in
+// whole groups of 32 columns, when a warp's share of a tile is at least 64 columns wide.  The
+// staging buffers cost ring stages, and a hand-over per box where a CTA has a single tile, so the
+// output (and residual) bytes of a tile have to weigh at least 5/8 of its operands': 56x56x64 ->
+// 256 with a residual 44 -> 33 us, 14x14x256 -> 1024 with one 16 -> 15; 28x28x256 -> 512 without
+// one would lose (19 -> 20.5), 7x7x512 -> 2048 with one too (13.0 -> 13.6).
+static int output_maps(GemmMaps *m, GemmArgs *g, int mode, int bn, int64_t tiles, int grid)
+{
+    g->out_box = 0;
+    if (!make_epi_view(*g).lean || tiles <= grid) return SPARQ_OK;
+    const int64_t out_bytes = (int64_t)kBM * bn * (g->residual ? 2 : 1), operand_bytes = (int64_t)(kBM + bn) * g->K;
+    if (8 * out_bytes < 5 * operand_bytes) return SPARQ_OK;
+    const int groups = epi_warps(mode) / 4, acc = bn == 256 ? 2 : 4;
+    const int teams = groups < acc ? groups : acc;
+    const int cols = bn / epi_parts(groups, teams, bn), widest = mode == SPARQ_MODE_NONE ? 64 : 128;
+    const int box = cols < widest ? cols : widest;
+    if (box < 64) return SPARQ_OK;
+    g->out_box = box;
+    int rc = encode_2d(&m->out, g->u8_out, g->N, g->M, g->N, box, 32);
+    if (rc == SPARQ_OK && g->residual) rc = encode_2d(&m->res, g->residual, g->N, g->M, g->N, box, 32);
+    return rc;
 }
 
 int gemm_with_status(const uint8_t *A, int64_t lda, const int8_t *B, int64_t ldb, int64_t M, int64_t N, int64_t K,
@@ -423,20 +445,20 @@ static int try_window_conv(const uint8_t *x_in, int n, int h, int w, int c, cons
         // flight), which halves the weight traffic out of L2 -- the bound of these layers.
         batched = bn == 128;
         grp = batched ? (tiles_per_img < 2 ? tiles_per_img : 2) : gmax;
-        while (grp > 1 && kMaxDynSmem - 1024 - 2 * plane_for(grp) * c_blocks < 4 * b_block) --grp;
+        while (grp > 1 && kWindowMaxDynSmemStreamed - 1024 - 2 * plane_for(grp) * c_blocks < 4 * b_block) --grp;
         const int win_bytes1 = plane_for(grp) * c_blocks;
         // a CTA that owns a single group needs no second window buffer: the room goes to the
         // weight ring, whose depth (bytes in flight) bounds how fast one SM can pull the weights
         const int64_t groups_b = (int64_t)n * n_tiles * ((tiles_per_img + grp - 1) / grp);
         if (batched && groups_b <= sms) win_bufs = 1;
-        const int left = kMaxDynSmem - 1024 - win_bufs * win_bytes1;
+        const int left = kWindowMaxDynSmemStreamed - 1024 - win_bufs * win_bytes1;
         b_stages = left / b_block;
         if (b_stages > kMaxBStages) b_stages = kMaxBStages;
         if (b_stages < 2) return 0;
         // spare room beyond four weight stages goes to a third window buffer
-        if (win_bufs == 2 && b_stages > 4 && 1024 + 3 * win_bytes1 + 4 * b_block <= kMaxDynSmem) {
+        if (win_bufs == 2 && b_stages > 4 && 1024 + 3 * win_bytes1 + 4 * b_block <= kWindowMaxDynSmemStreamed) {
             win_bufs = 3;
-            b_stages = (kMaxDynSmem - 1024 - 3 * win_bytes1) / b_block;
+            b_stages = (kWindowMaxDynSmemStreamed - 1024 - 3 * win_bytes1) / b_block;
             if (b_stages > kMaxBStages) b_stages = kMaxBStages;
         }
     }
@@ -514,10 +536,10 @@ int gemm_with_status(const uint8_t *A, int64_t lda, const int8_t *B, int64_t ldb
     // step is a hand-off between three warp roles, which is what a small launch is made of)
     const int bk = (pad64 < pad128 && !(pad64 >= 320 && pad128 * 8 <= pad64 * 9)) ? 64 : 128;
     const int bn = pick_bn(M, N, sms, x.mode != SPARQ_MODE_NONE);
-    CUtensorMap ma, mb;
-    rc = encode_2d(&ma, A, K, M, lda, bk, kBM);
+    GemmMaps m = {};
+    rc = encode_2d(&m.a, A, K, M, lda, bk, kBM);
     if (rc != SPARQ_OK) return rc;
-    rc = encode_2d(&mb, B, K, N, ldb, bk, bn);
+    rc = encode_2d(&m.b, B, K, N, ldb, bk, bn);
     if (rc != SPARQ_OK) return rc;
     GemmArgs g;
     memset(&g, 0, sizeof(g));
@@ -528,8 +550,9 @@ int gemm_with_status(const uint8_t *A, int64_t lda, const int8_t *B, int64_t ldb
     const int64_t tiles = ((M + kBM - 1) / kBM) * ((N + bn - 1) / bn);
     if (tiles >= ((int64_t)1 << 31)) return set_error(SPARQ_ERR_UNSUPPORTED, "more than 2^31 output tiles");
     const int grid = (int)(tiles < sms ? tiles : sms);
+    if ((rc = output_maps(&m, &g, x.mode, bn, tiles, grid)) != SPARQ_OK) return rc;
     record_launch_weights_clear(st, e, (size_t)M * (size_t)N, B, (size_t)N * (size_t)ldb);
-    cudaError_t ce = launch(bn, bk, ma, mb, g, x, grid, st);
+    cudaError_t ce = launch(bn, bk, m, g, x, grid, st);
     if (ce != cudaSuccess) return cuda_error(ce, "sparq_gemm_kernel launch");
     return SPARQ_OK;
 }
@@ -603,10 +626,10 @@ extern "C" int sparq_conv2d_nhwc_s8(const uint8_t *x_in, int n, int h, int w, in
     }
     const int bk = (c % 128 == 0) ? 128 : 64;
     const int bn = pick_bn(M, cout, sms, x.mode != SPARQ_MODE_NONE);
-    CUtensorMap ma, mb;
-    rc = encode_im2col(&ma, x_in, n, h, w, c, r, s, stride_h, stride_w, pad_h, pad_w, bk);
+    GemmMaps m = {};
+    rc = encode_im2col(&m.a, x_in, n, h, w, c, r, s, stride_h, stride_w, pad_h, pad_w, bk);
     if (rc != SPARQ_OK) return rc;
-    rc = encode_2d(&mb, wgt, K, cout, K, bk, bn);
+    rc = encode_2d(&m.b, wgt, K, cout, K, bk, bn);
     if (rc != SPARQ_OK) return rc;
     GemmArgs g;
     memset(&g, 0, sizeof(g));
@@ -625,8 +648,9 @@ extern "C" int sparq_conv2d_nhwc_s8(const uint8_t *x_in, int n, int h, int w, in
     const int64_t tiles = ((M + kBM - 1) / kBM) * ((cout + bn - 1) / bn);
     if (tiles >= ((int64_t)1 << 31)) return set_error(SPARQ_ERR_UNSUPPORTED, "more than 2^31 output tiles");
     const int grid = (int)(tiles < sms ? tiles : sms);
+    if ((rc = output_maps(&m, &g, x.mode, bn, tiles, grid)) != SPARQ_OK) return rc;
     record_launch_weights_clear(st, e, (size_t)M * (size_t)cout, wgt, (size_t)cout * (size_t)K);
-    cudaError_t ce = launch(bn, bk, ma, mb, g, x, grid, st);
+    cudaError_t ce = launch(bn, bk, m, g, x, grid, st);
     if (ce != cudaSuccess) return cuda_error(ce, "sparq_gemm_kernel (convolution) launch");
     return SPARQ_OK;
 }

@@ -44,6 +44,10 @@ constexpr int kFirstXfWarp = kFirstEpiWarp + kNumEpiWarps;
 constexpr int kGemmThreads = 32 * (kFirstXfWarp + kNumXfWarps);
 // Epilogue warps of a kernel instantiated for `mode`.
 __host__ __device__ constexpr int epi_warps(int mode) { return mode == SPARQ_MODE_NONE ? kNumEpiWarps + kNumXfWarps : kNumEpiWarps; }
+// Shares that a tile's columns are split into over the groups of one epilogue team.
+__host__ __device__ constexpr int epi_parts(int groups, int teams, int bn) { return groups / teams < bn / 32 ? groups / teams : bn / 32; }
+constexpr int kMaxStages = 8;
+constexpr int kMaxDynSmemGemm = 232448 - 6144;   // 227 KB minus room for the static variables
 constexpr int kSmemBudget = 200 * 1024;  // for the stage ring
 // Default limit of every device-side wait, in SM clock cycles (about a second).  The limit is a
 // kernel argument, so that a diagnostic launch can make a wait run out in microseconds.
@@ -78,6 +82,10 @@ struct GemmArgs {
     // residual input of the epilogue (nullptr = none)
     const uint8_t *residual;
     float residual_scale;
+    int stages;             // of the operand ring
+    // staged output: bytes per row of the boxes that the epilogue warps store (and fetch the residual)
+    // with through shared memory, 0 = straight from registers.  See epi_staged.
+    int out_box;
 };
 
 // ---- PTX wrappers ---------------------------------------------------------------------
@@ -185,6 +193,19 @@ __device__ __forceinline__ void tma_load_im2col_4d(uint32_t dst, const CUtensorM
         :: "r"(dst), "l"(map), "r"(bar), "r"(c), "r"(w), "r"(h), "r"(n), "h"(woff), "h"(hoff) : "memory");
 }
 
+// A box of shared memory into global memory (what lies outside the tensor is clipped); stores of a
+// thread form one group per tma_store_commit, and tma_store_wait_read<N> returns once all but
+// the last N groups have been read out of shared memory.
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, uint32_t src, int x, int y)
+{
+    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%2, %3}], [%1];"
+                 :: "l"(map), "r"(src), "r"(x), "r"(y) : "memory");
+}
+__device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read %0;" :: "n"(N) : "memory"); }
+__device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+
 __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap *map)
 {
     asm volatile("prefetch.tensormap [%0];" :: "l"(map) : "memory");
@@ -269,13 +290,6 @@ __device__ __forceinline__ constexpr uint32_t make_idesc_i8(int n)
 
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// Barrier among the epilogue warps only (hardware barrier 1).
-template <int WARPS>
-__device__ __forceinline__ void epi_bar_sync()
-{
-    asm volatile("bar.sync 1, %0;" :: "n"(WARPS * 32) : "memory");
-}
-
 // 32 contiguous bytes with one 256-bit store (dst 32-byte aligned).
 __device__ __forceinline__ void st_global_v8(void *dst, const uint32_t (&w)[8])
 {
@@ -297,29 +311,7 @@ __device__ __forceinline__ void tmem_ld_32x32_issue(uint32_t taddr, uint32_t (&r
         : "r"(taddr) : "memory");
 }
 
-__device__ __forceinline__ void tmem_ld_32x16_issue(uint32_t taddr, uint32_t (&r)[16])
-{
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr) : "memory");
-}
-
 // ---- epilogue arithmetic ----------------------------------------------------------------
-
-// int32 accumulator -> fp32 value, one IEEE operation per step.  SMALL: the caller
-// guarantees |acc| < 2^22, where (float)acc is exact and equals
-// bits(acc + bits(1.5 * 2^23)) - 1.5 * 2^23.
-template <bool SMALL>
-__device__ __forceinline__ float dequant(int32_t acc, float scale, float bias, int relu)
-{
-    float t = SMALL ? __fadd_rn(__int_as_float(acc + 0x4B400000), -12582912.0f) : __int2float_rn(acc);
-    float y = __fmaf_rn(t, scale, bias);
-    if (relu) y = fmaxf(y, 0.0f);        // NaN -> 0, like (y > 0 ? y : 0)
-    return y;
-}
 
 // Four fp32 values on the output grid -> four bytes clamp(rint(z), 0, 255) in one word, z0 in
 // the low byte: a round-to-nearest-even conversion to int32 each (NaN gives 0, the infinities
@@ -365,10 +357,9 @@ struct EpiView {
     float inv_out_scale;
     bool need_f;      // a dequantized output is requested
     bool relu_op;     // the ReLU select has to be executed (see below)
-    bool small_acc;   // |acc| < 2^22 guaranteed
-    bool vec_ok;      // rows allow 16/32-byte vector stores
-    bool u8_wide;     // 256-bit stores allowed on u8_out
-    bool lean;        // only requantized bytes are wanted and whole 32-byte groups can be stored: see epi_chunk_u8
+    bool vec_ok;      // rows allow 16-byte vector accesses
+    bool wide;        // rows come in whole groups of 32 columns, and every output and the residual allow 32-byte accesses
+    bool lean;        // wide, and only requantized bytes are wanted: see epi_lean
     int next_mode;    // SPARQ mode applied to the requantized bytes (producer-side transform)
     int next_rnd;
     XformDev next_xf;
@@ -377,7 +368,7 @@ struct EpiView {
 };
 
 template <class Args>
-__device__ __forceinline__ EpiView make_epi_view(const Args &g)
+__host__ __device__ __forceinline__ EpiView make_epi_view(const Args &g)
 {
     EpiView e;
     e.N = g.N;
@@ -389,134 +380,16 @@ __device__ __forceinline__ EpiView make_epi_view(const Args &g)
     // relu(y) * inv clamped to [0, 255] equals y * inv clamped when inv > 0, so the ReLU
     // select is only needed when the fp32 value itself is an output
     e.relu_op = g.relu && (g.f32_out != nullptr || !(g.inv_out_scale > 0.0f));
-    // |acc| <= K * 255 * 128; below 2^22 the int -> float conversion is exact and can be
-    // done with an integer add and a float subtract instead of the conversion unit
-    e.small_acc = g.K * (255 * 128) < (1 << 22);
-    e.vec_ok = (g.N % 32) == 0;
-    e.u8_wide = (reinterpret_cast<uintptr_t>(g.u8_out) & 31u) == 0;
-    e.lean = e.u8_out && !g.acc_out && !g.f32_out && !g.residual && g.next_mode == SPARQ_MODE_NONE && !e.relu_op &&
-             e.vec_ok && e.u8_wide;
+    e.vec_ok = (g.N % 16) == 0;
+    e.wide = (g.N % 32) == 0 && ((reinterpret_cast<uintptr_t>(g.u8_out) | reinterpret_cast<uintptr_t>(g.f32_out) |
+                                  reinterpret_cast<uintptr_t>(g.acc_out) | reinterpret_cast<uintptr_t>(g.residual)) & 31u) == 0;
+    e.lean = e.u8_out && !g.acc_out && !g.f32_out && g.next_mode == SPARQ_MODE_NONE && !e.relu_op && e.wide;
     e.next_mode = g.next_mode;
     e.next_rnd = g.next_rnd;
     e.next_xf = g.next_xf;
     e.residual = g.residual;
     e.residual_scale = g.residual_scale;
     return e;
-}
-
-// One thread's NV (32 or 16) consecutive accumulators of output row `row` (columns col0 ..
-// col0+NV-1, tile-local column ct): optional raw store, dequantize, optional fp32 store,
-// requantize and store.  v is overwritten.
-// REG: scale and bias of the NV columns come from the caller's registers rs / rb instead of
-// shared memory (shared-memory reads queue behind the tensor core's operand fetches).
-template <int NV = 32, bool REG = false>
-__device__ __forceinline__ void epi_chunk(const EpiView &e, uint32_t (&v)[NV], int64_t row, int64_t col0, int ct,
-                                          const float *s_scale, const float *s_bias,
-                                          const float *rs = nullptr, const float *rb = nullptr)
-{
-    static_assert(NV == 32 || NV == 16, "chunk width");
-    constexpr int NQ = NV / 4;      // groups of four columns = words of packed bytes
-    const int64_t off = row * e.N + col0;
-    const bool full = e.vec_ok && (col0 + NV <= e.N);
-    if (e.acc_out) {
-        if (full) {
-            int4 *dst = reinterpret_cast<int4 *>(e.acc_out + off);
-#pragma unroll
-            for (int q = 0; q < NQ; ++q)
-                dst[q] = make_int4((int)v[4 * q], (int)v[4 * q + 1], (int)v[4 * q + 2], (int)v[4 * q + 3]);
-        } else {
-            for (int i = 0; i < NV && col0 + i < e.N; ++i) e.acc_out[off + i] = (int32_t)v[i];
-        }
-    }
-    if (!e.need_f) return;
-    // with a residual input the ReLU comes after the sum
-    const int relu_first = e.residual ? 0 : (int)e.relu_op;
-    // v[i] becomes the fp32 value's bits in place
-    // scale and bias of 16 columns at a time: the eight 16-byte shared-memory reads are issued
-    // together, so that their latencies (long while the tensor core is fetching operands)
-    // overlap instead of adding up
-#pragma unroll
-    for (int h = 0; h < NV / 16; ++h) {
-        float hs[16], hb[16];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            if (REG) {
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    hs[4 * q + j] = rs[16 * h + 4 * q + j];
-                    hb[4 * q + j] = rb[16 * h + 4 * q + j];
-                }
-            } else {
-                const float4 sc = *reinterpret_cast<const float4 *>(&s_scale[ct + 16 * h + 4 * q]);
-                const float4 bi = *reinterpret_cast<const float4 *>(&s_bias[ct + 16 * h + 4 * q]);
-                hs[4 * q] = sc.x; hs[4 * q + 1] = sc.y; hs[4 * q + 2] = sc.z; hs[4 * q + 3] = sc.w;
-                hb[4 * q] = bi.x; hb[4 * q + 1] = bi.y; hb[4 * q + 2] = bi.z; hb[4 * q + 3] = bi.w;
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const int c = 16 * h + i;
-            v[c] = __float_as_uint(e.small_acc ? dequant<true>((int32_t)v[c], hs[i], hb[i], relu_first)
-                                               : dequant<false>((int32_t)v[c], hs[i], hb[i], relu_first));
-        }
-    }
-    if (e.residual) {
-        uint32_t r[NQ];
-        if (full) {
-#pragma unroll
-            for (int h = 0; h < NV / 16; ++h) {
-                const uint4 rr = __ldg(reinterpret_cast<const uint4 *>(e.residual + off) + h);
-                r[4 * h] = rr.x; r[4 * h + 1] = rr.y; r[4 * h + 2] = rr.z; r[4 * h + 3] = rr.w;
-            }
-        } else {
-#pragma unroll
-            for (int q = 0; q < NQ; ++q) r[q] = 0u;
-            for (int i = 0; i < NV && col0 + i < e.N; ++i)
-                r[i >> 2] |= (uint32_t)__ldg(e.residual + off + i) << (8 * (i & 3));
-        }
-#pragma unroll
-        for (int i = 0; i < NV; ++i) {
-            const float rv = __uint2float_rn((r[i >> 2] >> (8 * (i & 3))) & 0xFFu);
-            float y = __fmaf_rn(rv, e.residual_scale, __uint_as_float(v[i]));
-            if (e.relu_op) y = fmaxf(y, 0.0f);
-            v[i] = __float_as_uint(y);
-        }
-    }
-    if (e.f32_out) {
-        if (full) {
-            uint4 *dst = reinterpret_cast<uint4 *>(e.f32_out + off);
-#pragma unroll
-            for (int q = 0; q < NQ; ++q) dst[q] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-        } else {
-            for (int i = 0; i < NV && col0 + i < e.N; ++i) e.f32_out[off + i] = __uint_as_float(v[i]);
-        }
-    }
-    if (e.u8_out) {
-        uint32_t w[NQ];
-#pragma unroll
-        for (int q = 0; q < NQ; ++q)
-            w[q] = requant_pack4(__fmul_rn(__uint_as_float(v[4 * q]), e.inv_out_scale),
-                                 __fmul_rn(__uint_as_float(v[4 * q + 1]), e.inv_out_scale),
-                                 __fmul_rn(__uint_as_float(v[4 * q + 2]), e.inv_out_scale),
-                                 __fmul_rn(__uint_as_float(v[4 * q + 3]), e.inv_out_scale));
-        if (e.next_mode != SPARQ_MODE_NONE) next_xform_words(w, NQ, e.next_mode, e.next_rnd, e.next_xf);
-        if (full) {
-            if constexpr (NV == 32) {
-                if (e.u8_wide) {
-                    st_global_v8(e.u8_out + off, w);
-                } else {
-                    uint4 *dst = reinterpret_cast<uint4 *>(e.u8_out + off);
-                    dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
-                    dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
-                }
-            } else {
-                *reinterpret_cast<uint4 *>(e.u8_out + off) = make_uint4(w[0], w[1], w[2], w[3]);
-            }
-        } else {
-            for (int i = 0; i < NV && col0 + i < e.N; ++i)
-                e.u8_out[off + i] = (uint8_t)(w[i >> 2] >> (8 * (i & 3)));
-        }
-    }
 }
 
 // Two fp32 values in one 64-bit register and the packed arithmetic of sm_100: each instruction
@@ -551,93 +424,254 @@ __device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c)
     return d;
 }
 
-// The form every layer of a network uses -- requantized bytes only, no residual, full 32-column
-// groups -- as straight-line code with nothing decided per element and the fp32 steps done two
-// columns at a time: per accumulator an exact int -> float step, one fma, one multiply and the
-// conversion back to an integer, then two saturating packs per four columns.  Same IEEE
-// sequence per element as epi_chunk.
-template <bool SMALL>
-__device__ __forceinline__ void epi_chunk_u8(const EpiView &e, uint32_t (&v)[32], int64_t row, int64_t col0, int ct,
-                                             const float *s_scale, const float *s_bias)
+// 32 contiguous bytes (src 32-byte aligned) through the read-only path.
+__device__ __forceinline__ void ld_global_v8(const void *src, uint32_t (&w)[8])
 {
-    const uint64_t inv2 = f2_pack(e.inv_out_scale, e.inv_out_scale);
-    const uint64_t neg_magic2 = f2_pack(-12582912.0f, -12582912.0f);
-    uint32_t w[8];
+    asm volatile("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
+                 : "l"(src));
+}
+
+// Bytes 2H and 2H + 1 of w as two fp32 values: 2^23 + byte as a bit pattern (one permute), minus
+// 2^23, both exact.
+template <int H>
+__device__ __forceinline__ uint64_t bytes_to_f2(uint32_t w)
+{
+    const uint32_t a = prmt(w, 0x4B000000u, 0x7440u + (2 * H)), b = prmt(w, 0x4B000000u, 0x7440u + (2 * H + 1));
+    return f2_add(f2_pack(__uint_as_float(a), __uint_as_float(b)), f2_pack(-8388608.0f, -8388608.0f));
+}
+
+// The form every layer of a network uses -- requantized bytes only, whole groups of 32 columns --
+// as straight-line code with nothing decided per element and the fp32 steps done two columns at
+// a time: per accumulator one int -> float conversion, one fma, (with a residual one more fma,) one
+// multiply and the conversion back to an integer, then two saturating packs per four columns.
+// Same IEEE sequence per element as epi_general.  (The int -> float conversion beats the add-based
+// form for small accumulators: 46.6 against 42.7 outputs per clock and SM, arithmetic alone.)
+// res: the 32 columns' residual bytes.
+template <bool RES>
+__device__ __forceinline__ void epi_lean(const uint32_t (&v)[32], const float *s_scale, const float *s_bias, float inv, float res_scale,
+                                         const uint32_t (&res)[8], uint32_t (&w)[8])
+{
+    const uint64_t inv2 = f2_pack(inv, inv), rs2 = f2_pack(res_scale, res_scale);
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-        const float4 sc = *reinterpret_cast<const float4 *>(&s_scale[ct + 4 * q]);
-        const float4 bi = *reinterpret_cast<const float4 *>(&s_bias[ct + 4 * q]);
+        const float4 sc = *reinterpret_cast<const float4 *>(&s_scale[4 * q]);
+        const float4 bi = *reinterpret_cast<const float4 *>(&s_bias[4 * q]);
         float z[4];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int32_t a0 = (int32_t)v[4 * q + 2 * h], a1 = (int32_t)v[4 * q + 2 * h + 1];
-            // (float)acc: exact through the add-based form when |acc| < 2^22
-            const uint64_t t = SMALL ? f2_add(f2_pack(__int_as_float(a0 + 0x4B400000), __int_as_float(a1 + 0x4B400000)), neg_magic2)
-                                     : f2_pack(__int2float_rn(a0), __int2float_rn(a1));
-            const uint64_t y = f2_fma(t, h ? f2_pack(sc.z, sc.w) : f2_pack(sc.x, sc.y), h ? f2_pack(bi.z, bi.w) : f2_pack(bi.x, bi.y));
-            f2_unpack(f2_mul(y, inv2), z[2 * h], z[2 * h + 1]);
+        uint64_t y0 = f2_fma(f2_pack(__int2float_rn((int)v[4 * q]), __int2float_rn((int)v[4 * q + 1])), f2_pack(sc.x, sc.y), f2_pack(bi.x, bi.y));
+        uint64_t y1 = f2_fma(f2_pack(__int2float_rn((int)v[4 * q + 2]), __int2float_rn((int)v[4 * q + 3])), f2_pack(sc.z, sc.w), f2_pack(bi.z, bi.w));
+        if (RES) {
+            y0 = f2_fma(bytes_to_f2<0>(res[q]), rs2, y0);
+            y1 = f2_fma(bytes_to_f2<1>(res[q]), rs2, y1);
         }
+        f2_unpack(f2_mul(y0, inv2), z[0], z[1]);
+        f2_unpack(f2_mul(y1, inv2), z[2], z[3]);
         w[q] = requant_pack4(z[0], z[1], z[2], z[3]);
     }
-    st_global_v8(e.u8_out + row * e.N + col0, w);
 }
 
-// A warp's share of one accumulator: CW (16, 32, 64 or 128) columns starting at
-// tensor-memory address taddr0 (tile-local column cbase), for this thread's output row.
-// After the last load has landed in registers the warp hands the accumulator back by
-// arriving on acc_empty_bar.
-template <int CW>
-__device__ __forceinline__ void epi_warp_columns(const EpiView &e, uint32_t taddr0, int cbase, int64_t row, bool row_ok,
-                                                 int64_t n0, const float *s_scale, const float *s_bias,
-                                                 uint32_t acc_empty_bar, int lane)
+// 32 accumulators of one output row (columns col0 .. col0 + 31) with any combination of outputs and
+// any N: optional raw store, dequantize, optional fp32 store, requantize and store.  v is
+// overwritten.
+__device__ __forceinline__ void epi_general(const EpiView &e, uint32_t (&v)[32], int64_t row, int64_t col0,
+                                            const float *s_scale, const float *s_bias)
 {
-    if constexpr (CW == 16) {
-        uint32_t v[16];
-        tmem_ld_32x16_issue(taddr0, v);
-        tmem_ld_wait();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(acc_empty_bar);
-        const int64_t col0 = n0 + cbase;
-        if (row_ok && col0 < e.N) epi_chunk<16, false>(e, v, row, col0, cbase, s_scale, s_bias);
-    } else {
-        constexpr int CHUNKS = CW / 32;
-#pragma unroll 1
-        for (int ch = 0; ch < CHUNKS; ++ch) {
-            uint32_t v[32];
-            tmem_ld_32x32_issue(taddr0 + (uint32_t)(ch * 32), v);
-            tmem_ld_wait();
-            if (ch + 1 == CHUNKS) {
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(acc_empty_bar);
+    const int64_t off = row * e.N + col0;
+    const int cols = (int)(e.N - col0 < 32 ? e.N - col0 : 32);
+    const bool wide = e.wide, full = e.vec_ok && cols == 32;
+    auto store32 = [&](void *base) {       // 32 words
+        uint32_t *dst = reinterpret_cast<uint32_t *>(base) + off;
+        if (wide) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) st_global_v8(dst + 8 * q, reinterpret_cast<const uint32_t(&)[8]>(v[8 * q]));
+        } else if (full) {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) reinterpret_cast<uint4 *>(dst)[q] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 32; ++i)
+                if (i < cols) dst[i] = v[i];
+        }
+    };
+    if (e.acc_out) store32(e.acc_out);
+    if (!e.need_f) return;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const float4 sc = *reinterpret_cast<const float4 *>(&s_scale[4 * q]);
+        const float4 bi = *reinterpret_cast<const float4 *>(&s_bias[4 * q]);
+        const float ss[4] = {sc.x, sc.y, sc.z, sc.w}, bb[4] = {bi.x, bi.y, bi.z, bi.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            float y = __fmaf_rn(__int2float_rn((int)v[4 * q + i]), ss[i], bb[i]);
+            if (e.relu_op && !e.residual) y = fmaxf(y, 0.0f);    // NaN -> 0, like (y > 0 ? y : 0)
+            v[4 * q + i] = __float_as_uint(y);
+        }
+    }
+    if (e.residual) {                                            // with a residual input the ReLU comes after the sum
+        uint32_t r[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+        if (full) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const uint4 rr = __ldg(reinterpret_cast<const uint4 *>(e.residual + off) + h);
+                r[4 * h] = rr.x; r[4 * h + 1] = rr.y; r[4 * h + 2] = rr.z; r[4 * h + 3] = rr.w;
             }
-            const int ct = cbase + ch * 32;              // column inside the tile
-            const int64_t col0 = n0 + ct;
-            if (!row_ok || col0 >= e.N) continue;
-            if (e.lean && col0 + 32 <= e.N) {
-                if (e.small_acc) epi_chunk_u8<true>(e, v, row, col0, ct, s_scale, s_bias);
-                else epi_chunk_u8<false>(e, v, row, col0, ct, s_scale, s_bias);
-            } else {
-                epi_chunk<32, false>(e, v, row, col0, ct, s_scale, s_bias);
-            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 32; ++i)
+                if (i < cols) r[i >> 2] |= (uint32_t)__ldg(e.residual + off + i) << (8 * (i & 3));
+        }
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+            const float rv = __uint2float_rn((r[i >> 2] >> (8 * (i & 3))) & 0xFFu);
+            float y = __fmaf_rn(rv, e.residual_scale, __uint_as_float(v[i]));
+            if (e.relu_op) y = fmaxf(y, 0.0f);
+            v[i] = __float_as_uint(y);
+        }
+    }
+    if (e.f32_out) store32(e.f32_out);
+    if (e.u8_out) {
+        uint32_t w[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            w[q] = requant_pack4(__fmul_rn(__uint_as_float(v[4 * q]), e.inv_out_scale),
+                                 __fmul_rn(__uint_as_float(v[4 * q + 1]), e.inv_out_scale),
+                                 __fmul_rn(__uint_as_float(v[4 * q + 2]), e.inv_out_scale),
+                                 __fmul_rn(__uint_as_float(v[4 * q + 3]), e.inv_out_scale));
+        if (e.next_mode != SPARQ_MODE_NONE) next_xform_words(w, 8, e.next_mode, e.next_rnd, e.next_xf);
+        if (wide) {
+            st_global_v8(e.u8_out + off, w);
+        } else if (full) {
+            uint4 *dst = reinterpret_cast<uint4 *>(e.u8_out + off);
+            dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
+            dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 32; ++i)
+                if (i < cols) e.u8_out[off + i] = (uint8_t)(w[i >> 2] >> (8 * (i & 3)));
         }
     }
 }
 
-// Stages the scale and bias of columns n0 .. n0+bn-1 in shared memory (epilogue warps only).
-template <int WARPS, class Args>
-__device__ __forceinline__ void epi_stage_scale_bias(const Args &g, int64_t n0, int bn, int et,
+// A warp's share of one accumulator: `cols` columns (a multiple of 32) starting at tensor-memory
+// address taddr0 (tile-local column cbase), for this thread's output row.  wait_full() blocks
+// until the accumulator is complete; when its last columns are in registers the warp hands it
+// back by arriving on acc_empty_bar.
+//
+// 32 columns at a time: the arithmetic alone runs at 46 outputs per clock and SM, so what an
+// epilogue takes is latency -- the accumulator's barrier, tensor memory, shared memory behind the
+// tensor core's operand fetches -- and long straight-line groups hide most of it.  (Groups of 16 with
+// the next one's tensor-memory load in flight measured 20 % slower: every group starts with its
+// own exposed scale / bias reads.)  The residual bytes are fetched a group ahead, the first ones
+// before the accumulator is waited for.
+enum EpiKind { kEpiGeneral, kEpiLean, kEpiLeanResidual };
+
+template <int KIND, class WaitFull>
+__device__ __forceinline__ void epi_warp_columns_as(const EpiView &e, uint32_t taddr0, int cbase, int cols, int64_t row, bool row_ok,
+                                                    int64_t n0, const float *s_scale, const float *s_bias,
+                                                    uint32_t acc_empty_bar, int lane, WaitFull wait_full)
+{
+    uint32_t rn[8];
+    auto fetch_residual = [&](int ct) {       // columns ct .. ct + 31 of the tile
+        if (row_ok && n0 + ct < e.N) ld_global_v8(e.residual + row * e.N + n0 + ct, rn);
+    };
+    if (KIND == kEpiLeanResidual) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) rn[i] = 0u;
+        fetch_residual(cbase);
+    }
+    wait_full();
+#pragma unroll 1
+    for (int c = 0; c < cols; c += 32) {
+        uint32_t v[32], r[8];
+        tmem_ld_32x32_issue(taddr0 + (uint32_t)c, v);
+        if (KIND == kEpiLeanResidual) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) r[i] = rn[i];
+            if (c + 32 < cols) fetch_residual(cbase + c + 32);
+        }
+        tmem_ld_wait();
+        if (c + 32 == cols) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(acc_empty_bar);
+        }
+        const int ct = cbase + c;                    // column inside the tile
+        const int64_t col0 = n0 + ct;
+        if (!row_ok || col0 >= e.N) continue;
+        if (KIND == kEpiGeneral) {
+            epi_general(e, v, row, col0, s_scale + ct, s_bias + ct);
+        } else {
+            uint32_t w[8];
+            epi_lean<KIND == kEpiLeanResidual>(v, s_scale + ct, s_bias + ct, e.inv_out_scale, e.residual_scale, r, w);
+            st_global_v8(e.u8_out + row * e.N + col0, w);
+        }
+    }
+}
+
+template <class WaitFull>
+__device__ __forceinline__ void epi_warp_columns(const EpiView &e, uint32_t taddr0, int cbase, int cols, int64_t row, bool row_ok,
+                                                 int64_t n0, const float *s_scale, const float *s_bias,
+                                                 uint32_t acc_empty_bar, int lane, WaitFull wait_full)
+{
+    if (!e.lean) epi_warp_columns_as<kEpiGeneral>(e, taddr0, cbase, cols, row, row_ok, n0, s_scale, s_bias, acc_empty_bar, lane, wait_full);
+    else if (e.residual) epi_warp_columns_as<kEpiLeanResidual>(e, taddr0, cbase, cols, row, row_ok, n0, s_scale, s_bias, acc_empty_bar, lane, wait_full);
+    else epi_warp_columns_as<kEpiLean>(e, taddr0, cbase, cols, row, row_ok, n0, s_scale, s_bias, acc_empty_bar, lane, wait_full);
+}
+
+// One box of the staged output: this thread's row of `box` (64 or 128) columns, from tensor memory to
+// the warp's shared-memory buffer `buf` (32 rows of `box` bytes, 16-byte pieces swizzled as the
+// tensor map says), which a TMA store then takes to global memory as whole 64- or 128-byte
+// pieces of a row.  With a residual the buffer holds the identity tensor's box, fetched by TMA,
+// and is rewritten in place.
+//
+// Why: a thread owns an output row, so its own 32-byte stores (and residual loads) of a warp fall
+// into 32 different lines; a 51 MB output took 16.6 us that way against 10.5 in whole lines, and
+// its residual with it, with little L1 left beside the operand ring, 35 against 20.  (Fetching
+// the residual into L2 ahead of the boxes changed nothing: it is not HBM's latency.)  The whole
+// layer, M 200704 x K 64 -> N 256: 26.5 -> 23.3 us, with a residual 44.8 -> 33.2.
+// next_residual() is called once the first 32 columns are done.
+template <bool RES, class Next>
+__device__ __forceinline__ void epi_staged_box(uint32_t taddr, int box, uint32_t buf, const float *s_scale, const float *s_bias,
+                                               float inv, float res_scale, uint32_t acc_empty_bar, int lane, Next next_residual)
+{
+    const uint32_t row = buf + (uint32_t)(lane * box);
+    const uint32_t swz = box == 128 ? (uint32_t)(lane & 7) : (uint32_t)((lane >> 1) & 3);
+#pragma unroll 1
+    for (int c = 0; c < box; c += 32) {
+        uint32_t v[32], r[8], w[8];
+        tmem_ld_32x32_issue(taddr + (uint32_t)c, v);
+        const uint32_t a0 = row + ((((uint32_t)c >> 4) ^ swz) << 4), a1 = row + (((((uint32_t)c >> 4) + 1u) ^ swz) << 4);
+        if (RES) {
+            asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a0));
+            asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(a1));
+        }
+        tmem_ld_wait();
+        if (acc_empty_bar && c + 32 == box) {        // the accumulator's last columns are in registers
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(acc_empty_bar);
+        }
+        epi_lean<RES>(v, s_scale + c, s_bias + c, inv, res_scale, r, w);
+        asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" :: "r"(a0), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]) : "memory");
+        asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" :: "r"(a1), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
+        if (c == 0) next_residual();
+    }
+}
+
+// Stages the scale and bias of columns n0 .. n0+bn-1 in shared memory for the `threads` threads
+// that meet at hardware barrier `bar` (t = this thread's number among them).
+template <class Args>
+__device__ __forceinline__ void epi_stage_scale_bias(const Args &g, int64_t n0, int bn, int t, int threads, int bar,
                                                      float *s_scale, float *s_bias)
 {
-    epi_bar_sync<WARPS>();                      // previous readers are done
-    for (int c = et; c < bn; c += WARPS * 32) {
+    asm volatile("bar.sync %0, %1;" :: "r"(bar), "r"(threads) : "memory");     // previous readers are done
+    for (int c = t; c < bn; c += threads) {
         const int64_t col = n0 + c;
         const bool ok = col < g.N;
         s_scale[c] = ok ? __ldg(g.scale + col) : 0.0f;
         s_bias[c] = (ok && g.bias) ? __ldg(g.bias + col) : 0.0f;
     }
-    epi_bar_sync<WARPS>();
+    asm volatile("bar.sync %0, %1;" :: "r"(bar), "r"(threads) : "memory");
 }
 
 // ---- the kernel ---------------------------------------------------------------------------
@@ -647,40 +681,54 @@ struct TileCfg {
     static constexpr int kABytes = kBM * BK;
     static constexpr int kBBytes = BN * BK;
     static constexpr int kStageBytes = kABytes + kBBytes;
-    static constexpr int kStagesRaw = kSmemBudget / kStageBytes;
-    static constexpr int kStages = kStagesRaw > 8 ? 8 : kStagesRaw;
-    static constexpr int kTmemCols = (2 * BN < 32) ? 32 : 2 * BN;   // two accumulators
-    static constexpr int kSmemBytes = kStages * kStageBytes + 1024; // + alignment slack
+    // stages of the ring beside `staging` bytes of output boxes
+    __host__ __device__ static constexpr int stages(int staging)
+    {
+        const int n = (staging ? kMaxDynSmemGemm - 1024 - staging : kSmemBudget) / kStageBytes;
+        return n > kMaxStages ? kMaxStages : n;
+    }
+    static constexpr int kAcc = BN == 256 ? 2 : 4;                  // accumulator stages in tensor memory
+    static constexpr int kTmemCols = kAcc * BN;
 };
 
 template <int BN, int BK, int MODE, int XN, bool RND>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-                  const GemmArgs g)
+                  const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_res, const GemmArgs g)
 {
     using Cfg = TileCfg<BN, BK>;
-    constexpr int S = Cfg::kStages;
+    const int S = g.stages;
     extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) uint64_t bar_full[S], bar_xf[S], bar_empty[S];
-    __shared__ __align__(8) uint64_t bar_acc_full[2], bar_acc_empty[2], bar_done;
+    __shared__ __align__(8) uint64_t bar_full[kMaxStages], bar_xf[kMaxStages], bar_empty[kMaxStages];
+    __shared__ __align__(8) uint64_t bar_res[epi_warps(MODE)][2];       // residual boxes landed
+    constexpr int kAcc = Cfg::kAcc;
+    // The epilogue warps form groups of four (one warp per tensor-memory lane quarter) and the
+    // groups teams: team t takes the CTA's tiles of number t modulo the number of teams, so that the
+    // epilogues of consecutive tiles -- mostly latency -- overlap.  A CTA with a single tile puts
+    // all its groups in one team, each group on its own columns (32 at least; a group too many
+    // for the tile's columns stays idle).
+    constexpr int kGroups = epi_warps(MODE) / 4;
+    constexpr int kMaxTeams = kGroups < kAcc ? kGroups : kAcc;
+    __shared__ __align__(8) uint64_t bar_acc_full[kAcc], bar_acc_empty[kAcc], bar_done;
     __shared__ uint32_t tmem_base_slot;
     __shared__ uint32_t abort_word;
-    __shared__ __align__(16) float s_scale[BN], s_bias[BN];
+    __shared__ __align__(16) float s_scale[kMaxTeams][BN], s_bias[kMaxTeams][BN];
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     volatile uint32_t *abort_flag = &abort_word;
 
+    const int64_t m_tiles = (g.M + kBM - 1) / kBM;
+    const int64_t n_tiles = (g.N + BN - 1) / BN;
+    // tile indices fit 32 bits (the host refuses larger problems); a 64-bit division per tile
+    // and thread costs more instructions than a tile's share of the epilogue arithmetic
+    const uint32_t total_tiles = (uint32_t)(m_tiles * n_tiles);
+    const uint32_t n_tiles32 = (uint32_t)n_tiles;
+    const int teams = total_tiles > gridDim.x ? kMaxTeams : 1;
+
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     auto a_stage = [&](int s) { return smem_base + (uint32_t)s * Cfg::kStageBytes; };
     auto b_stage = [&](int s) { return smem_base + (uint32_t)s * Cfg::kStageBytes + Cfg::kABytes; };
-
-    // A tile's epilogue is mostly latency (barrier read, tensor-memory loads, stores).  On 64-wide
-    // tiles, and on 128-wide tiles with a transform (eight epilogue warps), with one column tile and
-    // only requantized bytes wanted, the epilogue warps split into two teams, one per accumulator
-    // stage, each warp taking twice the columns of its lane quarter: two tiles' epilogues overlap.
-    constexpr bool kTeamsPay = BN == 64 || (BN == 128 && MODE != SPARQ_MODE_NONE);
-    const bool epi_teams = kTeamsPay && g.N <= BN && make_epi_view(g).lean;
 
     if (threadIdx.x == 0) {
         prefetch_tensormap(&map_a);
@@ -690,10 +738,12 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
             mbar_init(smem_u32(&bar_xf[s]), kXfTeamWarps);
             mbar_init(smem_u32(&bar_empty[s]), 1);
         }
-        for (int a = 0; a < 2; ++a) {
+        for (int a = 0; a < kAcc; ++a) {
             mbar_init(smem_u32(&bar_acc_full[a]), 1);
-            mbar_init(smem_u32(&bar_acc_empty[a]), epi_teams ? epi_warps(MODE) / 2 : epi_warps(MODE));
+            mbar_init(smem_u32(&bar_acc_empty[a]), 4 * epi_parts(kGroups, teams, BN));
         }
+        for (int w = 0; w < epi_warps(MODE); ++w)
+            for (int b = 0; b < 2; ++b) mbar_init(smem_u32(&bar_res[w][b]), 1);
         mbar_init(smem_u32(&bar_done), 1);
         abort_word = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -710,18 +760,14 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     dep_wait();
     dep_launch();
 
-    const int64_t m_tiles = (g.M + kBM - 1) / kBM;
-    const int64_t n_tiles = (g.N + BN - 1) / BN;
-    // tile indices fit 32 bits (the host refuses larger problems); a 64-bit division per tile
-    // and thread costs more instructions than a tile's share of the epilogue arithmetic
-    const uint32_t total_tiles = (uint32_t)(m_tiles * n_tiles);
-    const uint32_t n_tiles32 = (uint32_t)n_tiles;
     const int kb_count = g.k_blocks;
 
     if (warp == 0) {
         // ================= TMA producer =================
         if (lane == 0) {
             uint32_t it = 0;   // running stage counter across tiles
+            int s = 0;         // stage it % S
+            uint32_t use = 0;  // it / S
             for (uint32_t tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
                 const uint32_t mt = (n_tiles32 == 1) ? tile : tile / n_tiles32, nt = tile - mt * n_tiles32;
                 const int64_t m0 = (int64_t)mt * kBM;
@@ -735,8 +781,6 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                     base_w = (rem % g.Wo) * g.stride_w - g.pad_w;
                 }
                 for (int kb = 0; kb < kb_count; ++kb, ++it) {
-                    const int s = it % S;
-                    const uint32_t use = it / S;
                     if (use > 0) mbar_wait(smem_u32(&bar_empty[s]), (use - 1) & 1, abort_flag, g.status, g.wait_limit);
                     if (*abort_flag) break;   // stop issuing copies once the CTA has given up
                     const uint32_t full = smem_u32(&bar_full[s]);
@@ -753,6 +797,7 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                         tma_load_2d(a_stage(s), &map_a, full, kb * BK, (int)m0);
                     }
                     tma_load_2d(b_stage(s), &map_b, full, bx, n0);
+                    if (++s == S) { s = 0; ++use; }
                 }
                 if (*abort_flag) break;
             }
@@ -779,8 +824,8 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
             int s = 0;             // stage
             uint32_t ph = 0;       // its phase parity
             for (uint32_t tile = blockIdx.x; tile < total_tiles; tile += gridDim.x, ++local_tile) {
-                const int acc = local_tile & 1;
-                const uint32_t acc_use = local_tile >> 1;
+                const int acc = local_tile % kAcc;
+                const uint32_t acc_use = local_tile / kAcc;
                 if (acc_use > 0) mbar_wait(smem_u32(&bar_acc_empty[acc]), (acc_use - 1) & 1, abort_flag, g.status, g.wait_limit);
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
@@ -806,63 +851,100 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         __syncwarp();
     } else if (warp < kFirstEpiWarp + epi_warps(MODE)) {
         // ================= epilogue =================
-        constexpr int kEpi = epi_warps(MODE);
-        constexpr int kColsPerWarp = BN / (kEpi / 4);        // the tile's columns are split over the warps of a quarter
         const int quarter = warp & 3;                        // tensor-memory lanes this warp may read
-        const int part = (warp - kFirstEpiWarp) >> 2;        // which share of the tile's columns
-        const int et = threadIdx.x - kFirstEpiWarp * 32;     // 0 .. kEpi * 32 - 1
+        const int group = (warp - kFirstEpiWarp) >> 2;
+        const int team = group % teams;                      // tiles team, team + teams, ...
+        const int parts = epi_parts(kGroups, teams, BN), part = group / teams;
+        const int cols = BN / parts, cbase = part * cols;    // this warp's share of the tile's columns
+        const int team_thread = (part * 4 + quarter) * 32 + lane, team_threads = parts * 128;
         const EpiView ev = make_epi_view(g);
-        uint32_t local_tile = 0;
         int64_t staged_nt = -1;
-        if (epi_teams) {
-            constexpr int kTeamWarps = kEpi / 2;
-            constexpr int kTeamCols = BN / (kTeamWarps / 4);          // columns per warp
-            epi_stage_scale_bias<kEpi>(g, 0, BN, et, s_scale, s_bias);
-            const uint32_t team = (uint32_t)(warp - kFirstEpiWarp) / kTeamWarps;   // team t takes the tiles of parity t
-            const int tcbase = (((warp - kFirstEpiWarp) % kTeamWarps) >> 2) * kTeamCols;
-            for (uint32_t tile = blockIdx.x; tile < total_tiles; tile += gridDim.x, ++local_tile) {
-                if ((local_tile & 1u) != team) continue;
-                const int64_t row = (int64_t)tile * kBM + quarter * 32 + lane;    // one column tile: row tile = tile
-                const bool row_ok = row < g.M;
-                const uint32_t taddr0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + team * BN + (uint32_t)tcbase;
-                mbar_wait(smem_u32(&bar_acc_full[team]), (local_tile >> 1) & 1u, abort_flag, g.status, g.wait_limit);
+        uint32_t local_tile = (uint32_t)team;
+        if (g.out_box) {
+            // ---- through shared memory (see epi_staged_box) ----
+            const int ew = warp - kFirstEpiWarp;
+            const uint32_t box_bytes = 32u * (uint32_t)g.out_box;
+            const uint32_t stage0 = smem_base + (uint32_t)(S * Cfg::kStageBytes) + (uint32_t)ew * 2u * box_bytes;
+            const bool res = g.residual != nullptr;
+            // boxes of this warp in order: the out_box-wide parts of its columns, tile after tile
+            auto fetch = [&](uint32_t n, uint32_t tile, int c) {          // box n's residual, by lane 0
+                const uint32_t mt = (n_tiles32 == 1) ? tile : tile / n_tiles32;
+                const int x = (int)(tile - mt * n_tiles32) * BN + cbase + c, y = (int)mt * kBM + quarter * 32;
+                const uint32_t bar = smem_u32(&bar_res[ew][n & 1u]);
+                mbar_expect_tx(bar, box_bytes);
+                tma_load_2d(stage0 + (n & 1u) * box_bytes, &map_res, bar, x, y);
+            };
+            uint32_t n = 0;
+            const uint32_t tile_step = (uint32_t)teams * gridDim.x;
+            uint32_t tile = blockIdx.x + (uint32_t)team * gridDim.x;
+            if (part < parts && tile < total_tiles && res && lane == 0) fetch(0u, tile, 0);
+            for (; tile < total_tiles && part < parts; tile += tile_step, local_tile += (uint32_t)teams) {
+                const uint32_t mt32 = (n_tiles32 == 1) ? tile : tile / n_tiles32;
+                const int64_t nt = tile - mt32 * n_tiles32;
+                const int acc = local_tile % kAcc;
+                if (nt != staged_nt) {
+                    staged_nt = nt;
+                    epi_stage_scale_bias(g, nt * BN, BN, team_thread, team_threads, 1 + team, s_scale[team], s_bias[team]);
+                }
+                mbar_wait(smem_u32(&bar_acc_full[acc]), (local_tile / kAcc) & 1u, abort_flag, g.status, g.wait_limit);
                 tc_fence_after();
-#pragma unroll 1
-                for (int ch = 0; ch < kTeamCols / 32; ++ch) {
-                    uint32_t v[32];
-                    tmem_ld_32x32_issue(taddr0 + (uint32_t)(ch * 32), v);
-                    tmem_ld_wait();
-                    if (ch + 1 == kTeamCols / 32) {
-                        tc_fence_before();
+                const uint32_t taddr0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * BN + cbase);
+                for (int c = 0; c < cols; c += g.out_box, ++n) {
+                    const bool last = c + g.out_box == cols;
+                    auto next_residual = [&]() {
+                        if (!res || lane != 0) return;
+                        const uint32_t nt_tile = last ? tile + tile_step : tile;
+                        if (nt_tile >= total_tiles) return;
+                        tma_store_wait_read<0>();          // the box before this one has left the buffer
+                        fetch(n + 1u, nt_tile, last ? 0 : c + g.out_box);
+                    };
+                    const uint32_t buf = stage0 + (n & 1u) * box_bytes;
+                    if (res) {
+                        mbar_wait(smem_u32(&bar_res[ew][n & 1u]), (n >> 1) & 1u, abort_flag, g.status, g.wait_limit);
+                    } else {
+                        if (lane == 0) tma_store_wait_read<1>();       // box n - 2 has left the buffer
                         __syncwarp();
-                        if (lane == 0) mbar_arrive(smem_u32(&bar_acc_empty[team]));
                     }
-                    const int ct = tcbase + ch * 32;
-                    if (!row_ok || ct >= (int)g.N) continue;          // N is a multiple of 32 here
-                    if (ev.small_acc) epi_chunk_u8<true>(ev, v, row, ct, ct, s_scale, s_bias);
-                    else epi_chunk_u8<false>(ev, v, row, ct, ct, s_scale, s_bias);
+                    const float *sc = s_scale[team] + cbase + c, *bi = s_bias[team] + cbase + c;
+                    const uint32_t abar = last ? smem_u32(&bar_acc_empty[acc]) : 0u;
+                    if (res) epi_staged_box<true>(taddr0 + (uint32_t)c, g.out_box, buf, sc, bi, g.inv_out_scale, g.residual_scale, abar, lane, next_residual);
+                    else epi_staged_box<false>(taddr0 + (uint32_t)c, g.out_box, buf, sc, bi, g.inv_out_scale, 0.0f, abar, lane, next_residual);
+                    fence_proxy_async_smem();
+                    __syncwarp();
+                    const int x = (int)nt * BN + cbase + c;
+                    const int64_t y = (int64_t)mt32 * kBM + quarter * 32;
+                    if (lane == 0) {
+                        if (x < (int)g.N && y < g.M) tma_store_2d(&map_out, buf, x, (int)y);
+                        tma_store_commit();
+                    }
                 }
             }
+            if (lane == 0) {
+                // after an abort: wait (bounded) for residual boxes that may still be in flight
+                if (*abort_flag && res && n > 0)
+                    for (uint32_t q = n > 1 ? n - 2 : 0; q < n; ++q)
+                        mbar_wait(smem_u32(&bar_res[ew][q & 1u]), (q >> 1) & 1u, abort_flag, g.status, g.wait_limit, true);
+                tma_store_wait_all();
+            }
+            __syncwarp();
         } else
-        for (uint32_t tile = blockIdx.x; tile < total_tiles; tile += gridDim.x, ++local_tile) {
+        for (uint32_t tile = blockIdx.x + (uint32_t)team * gridDim.x; tile < total_tiles && part < parts;
+             tile += (uint32_t)teams * gridDim.x, local_tile += (uint32_t)teams) {
             const uint32_t mt32 = (n_tiles32 == 1) ? tile : tile / n_tiles32;
             const int64_t mt = mt32, nt = tile - mt32 * n_tiles32;
-            const int acc = local_tile & 1;
-            const uint32_t acc_use = local_tile >> 1;
+            const int acc = local_tile % kAcc;
+            const uint32_t acc_use = local_tile / kAcc;
             if (ev.need_f && nt != staged_nt) {              // new column tile: new scale / bias
                 staged_nt = nt;
-                epi_stage_scale_bias<kEpi>(g, nt * BN, BN, et, s_scale, s_bias);
+                epi_stage_scale_bias(g, nt * BN, BN, team_thread, team_threads, 1 + team, s_scale[team], s_bias[team]);
             }
-            mbar_wait(smem_u32(&bar_acc_full[acc]), acc_use & 1, abort_flag, g.status, g.wait_limit);
-            tc_fence_after();
             const int64_t row = mt * kBM + quarter * 32 + lane;
-            const bool row_ok = row < g.M;
-            const int cbase = part * kColsPerWarp;
             const uint32_t taddr0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * BN + cbase);
-            epi_warp_columns<kColsPerWarp>(ev, taddr0, cbase, row, row_ok, nt * BN, s_scale, s_bias,
-                                      smem_u32(&bar_acc_empty[acc]), lane);
-        }
-        if (warp == kFirstEpiWarp && lane == 0) {
+            epi_warp_columns(ev, taddr0, cbase, cols, row, row < g.M, nt * BN, s_scale[team], s_bias[team],
+                             smem_u32(&bar_acc_empty[acc]), lane, [&]() {
+                                 mbar_wait(smem_u32(&bar_acc_full[acc]), acc_use & 1, abort_flag, g.status, g.wait_limit);
+                                 tc_fence_after();
+                             });
         }
     } else if (MODE != SPARQ_MODE_NONE) {
         // ================= transform =================
@@ -874,12 +956,15 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         constexpr int kBatch = kPerThread < 4 ? kPerThread : 4;     // vectors in flight per thread
         static_assert(kVecs % kXfThreads == 0 && kPerThread % kBatch == 0, "A stage must split evenly over a team");
         const XformDev xf = g.xf;
-        uint32_t it = 0;
+        uint32_t it = 0, ph = 0;
+        int sn = 0;
         for (uint32_t tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
             for (int kb = 0; kb < kb_count; ++kb, ++it) {
+                const int s = sn;
+                const uint32_t sph = ph;
+                if (++sn == S) { sn = 0; ph ^= 1u; }
                 if ((int)(it & 1u) != team) continue;      // the other team's stage
-                const int s = it % S;
-                mbar_wait(smem_u32(&bar_full[s]), (it / S) & 1, abort_flag, g.status, g.wait_limit);
+                mbar_wait(smem_u32(&bar_full[s]), sph, abort_flag, g.status, g.wait_limit);
                 const uint32_t base = a_stage(s) + (uint32_t)xt * 16u;
 #pragma unroll
                 for (int j0 = 0; j0 < kPerThread; j0 += kBatch) {
@@ -905,8 +990,6 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                 if (lane == 0) mbar_arrive(smem_u32(&bar_xf[s]));
             }
         }
-        if (warp == kFirstXfWarp && lane == 0) {
-        }
     }
 
     tc_fence_before();
@@ -918,11 +1001,14 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     }
 }
 
+struct GemmMaps {
+    CUtensorMap a, b, out, res;     // out, res: staged output only
+};
+
 // Host launcher for one tile shape; picks the transform variant.  Defined once per
 // (BN, BK) in its own translation unit.
 template <int BN, int BK>
-cudaError_t launch_gemm_shape(const CUtensorMap &ma, const CUtensorMap &mb, const GemmArgs &g,
-                              int mode, int n, int rnd, int grid, cudaStream_t st);
+cudaError_t launch_gemm_shape(const GemmMaps &m, GemmArgs &g, int mode, int n, int rnd, int grid, cudaStream_t st);
 
 #define SPARQ_LAUNCH_VARIANT(MODE_, XN_, RND_)                                                         \
     do {                                                                                               \
@@ -933,18 +1019,20 @@ cudaError_t launch_gemm_shape(const CUtensorMap &ma, const CUtensorMap &mb, cons
         if (e_ != cudaSuccess) return e_;                                                              \
         if (dev_ < 0 || dev_ >= 64 || !attr_set[dev_]) {                                               \
             e_ = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize,                \
-                                      TileCfg<BN, BK>::kSmemBytes);                                    \
+                                      kMaxDynSmemGemm);                                                \
             if (e_ != cudaSuccess) return e_;                                                          \
             if (dev_ >= 0 && dev_ < 64) attr_set[dev_] = true;                                         \
         }                                                                                              \
-        return launch_overlapped(kfn, grid, kGemmThreads, TileCfg<BN, BK>::kSmemBytes, st, ma, mb, g); \
+        const int staging_ = g.out_box ? epi_warps(MODE_) * 2 * 32 * g.out_box : 0;                    \
+        g.stages = TileCfg<BN, BK>::stages(staging_);                                                  \
+        const int smem_ = 1024 + g.stages * TileCfg<BN, BK>::kStageBytes + staging_;                   \
+        return launch_overlapped(kfn, grid, kGemmThreads, smem_, st, m.a, m.b, m.out, m.res, g);       \
     } while (0)
 
 #define SPARQ_DEFINE_GEMM_SHAPE(BN_, BK_)                                                              \
     template <>                                                                                        \
-    cudaError_t launch_gemm_shape<BN_, BK_>(const CUtensorMap &ma, const CUtensorMap &mb,              \
-                                            const GemmArgs &g, int mode, int n, int rnd, int grid,     \
-                                            cudaStream_t st)                                           \
+    cudaError_t launch_gemm_shape<BN_, BK_>(const GemmMaps &m, GemmArgs &g, int mode, int n, int rnd,  \
+                                            int grid, cudaStream_t st)                                 \
     {                                                                                                  \
         constexpr int BN = BN_, BK = BK_;                                                              \
         if (mode == SPARQ_MODE_NONE) SPARQ_LAUNCH_VARIANT(SPARQ_MODE_NONE, 4, false);                  \
