@@ -27,6 +27,10 @@
  *     fetches weights early only when they are clear of them, so a layer whose weights the
  *     previous layer has just written still sees the finished values; kernels of other
  *     libraries never release their successor early.  Nothing for the caller to do.
+ *   - Where a fused call would transform the same activations many times (several column tiles,
+ *     several filter taps), it runs as transform + plain contraction with the transformed
+ *     activations in stream-ordered scratch memory from a pool of the library's own; without
+ *     memory to be had it runs fused.  Same results.
  *   - The library is thread-compatible: concurrent calls are allowed, the error string
  *     is per host thread.
  */
@@ -367,7 +371,7 @@ SPARQ_API int sparq_selftest_mma_rate(int bn, int iters, int64_t *cycles_out, vo
 SPARQ_API const char *sparq_last_error(void);
 
 /* Releases what the library itself holds on the current device (the status word, the
- * host-buffer forms' staging buffers) and forgets the cached tensor-map encodings.  Safe to call more than once; later calls re-create what they need. */
+ * scratch pool, the host-buffer forms' staging buffers) and forgets the cached tensor-map encodings.  Safe to call more than once; later calls re-create what they need. */
 SPARQ_API int sparq_shutdown(void);
 
 #ifdef __cplusplus

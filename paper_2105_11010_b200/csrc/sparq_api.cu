@@ -97,6 +97,7 @@ int get_status_word(unsigned int **dptr)
 
 void release_gemm_state();     // sparq_gemm.cu
 void release_host_staging();   // sparq_host.cu
+void release_workspace();      // sparq_workspace.cu
 
 }  // namespace sparq
 
@@ -138,6 +139,7 @@ extern "C" int sparq_shutdown(void)
         cudaGetLastError();
         return SPARQ_OK;  // no device: nothing is held
     }
+    release_workspace();
     std::lock_guard<std::mutex> lk(g_mu);
     if (dev >= 0 && dev < kMaxDevices && g_status[dev]) {
         cudaFree(g_status[dev]);

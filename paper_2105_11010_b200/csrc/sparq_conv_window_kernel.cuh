@@ -38,10 +38,10 @@ struct WindowArgs {
     int64_t K;              // r * s * c
     // geometry
     int n_img, H, W, C, R, S, pad_h, pad_w, Ho, Wo;
-    int Wp;                 // W + 2 * pad_w
+    int Wp;                 // W + 2 * pad_w, rounded up to even where that costs no row (host)
     int TR;                 // output rows per tile
     int tiles_per_img;      // ceil(Ho / TR)
-    int c_blocks;           // C / CB
+    int c_blocks;           // ceil(C / CB); channels past C arrive as zeros, activations and weights alike
     int G;                  // most tiles that share one window (1 when there are several column tiles)
     int piece0_bytes;       // CB * Wp * (TR + R - 1): first piece of a group, one channel block
     int piece_bytes;        // CB * Wp * TR: every later piece
@@ -50,7 +50,6 @@ struct WindowArgs {
     int b_stages;           // weight stages (stream mode) or resident blocks (resident mode)
     int early_weights;      // resident weights may be fetched before the previous kernel on the stream has finished
     int issuers;            // 2: the two issuer warps alternate (resident weights); 1: warp 1 issues every tile (streamed weights)
-    int w_one_copy;         // resident weights: map_w is the 3-D (bytes, rows, blocks) view and one copy brings all blocks
     uint32_t n_tiles;       // column tiles
     uint32_t units;         // n_img * tiles_per_img * n_tiles, column tile fastest
     uint32_t groups;        // streamed weights on 128-wide tiles: n_img * n_tiles * ceil(tiles_per_img / G) whole
@@ -238,16 +237,12 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
     bool have = walk.next();       // the first group, too
     // All weight blocks, once per CTA, on stage barrier 0: every CTA reads the same bytes, so
     // they come out of L2 one reader after the other, and they are what the first tile waits
-    // for longest.  Block (tap, cb) = bytes [tap*C + cb*CB, +CB) of every filter lands in slot
-    // tap * c_blocks + cb.
+    // for longest.  map_w is the (channels, filters, taps) view; one copy brings a channel block of
+    // every tap, tap t of channel block cb into slot cb * taps + t.
     auto issue_resident_weights = [&]() {
         const uint32_t full = smem_u32(&bar_b_full[0]);
         mbar_expect_tx(full, (uint32_t)kb_count * kBBlock);
-        if (g.w_one_copy) {
-            tma_load_3d(b_slot(0), &map_w, full, 0, 0, 0);
-        } else {
-            for (int kb = 0; kb < kb_count; ++kb) tma_load_2d(b_slot(kb), &map_w, full, kb * CB, 0);
-        }
+        for (int cb = 0; cb < g.c_blocks; ++cb) tma_load_3d(b_slot(cb * taps), &map_w, full, cb * CB, 0, 0);
     };
     // The weights are not an output of the kernel that runs before this one (the host checks
     // that and sets early_weights), so their copy may start before that kernel has finished:
@@ -305,7 +300,7 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
                                 if (*abort_flag) { stop = true; break; }
                                 const uint32_t full = smem_u32(&bar_b_full[s]);
                                 mbar_expect_tx(full, kBBlock);
-                                tma_load_2d(b_slot(s), &map_w, full, tap * g.C + cb * CB, (int)(walk.nt * BN));
+                                tma_load_3d(b_slot(s), &map_w, full, cb * CB, (int)(walk.nt * BN), tap);
                             }
                         }
                     }
@@ -473,16 +468,17 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
                             if (++s == g.b_stages) { s = 0; bph ^= 1u; }
                         }
                     };
-                    // channel block outer, tap inner; the resident slot of (tap, cb) is tap * c_blocks + cb
+                    // channel block outer, tap inner: the order of the resident slots
                     uint64_t a_cb = a_desc0;
                     const uint32_t cbs = (uint32_t)g.c_blocks;
+                    uint32_t slot = 0;
                     if (g.R == 3 && g.S == 3) {
-                        for (uint32_t cb = 0; cb < cbs; ++cb, a_cb += plane16) {
+                        for (uint32_t cb = 0; cb < cbs; ++cb, a_cb += plane16, slot += 9u) {
 #pragma unroll
                             for (int r = 0; r < 3; ++r) {
 #pragma unroll
                                 for (int sx = 0; sx < 3; ++sx)
-                                    issue_block(cb == 0 && r == 0 && sx == 0, (uint32_t)(r * 3 + sx) * cbs + cb,
+                                    issue_block(cb == 0 && r == 0 && sx == 0, slot + (uint32_t)(r * 3 + sx),
                                                 a_cb + (uint64_t)((uint32_t)r * row16 + (uint32_t)(sx * (CB >> 4))));
                                 if (r == 0 && cb == 0) look();
                             }
@@ -490,9 +486,8 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
                     } else {
                         for (uint32_t cb = 0; cb < cbs; ++cb, a_cb += plane16) {
                             uint64_t a_r = a_cb;
-                            uint32_t slot = cb;
                             for (int r = 0; r < g.R; ++r, a_r += row16) {
-                                for (int sx = 0; sx < g.S; ++sx, slot += cbs)
+                                for (int sx = 0; sx < g.S; ++sx, ++slot)
                                     issue_block(cb == 0 && r == 0 && sx == 0, slot, a_r + (uint64_t)(uint32_t)(sx * (CB >> 4)));
                                 if (r == 0 && cb == 0) look();
                             }

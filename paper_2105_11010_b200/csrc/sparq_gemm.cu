@@ -175,34 +175,56 @@ static int check_epilogue(const sparq_epilogue *e)
     return SPARQ_OK;
 }
 
-// Tile width for the 128 x BN kernel.  Per reduction step (128 bytes of K) a CTA needs about
-//   max( transform of the A stage  ~1250 cycles when a SPARQ mode is on,
-//        MMA                       2 * BN cycles,
-//        operand fetch from L2     ~4.4 cycles per 128-byte row of A and B )
-// and the kernel takes ceil(tiles / SMs) such passes; narrow tiles add CTAs but re-fetch
-// and re-transform A once per column tile.  Pick the width with the lowest estimate.
-static int pick_bn(int64_t M, int64_t N, int sms, bool transform)
+// Cycles that one CTA spends on its reduction steps (128 bytes of K each) with 128 x bn tiles, the
+// estimate that tile width and form are chosen by.  A step takes the longest of
+//   transform of the A stage   1250 cycles when a SPARQ mode is on,
+//   MMA                        2 * bn cycles,
+//   operand fetch from L2      2.1 cycles per 128-byte row of A and B, 3.5 through an im2col map
+// plus a hand-over, in ceil(tiles / SMs) passes; narrow tiles add CTAs but re-fetch and
+// re-transform A once per column tile.  (16384 x 4096 x 4096 at 128 x 256: 802 cycles a step
+// measured without a transform, 1473 with one; 7x7x512 -> 512 3x3: 917 and 1530.)
+static double tile_cycles(int64_t M, int64_t N, int64_t steps, int bn, int sms, bool transform, bool im2col)
+{
+    const int64_t tiles = ((M + kBM - 1) / kBM) * ((N + bn - 1) / bn);
+    const int64_t rounds = (tiles + sms - 1) / sms;
+    double step = 2.0 * bn;
+    const double fetch = (im2col ? 3.5 : 2.1) * (kBM + bn);
+    if (fetch > step) step = fetch;
+    if (transform && step < 1250.0) step = 1250.0;
+    return (double)rounds * (double)steps * (step + 150.0);
+}
+
+// The tile width with the lowest estimate.
+static int pick_bn(int64_t M, int64_t N, int64_t steps, int sms, bool transform, bool im2col, double *cycles = nullptr)
 {
     const int cand[3] = {256, 128, 64};
-    const int64_t m_tiles = (M + kBM - 1) / kBM;
     int best = 64;
     double best_cost = 0.0;
     for (int i = 0; i < 3; ++i) {
         const int bn = cand[i];
         if (bn > 64 && N <= bn / 2) continue;          // would be mostly padding
-        const int64_t tiles = m_tiles * ((N + bn - 1) / bn);
-        const int64_t rounds = (tiles + sms - 1) / sms;
-        double step = 2.0 * bn;
-        const double fetch = 4.4 * (kBM + bn);
-        if (fetch > step) step = fetch;
-        if (transform && step < 1250.0) step = 1250.0;
-        const double cost = (double)rounds * (step + 150.0);   // + fixed per-step hand-off cost
+        const double cost = tile_cycles(M, N, steps, bn, sms, transform, im2col);
         if (best_cost == 0.0 || cost < best_cost) {
             best_cost = cost;
             best = bn;
         }
     }
+    if (cycles) *cycles = best_cost;
     return best;
+}
+
+// Whether to write T(A) to scratch memory once and contract that, instead of transforming every
+// staged tile: worth it when A is staged several times -- several column tiles, several filter
+// taps -- because the in-kernel transform is what such a step takes.  The extra pass costs about
+// 2.5 us and 2 bytes of traffic per activation (2.9 TB/s of activations).  A margin of 7 % keeps the
+// fused form, which needs no memory, where the two are close.
+static bool transform_first(int64_t M, int64_t N, int64_t steps, size_t act_bytes, int sms, bool im2col)
+{
+    double fused, plain;
+    pick_bn(M, N, steps, sms, true, im2col, &fused);
+    pick_bn(M, N, steps, sms, false, im2col, &plain);
+    const double clk = 1900.0;      // cycles per us
+    return plain + clk * (2.5 + (double)act_bytes / 2.9e6) < 0.93 * fused;
 }
 
 // ---- what the previous launch on a stream wrote ----------------------------------------------------
@@ -323,6 +345,15 @@ static int output_maps(GemmMaps *m, GemmArgs *g, int mode, int bn, int64_t tiles
 int gemm_with_status(const uint8_t *A, int64_t lda, const int8_t *B, int64_t ldb, int64_t M, int64_t N, int64_t K,
                      const XformArgs &x, const sparq_epilogue *e, unsigned int *status, cudaStream_t st);
 
+// Parameters of a contraction whose activations are already transformed.
+static XformArgs plain_a8w8()
+{
+    XformArgs x = {};
+    x.mode = SPARQ_MODE_NONE;
+    x.n = 4;
+    return x;
+}
+
 // The fused GEMM with the library's own status word (allocated on first use).
 static int gemm_impl(const uint8_t *A, int64_t lda, const int8_t *B, int64_t ldb, int64_t M, int64_t N, int64_t K,
                      const XformArgs &x, const sparq_epilogue *e, cudaStream_t st)
@@ -330,6 +361,16 @@ static int gemm_impl(const uint8_t *A, int64_t lda, const int8_t *B, int64_t ldb
     unsigned int *status = nullptr;
     int rc = get_status_word(&status);
     if (rc != SPARQ_OK) return rc;
+    int sms = 0;
+    if (x.mode != SPARQ_MODE_NONE && lda == K && (rc = device_info(&sms)) == SPARQ_OK &&
+        transform_first(M, N, (K + 127) / 128, (size_t)M * (size_t)K, sms, false)) {
+        if (uint8_t *ta = (uint8_t *)workspace_alloc((size_t)M * (size_t)K, st)) {
+            rc = quantize_rows(A, ta, (size_t)M, (size_t)K, x, st);
+            if (rc == SPARQ_OK) rc = gemm_with_status(ta, K, B, ldb, M, N, K, plain_a8w8(), e, status, st);
+            workspace_free(ta, st);
+            return rc;
+        }
+    }
     return gemm_with_status(A, lda, B, ldb, M, N, K, x, e, status, st);
 }
 
@@ -356,24 +397,27 @@ static int encode_window(CUtensorMap *map, const void *ptr, int n, int h, int w,
     return SPARQ_OK;
 }
 
-// Weights [cout][K] seen as (cb bytes, cout rows, K / cb blocks): one box brings every
-// (tap, channel block) of bn filters into consecutive bn x cb shared-memory blocks.
-// Returns the driver's result; the caller falls back to one copy per block if it is refused.
-static CUresult encode_weight_blocks(CUtensorMap *map, const void *ptr, int64_t K, int cout, int cb, int bn, int blocks)
+// Weights [cout][taps][c] as (channels, filters, taps): a box brings cb channels of bn filters and
+// box_taps taps into consecutive bn x cb shared-memory blocks; channels past c arrive as zeros.
+static int encode_weights(CUtensorMap *map, const void *ptr, int c, int cout, int taps, int cb, int bn, int box_taps)
 {
     static EncodeTiledFn fn = nullptr;
-    if (!fn && driver_fn("cuTensorMapEncodeTiled", (void **)&fn) != SPARQ_OK) return CUDA_ERROR_NOT_FOUND;
-    const MapKey key = {{4, (uint64_t)(uintptr_t)ptr, (uint64_t)K, (uint64_t)cout, (uint64_t)cb, (uint64_t)bn, (uint64_t)blocks}};
-    if (map_lookup(key, map)) return CUDA_SUCCESS;
-    cuuint64_t dims[3] = {(cuuint64_t)cb, (cuuint64_t)cout, (cuuint64_t)blocks};
-    cuuint64_t strides[2] = {(cuuint64_t)K, (cuuint64_t)cb};
-    cuuint32_t box[3] = {(cuuint32_t)cb, (cuuint32_t)bn, (cuuint32_t)blocks};
+    if (!fn) {
+        int rc = driver_fn("cuTensorMapEncodeTiled", (void **)&fn);
+        if (rc != SPARQ_OK) return rc;
+    }
+    const MapKey key = {{4, (uint64_t)(uintptr_t)ptr, (uint64_t)c, (uint64_t)cout, (uint64_t)taps, (uint64_t)cb, (uint64_t)bn, (uint64_t)box_taps}};
+    if (map_lookup(key, map)) return SPARQ_OK;
+    cuuint64_t dims[3] = {(cuuint64_t)c, (cuuint64_t)cout, (cuuint64_t)taps};
+    cuuint64_t strides[2] = {(cuuint64_t)c * taps, (cuuint64_t)c};
+    cuuint32_t box[3] = {(cuuint32_t)cb, (cuuint32_t)bn, (cuuint32_t)box_taps};
     cuuint32_t estr[3] = {1, 1, 1};
     const CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, const_cast<void *>(ptr), dims, strides, box, estr,
                           CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_for(cb), CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r == CUDA_SUCCESS) map_store(key, *map);
-    return r;
+    if (r != CUDA_SUCCESS) return set_error(SPARQ_ERR_CUDA, "cuTensorMapEncodeTiled (weights) failed with CUresult %d", (int)r);
+    map_store(key, *map);
+    return SPARQ_OK;
 }
 
 constexpr int kMaxDynSmem = kWindowMaxDynSmem;
@@ -384,14 +428,18 @@ static int try_window_conv(const uint8_t *x_in, int n, int h, int w, int c, cons
                            int pad_h, int pad_w, int ho, int wo, const XformArgs &x, const sparq_epilogue *e,
                            int sms, unsigned int *status, cudaStream_t st)
 {
-    const int wp = w + 2 * pad_w;
+    int wp = w + 2 * pad_w;
     if (wp > 128 || wo < 1) return 0;
-    const int cb = (c % 128 == 0) ? 128 : (c == 64 ? 64 : 0);
-    if (!cb) return 0;
+    // channel blocks; the last one's tail is zero fill.  Few channels and many filters: 128-wide blocks
+    // that are half empty, because 64-channel blocks exist on 64-wide tiles only.
+    const int cb = (c <= 64 && cout <= 64) ? 64 : 128;
     int tr = 128 / wp;
     if (tr > ho) tr = ho;
     if (tr < 1 || tr * wo < 64) return 0;               // less than half of the MMA rows would be useful
-    const int c_blocks = c / cb;
+    // Pieces land at multiples of tr * wp rows, which must be a multiple of 128 bytes: an even row
+    // width makes it so for 64-byte rows.
+    if (cb == 64 && (wp & 1) && wp + 1 <= 128 && (128 / (wp + 1) >= tr)) ++wp;
+    const int c_blocks = (c + cb - 1) / cb;
     const int taps = r * s;
     const int kb_count = taps * c_blocks;
     const int tiles_per_img = (ho + tr - 1) / tr;
@@ -399,10 +447,8 @@ static int try_window_conv(const uint8_t *x_in, int n, int h, int w, int c, cons
 
     int bn;
     if (cb == 64) {
-        if (cout > 64) return 0;
         bn = 64;
     } else {
-        if (cout <= 64) return 0;
         bn = (cout > 128 && m_tiles * ((cout + 255) / 256) >= sms) ? 256 : 128;
     }
     const int b_block = bn * cb;
@@ -472,16 +518,11 @@ static int try_window_conv(const uint8_t *x_in, int n, int h, int w, int c, cons
     rc = encode_window(&mx1, x_in, n, h, w, c, cb, wp, tr);
     if (rc != SPARQ_OK) return rc;
     const int64_t K = (int64_t)r * s * c;
-    bool w_one_copy = resident && kb_count <= 256 &&
-                      encode_weight_blocks(&mw, wgt, K, cout, cb, bn, kb_count) == CUDA_SUCCESS;
-    if (!w_one_copy) {
-        rc = encode_2d(&mw, wgt, K, cout, K, cb, bn);
-        if (rc != SPARQ_OK) return rc;
-    }
+    rc = encode_weights(&mw, wgt, c, cout, taps, cb, bn, resident ? taps : 1);
+    if (rc != SPARQ_OK) return rc;
 
     WindowArgs g;
     memset(&g, 0, sizeof(g));
-    g.w_one_copy = w_one_copy ? 1 : 0;
     // Streamed weights pass through a ring that is shorter than one tile's blocks, in tile order:
     // two issuers on different tiles would wait on the same stage barriers several phases apart,
     // which a parity wait cannot tell apart.  One issuer then; two with resident weights.
@@ -535,7 +576,7 @@ int gemm_with_status(const uint8_t *A, int64_t lda, const int8_t *B, int64_t ldb
     // padding stays below an eighth (K = 576: five 128-byte steps instead of nine 64-byte ones: each
     // step is a hand-off between three warp roles, which is what a small launch is made of)
     const int bk = (pad64 < pad128 && !(pad64 >= 320 && pad128 * 8 <= pad64 * 9)) ? 64 : 128;
-    const int bn = pick_bn(M, N, sms, x.mode != SPARQ_MODE_NONE);
+    const int bn = pick_bn(M, N, (K + 127) / 128, sms, x.mode != SPARQ_MODE_NONE, false);
     GemmMaps m = {};
     rc = encode_2d(&m.a, A, K, M, lda, bk, kBM);
     if (rc != SPARQ_OK) return rc;
@@ -554,6 +595,44 @@ int gemm_with_status(const uint8_t *A, int64_t lda, const int8_t *B, int64_t ldb
     record_launch_weights_clear(st, e, (size_t)M * (size_t)N, B, (size_t)N * (size_t)ldb);
     cudaError_t ce = launch(bn, bk, m, g, x, grid, st);
     if (ce != cudaSuccess) return cuda_error(ce, "sparq_gemm_kernel launch");
+    return SPARQ_OK;
+}
+
+// The convolution through an im2col tensor map (strides, and whatever the window kernel does not tile).
+static int im2col_conv(const uint8_t *x_in, int n, int h, int w, int c, const int8_t *wgt, int cout, int r, int s,
+                       int stride_h, int stride_w, int pad_h, int pad_w, int ho, int wo, const XformArgs &x, const sparq_epilogue *e,
+                       int sms, unsigned int *status, cudaStream_t st)
+{
+    const int64_t M = (int64_t)n * ho * wo, K = (int64_t)r * s * c;
+    const int bk = (c % 128 == 0) ? 128 : 64;
+    const int bn = pick_bn(M, cout, (int64_t)r * s * ((c + 127) / 128), sms, x.mode != SPARQ_MODE_NONE, true);
+    int rc;
+    GemmMaps m = {};
+    rc = encode_im2col(&m.a, x_in, n, h, w, c, r, s, stride_h, stride_w, pad_h, pad_w, bk);
+    if (rc != SPARQ_OK) return rc;
+    rc = encode_2d(&m.b, wgt, K, cout, K, bk, bn);
+    if (rc != SPARQ_OK) return rc;
+    GemmArgs g;
+    memset(&g, 0, sizeof(g));
+    g.M = M; g.N = cout; g.K = K;
+    // A channel count that is not a multiple of 64 takes a last block that reaches past C: the
+    // im2col copy fills those channels with zeros.
+    g.c_blocks = (c + bk - 1) / bk;
+    g.k_blocks = r * s * g.c_blocks;
+    g.conv = 1;
+    g.tap_k = c;
+    g.S = s;
+    g.Ho = ho; g.Wo = wo;
+    g.stride_h = stride_h; g.stride_w = stride_w; g.pad_h = pad_h; g.pad_w = pad_w;
+    rc = fill_common(&g, x, e, status);
+    if (rc != SPARQ_OK) return rc;
+    const int64_t tiles = ((M + kBM - 1) / kBM) * ((cout + bn - 1) / bn);
+    if (tiles >= ((int64_t)1 << 31)) return set_error(SPARQ_ERR_UNSUPPORTED, "more than 2^31 output tiles");
+    const int grid = (int)(tiles < sms ? tiles : sms);
+    if ((rc = output_maps(&m, &g, x.mode, bn, tiles, grid)) != SPARQ_OK) return rc;
+    record_launch_weights_clear(st, e, (size_t)M * (size_t)cout, wgt, (size_t)cout * (size_t)K);
+    cudaError_t ce = launch(bn, bk, m, g, x, grid, st);
+    if (ce != cudaSuccess) return cuda_error(ce, "sparq_gemm_kernel (convolution) launch");
     return SPARQ_OK;
 }
 
@@ -624,34 +703,15 @@ extern "C" int sparq_conv2d_nhwc_s8(const uint8_t *x_in, int n, int h, int w, in
         rc = try_window_conv(x_in, n, h, w, c, wgt, cout, r, s, pad_h, pad_w, ho, wo, x, e, sms, status, st);
         if (rc != 0) return rc < 0 ? rc : SPARQ_OK;
     }
-    const int bk = (c % 128 == 0) ? 128 : 64;
-    const int bn = pick_bn(M, cout, sms, x.mode != SPARQ_MODE_NONE);
-    GemmMaps m = {};
-    rc = encode_im2col(&m.a, x_in, n, h, w, c, r, s, stride_h, stride_w, pad_h, pad_w, bk);
-    if (rc != SPARQ_OK) return rc;
-    rc = encode_2d(&m.b, wgt, K, cout, K, bk, bn);
-    if (rc != SPARQ_OK) return rc;
-    GemmArgs g;
-    memset(&g, 0, sizeof(g));
-    g.M = M; g.N = cout; g.K = K;
-    // A channel count that is not a multiple of 64 takes a last block that reaches past C: the
-    // im2col copy fills those channels with zeros.
-    g.c_blocks = (c + bk - 1) / bk;
-    g.k_blocks = r * s * g.c_blocks;
-    g.conv = 1;
-    g.tap_k = c;
-    g.S = s;
-    g.Ho = ho; g.Wo = wo;
-    g.stride_h = stride_h; g.stride_w = stride_w; g.pad_h = pad_h; g.pad_w = pad_w;
-    rc = fill_common(&g, x, e, status);
-    if (rc != SPARQ_OK) return rc;
-    const int64_t tiles = ((M + kBM - 1) / kBM) * ((cout + bn - 1) / bn);
-    if (tiles >= ((int64_t)1 << 31)) return set_error(SPARQ_ERR_UNSUPPORTED, "more than 2^31 output tiles");
-    const int grid = (int)(tiles < sms ? tiles : sms);
-    if ((rc = output_maps(&m, &g, x.mode, bn, tiles, grid)) != SPARQ_OK) return rc;
-    record_launch_weights_clear(st, e, (size_t)M * (size_t)cout, wgt, (size_t)cout * (size_t)K);
-    cudaError_t ce = launch(bn, bk, m, g, x, grid, st);
-    if (ce != cudaSuccess) return cuda_error(ce, "sparq_gemm_kernel (convolution) launch");
-    return SPARQ_OK;
+    const int64_t steps = (int64_t)r * s * ((c + 127) / 128);
+    const size_t act_bytes = (size_t)n * h * w * (size_t)c;
+    if (x.mode != SPARQ_MODE_NONE && transform_first(M, cout, steps, act_bytes, sms, true)) {
+        if (uint8_t *tx = (uint8_t *)workspace_alloc(act_bytes, st)) {
+            rc = quantize_rows(x_in, tx, (size_t)n * h * w, (size_t)c, x, st);
+            if (rc == SPARQ_OK) rc = im2col_conv(tx, n, h, w, c, wgt, cout, r, s, stride_h, stride_w, pad_h, pad_w, ho, wo, plain_a8w8(), e, sms, status, st);
+            workspace_free(tx, st);
+            return rc;
+        }
+    }
+    return im2col_conv(x_in, n, h, w, c, wgt, cout, r, s, stride_h, stride_w, pad_h, pad_w, ho, wo, x, e, sms, status, st);
 }
-

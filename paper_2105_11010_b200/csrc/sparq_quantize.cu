@@ -33,6 +33,8 @@ template <int MODE, int N, bool RND, bool WIDEN>
 __global__ void __launch_bounds__(kThreads)
 quantize_vec_kernel(const uint4 *in, uint4 *out, size_t nvec, XformDev d)
 {
+    dep_wait();
+    dep_launch();
     const size_t tile = (size_t)kThreads * kVec;
     for (size_t base = (size_t)blockIdx.x * tile; base < nvec; base += (size_t)gridDim.x * tile) {
         uint4 v[kVec];
@@ -77,6 +79,8 @@ __device__ unsigned scalar_window(unsigned x, int w, unsigned mask, int rnd)
 __global__ void quantize_pair_kernel(const uint8_t *in, uint8_t *out,
                                      size_t rows, size_t row_len, XformArgs a)
 {
+    dep_wait();
+    dep_launch();
     const size_t pairs_per_row = (row_len + 1) / 2;
     const size_t total = rows * pairs_per_row;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
@@ -109,11 +113,12 @@ static cudaError_t launch_vec(const uint4 *in, uint4 *out, size_t nvec, const Xf
 {
     XformDev d{a.widen_c, a.widen_rounds, a.n};
     const bool widen = a.widen_rounds > 0;   // restricted placement set
-    if (a.rnd && widen) quantize_vec_kernel<MODE, N, true, true><<<blocks, kThreads, 0, st>>>(in, out, nvec, d);
-    else if (a.rnd) quantize_vec_kernel<MODE, N, true, false><<<blocks, kThreads, 0, st>>>(in, out, nvec, d);
-    else if (widen) quantize_vec_kernel<MODE, N, false, true><<<blocks, kThreads, 0, st>>>(in, out, nvec, d);
-    else quantize_vec_kernel<MODE, N, false, false><<<blocks, kThreads, 0, st>>>(in, out, nvec, d);
-    return cudaGetLastError();
+    cudaError_t e;
+    if (a.rnd && widen) e = launch_overlapped(quantize_vec_kernel<MODE, N, true, true>, blocks, kThreads, 0, st, in, out, nvec, d);
+    else if (a.rnd) e = launch_overlapped(quantize_vec_kernel<MODE, N, true, false>, blocks, kThreads, 0, st, in, out, nvec, d);
+    else if (widen) e = launch_overlapped(quantize_vec_kernel<MODE, N, false, true>, blocks, kThreads, 0, st, in, out, nvec, d);
+    else e = launch_overlapped(quantize_vec_kernel<MODE, N, false, false>, blocks, kThreads, 0, st, in, out, nvec, d);
+    return e;
 }
 
 template <int MODE>
@@ -127,16 +132,8 @@ static cudaError_t launch_vec_n(const uint4 *in, uint4 *out, size_t nvec, const 
     }
 }
 
-}  // namespace sparq
-
-using namespace sparq;
-
-extern "C" int sparq_quantize(const uint8_t *in, uint8_t *out, size_t rows, size_t row_len,
-                              const sparq_params *p, void *stream)
+int quantize_rows(const uint8_t *in, uint8_t *out, size_t rows, size_t row_len, const XformArgs &a, cudaStream_t st)
 {
-    XformArgs a;
-    int rc = validate_params(p, &a);
-    if (rc != SPARQ_OK) return rc;
     if (rows == 0 || row_len == 0) return SPARQ_OK;
     if (!in || !out) return set_error(SPARQ_ERR_INVALID_ARG, "in/out pointer is NULL");
     if (rows > ((size_t)1 << 62) / row_len) return set_error(SPARQ_ERR_INVALID_ARG, "rows * row_len overflows");
@@ -146,7 +143,7 @@ extern "C" int sparq_quantize(const uint8_t *in, uint8_t *out, size_t rows, size
         const uint8_t *hi = in < (const uint8_t *)out ? out : in;
         if (lo + total > hi) return set_error(SPARQ_ERR_INVALID_ARG, "in and out overlap partially");
     }
-    cudaStream_t st = (cudaStream_t)stream;
+    note_outputs(st, {{out, total}, {nullptr, 0}, {nullptr, 0}});
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -179,8 +176,19 @@ extern "C" int sparq_quantize(const uint8_t *in, uint8_t *out, size_t rows, size
     size_t cap = (size_t)sms * 32;
     int blocks = (int)(want < cap ? want : cap);
     if (blocks < 1) blocks = 1;
-    quantize_pair_kernel<<<blocks, 256, 0, st>>>(in + done, out + done, g_rows, g_len, a);
-    e = cudaGetLastError();
+    e = launch_overlapped(quantize_pair_kernel, blocks, 256, 0, st, in + done, out + done, g_rows, g_len, a);
     if (e != cudaSuccess) return cuda_error(e, "quantize_pair_kernel launch");
     return SPARQ_OK;
+}
+
+}  // namespace sparq
+
+using namespace sparq;
+
+extern "C" int sparq_quantize(const uint8_t *in, uint8_t *out, size_t rows, size_t row_len,
+                              const sparq_params *p, void *stream)
+{
+    XformArgs a;
+    const int rc = validate_params(p, &a);
+    return rc != SPARQ_OK ? rc : quantize_rows(in, out, rows, row_len, a, (cudaStream_t)stream);
 }

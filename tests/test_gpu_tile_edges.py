@@ -58,3 +58,61 @@ def test_staged_output(mode, residual, n):
     got = out.cpu().numpy()
     assert np.array_equal(got[:m * n].reshape(m, n), want)
     assert (got[m * n:] == 0xA5).all()
+
+
+@pytest.mark.parametrize("mode,n", [(sparq.MODE_VSPARQ, 4), (sparq.MODE_BSPARQ, 3)])
+def test_transform_first_gemm(mode, n):
+    """Long reductions with many column tiles run as transform + plain contraction: two streams at
+    once, each with scratch memory of its own, and again inside a captured graph."""
+    m, cols, k = 1024 + 45, 2048, 1040
+    mask = {4: 0x1F, 3: 0x3F}[n]
+    p = sparq.SparqParams(mode, n, mask, 1)
+    A = [synth.activations(70 + i, (m, k), 0.5) for i in range(2)]
+    B = synth.weights(72, (k, cols))
+    want = [oracle.gemm(a, B, mode, n, mask, 1) for a in A]
+    Ad = [torch.from_numpy(a).cuda() for a in A]
+    Bd = torch.from_numpy(np.ascontiguousarray(B.T)).cuda()
+    out = [torch.zeros((m, cols), dtype=torch.int32, device="cuda") for _ in A]
+    streams = [torch.cuda.Stream() for _ in A]
+    torch.cuda.synchronize()
+    for _ in range(3):
+        for i, s in enumerate(streams):
+            sparq.sparq_gemm_s8(Ad[i], Bd, p, acc_out=out[i], stream=s)
+    for s in streams:
+        sparq.sparq_check(s)
+    for i in range(2):
+        assert np.array_equal(out[i].cpu().numpy(), want[i])
+    out[0].zero_()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=streams[0]):
+        sparq.sparq_gemm_s8(Ad[0], Bd, p, acc_out=out[0])
+    for _ in range(2):
+        g.replay()
+    sparq.sparq_check()
+    assert np.array_equal(out[0].cpu().numpy(), want[0])
+
+
+@pytest.mark.parametrize("c,cout,r,hw,nb,stride", [
+    (48, 64, 5, 35, 3, 1),      # one partial 64-channel block, 25 resident taps, odd image
+    (16, 40, 3, 56, 2, 1),      # mostly fill
+    (80, 48, 3, 28, 2, 1),      # few filters on a partial 128-channel block
+    (64, 128, 3, 28, 2, 1),     # half-empty 128-channel block
+    (192, 192, 3, 17, 2, 1),    # two channel blocks, the second partial, streamed weights
+    (144, 300, 3, 14, 40, 1),   # 256-wide tiles, partial block and partial column tile
+    (512, 264, 3, 7, 20, 1),    # small maps: transform first, then im2col
+    (256, 512, 3, 14, 9, 2),    # strided
+])
+@pytest.mark.parametrize("mode", [sparq.MODE_NONE, sparq.MODE_VSPARQ])
+def test_conv_channel_blocks(c, cout, r, hw, nb, stride, mode):
+    x = synth.activations(c + cout, (nb, hw, hw, c), 0.5)
+    w = synth.weights(c + cout, (cout, r, r, c))
+    p = sparq.SparqParams(mode, 4, 0x1F, 1)
+    ho = (hw + 2 * (r // 2) - r) // stride + 1
+    acc = torch.full((nb * ho * ho * cout + 16,), -7, dtype=torch.int32, device="cuda")
+    sparq.sparq_conv2d_nhwc_s8(torch.from_numpy(x).cuda(), torch.from_numpy(w).cuda(), (stride, stride), (r // 2, r // 2), p,
+                               acc_out=acc)
+    sparq.sparq_check()
+    got = acc.cpu().numpy()
+    want = oracle.conv2d_nhwc(x, w, (stride, stride), (r // 2, r // 2), mode, 4, 0x1F, 1)
+    assert np.array_equal(got[:-16], want.reshape(-1))
+    assert (got[-16:] == -7).all()
