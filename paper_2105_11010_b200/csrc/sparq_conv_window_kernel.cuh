@@ -261,12 +261,12 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
         if (lane == 0) {
             uint32_t gi = 0;                   // group counter
             int rb = 0; uint32_t ruse = 0;     // its window buffer (gi % win_bufs) and that buffer's use count (gi / win_bufs)
-            uint32_t it = 0;      // streamed weight-block counter
+            uint32_t it = 0;      // streamed weight-block counter,
+            int bs = 0; uint32_t buse = 0;     // its stage (it % b_stages) and that stage's use count
             for (; have; have = walk.next()) {
                 const int b = rb;                 // window buffer of this group and how often it was used before
                 const uint32_t use = ruse;
-                if (use > 0) mbar_wait(smem_u32(&bar_win_empty[b]), (use - 1) & 1, abort_flag, g.status, g.wait_limit);
-                if (*abort_flag) break;
+                if (use > 0 && !mbar_wait(smem_u32(&bar_win_empty[b]), (use - 1) & 1, abort_flag, g.status, g.wait_limit)) break;
                 const int oh0 = (int)walk.tin * g.TR;
                 if (B_RESIDENT && !b_issued) {
                     issue_resident_weights();
@@ -294,13 +294,12 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
                     for (int j = 0; j < passes && !stop; ++j) {
                         for (int cb = 0; cb < g.c_blocks && !stop; ++cb) {
                             for (int tap = 0; tap < taps; ++tap, ++it) {
-                                const int s = it % g.b_stages;
-                                const uint32_t buse = it / g.b_stages;
-                                if (buse > 0) mbar_wait(smem_u32(&bar_b_empty[s]), (buse - 1) & 1, abort_flag, g.status, g.wait_limit);
-                                if (*abort_flag) { stop = true; break; }
-                                const uint32_t full = smem_u32(&bar_b_full[s]);
+                                const int sb = bs;
+                                if (buse > 0 && !mbar_wait(smem_u32(&bar_b_empty[sb]), (buse - 1) & 1, abort_flag, g.status, g.wait_limit)) { stop = true; break; }
+                                const uint32_t full = smem_u32(&bar_b_full[sb]);
                                 mbar_expect_tx(full, kBBlock);
-                                tma_load_3d(b_slot(s), &map_w, full, cb * CB, (int)(walk.nt * BN), tap);
+                                tma_load_3d(b_slot(sb), &map_w, full, cb * CB, (int)(walk.nt * BN), tap);
+                                if (++bs == g.b_stages) { bs = 0; ++buse; }
                             }
                         }
                     }

@@ -86,6 +86,9 @@ struct GemmArgs {
     // staged output: bytes per row of the boxes that the epilogue warps store (and fetch the residual)
     // with through shared memory, 0 = straight from registers.  See epi_staged.
     int out_box;
+    // small form only: the weights are not an output of the previous launch, so fetch them before waiting
+    // for it; rows of a tile; CTAs of a cluster that share a tile (1 = none)
+    int early_weights, tile_rows, split;
 };
 
 // ---- PTX wrappers ---------------------------------------------------------------------
@@ -283,9 +286,9 @@ __device__ __forceinline__ uint64_t make_smem_desc(uint32_t saddr)
 }
 
 // kind::i8 instruction descriptor: s32 accumulator, unsigned A, signed B, both K-major.
-__device__ __forceinline__ constexpr uint32_t make_idesc_i8(int n)
+__device__ __forceinline__ constexpr uint32_t make_idesc_i8(int n, int m = kBM)
 {
-    return (2u << 4) | (0u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
+    return (2u << 4) | (0u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
@@ -310,6 +313,34 @@ __device__ __forceinline__ void tmem_ld_32x32_issue(uint32_t taddr, uint32_t (&r
           "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
         : "r"(taddr) : "memory");
 }
+
+// Reduction steps of a convolution in order, from step `first`: filter tap (r, s), channel block
+// starting at c, and the block's first byte k of a filter.
+struct TapWalk {
+    int c, r, s, k, tap_k, bk, S;
+    __device__ __forceinline__ TapWalk(const GemmArgs &g, int bk_, int first)
+    {
+        tap_k = g.tap_k; bk = bk_; S = g.S;
+        c = r = s = k = 0;
+        if (g.conv && first) {
+            const int tap = first / g.c_blocks;
+            c = (first - tap * g.c_blocks) * bk;
+            r = tap / S;
+            s = tap - r * S;
+            k = tap * tap_k + c;
+        }
+    }
+    __device__ __forceinline__ void next()
+    {
+        c += bk;
+        k += bk;
+        if (c >= tap_k) {
+            k += tap_k - c;
+            c = 0;
+            if (++s == S) { s = 0; ++r; }
+        }
+    }
+};
 
 // ---- epilogue arithmetic ----------------------------------------------------------------
 
@@ -765,10 +796,14 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     if (warp == 0) {
         // ================= TMA producer =================
         if (lane == 0) {
+            // One thread feeds the whole CTA, a few hundred cycles a step: positions are counters, not
+            // divisions, and the abort flag is read only where a wait has given up (every read of
+            // shared memory queues behind the tensor core's operand fetches).
             uint32_t it = 0;   // running stage counter across tiles
             int s = 0;         // stage it % S
             uint32_t use = 0;  // it / S
-            for (uint32_t tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
+            bool live = true;
+            for (uint32_t tile = blockIdx.x; tile < total_tiles && live; tile += gridDim.x) {
                 const uint32_t mt = (n_tiles32 == 1) ? tile : tile / n_tiles32, nt = tile - mt * n_tiles32;
                 const int64_t m0 = (int64_t)mt * kBM;
                 const int n0 = (int)(nt * BN);
@@ -780,26 +815,24 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                     base_h = (rem / g.Wo) * g.stride_h - g.pad_h;
                     base_w = (rem % g.Wo) * g.stride_w - g.pad_w;
                 }
+                TapWalk tap(g, BK, 0);
                 for (int kb = 0; kb < kb_count; ++kb, ++it) {
-                    if (use > 0) mbar_wait(smem_u32(&bar_empty[s]), (use - 1) & 1, abort_flag, g.status, g.wait_limit);
-                    if (*abort_flag) break;   // stop issuing copies once the CTA has given up
+                    // stop issuing copies once the CTA has given up
+                    if (use > 0 && !mbar_wait(smem_u32(&bar_empty[s]), (use - 1) & 1, abort_flag, g.status, g.wait_limit)) { live = false; break; }
                     const uint32_t full = smem_u32(&bar_full[s]);
                     mbar_expect_tx(full, Cfg::kStageBytes);
-                    int bx = kb * BK;
                     if (g.conv) {
                         // Channels past C arrive as zeros, so whatever the weight block holds
                         // there (the next tap's first bytes) adds nothing.
-                        const int tap = kb / g.c_blocks, cb = kb % g.c_blocks;
-                        tma_load_im2col_4d(a_stage(s), &map_a, full, cb * BK, base_w, base_h, base_n,
-                                           (uint16_t)(tap % g.S), (uint16_t)(tap / g.S));
-                        bx = tap * g.tap_k + cb * BK;
+                        tma_load_im2col_4d(a_stage(s), &map_a, full, tap.c, base_w, base_h, base_n, (uint16_t)tap.s, (uint16_t)tap.r);
+                        tma_load_2d(b_stage(s), &map_b, full, tap.k, n0);
+                        tap.next();
                     } else {
                         tma_load_2d(a_stage(s), &map_a, full, kb * BK, (int)m0);
+                        tma_load_2d(b_stage(s), &map_b, full, kb * BK, n0);
                     }
-                    tma_load_2d(b_stage(s), &map_b, full, bx, n0);
                     if (++s == S) { s = 0; ++use; }
                 }
-                if (*abort_flag) break;
             }
             // After an abort: wait (bounded) for the copies this thread still has in
             // flight, so that none lands after the CTA has exited.
