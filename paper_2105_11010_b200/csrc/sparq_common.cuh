@@ -62,19 +62,28 @@ __device__ __forceinline__ void dep_launch() { asm volatile("griddepcontrol.laun
 __device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <class Kernel, class... Args>
-cudaError_t launch_overlapped(Kernel kernel, int grid, int threads, int smem_bytes, cudaStream_t st, const Args &...args)
+cudaError_t launch_overlapped_cluster(Kernel kernel, int grid, int cluster, int threads, int smem_bytes, cudaStream_t st, const Args &...args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = (size_t)smem_bytes;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+template <class Kernel, class... Args>
+cudaError_t launch_overlapped(Kernel kernel, int grid, int threads, int smem_bytes, cudaStream_t st, const Args &...args)
+{
+    return launch_overlapped_cluster(kernel, grid, 1, threads, smem_bytes, st, args...);
 }
 #endif
 

@@ -7,6 +7,7 @@
 #include <mutex>
 
 #include "sparq_conv_window_kernel.cuh"
+#include "sparq_gemm_small_kernel.cuh"
 
 namespace sparq {
 
@@ -99,9 +100,9 @@ static int encode_2d(CUtensorMap *map, const void *ptr, int64_t K, int64_t rows,
     return SPARQ_OK;
 }
 
-// NHWC activation tensor read as im2col columns of 128 output pixels x bk channels.
+// NHWC activation tensor read as im2col columns of `rows` output pixels x bk channels.
 static int encode_im2col(CUtensorMap *map, const void *ptr, int n, int h, int w, int c, int r, int s,
-                         int stride_h, int stride_w, int pad_h, int pad_w, int bk)
+                         int stride_h, int stride_w, int pad_h, int pad_w, int bk, int rows)
 {
     static EncodeIm2colFn fn = nullptr;
     if (!fn) {
@@ -109,7 +110,7 @@ static int encode_im2col(CUtensorMap *map, const void *ptr, int n, int h, int w,
         if (rc != SPARQ_OK) return rc;
     }
     const MapKey key = {{2, (uint64_t)(uintptr_t)ptr, (uint64_t)n, (uint64_t)h, (uint64_t)w, (uint64_t)c, (uint64_t)r, (uint64_t)s,
-                         (uint64_t)stride_h, (uint64_t)stride_w, (uint64_t)(int64_t)pad_h, (uint64_t)(int64_t)pad_w, (uint64_t)bk}};
+                         (uint64_t)stride_h, (uint64_t)stride_w, (uint64_t)(int64_t)pad_h, (uint64_t)(int64_t)pad_w, (uint64_t)bk, (uint64_t)rows}};
     if (map_lookup(key, map)) return SPARQ_OK;
     cuuint64_t dims[4] = {(cuuint64_t)c, (cuuint64_t)w, (cuuint64_t)h, (cuuint64_t)n};
     cuuint64_t strides[3] = {(cuuint64_t)c, (cuuint64_t)c * w, (cuuint64_t)c * w * h};
@@ -118,7 +119,7 @@ static int encode_im2col(CUtensorMap *map, const void *ptr, int n, int h, int w,
     int upper[2] = {pad_w - (s - 1), pad_h - (r - 1)};
     cuuint32_t estr[4] = {1, (cuuint32_t)stride_w, (cuuint32_t)stride_h, 1};
     CUresult res = fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, const_cast<void *>(ptr), dims, strides, lower, upper,
-                      (cuuint32_t)bk, (cuuint32_t)kBM, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_for(bk),
+                      (cuuint32_t)bk, (cuuint32_t)rows, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_for(bk),
                       CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (res != CUDA_SUCCESS) return set_error(SPARQ_ERR_CUDA, "cuTensorMapEncodeIm2col failed with CUresult %d", (int)res);
     map_store(key, *map);
@@ -191,7 +192,7 @@ static double tile_cycles(int64_t M, int64_t N, int64_t steps, int bn, int sms, 
     const double fetch = (im2col ? 3.5 : 2.1) * (kBM + bn);
     if (fetch > step) step = fetch;
     if (transform && step < 1250.0) step = 1250.0;
-    return (double)rounds * (double)steps * (step + 150.0);
+    return (double)rounds * (double)steps * (step + 150.0) + 3.0 * bn;     // + the last tile's epilogue
 }
 
 // The tile width with the lowest estimate.
@@ -213,6 +214,34 @@ static int pick_bn(int64_t M, int64_t N, int64_t steps, int sms, bool transform,
     return best;
 }
 
+// The small form (sparq_gemm_small_kernel): launches whose 64-wide tiles all run at once.  tile_rows = 0
+// where they do not.  Tiles of 64 or 128 rows, and 1 to 8 CTAs of a cluster on a tile, by the time
+// of the serial walk along K: a step takes such a launch about 0.25 us, and 0.35 us more for the
+// transform of 128 rows; sharing a tile costs about 1.6 us.  Measured (us, one image, 128-row
+// tiles, 1 / 2 / 4 / 8 CTAs on each): 7x7x2048 -> 512 9.4 / 9.1 / 6.1 / 4.8, 14x14x1024 -> 256 6.9 /
+// 8.7 / 6.3 / 5.0, 28x28x512 -> 128 5.6 / 7.1 / 5.6, 7x7x512 -> 2048 4.7 / 6.3 / 5.1; chosen by this
+// rule, against the full kernel before: 7x7x512 -> 512 3x3 30.1 -> 6.7, 14x14x256 -> 256 3x3 14.9 ->
+// 5.5, 14x14x1024 -> 256 8.9 -> 4.2, 28x28x128 -> 512 with a residual 4.6 -> 3.1, 256 x 64 x 576
+// with int32 and fp32 outputs 8.7 -> 6.5.
+struct SmallForm {
+    int tile_rows, split;
+};
+static SmallForm pick_small(int64_t M, int64_t N, int64_t k_blocks, int sms, bool transform)
+{
+    SmallForm best = {0, 1};
+    double best_cost = 0.0;
+    const int64_t n_tiles = (N + kSmallBN - 1) / kSmallBN;
+    for (int rows = kBM; rows >= 64; rows /= 2) {
+        const int64_t tiles = (M + rows - 1) / rows * n_tiles;
+        const double step = 0.25 + (transform ? 0.35 * (double)(M < rows ? M : rows) / kBM : 0.0);
+        for (int split = 1; split <= kMaxSplit && tiles * split <= sms && k_blocks >= split; split *= 2) {
+            const double cost = (double)((k_blocks + split - 1) / split) * step + (split > 1 ? 1.6 : 0.0) + (split == 2 ? 0.4 : 0.0);
+            if (!best.tile_rows || cost < best_cost - 0.05) { best = {rows, split}; best_cost = cost; }
+        }
+    }
+    return best;
+}
+
 // Whether to write T(A) to scratch memory once and contract that, instead of transforming every
 // staged tile: worth it when A is staged several times -- several column tiles, several filter
 // taps -- because the in-kernel transform is what such a step takes.  The extra pass costs about
@@ -220,6 +249,7 @@ static int pick_bn(int64_t M, int64_t N, int64_t steps, int sms, bool transform,
 // fused form, which needs no memory, where the two are close.
 static bool transform_first(int64_t M, int64_t N, int64_t steps, size_t act_bytes, int sms, bool im2col)
 {
+    if (pick_small(M, N, steps, sms, true).tile_rows) return false;
     double fused, plain;
     pick_bn(M, N, steps, sms, true, im2col, &fused);
     pick_bn(M, N, steps, sms, false, im2col, &plain);
@@ -292,8 +322,10 @@ static XformDev xform_dev(const XformArgs &x)
     return d;
 }
 
-static cudaError_t launch(int bn, int bk, const GemmMaps &m, GemmArgs &g, const XformArgs &x, int grid, cudaStream_t st)
+static cudaError_t launch(int bn, int bk, bool small, const GemmMaps &m, GemmArgs &g, const XformArgs &x, int grid, cudaStream_t st)
 {
+    if (small && bk == 64) return launch_gemm_small<64>(m, g, x.mode, variant_n(x), x.rnd, grid, st);
+    if (small) return launch_gemm_small<128>(m, g, x.mode, variant_n(x), x.rnd, grid, st);
     if (bn == 64 && bk == 64) return launch_gemm_shape<64, 64>(m, g, x.mode, variant_n(x), x.rnd, grid, st);
     if (bn == 64) return launch_gemm_shape<64, 128>(m, g, x.mode, variant_n(x), x.rnd, grid, st);
     if (bn == 128 && bk == 64) return launch_gemm_shape<128, 64>(m, g, x.mode, variant_n(x), x.rnd, grid, st);
@@ -486,6 +518,9 @@ static int try_window_conv(const uint8_t *x_in, int n, int h, int w, int c, cons
                1024 + (win_bufs + 1) * plane_for(grp) * c_blocks + kb_count * b_block <= kMaxDynSmem) ++win_bufs;
     } else {
         if (bn == 64) return 0;                          // only the resident form is built for 64-wide tiles
+        // Few tiles: the im2col form, whose long reduction a cluster can share (one image of
+        // 14x14x256 -> 256 3x3: 6.9 us against 14.6; with resident weights the window kernel wins).
+        if (pick_small((int64_t)n * ho * wo, cout, kb_count, sms, x.mode != SPARQ_MODE_NONE).split > 1) return 0;
         // 128-wide tiles: up to two row tiles of one (image, column tile) are accumulated together
         // during ONE pass over the streamed weights (four accumulator stages: two groups in
         // flight), which halves the weight traffic out of L2 -- the bound of these layers.
@@ -576,9 +611,11 @@ int gemm_with_status(const uint8_t *A, int64_t lda, const int8_t *B, int64_t ldb
     // padding stays below an eighth (K = 576: five 128-byte steps instead of nine 64-byte ones: each
     // step is a hand-off between three warp roles, which is what a small launch is made of)
     const int bk = (pad64 < pad128 && !(pad64 >= 320 && pad128 * 8 <= pad64 * 9)) ? 64 : 128;
-    const int bn = pick_bn(M, N, (K + 127) / 128, sms, x.mode != SPARQ_MODE_NONE, false);
+    const SmallForm small = pick_small(M, N, (K + bk - 1) / bk, sms, x.mode != SPARQ_MODE_NONE);
+    const int bn = small.tile_rows ? kSmallBN : pick_bn(M, N, (K + 127) / 128, sms, x.mode != SPARQ_MODE_NONE, false);
+    const int tile_rows = small.tile_rows ? small.tile_rows : kBM;
     GemmMaps m = {};
-    rc = encode_2d(&m.a, A, K, M, lda, bk, kBM);
+    rc = encode_2d(&m.a, A, K, M, lda, bk, tile_rows);
     if (rc != SPARQ_OK) return rc;
     rc = encode_2d(&m.b, B, K, N, ldb, bk, bn);
     if (rc != SPARQ_OK) return rc;
@@ -588,12 +625,14 @@ int gemm_with_status(const uint8_t *A, int64_t lda, const int8_t *B, int64_t ldb
     g.k_blocks = (int)((K + bk - 1) / bk);
     rc = fill_common(&g, x, e, status);
     if (rc != SPARQ_OK) return rc;
-    const int64_t tiles = ((M + kBM - 1) / kBM) * ((N + bn - 1) / bn);
+    const int64_t tiles = ((M + tile_rows - 1) / tile_rows) * ((N + bn - 1) / bn);
     if (tiles >= ((int64_t)1 << 31)) return set_error(SPARQ_ERR_UNSUPPORTED, "more than 2^31 output tiles");
-    const int grid = (int)(tiles < sms ? tiles : sms);
+    g.tile_rows = tile_rows;
+    g.split = small.split;
+    const int grid = small.tile_rows ? (int)tiles * small.split : (int)(tiles < sms ? tiles : sms);
     if ((rc = output_maps(&m, &g, x.mode, bn, tiles, grid)) != SPARQ_OK) return rc;
-    record_launch_weights_clear(st, e, (size_t)M * (size_t)N, B, (size_t)N * (size_t)ldb);
-    cudaError_t ce = launch(bn, bk, m, g, x, grid, st);
+    g.early_weights = record_launch_weights_clear(st, e, (size_t)M * (size_t)N, B, (size_t)N * (size_t)ldb) ? 1 : 0;
+    cudaError_t ce = launch(bn, bk, small.tile_rows != 0, m, g, x, grid, st);
     if (ce != cudaSuccess) return cuda_error(ce, "sparq_gemm_kernel launch");
     return SPARQ_OK;
 }
@@ -605,10 +644,12 @@ static int im2col_conv(const uint8_t *x_in, int n, int h, int w, int c, const in
 {
     const int64_t M = (int64_t)n * ho * wo, K = (int64_t)r * s * c;
     const int bk = (c % 128 == 0) ? 128 : 64;
-    const int bn = pick_bn(M, cout, (int64_t)r * s * ((c + 127) / 128), sms, x.mode != SPARQ_MODE_NONE, true);
+    const SmallForm small = pick_small(M, cout, (int64_t)r * s * ((c + bk - 1) / bk), sms, x.mode != SPARQ_MODE_NONE);
+    const int bn = small.tile_rows ? kSmallBN : pick_bn(M, cout, (int64_t)r * s * ((c + 127) / 128), sms, x.mode != SPARQ_MODE_NONE, true);
     int rc;
+    const int tile_rows = small.tile_rows ? small.tile_rows : kBM;
     GemmMaps m = {};
-    rc = encode_im2col(&m.a, x_in, n, h, w, c, r, s, stride_h, stride_w, pad_h, pad_w, bk);
+    rc = encode_im2col(&m.a, x_in, n, h, w, c, r, s, stride_h, stride_w, pad_h, pad_w, bk, tile_rows);
     if (rc != SPARQ_OK) return rc;
     rc = encode_2d(&m.b, wgt, K, cout, K, bk, bn);
     if (rc != SPARQ_OK) return rc;
@@ -626,12 +667,14 @@ static int im2col_conv(const uint8_t *x_in, int n, int h, int w, int c, const in
     g.stride_h = stride_h; g.stride_w = stride_w; g.pad_h = pad_h; g.pad_w = pad_w;
     rc = fill_common(&g, x, e, status);
     if (rc != SPARQ_OK) return rc;
-    const int64_t tiles = ((M + kBM - 1) / kBM) * ((cout + bn - 1) / bn);
+    const int64_t tiles = ((M + tile_rows - 1) / tile_rows) * ((cout + bn - 1) / bn);
     if (tiles >= ((int64_t)1 << 31)) return set_error(SPARQ_ERR_UNSUPPORTED, "more than 2^31 output tiles");
-    const int grid = (int)(tiles < sms ? tiles : sms);
+    g.tile_rows = tile_rows;
+    g.split = small.split;
+    const int grid = small.tile_rows ? (int)tiles * small.split : (int)(tiles < sms ? tiles : sms);
     if ((rc = output_maps(&m, &g, x.mode, bn, tiles, grid)) != SPARQ_OK) return rc;
-    record_launch_weights_clear(st, e, (size_t)M * (size_t)cout, wgt, (size_t)cout * (size_t)K);
-    cudaError_t ce = launch(bn, bk, m, g, x, grid, st);
+    g.early_weights = record_launch_weights_clear(st, e, (size_t)M * (size_t)cout, wgt, (size_t)cout * (size_t)K) ? 1 : 0;
+    cudaError_t ce = launch(bn, bk, small.tile_rows != 0, m, g, x, grid, st);
     if (ce != cudaSuccess) return cuda_error(ce, "sparq_gemm_kernel (convolution) launch");
     return SPARQ_OK;
 }

@@ -116,3 +116,54 @@ def test_conv_channel_blocks(c, cout, r, hw, nb, stride, mode):
     want = oracle.conv2d_nhwc(x, w, (stride, stride), (r // 2, r // 2), mode, 4, 0x1F, 1)
     assert np.array_equal(got[:-16], want.reshape(-1))
     assert (got[-16:] == -7).all()
+
+
+@pytest.mark.parametrize("m,n,k", [
+    (1, 64, 2048),       # one row: most CTAs of a cluster of eight own nothing
+    (49, 512, 2048),     # rows that do not divide over the cluster
+    (64, 61, 576),       # one 64-row tile, ragged columns (scalar accesses), five steps
+    (65, 264, 1040),     # a second tile of one row, a partial last reduction step
+    (200, 72, 1024),     # partial last tile
+    (333, 128, 16),      # one step: not shared
+    (700, 136, 320),     # 64-byte steps
+])
+@pytest.mark.parametrize("mode", [sparq.MODE_NONE, sparq.MODE_VSPARQ])
+@pytest.mark.parametrize("outputs", ["u8", "all"])
+def test_few_tiles_gemm(m, n, k, mode, outputs):
+    A = synth.activations(m + k, (m, k), 0.5)
+    B = synth.weights(m + k, (k, n))
+    scale, bias, inv = synth.scales(n, n), synth.bias(n, n), synth.inv_out_scale(k)
+    res = synth.activations(m + n, (m, n), 0.5)
+    p = sparq.SparqParams(mode, 4, 0x1F, 1)
+    acc = oracle.gemm(A, B, mode, 4, 0x1F, 1)
+    f32, u8 = oracle.epilogue(acc, scale, bias, True, inv, residual=res, residual_scale=0.02)
+    d = lambda x: torch.from_numpy(x).cuda()  # noqa: E731
+    guard = lambda dt, v: torch.full((m * n + 64,), v, dtype=dt, device="cuda")  # noqa: E731
+    out = {"u8_out": guard(torch.uint8, 0xA5)}
+    if outputs == "all":
+        out.update(acc_out=guard(torch.int32, -7), f32_out=guard(torch.float32, -7.0))
+    for _ in range(2):       # the second launch starts beside the first
+        sparq.sparq_gemm_s8(d(A), d(np.ascontiguousarray(B.T)), p, scale=d(scale), bias=d(bias), relu=True, inv_out_scale=inv,
+                            residual=d(res), residual_scale=0.02, **out)
+    sparq.sparq_check()
+    for name, want, fill in (("u8_out", u8, 0xA5), ("acc_out", acc, -7), ("f32_out", f32, -7.0)):
+        if name in out:
+            got = out[name].cpu().numpy()
+            assert np.array_equal(got[:m * n].reshape(m, n), want), name
+            assert (got[m * n:] == fill).all()
+
+
+@pytest.mark.parametrize("nb,hw,c,cout,r,stride", [(1, 7, 512, 512, 3, 1), (1, 14, 256, 256, 3, 1), (1, 14, 144, 200, 3, 2),
+                                                   (3, 9, 80, 130, 5, 1), (1, 28, 48, 512, 1, 2)])
+@pytest.mark.parametrize("mode", [sparq.MODE_NONE, sparq.MODE_VSPARQ])
+def test_few_tiles_conv(nb, hw, c, cout, r, stride, mode):
+    x = synth.activations(c + cout, (nb, hw, hw, c), 0.5)
+    w = synth.weights(c + cout, (cout, r, r, c))
+    ho = (hw + 2 * (r // 2) - r) // stride + 1
+    acc = torch.full((nb * ho * ho * cout + 16,), -7, dtype=torch.int32, device="cuda")
+    sparq.sparq_conv2d_nhwc_s8(torch.from_numpy(x).cuda(), torch.from_numpy(w).cuda(), (stride, stride), (r // 2, r // 2),
+                               sparq.SparqParams(mode, 4, 0x1F, 1), acc_out=acc)
+    sparq.sparq_check()
+    got = acc.cpu().numpy()
+    assert np.array_equal(got[:-16], oracle.conv2d_nhwc(x, w, (stride, stride), (r // 2, r // 2), mode, 4, 0x1F, 1).reshape(-1))
+    assert (got[-16:] == -7).all()
