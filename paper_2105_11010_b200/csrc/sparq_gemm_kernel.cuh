@@ -388,9 +388,8 @@ struct EpiView {
     float inv_out_scale;
     bool need_f;      // a dequantized output is requested
     bool relu_op;     // the ReLU select has to be executed (see below)
-    bool vec_ok;      // rows allow 16-byte vector accesses
-    bool wide;        // rows come in whole groups of 32 columns, and every output and the residual allow 32-byte accesses
-    bool lean;        // wide, and only requantized bytes are wanted: see epi_lean
+    int gran;         // bytes (columns) that one access to a u8 row may take: 32, 16, 8, 4 or 1, whichever divides N
+    bool lean;        // gran = 32, and only requantized bytes are wanted: see epi_lean
     int next_mode;    // SPARQ mode applied to the requantized bytes (producer-side transform)
     int next_rnd;
     XformDev next_xf;
@@ -411,10 +410,10 @@ __host__ __device__ __forceinline__ EpiView make_epi_view(const Args &g)
     // relu(y) * inv clamped to [0, 255] equals y * inv clamped when inv > 0, so the ReLU
     // select is only needed when the fp32 value itself is an output
     e.relu_op = g.relu && (g.f32_out != nullptr || !(g.inv_out_scale > 0.0f));
-    e.vec_ok = (g.N % 16) == 0;
-    e.wide = (g.N % 32) == 0 && ((reinterpret_cast<uintptr_t>(g.u8_out) | reinterpret_cast<uintptr_t>(g.f32_out) |
-                                  reinterpret_cast<uintptr_t>(g.acc_out) | reinterpret_cast<uintptr_t>(g.residual)) & 31u) == 0;
-    e.lean = e.u8_out && !g.acc_out && !g.f32_out && g.next_mode == SPARQ_MODE_NONE && !e.relu_op && e.wide;
+    const bool aligned32 = ((reinterpret_cast<uintptr_t>(g.u8_out) | reinterpret_cast<uintptr_t>(g.f32_out) |
+                             reinterpret_cast<uintptr_t>(g.acc_out) | reinterpret_cast<uintptr_t>(g.residual)) & 31u) == 0;
+    e.gran = g.N % 32 == 0 && aligned32 ? 32 : g.N % 16 == 0 ? 16 : g.N % 8 == 0 ? 8 : g.N % 4 == 0 ? 4 : 1;
+    e.lean = e.u8_out && !g.acc_out && !g.f32_out && g.next_mode == SPARQ_MODE_NONE && !e.relu_op && e.gran == 32;
     e.next_mode = g.next_mode;
     e.next_rnd = g.next_rnd;
     e.next_xf = g.next_xf;
@@ -501,27 +500,101 @@ __device__ __forceinline__ void epi_lean(const uint32_t (&v)[32], const float *s
     }
 }
 
+// The first `cols` of 32 bytes / words at any byte / word address: aligned words / 16-byte pieces put
+// together from their neighbours, and single bytes / words at the ends.  (A thread owns a row, so
+// every store of a warp falls into 32 lines: their number is what such an epilogue takes.  Row
+// lengths that are no multiple of 4 only: 16384 x 1021, K 512, 171 -> 44 us.)
+__device__ __forceinline__ void store_bytes_unaligned(uint8_t *dst, const uint32_t (&w)[8], int cols)
+{
+    const int head = (int)(-reinterpret_cast<uintptr_t>(dst) & 3u), sh = 8 * head;
+    const int words = cols > head ? (cols - head) >> 2 : 0, done = head + 4 * words;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+        if (i < head && i < cols) dst[i] = (uint8_t)(w[0] >> (8 * i));
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+        if (q < words) *reinterpret_cast<uint32_t *>(dst + head + 4 * q) = __funnelshift_r(w[q], q < 7 ? w[q + 1] : 0u, sh);
+#pragma unroll
+    for (int i = 0; i < 32; ++i)
+        if ((cols != 32 || i >= 28) && i >= done && i < cols) dst[i] = (uint8_t)(w[i >> 2] >> (8 * (i & 3)));
+}
+__device__ __forceinline__ void store_words_unaligned(uint32_t *dst, const uint32_t (&v)[32], int cols)
+{
+    const int head = (int)(-(reinterpret_cast<uintptr_t>(dst) >> 2) & 3u);
+    const int quads = cols > head ? (cols - head) >> 2 : 0, done = head + 4 * quads;
+    auto at = [&](int i) {      // v[i + head]
+        const uint32_t a = head & 1 ? v[i + 1 < 32 ? i + 1 : 31] : v[i], b = head & 1 ? v[i + 3 < 32 ? i + 3 : 31] : v[i + 2 < 32 ? i + 2 : 31];
+        return head & 2 ? b : a;
+    };
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+        if (i < head && i < cols) dst[i] = v[i];
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+        if (q < quads) *reinterpret_cast<uint4 *>(dst + head + 4 * q) = make_uint4(at(4 * q), at(4 * q + 1), at(4 * q + 2), at(4 * q + 3));
+#pragma unroll
+    for (int i = 0; i < 32; ++i)
+        if ((cols != 32 || i >= 28) && i >= done && i < cols) dst[i] = v[i];
+}
+
+// The first `cols` of 32 bytes, in accesses of `gran` >= 4 bytes (a divisor of the row length).
+__device__ __forceinline__ void store_bytes32(uint8_t *dst, const uint32_t (&w)[8], int cols, int gran)
+{
+    if (gran == 32) {
+        st_global_v8(dst, w);
+    } else if (gran == 16) {
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            if (16 * i < cols) reinterpret_cast<uint4 *>(dst)[i] = make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
+    } else if (gran == 8) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (8 * i < cols) reinterpret_cast<uint2 *>(dst)[i] = make_uint2(w[2 * i], w[2 * i + 1]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (4 * i < cols) reinterpret_cast<uint32_t *>(dst)[i] = w[i];
+    }
+}
+
+__device__ __forceinline__ void load_bytes32(const uint8_t *src, uint32_t (&w)[8], int cols, int gran)
+{
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[i] = 0u;
+    if (gran >= 16) {
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            if (16 * i < cols) {
+                const uint4 r = __ldg(reinterpret_cast<const uint4 *>(src) + i);
+                w[4 * i] = r.x; w[4 * i + 1] = r.y; w[4 * i + 2] = r.z; w[4 * i + 3] = r.w;
+            }
+    } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (4 * i < cols) w[i] = __ldg(reinterpret_cast<const uint32_t *>(src) + i);
+    }
+}
+
 // 32 accumulators of one output row (columns col0 .. col0 + 31) with any combination of outputs and
-// any N: optional raw store, dequantize, optional fp32 store, requantize and store.  v is
-// overwritten.
+// any N (ODD: N is no multiple of 4): optional raw store, dequantize, optional fp32 store, requantize
+// and store.  v is overwritten.
+template <bool ODD>
 __device__ __forceinline__ void epi_general(const EpiView &e, uint32_t (&v)[32], int64_t row, int64_t col0,
                                             const float *s_scale, const float *s_bias)
 {
     const int64_t off = row * e.N + col0;
     const int cols = (int)(e.N - col0 < 32 ? e.N - col0 : 32);
-    const bool wide = e.wide, full = e.vec_ok && cols == 32;
     auto store32 = [&](void *base) {       // 32 words
         uint32_t *dst = reinterpret_cast<uint32_t *>(base) + off;
-        if (wide) {
+        if (ODD) {
+            store_words_unaligned(dst, v, cols);
+        } else if (e.gran == 32) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) st_global_v8(dst + 8 * q, reinterpret_cast<const uint32_t(&)[8]>(v[8 * q]));
-        } else if (full) {
-#pragma unroll
-            for (int q = 0; q < 8; ++q) reinterpret_cast<uint4 *>(dst)[q] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
         } else {
 #pragma unroll
-            for (int i = 0; i < 32; ++i)
-                if (i < cols) dst[i] = v[i];
+            for (int q = 0; q < 8; ++q)
+                if (4 * q < cols) reinterpret_cast<uint4 *>(dst)[q] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
         }
     };
     if (e.acc_out) store32(e.acc_out);
@@ -530,56 +603,51 @@ __device__ __forceinline__ void epi_general(const EpiView &e, uint32_t (&v)[32],
     for (int q = 0; q < 8; ++q) {
         const float4 sc = *reinterpret_cast<const float4 *>(&s_scale[4 * q]);
         const float4 bi = *reinterpret_cast<const float4 *>(&s_bias[4 * q]);
-        const float ss[4] = {sc.x, sc.y, sc.z, sc.w}, bb[4] = {bi.x, bi.y, bi.z, bi.w};
+        float y[4];
+        f2_unpack(f2_fma(f2_pack(__int2float_rn((int)v[4 * q]), __int2float_rn((int)v[4 * q + 1])), f2_pack(sc.x, sc.y), f2_pack(bi.x, bi.y)), y[0], y[1]);
+        f2_unpack(f2_fma(f2_pack(__int2float_rn((int)v[4 * q + 2]), __int2float_rn((int)v[4 * q + 3])), f2_pack(sc.z, sc.w), f2_pack(bi.z, bi.w)), y[2], y[3]);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            float y = __fmaf_rn(__int2float_rn((int)v[4 * q + i]), ss[i], bb[i]);
-            if (e.relu_op && !e.residual) y = fmaxf(y, 0.0f);    // NaN -> 0, like (y > 0 ? y : 0)
-            v[4 * q + i] = __float_as_uint(y);
-        }
+        for (int i = 0; i < 4; ++i) v[4 * q + i] = __float_as_uint(y[i]);
     }
-    if (e.residual) {                                            // with a residual input the ReLU comes after the sum
-        uint32_t r[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
-        if (full) {
+    if (e.residual) {
+        uint32_t r[8];
+        if (ODD) {
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const uint4 rr = __ldg(reinterpret_cast<const uint4 *>(e.residual + off) + h);
-                r[4 * h] = rr.x; r[4 * h + 1] = rr.y; r[4 * h + 2] = rr.z; r[4 * h + 3] = rr.w;
-            }
-        } else {
+            for (int i = 0; i < 8; ++i) r[i] = 0u;
 #pragma unroll
             for (int i = 0; i < 32; ++i)
                 if (i < cols) r[i >> 2] |= (uint32_t)__ldg(e.residual + off + i) << (8 * (i & 3));
+        } else {
+            load_bytes32(e.residual + off, r, cols, e.gran);
         }
+        const uint64_t rs2 = f2_pack(e.residual_scale, e.residual_scale);
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-            const float rv = __uint2float_rn((r[i >> 2] >> (8 * (i & 3))) & 0xFFu);
-            float y = __fmaf_rn(rv, e.residual_scale, __uint_as_float(v[i]));
-            if (e.relu_op) y = fmaxf(y, 0.0f);
-            v[i] = __float_as_uint(y);
+        for (int q = 0; q < 8; ++q) {
+            float y[4];
+            f2_unpack(f2_fma(bytes_to_f2<0>(r[q]), rs2, f2_pack(__uint_as_float(v[4 * q]), __uint_as_float(v[4 * q + 1]))), y[0], y[1]);
+            f2_unpack(f2_fma(bytes_to_f2<1>(r[q]), rs2, f2_pack(__uint_as_float(v[4 * q + 2]), __uint_as_float(v[4 * q + 3]))), y[2], y[3]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[4 * q + i] = __float_as_uint(y[i]);
         }
+    }
+    if (e.relu_op) {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) v[i] = __float_as_uint(fmaxf(__uint_as_float(v[i]), 0.0f));    // NaN -> 0, like (y > 0 ? y : 0)
     }
     if (e.f32_out) store32(e.f32_out);
     if (e.u8_out) {
         uint32_t w[8];
+        const uint64_t inv2 = f2_pack(e.inv_out_scale, e.inv_out_scale);
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-            w[q] = requant_pack4(__fmul_rn(__uint_as_float(v[4 * q]), e.inv_out_scale),
-                                 __fmul_rn(__uint_as_float(v[4 * q + 1]), e.inv_out_scale),
-                                 __fmul_rn(__uint_as_float(v[4 * q + 2]), e.inv_out_scale),
-                                 __fmul_rn(__uint_as_float(v[4 * q + 3]), e.inv_out_scale));
-        if (e.next_mode != SPARQ_MODE_NONE) next_xform_words(w, 8, e.next_mode, e.next_rnd, e.next_xf);
-        if (wide) {
-            st_global_v8(e.u8_out + off, w);
-        } else if (full) {
-            uint4 *dst = reinterpret_cast<uint4 *>(e.u8_out + off);
-            dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
-            dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
-        } else {
-#pragma unroll
-            for (int i = 0; i < 32; ++i)
-                if (i < cols) e.u8_out[off + i] = (uint8_t)(w[i >> 2] >> (8 * (i & 3)));
+        for (int q = 0; q < 8; ++q) {
+            float z[4];
+            f2_unpack(f2_mul(f2_pack(__uint_as_float(v[4 * q]), __uint_as_float(v[4 * q + 1])), inv2), z[0], z[1]);
+            f2_unpack(f2_mul(f2_pack(__uint_as_float(v[4 * q + 2]), __uint_as_float(v[4 * q + 3])), inv2), z[2], z[3]);
+            w[q] = requant_pack4(z[0], z[1], z[2], z[3]);
         }
+        if (e.next_mode != SPARQ_MODE_NONE) next_xform_words(w, 8, e.next_mode, e.next_rnd, e.next_xf);
+        if (ODD) store_bytes_unaligned(e.u8_out + off, w, cols);
+        else store_bytes32(e.u8_out + off, w, cols, e.gran);
     }
 }
 
@@ -594,7 +662,7 @@ __device__ __forceinline__ void epi_general(const EpiView &e, uint32_t (&v)[32],
 // the next one's tensor-memory load in flight measured 20 % slower: every group starts with its
 // own exposed scale / bias reads.)  The residual bytes are fetched a group ahead, the first ones
 // before the accumulator is waited for.
-enum EpiKind { kEpiGeneral, kEpiLean, kEpiLeanResidual };
+enum EpiKind { kEpiGeneral, kEpiGeneralOdd, kEpiLean, kEpiLeanResidual };
 
 template <int KIND, class WaitFull>
 __device__ __forceinline__ void epi_warp_columns_as(const EpiView &e, uint32_t taddr0, int cbase, int cols, int64_t row, bool row_ok,
@@ -629,8 +697,8 @@ __device__ __forceinline__ void epi_warp_columns_as(const EpiView &e, uint32_t t
         const int ct = cbase + c;                    // column inside the tile
         const int64_t col0 = n0 + ct;
         if (!row_ok || col0 >= e.N) continue;
-        if (KIND == kEpiGeneral) {
-            epi_general(e, v, row, col0, s_scale + ct, s_bias + ct);
+        if (KIND == kEpiGeneral || KIND == kEpiGeneralOdd) {
+            epi_general<KIND == kEpiGeneralOdd>(e, v, row, col0, s_scale + ct, s_bias + ct);
         } else {
             uint32_t w[8];
             epi_lean<KIND == kEpiLeanResidual>(v, s_scale + ct, s_bias + ct, e.inv_out_scale, e.residual_scale, r, w);
@@ -644,7 +712,8 @@ __device__ __forceinline__ void epi_warp_columns(const EpiView &e, uint32_t tadd
                                                  int64_t n0, const float *s_scale, const float *s_bias,
                                                  uint32_t acc_empty_bar, int lane, WaitFull wait_full)
 {
-    if (!e.lean) epi_warp_columns_as<kEpiGeneral>(e, taddr0, cbase, cols, row, row_ok, n0, s_scale, s_bias, acc_empty_bar, lane, wait_full);
+    if (e.gran == 1) epi_warp_columns_as<kEpiGeneralOdd>(e, taddr0, cbase, cols, row, row_ok, n0, s_scale, s_bias, acc_empty_bar, lane, wait_full);
+    else if (!e.lean) epi_warp_columns_as<kEpiGeneral>(e, taddr0, cbase, cols, row, row_ok, n0, s_scale, s_bias, acc_empty_bar, lane, wait_full);
     else if (e.residual) epi_warp_columns_as<kEpiLeanResidual>(e, taddr0, cbase, cols, row, row_ok, n0, s_scale, s_bias, acc_empty_bar, lane, wait_full);
     else epi_warp_columns_as<kEpiLean>(e, taddr0, cbase, cols, row, row_ok, n0, s_scale, s_bias, acc_empty_bar, lane, wait_full);
 }
