@@ -679,6 +679,43 @@ static int im2col_conv(const uint8_t *x_in, int n, int h, int w, int c, const in
     return SPARQ_OK;
 }
 
+cudaError_t launch_x24(int bn, const CUtensorMap &ma, const CUtensorMap &mb, const GemmArgs &g, int n, int rnd, int grid, cudaStream_t st);
+
+// The 2:4 product with the expansion inside the kernel (sparq_gemm_sparse24_kernel).  Returns 1 if it
+// launched, 0 if expanding into the workspace first is expected to be faster, < 0 on error.
+int gemm_sparse24_fused(const uint8_t *A, const int8_t *w_exp, int64_t M, int64_t N, int64_t K, const XformArgs &x,
+                        const sparq_epilogue *e, cudaStream_t st)
+{
+    if (K == 0 || K % 16 || 3 * K > 65536 || (((uintptr_t)A | (uintptr_t)w_exp) & 15u) || M > (int64_t)1 << 31 || N > (int64_t)1 << 31)
+        return 0;                                        // the two-kernel form reports it
+    int sms = 0, rc = device_info(&sms);
+    if (rc != SPARQ_OK) return rc;
+    // A tile of 256 rows is expanded once per column tile, about 4200 cycles per 128 activations of its
+    // rows; the other form moves 4 bytes per activation through HBM and multiplies at K' = 3K.  Few
+    // tiles: that product can be shared by clusters.
+    const int64_t steps = (K + 127) / 128, steps3 = (3 * K + 127) / 128;
+    if (pick_small(M, N, steps3, sms, false).tile_rows) return 0;
+    const int bn = N <= 64 ? 64 : 128;
+    const int64_t tiles = (M + 255) / 256 * ((N + bn - 1) / bn);
+    double plain;
+    pick_bn(M, N, steps3, sms, false, false, &plain);
+    const double fused = (double)((tiles + sms - 1) / sms) * (double)steps * 4200.0;
+    if (tiles >= (int64_t)1 << 31 || fused > plain + 1900.0 * (2.5 + (double)M * (double)K * 4.0 / 6.0e6)) return 0;
+    CUtensorMap ma, mb;
+    if ((rc = encode_2d(&ma, A, K, M, K, 128, 256)) != SPARQ_OK) return rc;
+    if ((rc = encode_2d(&mb, w_exp, 3 * K, N, 3 * K, 128, bn)) != SPARQ_OK) return rc;
+    unsigned int *status = nullptr;
+    if ((rc = get_status_word(&status)) != SPARQ_OK) return rc;
+    GemmArgs g;
+    memset(&g, 0, sizeof(g));
+    g.M = M; g.N = N; g.K = 3 * K;
+    g.k_blocks = (int)steps;
+    if ((rc = fill_common(&g, x, e, status)) != SPARQ_OK) return rc;
+    record_launch_weights_clear(st, e, (size_t)M * (size_t)N, w_exp, (size_t)N * (size_t)(3 * K));
+    const cudaError_t ce = launch_x24(bn, ma, mb, g, variant_n(x), x.rnd, (int)(tiles < sms ? tiles : sms), st);
+    return ce == cudaSuccess ? 1 : cuda_error(ce, "sparq_gemm_sparse24_kernel launch");
+}
+
 int check_epilogue_args(const sparq_epilogue *e) { return check_epilogue(e); }
 
 }  // namespace sparq

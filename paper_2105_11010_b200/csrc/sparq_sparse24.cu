@@ -11,11 +11,13 @@
 // contraction (K' = 3K) that the existing GEMM / convolution kernels run with mode NONE.
 // Without the pair rule (modes NONE and BSPARQ) the transform is per element, commutes
 // with the selection, and the expansion is just the dense form of the weights (K' = K).
-#include "sparq_common.cuh"
+#include "sparq_expand24.cuh"
 
 namespace sparq {
 
 int check_epilogue_args(const sparq_epilogue *e);
+int gemm_sparse24_fused(const uint8_t *A, const int8_t *w_exp, int64_t M, int64_t N, int64_t K, const XformArgs &x,
+                        const sparq_epilogue *e, cudaStream_t st);
 
 namespace {
 
@@ -36,27 +38,20 @@ __device__ __forceinline__ void st_stream16(void *p, uint4 v)
                  :: "l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 
-// One group of four activations (bytes of x) -> the six transformed pairs, 12 bytes.
-template <int N, bool RND, bool WIDEN>
-__device__ __forceinline__ void expand_group(uint32_t x, const XformDev &d, uint32_t &o0, uint32_t &o1, uint32_t &o2)
-{
-    o0 = xform_word<SPARQ_MODE_VSPARQ, N, RND, WIDEN>(prmt(x, x, 0x2010u), d);   // (0,1) (0,2)
-    o1 = xform_word<SPARQ_MODE_VSPARQ, N, RND, WIDEN>(prmt(x, x, 0x2130u), d);   // (0,3) (1,2)
-    o2 = xform_word<SPARQ_MODE_VSPARQ, N, RND, WIDEN>(prmt(x, x, 0x3231u), d);   // (1,3) (2,3)
-}
-
 // in: vectors of 16 activations (4 groups); out: 48 bytes per vector
-template <int N, bool RND, bool WIDEN>
+template <int XN, bool RND>
 __global__ void __launch_bounds__(kThreads)
 expand_act_kernel(const uint4 *__restrict__ in, uint4 *__restrict__ out, size_t nvec, XformDev d)
 {
+    dep_wait();
+    dep_launch();
     for (size_t i = (size_t)blockIdx.x * kThreads + threadIdx.x; i < nvec; i += (size_t)gridDim.x * kThreads) {
         const uint4 v = ld_stream16(in + i);
         uint32_t g0[3], g1[3], g2[3], g3[3];
-        expand_group<N, RND, WIDEN>(v.x, d, g0[0], g0[1], g0[2]);
-        expand_group<N, RND, WIDEN>(v.y, d, g1[0], g1[1], g1[2]);
-        expand_group<N, RND, WIDEN>(v.z, d, g2[0], g2[1], g2[2]);
-        expand_group<N, RND, WIDEN>(v.w, d, g3[0], g3[1], g3[2]);
+        expand_group<XN, RND>(v.x, d, g0[0], g0[1], g0[2]);
+        expand_group<XN, RND>(v.y, d, g1[0], g1[1], g1[2]);
+        expand_group<XN, RND>(v.z, d, g2[0], g2[1], g2[2]);
+        expand_group<XN, RND>(v.w, d, g3[0], g3[1], g3[2]);
         st_stream16(out + 3 * i, make_uint4(g0[0], g0[1], g0[2], g1[0]));
         st_stream16(out + 3 * i + 1, make_uint4(g1[1], g1[2], g2[0], g2[1]));
         st_stream16(out + 3 * i + 2, make_uint4(g2[2], g3[0], g3[1], g3[2]));
@@ -102,16 +97,14 @@ int grid_for(size_t items, int per_sm, int *blocks)
     return SPARQ_OK;
 }
 
-template <int N>
 cudaError_t launch_expand_act(const uint4 *in, uint4 *out, size_t nvec, const XformArgs &a, int blocks, cudaStream_t st)
 {
-    const XformDev d{a.widen_c, a.widen_rounds, a.n};
-    const bool widen = a.widen_rounds > 0 || N == 0;
-    if (a.rnd && widen) expand_act_kernel<N, true, true><<<blocks, kThreads, 0, st>>>(in, out, nvec, d);
-    else if (a.rnd) expand_act_kernel<N, true, false><<<blocks, kThreads, 0, st>>>(in, out, nvec, d);
-    else if (widen) expand_act_kernel<N, false, true><<<blocks, kThreads, 0, st>>>(in, out, nvec, d);
-    else expand_act_kernel<N, false, false><<<blocks, kThreads, 0, st>>>(in, out, nvec, d);
-    return cudaGetLastError();
+    XformDev d{a.widen_c, a.widen_rounds, a.n};
+    fill_fullset(&d, a.n, a.rnd);
+    auto go = [&](auto kernel) { return launch_overlapped(kernel, blocks, kThreads, 0, st, in, out, nvec, d); };
+    if (a.widen_rounds > 0) return a.rnd ? go(expand_act_kernel<0, true>) : go(expand_act_kernel<0, false>);
+    if (a.n != 4) return go(expand_act_kernel<8, true>);
+    return a.rnd ? go(expand_act_kernel<4, true>) : go(expand_act_kernel<4, false>);
 }
 
 }  // namespace
@@ -171,8 +164,8 @@ extern "C" int sparq_sparse24_expand_activations(const uint8_t *A, size_t rows, 
     cudaStream_t st = (cudaStream_t)stream;
     const uint4 *in = reinterpret_cast<const uint4 *>(A);
     uint4 *out = reinterpret_cast<uint4 *>(a_exp);
-    cudaError_t e = (x.n == 4 && x.widen_rounds == 0) ? launch_expand_act<4>(in, out, nvec, x, blocks, st)
-                                                       : launch_expand_act<0>(in, out, nvec, x, blocks, st);
+    note_outputs(st, {{out, 48 * nvec}, {nullptr, 0}, {nullptr, 0}});
+    const cudaError_t e = launch_expand_act(in, out, nvec, x, blocks, st);
     if (e != cudaSuccess) return cuda_error(e, "expand_act_kernel launch");
     return SPARQ_OK;
 }
@@ -189,6 +182,7 @@ extern "C" int sparq_gemm_s8_sparse24(const uint8_t *A, const int8_t *w_exp, int
     if (x.mode != SPARQ_MODE_VSPARQ)   // dense form of the weights, transform fused as usual
         return sparq_gemm_s8(A, K, w_exp, K, M, N, K, p, e, stream);
     if (!workspace) return set_error(SPARQ_ERR_INVALID_ARG, "workspace is NULL (M * 3K bytes are needed with vSPARQ)");
+    if ((rc = gemm_sparse24_fused(A, w_exp, M, N, K, x, e, (cudaStream_t)stream)) != 0) return rc < 0 ? rc : SPARQ_OK;
     if ((rc = sparq_sparse24_expand_activations(A, (size_t)M, (size_t)K, p, workspace, stream)) != SPARQ_OK) return rc;
     const sparq_params none = {SPARQ_MODE_NONE, 4, 0x1Fu, 0};
     return sparq_gemm_s8(workspace, 3 * K, w_exp, 3 * K, M, N, 3 * K, &none, e, stream);

@@ -167,3 +167,49 @@ def test_few_tiles_conv(nb, hw, c, cout, r, stride, mode):
     got = acc.cpu().numpy()
     assert np.array_equal(got[:-16], oracle.conv2d_nhwc(x, w, (stride, stride), (r // 2, r // 2), mode, 4, 0x1F, 1).reshape(-1))
     assert (got[-16:] == -7).all()
+
+
+@pytest.mark.parametrize("n", [1, 3, 31, 33, 61, 68, 72, 80, 127, 130, 200, 261])
+@pytest.mark.parametrize("residual", [False, True])
+def test_ragged_columns(n, residual):
+    """Every row length modulo the store widths, in launches with several tiles per SM."""
+    m, k = 148 * 128 * 2 + 77, 48
+    A, B = synth.activations(n, (m, k), 0.5), synth.weights(n, (k, n))
+    scale, bias, inv = synth.scales(n, n), synth.bias(n, n), synth.inv_out_scale(k)
+    res = synth.activations(n + 1, (m, n), 0.5) if residual else None
+    p = sparq.SparqParams(sparq.MODE_VSPARQ, 4, 0x1F, 1)
+    acc = oracle.gemm(A, B, p.mode, 4, 0x1F, 1)
+    f32, u8 = oracle.epilogue(acc, scale, bias, True, inv, residual=res, residual_scale=0.02)
+    d = lambda x: torch.from_numpy(x).cuda()  # noqa: E731
+    for names in (["u8_out"], ["acc_out", "f32_out", "u8_out"]):
+        dt = {"u8_out": torch.uint8, "acc_out": torch.int32, "f32_out": torch.float32}
+        out = {q: torch.full((m * n + 64,), 3, dtype=dt[q], device="cuda") for q in names}
+        sparq.sparq_gemm_s8(d(A), d(np.ascontiguousarray(B.T)), p, scale=d(scale), bias=d(bias), relu=True, inv_out_scale=inv,
+                            residual=d(res) if residual else None, residual_scale=0.02, **out)
+        sparq.sparq_check()
+        for q in names:
+            got = out[q].cpu().numpy()
+            assert np.array_equal(got[:m * n].reshape(m, n), {"u8_out": u8, "acc_out": acc, "f32_out": f32}[q]), q
+            assert (got[m * n:] == 3).all()
+
+
+@pytest.mark.parametrize("m,n,k", [(148 * 256 + 300, 128, 256), (148 * 256 * 2 + 45, 104, 144), (148 * 128 + 31, 61, 528),
+                                   (148 * 256 + 1, 264, 96)])
+@pytest.mark.parametrize("nb,mask,rnd", [(4, 0x1F, 1), (4, 0x1F, 0), (4, 0x15, 1), (3, 0x3F, 1), (2, 0x7F, 0)])
+def test_sparse24_fused(m, n, k, nb, mask, rnd):
+    """Expansion inside the product: partial row tiles, partial reduction steps, ragged columns."""
+    A = synth.activations(m % 91, (m, k), 0.5)
+    vals, pos = synth.sparse24_weights(n, n, k)
+    p = sparq.SparqParams(sparq.MODE_VSPARQ, nb, mask, rnd)
+    kx = sparq.sparq_sparse24_expanded_k(k, p)
+    d = lambda x: torch.from_numpy(x).cuda()  # noqa: E731
+    w = torch.empty((n, kx), dtype=torch.int8, device="cuda")
+    sparq.sparq_sparse24_expand_weights(d(vals), d(pos), p, w)
+    acc = torch.full((m * n + 16,), -7, dtype=torch.int32, device="cuda")
+    sparq.sparq_gemm_s8_sparse24(d(A), w, p, workspace=torch.empty(m * kx, dtype=torch.uint8, device="cuda"), acc_out=acc)
+    sparq.sparq_check()
+    got = acc.cpu().numpy()
+    rows = np.unique(np.concatenate([np.arange(0, m, 997), np.arange(300), np.arange(m - 300, m)]))
+    want = oracle.gemm_sparse24(A[rows], vals, pos, p.mode, nb, mask, rnd)
+    assert np.array_equal(got[:-16].reshape(m, n)[rows], want)
+    assert (got[-16:] == -7).all()
