@@ -3,8 +3,12 @@
 //   activations  unsigned symmetric per layer:  q = clamp(rint(x * (255 / max)), 0, 255)
 //   weights      signed symmetric per kernel:   q = clamp(rint(w * (127 / max_j)), -127, 127)
 // with max the largest magnitude (gathered over calibration batches by sparq_absmax, which
-// folds each batch into a running maximum on the device).  All three kernels are
-// streaming kernels bound by HBM traffic; fp32, one IEEE operation per step.
+// folds each batch into a running maximum on the device).  fp32, one IEEE operation per step.
+//
+// All three kernels stream and are bound by HBM traffic.  Calibration reads a tensor for its maximum and
+// then again to quantize it; the first pass goes through the tensor forwards, streaming, and leaves
+// the last 64 MB in L2, and the second goes backwards and finds them there.  51.4 M bf16 values,
+// both passes: 42.3 us without, 41.2 / 38.2 / 36.6 / 37.5 / 37.6 us with 0 / 32 / 64 / 80 / 120 MB left.
 #include "sparq_common.cuh"
 
 namespace sparq {
@@ -13,7 +17,17 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kVec = 4;   // 16-byte vectors in flight per thread
+constexpr size_t kKeepVecs = (size_t)(64 << 20) / 16;   // of the end of a tensor, left in L2 by the first pass
 
+__device__ __forceinline__ uint4 ld16(const void *p)
+{
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+
+// The same, first in line to leave the caches.
 __device__ __forceinline__ uint4 ld_stream16(const void *p)
 {
     uint4 v;
@@ -65,9 +79,11 @@ __device__ __forceinline__ uint32_t block_max_bits(float m, uint32_t *s_red)
 // max_inout = max(max_inout, max |x|): one atomic per block on the running maximum
 template <bool BF16>
 __global__ void __launch_bounds__(kThreads)
-absmax_kernel(const void *__restrict__ x, size_t n, float *max_inout)
+absmax_kernel(const void *__restrict__ x, size_t n, float *max_inout, size_t keep_from)
 {
     __shared__ uint32_t s_red[kThreads / 32];
+    dep_wait();
+    dep_launch();
     constexpr int kPer = BF16 ? 8 : 4;
     const size_t nvec = n / kPer;
     const uint4 *xv = reinterpret_cast<const uint4 *>(x);
@@ -75,10 +91,11 @@ absmax_kernel(const void *__restrict__ x, size_t n, float *max_inout)
     const size_t tile = (size_t)kThreads * kVec;
     for (size_t base = (size_t)blockIdx.x * tile; base < nvec; base += (size_t)gridDim.x * tile) {
         uint4 v[kVec];
+        const bool keep = base >= keep_from;
 #pragma unroll
         for (int j = 0; j < kVec; ++j) {
             const size_t i = base + (size_t)j * kThreads + threadIdx.x;
-            v[j] = i < nvec ? ld_stream16(xv + i) : make_uint4(0u, 0u, 0u, 0u);
+            v[j] = i >= nvec ? make_uint4(0u, 0u, 0u, 0u) : keep ? ld16(xv + i) : ld_stream16(xv + i);
         }
 #pragma unroll
         for (int j = 0; j < kVec; ++j) m = vec_absmax<BF16>(v[j], m);
@@ -108,12 +125,16 @@ __global__ void __launch_bounds__(kThreads)
 quantize_act_kernel(const void *__restrict__ x, size_t n, const float *__restrict__ max_dev, uint8_t *__restrict__ out)
 {
     constexpr int kPer = BF16 ? 8 : 4;
-    const float mx = __ldg(max_dev);
+    dep_wait();
+    dep_launch();
+    const float mx = *max_dev;
     const float inv = mx > 0.0f ? __fdiv_rn(255.0f, mx) : 0.0f;
     const size_t nvec = n / kPer;
     const uint4 *xv = reinterpret_cast<const uint4 *>(x);
     const size_t tile = (size_t)kThreads * kVec;
-    for (size_t base = (size_t)blockIdx.x * tile; base < nvec; base += (size_t)gridDim.x * tile) {
+    const size_t tiles = (nvec + tile - 1) / tile;
+    for (size_t t = blockIdx.x; t < tiles; t += gridDim.x) {
+        const size_t base = (tiles - 1 - t) * tile;            // from the end, which L2 still holds
         uint4 v[kVec];
         size_t idx[kVec];
 #pragma unroll
@@ -142,27 +163,63 @@ quantize_act_kernel(const void *__restrict__ x, size_t n, const float *__restric
             out[i] = (uint8_t)quant_u8_bits(elem<BF16>(x, i), inv);
 }
 
-// One block per kernel (output channel): its largest magnitude, then its int8 row.
+__device__ __forceinline__ int quant_s8(float w, float inv)
+{
+    const float z = fminf(fmaxf(__fmul_rn(w, inv), -127.0f), 127.0f);      // NaN -> -127 -> fixed below
+    return w != w ? 0 : __float2int_rn(z);
+}
+
+// One block per kernel (output channel): its largest magnitude, then its int8 row.  early: the weights are
+// no output of the previous launch, so they may be read while that is finishing.  VEC: rows are whole
+// 16-byte vectors, and the first kWeightVecs per thread stay in registers between the two steps, which
+// is the whole row up to 4608 values (512 filters of 3x3); what lies beyond is read again.
+constexpr int kWeightVecs = 5;
+template <bool VEC>
 __global__ void __launch_bounds__(kThreads)
-quantize_weight_kernel(const float *__restrict__ w, int64_t k, int8_t *__restrict__ out, float *__restrict__ scale_out)
+quantize_weight_kernel(const float *__restrict__ w, int64_t k, int8_t *__restrict__ out, float *__restrict__ scale_out, int early)
 {
     __shared__ uint32_t s_red[kThreads / 32];
     __shared__ float s_max;
+    if (!early) dep_wait();
     const float *row = w + (int64_t)blockIdx.x * k;
     int8_t *orow = out + (int64_t)blockIdx.x * k;
+    const uint4 *rv = reinterpret_cast<const uint4 *>(row);
+    const int64_t nv = VEC ? k / 4 : 0;
+    uint4 v[kWeightVecs];
     float m = 0.0f;
-    for (int64_t i = threadIdx.x; i < k; i += kThreads) m = fmaxf(m, fabsf(row[i]));
+    if (VEC) {
+#pragma unroll
+        for (int j = 0; j < kWeightVecs; ++j) {
+            const int64_t i = threadIdx.x + (int64_t)j * kThreads;
+            v[j] = i < nv ? ld16(rv + i) : make_uint4(0u, 0u, 0u, 0u);
+        }
+#pragma unroll
+        for (int j = 0; j < kWeightVecs; ++j) m = vec_absmax<false>(v[j], m);
+        for (int64_t i = threadIdx.x + kWeightVecs * kThreads; i < nv; i += kThreads) m = vec_absmax<false>(ld16(rv + i), m);
+    } else {
+        for (int64_t i = threadIdx.x; i < k; i += kThreads) m = fmaxf(m, fabsf(row[i]));
+    }
     const uint32_t b = block_max_bits(m, s_red);
     if (threadIdx.x == 0) s_max = __uint_as_float(b);
+    if (early) dep_wait();
+    dep_launch();
     __syncthreads();
     const float a = s_max;
     const float inv = a > 0.0f ? __fdiv_rn(127.0f, a) : 0.0f;
-    for (int64_t i = threadIdx.x; i < k; i += kThreads) {
-        float z = __fmul_rn(row[i], inv);
-        z = fminf(fmaxf(z, -127.0f), 127.0f);                 // NaN -> -127 -> fixed below
-        int q = __float2int_rn(z);
-        if (row[i] != row[i]) q = 0;
-        orow[i] = (int8_t)q;
+    if (VEC) {
+        auto put = [&](int64_t i, uint4 x) {
+            const uint32_t q = bytes4((uint32_t)quant_s8(__uint_as_float(x.x), inv), (uint32_t)quant_s8(__uint_as_float(x.y), inv),
+                                      (uint32_t)quant_s8(__uint_as_float(x.z), inv), (uint32_t)quant_s8(__uint_as_float(x.w), inv));
+            reinterpret_cast<uint32_t *>(orow)[i] = q;
+        };
+#pragma unroll
+        for (int j = 0; j < kWeightVecs; ++j) {
+            const int64_t i = threadIdx.x + (int64_t)j * kThreads;
+            if (i < nv) put(i, v[j]);
+        }
+        for (int64_t i = threadIdx.x + kWeightVecs * kThreads; i < nv; i += kThreads) put(i, ld16(rv + i));
+    } else {
+        for (int64_t i = threadIdx.x; i < k; i += kThreads) orow[i] = (int8_t)quant_s8(row[i], inv);
     }
     if (threadIdx.x == 0) scale_out[blockIdx.x] = __fdiv_rn(a, 127.0f);
 }
@@ -207,9 +264,9 @@ extern "C" int sparq_absmax(const void *x, int dtype, size_t n, float *max_inout
     int blocks = 0;
     if ((rc = stream_grid(n / (bf16 ? 8 : 4), &blocks)) != SPARQ_OK) return rc;
     cudaStream_t st = (cudaStream_t)stream;
-    if (bf16) absmax_kernel<true><<<blocks, kThreads, 0, st>>>(x, n, max_inout);
-    else absmax_kernel<false><<<blocks, kThreads, 0, st>>>(x, n, max_inout);
-    cudaError_t e = cudaGetLastError();
+    note_outputs(st, {{max_inout, sizeof(float)}, {nullptr, 0}, {nullptr, 0}});
+    const size_t nvec = n / (bf16 ? 8 : 4), keep_from = nvec > kKeepVecs ? nvec - kKeepVecs : 0;
+    const cudaError_t e = launch_overlapped(bf16 ? absmax_kernel<true> : absmax_kernel<false>, blocks, kThreads, 0, st, x, n, max_inout, keep_from);
     if (e != cudaSuccess) return cuda_error(e, "absmax_kernel launch");
     return SPARQ_OK;
 }
@@ -228,9 +285,8 @@ extern "C" int sparq_quantize_act_u8(const void *x, int dtype, size_t n, const f
     int blocks = 0;
     if ((rc = stream_grid(n / (bf16 ? 8 : 4), &blocks)) != SPARQ_OK) return rc;
     cudaStream_t st = (cudaStream_t)stream;
-    if (bf16) quantize_act_kernel<true><<<blocks, kThreads, 0, st>>>(x, n, max_dev, out);
-    else quantize_act_kernel<false><<<blocks, kThreads, 0, st>>>(x, n, max_dev, out);
-    cudaError_t e = cudaGetLastError();
+    note_outputs(st, {{out, n}, {nullptr, 0}, {nullptr, 0}});
+    const cudaError_t e = launch_overlapped(bf16 ? quantize_act_kernel<true> : quantize_act_kernel<false>, blocks, kThreads, 0, st, x, n, max_dev, out);
     if (e != cudaSuccess) return cuda_error(e, "quantize_act_kernel launch");
     return SPARQ_OK;
 }
@@ -244,8 +300,12 @@ extern "C" int sparq_quantize_weight_s8(const float *w, int64_t cout, int64_t k,
     if (cout > 2147483647LL) return set_error(SPARQ_ERR_UNSUPPORTED, "more than 2^31-1 kernels");
     if (((uintptr_t)w | (uintptr_t)scale_out) & 3u)
         return set_error(SPARQ_ERR_UNSUPPORTED, "w and scale_out must be 4-byte aligned");
-    quantize_weight_kernel<<<(unsigned)cout, kThreads, 0, (cudaStream_t)stream>>>(w, k, out, scale_out);
-    cudaError_t e = cudaGetLastError();
+    cudaStream_t st = (cudaStream_t)stream;
+    const bool early = note_outputs(st, {{out, (size_t)cout * (size_t)k}, {scale_out, (size_t)cout * sizeof(float)}, {nullptr, 0}},
+                                    w, (size_t)cout * (size_t)k * sizeof(float));
+    const bool vec = k % 4 == 0 && ((uintptr_t)w & 15u) == 0 && ((uintptr_t)out & 3u) == 0;
+    const cudaError_t e = launch_overlapped(vec ? quantize_weight_kernel<true> : quantize_weight_kernel<false>, (int)cout, kThreads, 0, st,
+                                            w, k, out, scale_out, (int)early);
     if (e != cudaSuccess) return cuda_error(e, "quantize_weight_kernel launch");
     return SPARQ_OK;
 }

@@ -213,3 +213,31 @@ def test_sparse24_fused(m, n, k, nb, mask, rnd):
     want = oracle.gemm_sparse24(A[rows], vals, pos, p.mode, nb, mask, rnd)
     assert np.array_equal(got[:-16].reshape(m, n)[rows], want)
     assert (got[-16:] == -7).all()
+
+
+@pytest.mark.parametrize("cout,k", [(1, 4), (3, 5), (7, 1020), (5, 5120), (4, 5124), (3, 9001), (130, 64)])
+def test_quantize_weight_rows(cout, k):
+    """Row lengths around what a block keeps in registers, with and without whole vectors."""
+    w = np.random.default_rng(cout + k).standard_normal((cout, k)).astype(np.float32)
+    w[0, 0] = np.nan
+    out = torch.full((cout * k + 16,), 99, dtype=torch.int8, device="cuda")
+    sc = torch.zeros(cout, device="cuda")
+    sparq.sparq_quantize_weight_s8(torch.from_numpy(w).cuda(), out, sc)
+    want_q, want_s = oracle.quantize_weight(w)
+    got = out.cpu().numpy()
+    assert np.array_equal(got[:-16].reshape(cout, k), want_q) and (got[-16:] == 99).all()
+    assert np.array_equal(sc.cpu().numpy(), want_s)
+
+
+@pytest.mark.parametrize("n", [7, 4096, (64 << 20) // 4 + 4096 * 3 + 5])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_calibration_passes(n, dtype):
+    """Maximum and quantization of one tensor, beyond the part that the first pass leaves in L2."""
+    x = torch.randn(n, device="cuda").to(dtype)
+    mx, q = torch.zeros(1, device="cuda"), torch.full((n + 16,), 7, dtype=torch.uint8, device="cuda")
+    sparq.sparq_absmax(x, mx)
+    sparq.sparq_quantize_act_u8(x, mx, q)
+    xh = x.float().cpu().numpy()
+    assert mx.item() == oracle.absmax(xh)
+    got = q.cpu().numpy()
+    assert np.array_equal(got[:n], oracle.quantize_act(xh, mx.item())) and (got[n:] == 7).all()
