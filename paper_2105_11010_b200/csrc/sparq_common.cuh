@@ -275,15 +275,36 @@ __device__ __forceinline__ uint32_t xform_word_fullset(uint32_t x, const XformDe
 }
 
 // The transform of a fused kernel instantiated for (MODE, XN, RND): XN = 4 is n = 4 with all
-// five placements (packed-integer form, width fixed at compile time), XN = 8 any other full
-// placement set (6opt, 7opt; either rounding, through the constants; RND unused), XN = 0 the
-// general packed-integer form with run-time width and the placement widening.
+// five placements (packed-integer form, width fixed at compile time), XN = 5 the same with the
+// placement widening (any restricted set of n = 4: 3opt, 2opt), XN = 8 any other full placement set
+// (6opt, 7opt; either rounding, through the constants; RND unused), XN = 0 the general
+// packed-integer form with run-time width and the placement widening (restricted sets of n < 4).
 template <int MODE, int XN, bool RND>
 __device__ __forceinline__ uint32_t xform_fused(uint32_t x, const XformDev &d)
 {
     if (XN == 8) return xform_word_fullset<MODE>(x, d);
     if (XN == 4) return xform_word<MODE, 4, RND, false>(x, d);
+    if (XN == 5) return xform_word<MODE, 4, RND, true>(x, d);
     return xform_word<MODE, 0, RND, true>(x, d);
+}
+
+// The two values that vSPARQ chooses between for each of four activations, whatever pairs they form: q,
+// its own window, and l, what it keeps beside a zero (the whole byte for n = 4).  XN as above.
+template <int XN, bool RND>
+__device__ __forceinline__ void window_and_lone(uint32_t x, const XformDev &d, uint32_t &q, uint32_t &l)
+{
+    q = xform_fused<SPARQ_MODE_BSPARQ, XN, RND>(x, d);
+    l = x;
+    if (XN != 4 && XN != 5) {
+        if (XN == 8) {
+            const uint32_t k1024 = 0x64006400u;
+            const uint32_t lo = h2_sub(prmt(x, 0x64646464u, 0x4140u), k1024), hi = h2_sub(prmt(x, 0x64646464u, 0x4342u), k1024);
+            l = prmt(h2_add(h2_min((lo + d.l_add) & d.l_mask, d.l_sat), k1024),
+                     h2_add(h2_min((hi + d.l_add) & d.l_mask, d.l_sat), k1024), 0x6420u);
+        } else {
+            l = apply_mask<RND>(x, drop_mask<0, false>(x, 2 * d.n, 0u), 2 * d.n);
+        }
+    }
 }
 #endif
 

@@ -102,6 +102,7 @@ cudaError_t launch_expand_act(const uint4 *in, uint4 *out, size_t nvec, const Xf
     XformDev d{a.widen_c, a.widen_rounds, a.n};
     fill_fullset(&d, a.n, a.rnd);
     auto go = [&](auto kernel) { return launch_overlapped(kernel, blocks, kThreads, 0, st, in, out, nvec, d); };
+    if (a.widen_rounds > 0 && a.n == 4) return a.rnd ? go(expand_act_kernel<5, true>) : go(expand_act_kernel<5, false>);
     if (a.widen_rounds > 0) return a.rnd ? go(expand_act_kernel<0, true>) : go(expand_act_kernel<0, false>);
     if (a.n != 4) return go(expand_act_kernel<8, true>);
     return a.rnd ? go(expand_act_kernel<4, true>) : go(expand_act_kernel<4, false>);

@@ -241,3 +241,19 @@ def test_calibration_passes(n, dtype):
     assert mx.item() == oracle.absmax(xh)
     got = q.cpu().numpy()
     assert np.array_equal(got[:n], oracle.quantize_act(xh, mx.item())) and (got[n:] == 7).all()
+
+
+@pytest.mark.parametrize("rows,row_len", [(1, 17), (1, 31), (5, 17), (64, 19), (333, 33), (7, 4097), (1000, 1023), (3, 15), (257, 101)])
+@pytest.mark.parametrize("n,mask,rnd", [(4, 0x1F, 1), (4, 0x1F, 0), (4, 0x15, 1), (3, 0x3F, 1), (3, 0x29, 0), (2, 0x7F, 0)])
+def test_transform_odd_rows(rows, row_len, n, mask, rnd):
+    """Row boundaries at every place of a vector, a last partial vector, and in place."""
+    x = synth.activations(rows + row_len, (rows, row_len), 0.4)
+    p = sparq.SparqParams(sparq.MODE_VSPARQ, n, mask, rnd)
+    want = oracle.transform(x, p.mode, n, mask, rnd).reshape(-1)
+    xd = torch.from_numpy(x).cuda().reshape(-1)
+    out = torch.full((x.size + 16,), 0xA5, dtype=torch.uint8, device="cuda")
+    sparq.sparq_quantize(xd, out, rows, row_len, p)
+    got = out.cpu().numpy()
+    assert np.array_equal(got[:-16], want) and (got[-16:] == 0xA5).all()
+    sparq.sparq_quantize(xd, xd, rows, row_len, p)
+    assert np.array_equal(xd.cpu().numpy(), want)
