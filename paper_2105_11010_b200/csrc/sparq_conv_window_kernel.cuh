@@ -152,7 +152,7 @@ struct GroupWalk {
     }
 };
 
-template <int BN, int CB, int MODE, int XN, bool RND, bool B_RESIDENT>
+template <int BN, int CB, int MODE, int XN, bool RND, bool B_RESIDENT, bool LEAN>
 __global__ void __launch_bounds__(kWindowThreads, 1)
 sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __grid_constant__ CUtensorMap map_x1,
                          const __grid_constant__ CUtensorMap map_w, const WindowArgs g)
@@ -548,7 +548,7 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
                 const bool row_ok = slot_ok && (oh < g.Ho);
                 const int64_t row = ((int64_t)walk.img * g.Ho + oh) * g.Wo + ow;
                 const uint32_t taddr0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + (uint32_t)cbase;
-                epi_warp_columns(ev, taddr0, cbase, cols, row, row_ok, nt * BN, s_scale, s_bias,
+                epi_warp_columns<LEAN>(ev, taddr0, cbase, cols, row, row_ok, nt * BN, s_scale, s_bias,
                                  smem_u32(&bar_acc_empty[acc]), lane, [&]() {
                                      mbar_wait(smem_u32(&bar_acc_full[acc]), acc_use & 1u, abort_flag, g.status, g.wait_limit);
                                      tc_fence_after();
@@ -620,21 +620,27 @@ template <int BN, int CB, bool B_RESIDENT>
 cudaError_t launch_window_shape(const CUtensorMap &mx0, const CUtensorMap &mx1, const CUtensorMap &mw, const WindowArgs &g,
                                 int mode, int n, int rnd, int grid, int smem_bytes, cudaStream_t st);
 
+template <int BN, int CB, int MODE, int XN, bool RND, bool RES, bool LEAN>
+cudaError_t launch_window_kernel(const CUtensorMap &mx0, const CUtensorMap &mx1, const CUtensorMap &mw, const WindowArgs &g,
+                                 int grid, int smem_bytes, cudaStream_t st)
+{
+    auto kfn = sparq_conv_window_kernel<BN, CB, MODE, XN, RND, RES, LEAN>;
+    static bool attr_set[64] = {};   // per device ordinal
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64 || !attr_set[dev]) {
+        e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, RES ? kWindowMaxDynSmem : kWindowMaxDynSmemStreamed);
+        if (e != cudaSuccess) return e;
+        if (dev >= 0 && dev < 64) attr_set[dev] = true;
+    }
+    return launch_overlapped(kfn, grid, kWindowThreads, smem_bytes, st, mx0, mx1, mw, g);
+}
+
 #define SPARQ_LAUNCH_WINDOW_VARIANT(MODE_, XN_, RND_)                                                  \
-    do {                                                                                               \
-        auto kfn = sparq_conv_window_kernel<BN, CB, MODE_, XN_, RND_, RES>;                            \
-        static bool attr_set[64] = {};   /* per device ordinal */                                     \
-        int dev_ = 0;                                                                                  \
-        cudaError_t e_ = cudaGetDevice(&dev_);                                                         \
-        if (e_ != cudaSuccess) return e_;                                                              \
-        if (dev_ < 0 || dev_ >= 64 || !attr_set[dev_]) {                                               \
-            e_ = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize,                \
-                                      RES ? kWindowMaxDynSmem : kWindowMaxDynSmemStreamed);            \
-            if (e_ != cudaSuccess) return e_;                                                          \
-            if (dev_ >= 0 && dev_ < 64) attr_set[dev_] = true;                                         \
-        }                                                                                              \
-        return launch_overlapped(kfn, grid, kWindowThreads, smem_bytes, st, mx0, mx1, mw, g);         \
-    } while (0)
+    return make_epi_view(g).lean                                                                       \
+               ? launch_window_kernel<BN, CB, MODE_, XN_, RND_, RES, true>(mx0, mx1, mw, g, grid, smem_bytes, st)   \
+               : launch_window_kernel<BN, CB, MODE_, XN_, RND_, RES, false>(mx0, mx1, mw, g, grid, smem_bytes, st)
 
 #define SPARQ_DEFINE_WINDOW_SHAPE(BN_, CB_, RES_)                                                      \
     template <>                                                                                        \
@@ -648,12 +654,16 @@ cudaError_t launch_window_shape(const CUtensorMap &mx0, const CUtensorMap &mx1, 
         if (mode == SPARQ_MODE_NONE) SPARQ_LAUNCH_WINDOW_VARIANT(SPARQ_MODE_NONE, 4, false);           \
         if (mode == SPARQ_MODE_BSPARQ) {                                                               \
             if (n == 8) SPARQ_LAUNCH_WINDOW_VARIANT(SPARQ_MODE_BSPARQ, 8, true);                       \
+            if (n == 5) { if (rnd) SPARQ_LAUNCH_WINDOW_VARIANT(SPARQ_MODE_BSPARQ, 5, true);            \
+                          else SPARQ_LAUNCH_WINDOW_VARIANT(SPARQ_MODE_BSPARQ, 5, false); }             \
             if (n == 4) { if (rnd) SPARQ_LAUNCH_WINDOW_VARIANT(SPARQ_MODE_BSPARQ, 4, true);            \
                           else SPARQ_LAUNCH_WINDOW_VARIANT(SPARQ_MODE_BSPARQ, 4, false); }             \
             if (rnd) SPARQ_LAUNCH_WINDOW_VARIANT(SPARQ_MODE_BSPARQ, 0, true);                          \
             else SPARQ_LAUNCH_WINDOW_VARIANT(SPARQ_MODE_BSPARQ, 0, false);                             \
         }                                                                                              \
         if (n == 8) SPARQ_LAUNCH_WINDOW_VARIANT(SPARQ_MODE_VSPARQ, 8, true);                           \
+        if (n == 5) { if (rnd) SPARQ_LAUNCH_WINDOW_VARIANT(SPARQ_MODE_VSPARQ, 5, true);                \
+                      else SPARQ_LAUNCH_WINDOW_VARIANT(SPARQ_MODE_VSPARQ, 5, false); }                 \
         if (n == 4) { if (rnd) SPARQ_LAUNCH_WINDOW_VARIANT(SPARQ_MODE_VSPARQ, 4, true);                \
                       else SPARQ_LAUNCH_WINDOW_VARIANT(SPARQ_MODE_VSPARQ, 4, false); }                 \
         if (rnd) SPARQ_LAUNCH_WINDOW_VARIANT(SPARQ_MODE_VSPARQ, 0, true);                              \

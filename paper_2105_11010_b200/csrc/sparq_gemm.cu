@@ -310,9 +310,9 @@ static bool record_launch_weights_clear(cudaStream_t st, const sparq_epilogue *e
     return note_outputs(st, {{e->acc_out, 4 * out_elems}, {e->f32_out, 4 * out_elems}, {e->u8_out, out_elems}}, wgt, wgt_bytes);
 }
 
-// Variant argument of the launchers: 4 = n = 4 with all five placements, 8 = another full
-// placement set (6opt, 7opt), 0 = the general kernels.
-static int variant_n(const XformArgs &x) { return x.widen_rounds != 0 ? 0 : (x.n == 4 ? 4 : 8); }
+// Variant argument of the launchers (XN of xform_fused): 4 = n = 4 with all five placements, 5 = n = 4
+// with fewer, 8 = another full placement set (6opt, 7opt), 0 = restricted sets of n < 4.
+static int variant_n(const XformArgs &x) { return x.n == 4 ? (x.widen_rounds ? 5 : 4) : (x.widen_rounds ? 0 : 8); }
 
 // Kernel-side transform constants.
 static XformDev xform_dev(const XformArgs &x)

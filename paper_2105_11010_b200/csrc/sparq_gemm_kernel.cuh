@@ -707,15 +707,21 @@ __device__ __forceinline__ void epi_warp_columns_as(const EpiView &e, uint32_t t
     }
 }
 
-template <class WaitFull>
+// LEAN: the kernel is instantiated for requantized bytes only (EpiView::lean), else for everything else.
+// One kernel with both was slower wherever launches of different layers follow one another: the warp
+// roles share the instruction caches, and every kernel starts with cold ones.
+template <bool LEAN, class WaitFull>
 __device__ __forceinline__ void epi_warp_columns(const EpiView &e, uint32_t taddr0, int cbase, int cols, int64_t row, bool row_ok,
                                                  int64_t n0, const float *s_scale, const float *s_bias,
                                                  uint32_t acc_empty_bar, int lane, WaitFull wait_full)
 {
-    if (e.gran == 1) epi_warp_columns_as<kEpiGeneralOdd>(e, taddr0, cbase, cols, row, row_ok, n0, s_scale, s_bias, acc_empty_bar, lane, wait_full);
-    else if (!e.lean) epi_warp_columns_as<kEpiGeneral>(e, taddr0, cbase, cols, row, row_ok, n0, s_scale, s_bias, acc_empty_bar, lane, wait_full);
-    else if (e.residual) epi_warp_columns_as<kEpiLeanResidual>(e, taddr0, cbase, cols, row, row_ok, n0, s_scale, s_bias, acc_empty_bar, lane, wait_full);
-    else epi_warp_columns_as<kEpiLean>(e, taddr0, cbase, cols, row, row_ok, n0, s_scale, s_bias, acc_empty_bar, lane, wait_full);
+    if constexpr (LEAN) {
+        if (e.residual) epi_warp_columns_as<kEpiLeanResidual>(e, taddr0, cbase, cols, row, row_ok, n0, s_scale, s_bias, acc_empty_bar, lane, wait_full);
+        else epi_warp_columns_as<kEpiLean>(e, taddr0, cbase, cols, row, row_ok, n0, s_scale, s_bias, acc_empty_bar, lane, wait_full);
+    } else {
+        if (e.gran == 1) epi_warp_columns_as<kEpiGeneralOdd>(e, taddr0, cbase, cols, row, row_ok, n0, s_scale, s_bias, acc_empty_bar, lane, wait_full);
+        else epi_warp_columns_as<kEpiGeneral>(e, taddr0, cbase, cols, row, row_ok, n0, s_scale, s_bias, acc_empty_bar, lane, wait_full);
+    }
 }
 
 // One box of the staged output: this thread's row of `box` (64 or 128) columns, from tensor memory to
@@ -791,7 +797,7 @@ struct TileCfg {
     static constexpr int kTmemCols = kAcc * BN;
 };
 
-template <int BN, int BK, int MODE, int XN, bool RND>
+template <int BN, int BK, int MODE, int XN, bool RND, bool LEAN>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                   const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_res, const GemmArgs g)
@@ -962,7 +968,7 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         const EpiView ev = make_epi_view(g);
         int64_t staged_nt = -1;
         uint32_t local_tile = (uint32_t)team;
-        if (g.out_box) {
+        if (LEAN && g.out_box) {
             // ---- through shared memory (see epi_staged_box) ----
             const int ew = warp - kFirstEpiWarp;
             const uint32_t box_bytes = 32u * (uint32_t)g.out_box;
@@ -1042,7 +1048,7 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
             }
             const int64_t row = mt * kBM + quarter * 32 + lane;
             const uint32_t taddr0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * BN + cbase);
-            epi_warp_columns(ev, taddr0, cbase, cols, row, row < g.M, nt * BN, s_scale[team], s_bias[team],
+            epi_warp_columns<LEAN>(ev, taddr0, cbase, cols, row, row < g.M, nt * BN, s_scale[team], s_bias[team],
                              smem_u32(&bar_acc_empty[acc]), lane, [&]() {
                                  mbar_wait(smem_u32(&bar_acc_full[acc]), acc_use & 1, abort_flag, g.status, g.wait_limit);
                                  tc_fence_after();
@@ -1112,24 +1118,28 @@ struct GemmMaps {
 template <int BN, int BK>
 cudaError_t launch_gemm_shape(const GemmMaps &m, GemmArgs &g, int mode, int n, int rnd, int grid, cudaStream_t st);
 
+template <int BN, int BK, int MODE, int XN, bool RND, bool LEAN>
+cudaError_t launch_gemm_kernel(const GemmMaps &m, GemmArgs &g, int grid, cudaStream_t st)
+{
+    auto kfn = sparq_gemm_kernel<BN, BK, MODE, XN, RND, LEAN>;
+    static bool attr_set[64] = {};   // per device ordinal
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64 || !attr_set[dev]) {
+        e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmemGemm);
+        if (e != cudaSuccess) return e;
+        if (dev >= 0 && dev < 64) attr_set[dev] = true;
+    }
+    const int staging = g.out_box ? epi_warps(MODE) * 2 * 32 * g.out_box : 0;
+    g.stages = TileCfg<BN, BK>::stages(staging);
+    const int smem = 1024 + g.stages * TileCfg<BN, BK>::kStageBytes + staging;
+    return launch_overlapped(kfn, grid, kGemmThreads, smem, st, m.a, m.b, m.out, m.res, g);
+}
+
 #define SPARQ_LAUNCH_VARIANT(MODE_, XN_, RND_)                                                         \
-    do {                                                                                               \
-        auto kfn = sparq_gemm_kernel<BN, BK, MODE_, XN_, RND_>;                                        \
-        static bool attr_set[64] = {};   /* per device ordinal */                                     \
-        int dev_ = 0;                                                                                  \
-        cudaError_t e_ = cudaGetDevice(&dev_);                                                         \
-        if (e_ != cudaSuccess) return e_;                                                              \
-        if (dev_ < 0 || dev_ >= 64 || !attr_set[dev_]) {                                               \
-            e_ = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize,                \
-                                      kMaxDynSmemGemm);                                                \
-            if (e_ != cudaSuccess) return e_;                                                          \
-            if (dev_ >= 0 && dev_ < 64) attr_set[dev_] = true;                                         \
-        }                                                                                              \
-        const int staging_ = g.out_box ? epi_warps(MODE_) * 2 * 32 * g.out_box : 0;                    \
-        g.stages = TileCfg<BN, BK>::stages(staging_);                                                  \
-        const int smem_ = 1024 + g.stages * TileCfg<BN, BK>::kStageBytes + staging_;                   \
-        return launch_overlapped(kfn, grid, kGemmThreads, smem_, st, m.a, m.b, m.out, m.res, g);       \
-    } while (0)
+    return make_epi_view(g).lean ? launch_gemm_kernel<BN, BK, MODE_, XN_, RND_, true>(m, g, grid, st)  \
+                                 : launch_gemm_kernel<BN, BK, MODE_, XN_, RND_, false>(m, g, grid, st)
 
 #define SPARQ_DEFINE_GEMM_SHAPE(BN_, BK_)                                                              \
     template <>                                                                                        \
@@ -1140,12 +1150,16 @@ cudaError_t launch_gemm_shape(const GemmMaps &m, GemmArgs &g, int mode, int n, i
         if (mode == SPARQ_MODE_NONE) SPARQ_LAUNCH_VARIANT(SPARQ_MODE_NONE, 4, false);                  \
         if (mode == SPARQ_MODE_BSPARQ) {                                                               \
             if (n == 8) SPARQ_LAUNCH_VARIANT(SPARQ_MODE_BSPARQ, 8, true);                              \
+            if (n == 5) { if (rnd) SPARQ_LAUNCH_VARIANT(SPARQ_MODE_BSPARQ, 5, true);                   \
+                          else SPARQ_LAUNCH_VARIANT(SPARQ_MODE_BSPARQ, 5, false); }                    \
             if (n == 4) { if (rnd) SPARQ_LAUNCH_VARIANT(SPARQ_MODE_BSPARQ, 4, true);                   \
                           else SPARQ_LAUNCH_VARIANT(SPARQ_MODE_BSPARQ, 4, false); }                    \
             if (rnd) SPARQ_LAUNCH_VARIANT(SPARQ_MODE_BSPARQ, 0, true);                                 \
             else SPARQ_LAUNCH_VARIANT(SPARQ_MODE_BSPARQ, 0, false);                                    \
         }                                                                                              \
         if (n == 8) SPARQ_LAUNCH_VARIANT(SPARQ_MODE_VSPARQ, 8, true);                                  \
+        if (n == 5) { if (rnd) SPARQ_LAUNCH_VARIANT(SPARQ_MODE_VSPARQ, 5, true);                       \
+                      else SPARQ_LAUNCH_VARIANT(SPARQ_MODE_VSPARQ, 5, false); }                        \
         if (n == 4) { if (rnd) SPARQ_LAUNCH_VARIANT(SPARQ_MODE_VSPARQ, 4, true);                       \
                       else SPARQ_LAUNCH_VARIANT(SPARQ_MODE_VSPARQ, 4, false); }                        \
         if (rnd) SPARQ_LAUNCH_VARIANT(SPARQ_MODE_VSPARQ, 0, true);                                     \

@@ -290,7 +290,7 @@ sparq_gemm_small_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
                 asm volatile("bar.sync 1, %0;" :: "n"(kSmallWorkers * 32) : "memory");
             }
             // (handing the accumulator back is not needed here: the barrier named is never waited for)
-            epi_warp_columns(ev, taddr, cbase, 32, m0 + trow, trow < rows_left, n0, s_scale, s_bias, smem_u32(&bar_recv), lane, wait_acc);
+            epi_warp_columns<true>(ev, taddr, cbase, 32, m0 + trow, trow < rows_left, n0, s_scale, s_bias, smem_u32(&bar_recv), lane, wait_acc);
         } else {
             // residual bytes of this thread's four columns of the CTA's row lrow
             auto residual_of = [&](int lrow) {
@@ -402,12 +402,16 @@ cudaError_t launch_gemm_small_kernel(const GemmMaps &m, GemmArgs &g, int grid, c
         if (mode == SPARQ_MODE_NONE) SPARQ_LAUNCH_SMALL(SPARQ_MODE_NONE, 4, false);                    \
         if (mode == SPARQ_MODE_BSPARQ) {                                                               \
             if (n == 8) SPARQ_LAUNCH_SMALL(SPARQ_MODE_BSPARQ, 8, true);                                \
+            if (n == 5 && rnd) SPARQ_LAUNCH_SMALL(SPARQ_MODE_BSPARQ, 5, true);                         \
+            if (n == 5) SPARQ_LAUNCH_SMALL(SPARQ_MODE_BSPARQ, 5, false);                               \
             if (n == 4 && rnd) SPARQ_LAUNCH_SMALL(SPARQ_MODE_BSPARQ, 4, true);                         \
             if (n == 4) SPARQ_LAUNCH_SMALL(SPARQ_MODE_BSPARQ, 4, false);                               \
             if (rnd) SPARQ_LAUNCH_SMALL(SPARQ_MODE_BSPARQ, 0, true);                                   \
             SPARQ_LAUNCH_SMALL(SPARQ_MODE_BSPARQ, 0, false);                                           \
         }                                                                                              \
         if (n == 8) SPARQ_LAUNCH_SMALL(SPARQ_MODE_VSPARQ, 8, true);                                    \
+        if (n == 5 && rnd) SPARQ_LAUNCH_SMALL(SPARQ_MODE_VSPARQ, 5, true);                             \
+        if (n == 5) SPARQ_LAUNCH_SMALL(SPARQ_MODE_VSPARQ, 5, false);                                   \
         if (n == 4 && rnd) SPARQ_LAUNCH_SMALL(SPARQ_MODE_VSPARQ, 4, true);                             \
         if (n == 4) SPARQ_LAUNCH_SMALL(SPARQ_MODE_VSPARQ, 4, false);                                   \
         if (rnd) SPARQ_LAUNCH_SMALL(SPARQ_MODE_VSPARQ, 0, true);                                       \

@@ -23,6 +23,7 @@ template <int BN>
 static cudaError_t launch_x24_bn(const CUtensorMap &ma, const CUtensorMap &mb, const GemmArgs &g, int n, int rnd, int grid, cudaStream_t st)
 {
     if (n == 8) return launch_x24_kernel<BN, 8, true>(ma, mb, g, grid, st);
+    if (n == 5) return rnd ? launch_x24_kernel<BN, 5, true>(ma, mb, g, grid, st) : launch_x24_kernel<BN, 5, false>(ma, mb, g, grid, st);
     if (n == 4) return rnd ? launch_x24_kernel<BN, 4, true>(ma, mb, g, grid, st) : launch_x24_kernel<BN, 4, false>(ma, mb, g, grid, st);
     return rnd ? launch_x24_kernel<BN, 0, true>(ma, mb, g, grid, st) : launch_x24_kernel<BN, 0, false>(ma, mb, g, grid, st);
 }

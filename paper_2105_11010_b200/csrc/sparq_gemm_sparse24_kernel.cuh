@@ -178,10 +178,13 @@ sparq_gemm_sparse24_kernel(const __grid_constant__ CUtensorMap map_a, const __gr
             for (int h = 0; h < 2; ++h) {
                 const int64_t row = (int64_t)mt * kX24Rows + h * kBM + quarter * 32 + lane;
                 const uint32_t taddr0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * (uint32_t)(2 * BN) + (uint32_t)(h * BN);
-                epi_warp_columns(ev, taddr0, 0, BN, row, row < g.M, nt * BN, s_scale, s_bias, smem_u32(&bar_acc_empty[acc]), lane, [&]() {
+                auto wait_full = [&]() {
                     mbar_wait(smem_u32(&bar_acc_full[acc]), ph, abort_flag, g.status, g.wait_limit);
                     tc_fence_after();
-                });
+                };
+                const uint32_t empty = smem_u32(&bar_acc_empty[acc]);
+                if (ev.lean) epi_warp_columns<true>(ev, taddr0, 0, BN, row, row < g.M, nt * BN, s_scale, s_bias, empty, lane, wait_full);
+                else epi_warp_columns<false>(ev, taddr0, 0, BN, row, row < g.M, nt * BN, s_scale, s_bias, empty, lane, wait_full);
             }
         }
     } else {
