@@ -360,7 +360,7 @@ static int fill_common(GemmArgs *g, const XformArgs &x, const sparq_epilogue *e,
 static int output_maps(GemmMaps *m, GemmArgs *g, int mode, int bn, int64_t tiles, int grid)
 {
     g->out_box = 0;
-    if (!make_epi_view(*g).lean || tiles <= grid) return SPARQ_OK;
+    if (make_epi_view(*g).out == kOutGeneral || tiles <= grid) return SPARQ_OK;
     const int64_t out_bytes = (int64_t)kBM * bn * (g->residual ? 2 : 1), operand_bytes = (int64_t)(kBM + bn) * g->K;
     if (8 * out_bytes < 5 * operand_bytes) return SPARQ_OK;
     const int groups = epi_warps(mode) / 4, acc = bn == 256 ? 2 : 4;

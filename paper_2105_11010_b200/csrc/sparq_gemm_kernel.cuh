@@ -389,13 +389,21 @@ struct EpiView {
     bool need_f;      // a dequantized output is requested
     bool relu_op;     // the ReLU select has to be executed (see below)
     int gran;         // bytes (columns) that one access to a u8 row may take: 32, 16, 8, 4 or 1, whichever divides N
-    bool lean;        // gran = 32, and only requantized bytes are wanted: see epi_lean
+    int out;          // EpiOut: which instantiation of a kernel the launch takes
     int next_mode;    // SPARQ mode applied to the requantized bytes (producer-side transform)
     int next_rnd;
     XformDev next_xf;
     const uint8_t *residual;   // u8 identity tensor added before the ReLU, or nullptr
     float residual_scale;
 };
+
+// The kernels are instantiated per kind of output: requantized bytes only, in whole groups of 32
+// columns (epi_lean), the same with a residual, and everything else.  One kernel with all of them
+// was slower on every layer: the warp roles share the instruction caches, every kernel starts with
+// cold ones, and the code that a launch does not run still spreads the code it does over more
+// lines (and takes registers: the largest role decides for all).  128x28x28x128 -> 128 3x3:
+// 17.5 -> 16.9 us without the residual's code, 32x56x56x64 -> 64 10.75 -> 10.45.
+enum EpiOut { kOutGeneral, kOutBytes, kOutResidual };
 
 template <class Args>
 __host__ __device__ __forceinline__ EpiView make_epi_view(const Args &g)
@@ -413,7 +421,8 @@ __host__ __device__ __forceinline__ EpiView make_epi_view(const Args &g)
     const bool aligned32 = ((reinterpret_cast<uintptr_t>(g.u8_out) | reinterpret_cast<uintptr_t>(g.f32_out) |
                              reinterpret_cast<uintptr_t>(g.acc_out) | reinterpret_cast<uintptr_t>(g.residual)) & 31u) == 0;
     e.gran = g.N % 32 == 0 && aligned32 ? 32 : g.N % 16 == 0 ? 16 : g.N % 8 == 0 ? 8 : g.N % 4 == 0 ? 4 : 1;
-    e.lean = e.u8_out && !g.acc_out && !g.f32_out && g.next_mode == SPARQ_MODE_NONE && !e.relu_op && e.gran == 32;
+    const bool bytes_only = e.u8_out && !g.acc_out && !g.f32_out && g.next_mode == SPARQ_MODE_NONE && !e.relu_op && e.gran == 32;
+    e.out = !bytes_only ? kOutGeneral : g.residual ? kOutResidual : kOutBytes;
     e.next_mode = g.next_mode;
     e.next_rnd = g.next_rnd;
     e.next_xf = g.next_xf;
@@ -707,17 +716,15 @@ __device__ __forceinline__ void epi_warp_columns_as(const EpiView &e, uint32_t t
     }
 }
 
-// LEAN: the kernel is instantiated for requantized bytes only (EpiView::lean), else for everything else.
-// One kernel with both was slower wherever launches of different layers follow one another: the warp
-// roles share the instruction caches, and every kernel starts with cold ones.
-template <bool LEAN, class WaitFull>
+// OUT: the kind of output that the kernel is instantiated for (EpiOut).
+template <int OUT, class WaitFull>
 __device__ __forceinline__ void epi_warp_columns(const EpiView &e, uint32_t taddr0, int cbase, int cols, int64_t row, bool row_ok,
                                                  int64_t n0, const float *s_scale, const float *s_bias,
                                                  uint32_t acc_empty_bar, int lane, WaitFull wait_full)
 {
-    if constexpr (LEAN) {
-        if (e.residual) epi_warp_columns_as<kEpiLeanResidual>(e, taddr0, cbase, cols, row, row_ok, n0, s_scale, s_bias, acc_empty_bar, lane, wait_full);
-        else epi_warp_columns_as<kEpiLean>(e, taddr0, cbase, cols, row, row_ok, n0, s_scale, s_bias, acc_empty_bar, lane, wait_full);
+    if constexpr (OUT != kOutGeneral) {
+        epi_warp_columns_as<OUT == kOutResidual ? kEpiLeanResidual : kEpiLean>(e, taddr0, cbase, cols, row, row_ok, n0, s_scale, s_bias,
+                                                                               acc_empty_bar, lane, wait_full);
     } else {
         if (e.gran == 1) epi_warp_columns_as<kEpiGeneralOdd>(e, taddr0, cbase, cols, row, row_ok, n0, s_scale, s_bias, acc_empty_bar, lane, wait_full);
         else epi_warp_columns_as<kEpiGeneral>(e, taddr0, cbase, cols, row, row_ok, n0, s_scale, s_bias, acc_empty_bar, lane, wait_full);
@@ -797,7 +804,7 @@ struct TileCfg {
     static constexpr int kTmemCols = kAcc * BN;
 };
 
-template <int BN, int BK, int MODE, int XN, bool RND, bool LEAN>
+template <int BN, int BK, int MODE, int XN, bool RND, int OUT>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                   const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_res, const GemmArgs g)
@@ -968,12 +975,12 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         const EpiView ev = make_epi_view(g);
         int64_t staged_nt = -1;
         uint32_t local_tile = (uint32_t)team;
-        if (LEAN && g.out_box) {
+        if (OUT != kOutGeneral && g.out_box) {
             // ---- through shared memory (see epi_staged_box) ----
             const int ew = warp - kFirstEpiWarp;
             const uint32_t box_bytes = 32u * (uint32_t)g.out_box;
             const uint32_t stage0 = smem_base + (uint32_t)(S * Cfg::kStageBytes) + (uint32_t)ew * 2u * box_bytes;
-            const bool res = g.residual != nullptr;
+            constexpr bool res = OUT == kOutResidual;
             // boxes of this warp in order: the out_box-wide parts of its columns, tile after tile
             auto fetch = [&](uint32_t n, uint32_t tile, int c) {          // box n's residual, by lane 0
                 const uint32_t mt = (n_tiles32 == 1) ? tile : tile / n_tiles32;
@@ -1015,8 +1022,7 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                     }
                     const float *sc = s_scale[team] + cbase + c, *bi = s_bias[team] + cbase + c;
                     const uint32_t abar = last ? smem_u32(&bar_acc_empty[acc]) : 0u;
-                    if (res) epi_staged_box<true>(taddr0 + (uint32_t)c, g.out_box, buf, sc, bi, g.inv_out_scale, g.residual_scale, abar, lane, next_residual);
-                    else epi_staged_box<false>(taddr0 + (uint32_t)c, g.out_box, buf, sc, bi, g.inv_out_scale, 0.0f, abar, lane, next_residual);
+                    epi_staged_box<res>(taddr0 + (uint32_t)c, g.out_box, buf, sc, bi, g.inv_out_scale, g.residual_scale, abar, lane, next_residual);
                     fence_proxy_async_smem();
                     __syncwarp();
                     const int x = (int)nt * BN + cbase + c;
@@ -1048,7 +1054,7 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
             }
             const int64_t row = mt * kBM + quarter * 32 + lane;
             const uint32_t taddr0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * BN + cbase);
-            epi_warp_columns<LEAN>(ev, taddr0, cbase, cols, row, row < g.M, nt * BN, s_scale[team], s_bias[team],
+            epi_warp_columns<OUT>(ev, taddr0, cbase, cols, row, row < g.M, nt * BN, s_scale[team], s_bias[team],
                              smem_u32(&bar_acc_empty[acc]), lane, [&]() {
                                  mbar_wait(smem_u32(&bar_acc_full[acc]), acc_use & 1, abort_flag, g.status, g.wait_limit);
                                  tc_fence_after();
@@ -1118,10 +1124,10 @@ struct GemmMaps {
 template <int BN, int BK>
 cudaError_t launch_gemm_shape(const GemmMaps &m, GemmArgs &g, int mode, int n, int rnd, int grid, cudaStream_t st);
 
-template <int BN, int BK, int MODE, int XN, bool RND, bool LEAN>
+template <int BN, int BK, int MODE, int XN, bool RND, int OUT>
 cudaError_t launch_gemm_kernel(const GemmMaps &m, GemmArgs &g, int grid, cudaStream_t st)
 {
-    auto kfn = sparq_gemm_kernel<BN, BK, MODE, XN, RND, LEAN>;
+    auto kfn = sparq_gemm_kernel<BN, BK, MODE, XN, RND, OUT>;
     static bool attr_set[64] = {};   // per device ordinal
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -1137,9 +1143,16 @@ cudaError_t launch_gemm_kernel(const GemmMaps &m, GemmArgs &g, int grid, cudaStr
     return launch_overlapped(kfn, grid, kGemmThreads, smem, st, m.a, m.b, m.out, m.res, g);
 }
 
-#define SPARQ_LAUNCH_VARIANT(MODE_, XN_, RND_)                                                         \
-    return make_epi_view(g).lean ? launch_gemm_kernel<BN, BK, MODE_, XN_, RND_, true>(m, g, grid, st)  \
-                                 : launch_gemm_kernel<BN, BK, MODE_, XN_, RND_, false>(m, g, grid, st)
+template <int BN, int BK, int MODE, int XN, bool RND>
+cudaError_t launch_gemm_variant(const GemmMaps &m, GemmArgs &g, int grid, cudaStream_t st)
+{
+    const int out = make_epi_view(g).out;
+    if (out == kOutBytes) return launch_gemm_kernel<BN, BK, MODE, XN, RND, kOutBytes>(m, g, grid, st);
+    if (out == kOutResidual) return launch_gemm_kernel<BN, BK, MODE, XN, RND, kOutResidual>(m, g, grid, st);
+    return launch_gemm_kernel<BN, BK, MODE, XN, RND, kOutGeneral>(m, g, grid, st);
+}
+
+#define SPARQ_LAUNCH_VARIANT(MODE_, XN_, RND_) return launch_gemm_variant<BN, BK, MODE_, XN_, RND_>(m, g, grid, st)
 
 #define SPARQ_DEFINE_GEMM_SHAPE(BN_, BK_)                                                              \
     template <>                                                                                        \

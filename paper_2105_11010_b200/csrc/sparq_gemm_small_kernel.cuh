@@ -290,7 +290,10 @@ sparq_gemm_small_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
                 asm volatile("bar.sync 1, %0;" :: "n"(kSmallWorkers * 32) : "memory");
             }
             // (handing the accumulator back is not needed here: the barrier named is never waited for)
-            epi_warp_columns<true>(ev, taddr, cbase, 32, m0 + trow, trow < rows_left, n0, s_scale, s_bias, smem_u32(&bar_recv), lane, wait_acc);
+            if (ev.out == kOutResidual)
+                epi_warp_columns<kOutResidual>(ev, taddr, cbase, 32, m0 + trow, trow < rows_left, n0, s_scale, s_bias, smem_u32(&bar_recv), lane, wait_acc);
+            else
+                epi_warp_columns<kOutBytes>(ev, taddr, cbase, 32, m0 + trow, trow < rows_left, n0, s_scale, s_bias, smem_u32(&bar_recv), lane, wait_acc);
         } else {
             // residual bytes of this thread's four columns of the CTA's row lrow
             auto residual_of = [&](int lrow) {
@@ -390,7 +393,7 @@ cudaError_t launch_gemm_small_kernel(const GemmMaps &m, GemmArgs &g, int grid, c
 }
 
 #define SPARQ_LAUNCH_SMALL(MODE_, XN_, RND_)                                                           \
-    return g.split > 1 || !make_epi_view(g).lean ? launch_gemm_small_kernel<BK, MODE_, XN_, RND_, true>(m, g, grid, st)          \
+    return g.split > 1 || make_epi_view(g).out == kOutGeneral ? launch_gemm_small_kernel<BK, MODE_, XN_, RND_, true>(m, g, grid, st)          \
                        : launch_gemm_small_kernel<BK, MODE_, XN_, RND_, false>(m, g, grid, st)
 
 #define SPARQ_DEFINE_GEMM_SMALL(BK_)                                                                   \

@@ -183,8 +183,8 @@ sparq_gemm_sparse24_kernel(const __grid_constant__ CUtensorMap map_a, const __gr
                     tc_fence_after();
                 };
                 const uint32_t empty = smem_u32(&bar_acc_empty[acc]);
-                if (ev.lean) epi_warp_columns<true>(ev, taddr0, 0, BN, row, row < g.M, nt * BN, s_scale, s_bias, empty, lane, wait_full);
-                else epi_warp_columns<false>(ev, taddr0, 0, BN, row, row < g.M, nt * BN, s_scale, s_bias, empty, lane, wait_full);
+                if (ev.out == kOutBytes) epi_warp_columns<kOutBytes>(ev, taddr0, 0, BN, row, row < g.M, nt * BN, s_scale, s_bias, empty, lane, wait_full);
+                else epi_warp_columns<kOutGeneral>(ev, taddr0, 0, BN, row, row < g.M, nt * BN, s_scale, s_bias, empty, lane, wait_full);
             }
         }
     } else {

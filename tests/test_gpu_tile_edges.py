@@ -169,6 +169,30 @@ def test_few_tiles_conv(nb, hw, c, cout, r, stride, mode):
     assert (got[-16:] == -7).all()
 
 
+@pytest.mark.parametrize("nb,hw,c,cout", [(7, 20, 64, 64), (7, 20, 128, 128), (11, 14, 256, 256), (37, 28, 128, 320)])
+@pytest.mark.parametrize("kind", ["u8", "u8+residual", "all"])
+@pytest.mark.parametrize("mode", [sparq.MODE_NONE, sparq.MODE_VSPARQ])
+def test_window_output_kinds(nb, hw, c, cout, kind, mode):
+    """3x3 convolutions on every window tile, for each kind of output that a kernel is instantiated for."""
+    x, w = synth.activations(c, (nb, hw, hw, c), 0.5), synth.weights(c, (cout, 3, 3, c))
+    scale, bias, inv = synth.scales(c, cout), synth.bias(c, cout), synth.inv_out_scale(9 * c)
+    res = synth.activations(cout + 1, (nb * hw * hw, cout), 0.5) if "residual" in kind else None
+    f32, u8 = oracle.epilogue(oracle.conv2d_nhwc(x, w, (1, 1), (1, 1), mode, 4, 0x1F, 1).reshape(-1, cout), scale, bias, True, inv,
+                              residual=res, residual_scale=0.02)
+    d = lambda v: torch.from_numpy(v).cuda()  # noqa: E731
+    out = {"u8_out": torch.full((u8.size + 64,), 3, dtype=torch.uint8, device="cuda")}
+    if kind == "all":
+        out["f32_out"] = torch.full((u8.size + 64,), 3, dtype=torch.float32, device="cuda")
+    sparq.sparq_conv2d_nhwc_s8(d(x), d(w), (1, 1), (1, 1), sparq.SparqParams(mode, 4, 0x1F, 1), scale=d(scale), bias=d(bias), relu=True,
+                               inv_out_scale=inv, residual=None if res is None else d(res), residual_scale=0.02, **out)
+    sparq.sparq_check()
+    for name, want in (("u8_out", u8), ("f32_out", f32)):
+        if name in out:
+            got = out[name].cpu().numpy()
+            assert np.array_equal(got[:u8.size].reshape(-1, cout), want), name
+            assert (got[u8.size:] == 3).all()
+
+
 @pytest.mark.parametrize("n", [1, 3, 31, 33, 61, 68, 72, 80, 127, 130, 200, 261])
 @pytest.mark.parametrize("residual", [False, True])
 def test_ragged_columns(n, residual):
