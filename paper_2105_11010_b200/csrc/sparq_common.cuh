@@ -278,13 +278,17 @@ __device__ __forceinline__ uint32_t xform_word_fullset(uint32_t x, const XformDe
 // five placements (packed-integer form, width fixed at compile time), XN = 5 the same with the
 // placement widening (any restricted set of n = 4: 3opt, 2opt), XN = 8 any other full placement set
 // (6opt, 7opt; either rounding, through the constants; RND unused), XN = 0 the general
-// packed-integer form with run-time width and the placement widening (restricted sets of n < 4).
+// packed-integer form with run-time width and the placement widening (restricted sets of n < 4); XN = 3
+// and 2 are that with the width fixed, in the standalone kernels only, which the integer pipe bounds
+// there (the fused kernels would need two more instantiations of everything for rare sets).
 template <int MODE, int XN, bool RND>
 __device__ __forceinline__ uint32_t xform_fused(uint32_t x, const XformDev &d)
 {
     if (XN == 8) return xform_word_fullset<MODE>(x, d);
     if (XN == 4) return xform_word<MODE, 4, RND, false>(x, d);
     if (XN == 5) return xform_word<MODE, 4, RND, true>(x, d);
+    if (XN == 3) return xform_word<MODE, 3, RND, true>(x, d);
+    if (XN == 2) return xform_word<MODE, 2, RND, true>(x, d);
     return xform_word<MODE, 0, RND, true>(x, d);
 }
 

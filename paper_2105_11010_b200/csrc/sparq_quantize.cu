@@ -196,7 +196,8 @@ static cudaError_t by_variant(const XformArgs &a, F go)
 {
     using std::integral_constant;
     if (a.widen_rounds > 0 && a.n == 4) return a.rnd ? go(integral_constant<int, 5>(), std::true_type()) : go(integral_constant<int, 5>(), std::false_type());
-    if (a.widen_rounds > 0) return a.rnd ? go(integral_constant<int, 0>(), std::true_type()) : go(integral_constant<int, 0>(), std::false_type());
+    if (a.widen_rounds > 0 && a.n == 3) return a.rnd ? go(integral_constant<int, 3>(), std::true_type()) : go(integral_constant<int, 3>(), std::false_type());
+    if (a.widen_rounds > 0) return a.rnd ? go(integral_constant<int, 2>(), std::true_type()) : go(integral_constant<int, 2>(), std::false_type());
     if (a.n != 4) return go(integral_constant<int, 8>(), std::true_type());
     return a.rnd ? go(integral_constant<int, 4>(), std::true_type()) : go(integral_constant<int, 4>(), std::false_type());
 }
