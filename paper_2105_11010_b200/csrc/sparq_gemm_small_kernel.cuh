@@ -157,6 +157,7 @@ sparq_gemm_small_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
     // (A launch with split = 1 has no clusters, and executes none of their instructions.)
     if (SHARED && split > 1) {
         if (threadIdx.x == 0) mbar_expect_tx(smem_u32(&bar_recv), split * (uint32_t)own_valid * (BN * 4));
+        __syncwarp();
         cluster_arrive();       // "barriers ready": waited for before the first remote store
     }
     // weights before the previous kernel on the stream has finished
@@ -361,6 +362,18 @@ sparq_gemm_small_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
         cluster_wait();            // matches the arrival above
     }
     __syncthreads();
+    // No CTA leaves while a peer may still write to its shared memory.  In a normal run its barrier has
+    // counted every byte by now; a CTA that gave up a wait comes here early.  It stays until every
+    // other CTA of the cluster has left or is here too (both after its last remote store: every CTA
+    // sends all its rows, given up or not, and reaches this point by bounded waits only), and then
+    // until the bytes still on their way have landed.  All waits of the CTA lie before the barrier
+    // above, so its threads agree on the flag.  (A second cluster barrier in every run cost 0.1 us.)
+    if (SHARED && split > 1 && *abort_flag) {
+        __syncwarp();
+        cluster_arrive();
+        cluster_wait();
+        mbar_wait(smem_u32(&bar_recv), 0, abort_flag, g.status, g.wait_limit, true);
+    }
     if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem_base), "r"((uint32_t)BN) : "memory");
