@@ -41,22 +41,11 @@ int quantize_rows(const uint8_t *in, uint8_t *out, size_t rows, size_t row_len, 
 void *workspace_alloc(size_t bytes, cudaStream_t st);
 void workspace_free(void *p, cudaStream_t st);
 
-// Memory that a launch writes (ptr == nullptr: nothing).
-struct OutRange {
-    const void *ptr;
-    size_t bytes;
-};
-
-// Records what the launch about to be enqueued on `st` writes; returns whether the weights (may
-// be null) are known to be clear of what the previous launch on the stream writes.
-bool note_outputs(cudaStream_t st, const OutRange (&outs)[3], const void *wgt = nullptr, size_t wgt_bytes = 0);
-
 // ---- overlapped launches ----------------------------------------------------------------
 // The library's kernels are launched with programmatic stream serialization: a kernel may start,
 // and set itself up, while its predecessor on the stream is finishing.  dep_wait() blocks until
 // every earlier kernel has completed and its writes are visible; no thread touches the caller's
-// memory before it (the fused kernels' early weights aside, see note_outputs).  dep_launch()
-// lets the next kernel start.
+// memory before it.  dep_launch() lets the next kernel start.
 #ifdef __CUDACC__
 __device__ __forceinline__ void dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

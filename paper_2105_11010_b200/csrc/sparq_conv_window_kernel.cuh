@@ -48,7 +48,6 @@ struct WindowArgs {
     int plane_bytes;        // shared-memory bytes reserved per channel block (>= rows the MMA may touch)
     int win_bufs;           // window buffers in the ring
     int b_stages;           // weight stages (stream mode) or resident blocks (resident mode)
-    int early_weights;      // resident weights may be fetched before the previous kernel on the stream has finished
     int issuers;            // 2: the two issuer warps alternate (resident weights); 1: warp 1 issues every tile (streamed weights)
     uint32_t n_tiles;       // column tiles
     uint32_t units;         // n_img * tiles_per_img * n_tiles, column tile fastest
@@ -239,26 +238,27 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
     // integer divisions) while the previous kernel may still be running
     GroupWalk<kBatched> walk(g);
     bool have = walk.next();       // the first group, too
-    // All weight blocks, once per CTA, on stage barrier 0: every CTA reads the same bytes, so
-    // they come out of L2 one reader after the other, and they are what the first tile waits
-    // for longest.  map_w is the (channels, filters, taps) view; one copy brings a channel block of
-    // every tap, tap t of channel block cb into slot cb * taps + t.
+    // All weight blocks, once per CTA: every CTA reads the same bytes, so they come out of L2 one
+    // reader after the other.  They follow the first piece of activations, which the transform waits
+    // for.  map_w is the (channels, filters, taps) view; tap t of channel block cb goes into slot
+    // cb * taps + t.  3x3 filters arrive with one copy a channel block on stage barrier 0; other sizes with
+    // one a filter row, each on a barrier of its own, so that the first tile starts on the first row
+    // (17x35x35x48 -> 64 5x5: 12.9 -> 11.9 us; in the unrolled 3x3 loop the waits cost more than they gave,
+    // 128x28x28x128 -> 128 16.0 -> 16.5).
+    const bool by_row = B_RESIDENT && !(g.R == 3 && g.S == 3);
     auto issue_resident_weights = [&]() {
-        const uint32_t full = smem_u32(&bar_b_full[0]);
-        mbar_expect_tx(full, (uint32_t)kb_count * kBBlock);
-        for (int cb = 0; cb < g.c_blocks; ++cb) tma_load_3d(b_slot(cb * taps), &map_w, full, cb * CB, 0, 0);
+        const int copies = by_row ? g.R : 1, copy_taps = by_row ? g.S : taps;
+        if (!by_row) mbar_expect_tx(smem_u32(&bar_b_full[0]), (uint32_t)kb_count * kBBlock);
+        for (int cb = 0, q = 0; cb < g.c_blocks; ++cb)
+            for (int r = 0; r < copies; ++r, ++q) {
+                const uint32_t full = smem_u32(&bar_b_full[by_row ? q : 0]);
+                if (by_row) mbar_expect_tx(full, (uint32_t)copy_taps * kBBlock);
+                tma_load_3d(b_slot(cb * taps + r * copy_taps), &map_w, full, cb * CB, 0, r * copy_taps);
+            }
     };
-    // The weights are not an output of the kernel that runs before this one (the host checks
-    // that and sets early_weights), so their copy may start before that kernel has finished:
-    // in a chain of layers the wait for the weights then overlaps the predecessor's tail.
     bool b_issued = false;
-    if (B_RESIDENT && g.early_weights && threadIdx.x == 0 && have) {
-        issue_resident_weights();
-        b_issued = true;
-    }
     dep_wait();
     dep_launch();
-
 
     if (warp == 0) {
         // ================= TMA producer =================
@@ -272,10 +272,6 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
                 const uint32_t use = ruse;
                 if (use > 0 && !mbar_wait(smem_u32(&bar_win_empty[b]), (use - 1) & 1, abort_flag, g.status, g.wait_limit)) break;
                 const int oh0 = (int)walk.tin * g.TR;
-                if (B_RESIDENT && !b_issued) {
-                    issue_resident_weights();
-                    b_issued = true;
-                }
                 for (int j = 0; j < g.G; ++j) {
                     const uint32_t wfull = smem_u32(&bar_win_full[b * kMaxG + j]);
                     if (j < (int)walk.cnt) {
@@ -288,6 +284,10 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
                         // a piece this group does not have: complete its phase so that the
                         // parity of every barrier of the buffer advances once per use
                         mbar_arrive(wfull);
+                    }
+                    if (B_RESIDENT && !b_issued) {       // behind the first piece, which the transform waits for
+                        issue_resident_weights();
+                        b_issued = true;
                     }
                 }
                 ++gi;
@@ -318,7 +318,8 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
                         mbar_wait(smem_u32(&bar_win_full[(q % g.win_bufs) * kMaxG + j]), (q / g.win_bufs) & 1,
                                   abort_flag, g.status, g.wait_limit, true);
                 if (B_RESIDENT) {
-                    if (b_issued) mbar_wait(smem_u32(&bar_b_full[0]), 0, abort_flag, g.status, g.wait_limit, true);
+                    for (int q = 0; b_issued && q < (by_row ? g.c_blocks * g.R : 1); ++q)
+                        mbar_wait(smem_u32(&bar_b_full[q]), 0, abort_flag, g.status, g.wait_limit, true);
                 } else {
                     const uint32_t first = it > (uint32_t)g.b_stages ? it - g.b_stages : 0;
                     for (uint32_t q = first; q < it; ++q)
@@ -352,6 +353,7 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
             const uint32_t plane16 = (uint32_t)g.plane_bytes >> 4;
             const uint32_t tile16 = (uint32_t)(g.TR * g.Wp * CB) >> 4;
             if (B_RESIDENT) mbar_wait(smem_u32(&bar_b_full[0]), 0, abort_flag, g.status, g.wait_limit);
+            bool weights_there = !by_row;      // else waited for row by row, during this issuer's first tile
             for (; have; have = walk.next()) {
                 const int b = rb;
                 const uint32_t wph = ruse & 1u;
@@ -490,12 +492,17 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
                         for (uint32_t cb = 0; cb < cbs; ++cb, a_cb += plane16) {
                             uint64_t a_r = a_cb;
                             for (int r = 0; r < g.R; ++r, a_r += row16) {
+                                if (B_RESIDENT && !weights_there) {
+                                    mbar_wait(smem_u32(&bar_b_full[cb * (uint32_t)g.R + (uint32_t)r]), 0, abort_flag, g.status, g.wait_limit);
+                                    tc_fence_after();
+                                }
                                 for (int sx = 0; sx < g.S; ++sx, ++slot)
                                     issue_block(cb == 0 && r == 0 && sx == 0, slot, a_r + (uint64_t)(uint32_t)(sx * (CB >> 4)));
                                 if (r == 0 && cb == 0) look();
                             }
                         }
                     }
+                    weights_there = true;
                     tc_commit_if(smem_u32(&bar_acc_full[acc]), elected);      // accumulator complete
                 }
                 // The buffer goes back to the producer once both issuers have arrived and their

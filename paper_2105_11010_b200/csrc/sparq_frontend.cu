@@ -169,18 +169,18 @@ __device__ __forceinline__ int quant_s8(float w, float inv)
     return w != w ? 0 : __float2int_rn(z);
 }
 
-// One block per kernel (output channel): its largest magnitude, then its int8 row.  early: the weights are
-// no output of the previous launch, so they may be read while that is finishing.  VEC: rows are whole
+// One block per kernel (output channel): its largest magnitude, then its int8 row.  VEC: rows are whole
 // 16-byte vectors, and the first kWeightVecs per thread stay in registers between the two steps, which
 // is the whole row up to 4608 values (512 filters of 3x3); what lies beyond is read again.
 constexpr int kWeightVecs = 5;
 template <bool VEC>
 __global__ void __launch_bounds__(kThreads)
-quantize_weight_kernel(const float *__restrict__ w, int64_t k, int8_t *__restrict__ out, float *__restrict__ scale_out, int early)
+quantize_weight_kernel(const float *__restrict__ w, int64_t k, int8_t *__restrict__ out, float *__restrict__ scale_out)
 {
     __shared__ uint32_t s_red[kThreads / 32];
     __shared__ float s_max;
-    if (!early) dep_wait();
+    dep_wait();
+    dep_launch();
     const float *row = w + (int64_t)blockIdx.x * k;
     int8_t *orow = out + (int64_t)blockIdx.x * k;
     const uint4 *rv = reinterpret_cast<const uint4 *>(row);
@@ -201,8 +201,6 @@ quantize_weight_kernel(const float *__restrict__ w, int64_t k, int8_t *__restric
     }
     const uint32_t b = block_max_bits(m, s_red);
     if (threadIdx.x == 0) s_max = __uint_as_float(b);
-    if (early) dep_wait();
-    dep_launch();
     __syncthreads();
     const float a = s_max;
     const float inv = a > 0.0f ? __fdiv_rn(127.0f, a) : 0.0f;
@@ -264,7 +262,6 @@ extern "C" int sparq_absmax(const void *x, int dtype, size_t n, float *max_inout
     int blocks = 0;
     if ((rc = stream_grid(n / (bf16 ? 8 : 4), &blocks)) != SPARQ_OK) return rc;
     cudaStream_t st = (cudaStream_t)stream;
-    note_outputs(st, {{max_inout, sizeof(float)}, {nullptr, 0}, {nullptr, 0}});
     const size_t nvec = n / (bf16 ? 8 : 4), keep_from = nvec > kKeepVecs ? nvec - kKeepVecs : 0;
     const cudaError_t e = launch_overlapped(bf16 ? absmax_kernel<true> : absmax_kernel<false>, blocks, kThreads, 0, st, x, n, max_inout, keep_from);
     if (e != cudaSuccess) return cuda_error(e, "absmax_kernel launch");
@@ -285,7 +282,6 @@ extern "C" int sparq_quantize_act_u8(const void *x, int dtype, size_t n, const f
     int blocks = 0;
     if ((rc = stream_grid(n / (bf16 ? 8 : 4), &blocks)) != SPARQ_OK) return rc;
     cudaStream_t st = (cudaStream_t)stream;
-    note_outputs(st, {{out, n}, {nullptr, 0}, {nullptr, 0}});
     const cudaError_t e = launch_overlapped(bf16 ? quantize_act_kernel<true> : quantize_act_kernel<false>, blocks, kThreads, 0, st, x, n, max_dev, out);
     if (e != cudaSuccess) return cuda_error(e, "quantize_act_kernel launch");
     return SPARQ_OK;
@@ -301,11 +297,9 @@ extern "C" int sparq_quantize_weight_s8(const float *w, int64_t cout, int64_t k,
     if (((uintptr_t)w | (uintptr_t)scale_out) & 3u)
         return set_error(SPARQ_ERR_UNSUPPORTED, "w and scale_out must be 4-byte aligned");
     cudaStream_t st = (cudaStream_t)stream;
-    const bool early = note_outputs(st, {{out, (size_t)cout * (size_t)k}, {scale_out, (size_t)cout * sizeof(float)}, {nullptr, 0}},
-                                    w, (size_t)cout * (size_t)k * sizeof(float));
     const bool vec = k % 4 == 0 && ((uintptr_t)w & 15u) == 0 && ((uintptr_t)out & 3u) == 0;
     const cudaError_t e = launch_overlapped(vec ? quantize_weight_kernel<true> : quantize_weight_kernel<false>, (int)cout, kThreads, 0, st,
-                                            w, k, out, scale_out, (int)early);
+                                            w, k, out, scale_out);
     if (e != cudaSuccess) return cuda_error(e, "quantize_weight_kernel launch");
     return SPARQ_OK;
 }

@@ -257,59 +257,6 @@ static bool transform_first(int64_t M, int64_t N, int64_t steps, size_t act_byte
     return plain + clk * (2.5 + (double)act_bytes / 2.9e6) < 0.93 * fused;
 }
 
-// ---- what the previous launch on a stream wrote ----------------------------------------------------
-// The library's kernels are launched with programmatic stream serialization and let their
-// successor start once they themselves may run; a fused successor may fetch its WEIGHTS before it
-// waits for them -- provided the weights are not among their outputs.  Every launch that lets
-// its successor start early records its output ranges per (device, stream) here, and a fused one
-// learns whether its own weights are clear of the previous launch's.  (Launches before that one
-// have completed: a kernel releases its successor after its own wait.)  Kernels of other libraries
-// never release their successor early.  A stream that is not in the table (first launch, or
-// evicted) counts as "not clear".
-struct LastLaunch {
-    bool used;
-    int dev;
-    cudaStream_t stream;
-    uint64_t age;
-    uintptr_t lo[3], hi[3];
-};
-constexpr int kLastSlots = 32;
-static LastLaunch g_last[kLastSlots];
-static uint64_t g_last_age = 0;
-static std::mutex g_last_mutex;
-
-bool note_outputs(cudaStream_t st, const OutRange (&outs)[3], const void *wgt, size_t wgt_bytes)
-{
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return false; }
-    std::lock_guard<std::mutex> lock(g_last_mutex);
-    LastLaunch *slot = nullptr, *oldest = &g_last[0];
-    for (LastLaunch &l : g_last) {
-        if (l.used && l.dev == dev && l.stream == st) { slot = &l; break; }
-        if (!l.used || l.age < oldest->age || (oldest->used && !l.used)) oldest = &l;
-    }
-    bool clear = false;
-    if (slot) {
-        clear = true;
-        const uintptr_t w0 = (uintptr_t)wgt, w1 = w0 + wgt_bytes;
-        for (int i = 0; i < 3; ++i)
-            if (slot->lo[i] < w1 && w0 < slot->hi[i]) clear = false;
-    } else {
-        slot = oldest;
-    }
-    slot->used = true; slot->dev = dev; slot->stream = st; slot->age = ++g_last_age;
-    for (int i = 0; i < 3; ++i) {
-        slot->lo[i] = (uintptr_t)outs[i].ptr;
-        slot->hi[i] = outs[i].ptr ? (uintptr_t)outs[i].ptr + outs[i].bytes : 0;
-    }
-    return clear;
-}
-
-static bool record_launch_weights_clear(cudaStream_t st, const sparq_epilogue *e, size_t out_elems, const void *wgt, size_t wgt_bytes)
-{
-    return note_outputs(st, {{e->acc_out, 4 * out_elems}, {e->f32_out, 4 * out_elems}, {e->u8_out, out_elems}}, wgt, wgt_bytes);
-}
-
 // Variant argument of the launchers (XN of xform_fused): 4 = n = 4 with all five placements, 5 = n = 4
 // with fewer, 8 = another full placement set (6opt, 7opt), 0 = restricted sets of n < 4.
 static int variant_n(const XformArgs &x) { return x.n == 4 ? (x.widen_rounds ? 5 : 4) : (x.widen_rounds ? 0 : 8); }
@@ -430,7 +377,8 @@ static int encode_window(CUtensorMap *map, const void *ptr, int n, int h, int w,
 }
 
 // Weights [cout][taps][c] as (channels, filters, taps): a box brings cb channels of bn filters and
-// box_taps taps into consecutive bn x cb shared-memory blocks; channels past c arrive as zeros.
+// box_taps taps into consecutive bn x cb shared-memory blocks (a whole filter, a filter row, a tap);
+// channels past c arrive as zeros.
 static int encode_weights(CUtensorMap *map, const void *ptr, int c, int cout, int taps, int cb, int bn, int box_taps)
 {
     static EncodeTiledFn fn = nullptr;
@@ -507,7 +455,7 @@ static int try_window_conv(const uint8_t *x_in, int n, int h, int w, int c, cons
     }
     bool resident = false, batched = false;
     int win_bufs = 2, b_stages = 0, grp = 1;
-    if (bn != 256 && n_tiles == 1 && 1024 + 2 * plane_for(1) * c_blocks + kb_count * b_block <= kMaxDynSmem) {
+    if (bn != 256 && n_tiles == 1 && c_blocks * r <= kMaxBStages && 1024 + 2 * plane_for(1) * c_blocks + kb_count * b_block <= kMaxDynSmem) {
         resident = true;
         b_stages = kb_count;
         grp = gmax;
@@ -553,7 +501,7 @@ static int try_window_conv(const uint8_t *x_in, int n, int h, int w, int c, cons
     rc = encode_window(&mx1, x_in, n, h, w, c, cb, wp, tr);
     if (rc != SPARQ_OK) return rc;
     const int64_t K = (int64_t)r * s * c;
-    rc = encode_weights(&mw, wgt, c, cout, taps, cb, bn, resident ? taps : 1);
+    rc = encode_weights(&mw, wgt, c, cout, taps, cb, bn, !resident ? 1 : r == 3 && s == 3 ? taps : s);   // as the kernel copies them
     if (rc != SPARQ_OK) return rc;
 
     WindowArgs g;
@@ -588,7 +536,6 @@ static int try_window_conv(const uint8_t *x_in, int n, int h, int w, int c, cons
     g.residual_scale = e->residual_scale;
     rc = next_transform_args(e, g.N, &g.next_mode, &g.next_rnd, &g.next_xf);
     if (rc != SPARQ_OK) return rc;
-    g.early_weights = record_launch_weights_clear(st, e, (size_t)n * ho * wo * (size_t)cout, wgt, (size_t)cout * (size_t)K) ? 1 : 0;
     cudaError_t ce;
     if (bn == 64) ce = launch_window_shape<64, 64, true>(mx, mx1, mw, g, x.mode, variant_n(x), x.rnd, grid, smem_bytes, st);
     else if (bn == 128 && resident) ce = launch_window_shape<128, 128, true>(mx, mx1, mw, g, x.mode, variant_n(x), x.rnd, grid, smem_bytes, st);
@@ -631,7 +578,6 @@ int gemm_with_status(const uint8_t *A, int64_t lda, const int8_t *B, int64_t ldb
     g.split = small.split;
     const int grid = small.tile_rows ? (int)tiles * small.split : (int)(tiles < sms ? tiles : sms);
     if ((rc = output_maps(&m, &g, x.mode, bn, tiles, grid)) != SPARQ_OK) return rc;
-    g.early_weights = record_launch_weights_clear(st, e, (size_t)M * (size_t)N, B, (size_t)N * (size_t)ldb) ? 1 : 0;
     cudaError_t ce = launch(bn, bk, small.tile_rows != 0, m, g, x, grid, st);
     if (ce != cudaSuccess) return cuda_error(ce, "sparq_gemm_kernel launch");
     return SPARQ_OK;
@@ -673,7 +619,6 @@ static int im2col_conv(const uint8_t *x_in, int n, int h, int w, int c, const in
     g.split = small.split;
     const int grid = small.tile_rows ? (int)tiles * small.split : (int)(tiles < sms ? tiles : sms);
     if ((rc = output_maps(&m, &g, x.mode, bn, tiles, grid)) != SPARQ_OK) return rc;
-    g.early_weights = record_launch_weights_clear(st, e, (size_t)M * (size_t)cout, wgt, (size_t)cout * (size_t)K) ? 1 : 0;
     cudaError_t ce = launch(bn, bk, small.tile_rows != 0, m, g, x, grid, st);
     if (ce != cudaSuccess) return cuda_error(ce, "sparq_gemm_kernel (convolution) launch");
     return SPARQ_OK;
@@ -711,7 +656,6 @@ int gemm_sparse24_fused(const uint8_t *A, const int8_t *w_exp, int64_t M, int64_
     g.M = M; g.N = N; g.K = 3 * K;
     g.k_blocks = (int)steps;
     if ((rc = fill_common(&g, x, e, status)) != SPARQ_OK) return rc;
-    record_launch_weights_clear(st, e, (size_t)M * (size_t)N, w_exp, (size_t)N * (size_t)(3 * K));
     const cudaError_t ce = launch_x24(bn, ma, mb, g, variant_n(x), x.rnd, (int)(tiles < sms ? tiles : sms), st);
     return ce == cudaSuccess ? 1 : cuda_error(ce, "sparq_gemm_sparse24_kernel launch");
 }

@@ -86,9 +86,8 @@ struct GemmArgs {
     // staged output: bytes per row of the boxes that the epilogue warps store (and fetch the residual)
     // with through shared memory, 0 = straight from registers.  See epi_staged.
     int out_box;
-    // small form only: the weights are not an output of the previous launch, so fetch them before waiting
-    // for it; rows of a tile; CTAs of a cluster that share a tile (1 = none)
-    int early_weights, tile_rows, split;
+    // small form only: rows of a tile; CTAs of a cluster that share a tile (1 = none)
+    int tile_rows, split;
 };
 
 // ---- PTX wrappers ---------------------------------------------------------------------

@@ -2,7 +2,7 @@
 // of a network at batch 1, small matrices.  Such a launch is latency from end to end, so this
 // form of sparq_gemm_kernel (same operands, stage hand-offs and epilogue arithmetic)
 //   - runs ten warps and at most half of an SM's shared memory and registers, so that CTAs of the
-//     NEXT launch start beside it (barriers, tensor memory, tensor maps) and fetch their weights;
+//     NEXT launch start beside it (barriers, tensor memory, tensor maps);
 //   - has eight worker warps that first transform the stages and then run the epilogue, instead
 //     of separate roles of which one always waits;
 //   - has tiles of 64 rows as well as of 128 (x 64 columns): a step is bound by the transform of its
@@ -160,15 +160,6 @@ sparq_gemm_small_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
         __syncwarp();
         cluster_arrive();       // "barriers ready": waited for before the first remote store
     }
-    // weights before the previous kernel on the stream has finished
-    const int early = g.early_weights ? (steps < S ? steps : S) : 0;
-    if (threadIdx.x == 0) {
-        TapWalk tap(g, BK, kb_first);
-        for (int it = 0; it < early; ++it, tap.next()) {
-            mbar_expect_tx(smem_u32(&bar_full[it]), kStageBytes);
-            tma_load_2d(b_stage(it), &map_b, smem_u32(&bar_full[it]), g.conv ? tap.k : (kb_first + it) * BK, n0);
-        }
-    }
     dep_wait();
     dep_launch();
 
@@ -190,10 +181,10 @@ sparq_gemm_small_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
                 if (it >= S && !mbar_wait(smem_u32(&bar_empty[s]), ph, abort_flag, g.status, g.wait_limit)) break;
                 const uint32_t full = smem_u32(&bar_full[s]);
                 const int kx = g.conv ? tap.k : (kb_first + it) * BK;
-                if (it >= early) mbar_expect_tx(full, kStageBytes);
+                mbar_expect_tx(full, kStageBytes);
                 if (g.conv) tma_load_im2col_4d(a_stage(s), &map_a, full, tap.c, base_w, base_h, base_n, (uint16_t)tap.s, (uint16_t)tap.r);
                 else tma_load_2d(a_stage(s), &map_a, full, kx, (int)m0);
-                if (it >= early) tma_load_2d(b_stage(s), &map_b, full, kx, n0);
+                if (it >= S) tma_load_2d(b_stage(s), &map_b, full, kx, n0);
                 tap.next();
                 if (++s == S) { s = 0; ph ^= 1u; }
             }
@@ -205,6 +196,14 @@ sparq_gemm_small_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
     } else if (warp == 1) {
         // ================= MMA issuer =================
         const uint32_t elected = elect_one();
+        // The ring's first round of weights, beside the producer's activations: one thread takes about
+        // 0.1 us a stage to issue both, in front of the first MMA.
+        if (elected) {
+            TapWalk tap(g, BK, kb_first);
+            for (int it = 0; it < S && it < steps; ++it, tap.next())
+                tma_load_2d(b_stage(it), &map_b, smem_u32(&bar_full[it]), g.conv ? tap.k : (kb_first + it) * BK, n0);
+        }
+        __syncwarp();
         const uint32_t idesc = make_idesc_i8(BN, TM);
         const uint64_t adesc0 = make_smem_desc<BK>(smem_base);
         const uint64_t bdesc0 = make_smem_desc<BK>(smem_base + kABytes);

@@ -530,14 +530,12 @@ int launch_pack_b(const uint8_t *i, uint8_t *d, uint8_t *c, size_t u, const Xfor
 int pack_switch(const uint8_t *in, uint8_t *data, uint8_t *ctrl, size_t units, const XformArgs &x, cudaStream_t st)
 {
     const int cb = state_bits(x);
-    note_outputs(st, {{data, units * 2 * x.n}, {ctrl, units * cb}, {nullptr, 0}});
     if (x.mode == SPARQ_MODE_VSPARQ) SPARQ_CODEC_SWITCH(launch_pack_v, x.n, cb, in, data, ctrl, units, x, st);
     SPARQ_CODEC_SWITCH(launch_pack_b, x.n, cb, in, data, ctrl, units, x, st);
 }
 
 int unpack_switch(const uint8_t *data, const uint8_t *ctrl, uint8_t *out, size_t units, const XformArgs &x, cudaStream_t st)
 {
-    note_outputs(st, {{out, units * 16}, {nullptr, 0}, {nullptr, 0}});
     SPARQ_CODEC_SWITCH(launch_unpack, x.n, state_bits(x), data, ctrl, out, units, x, st);
 }
 

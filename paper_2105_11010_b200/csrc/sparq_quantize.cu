@@ -233,7 +233,6 @@ int quantize_rows(const uint8_t *in, uint8_t *out, size_t rows, size_t row_len, 
         const uint8_t *hi = in < (const uint8_t *)out ? out : in;
         if (lo + total > hi) return set_error(SPARQ_ERR_INVALID_ARG, "in and out overlap partially");
     }
-    note_outputs(st, {{out, total}, {nullptr, 0}, {nullptr, 0}});
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

@@ -165,7 +165,6 @@ extern "C" int sparq_sparse24_expand_activations(const uint8_t *A, size_t rows, 
     cudaStream_t st = (cudaStream_t)stream;
     const uint4 *in = reinterpret_cast<const uint4 *>(A);
     uint4 *out = reinterpret_cast<uint4 *>(a_exp);
-    note_outputs(st, {{out, 48 * nvec}, {nullptr, 0}, {nullptr, 0}});
     const cudaError_t e = launch_expand_act(in, out, nvec, x, blocks, st);
     if (e != cudaSuccess) return cuda_error(e, "expand_act_kernel launch");
     return SPARQ_OK;
