@@ -15,10 +15,10 @@
  *     validates its arguments on the host, enqueues its kernels on `stream` and returns
  *     without synchronizing.
  *   - Return value: SPARQ_OK (0) or a negative sparq_status.  On error nothing has been
- *     enqueued and sparq_last_error() describes the reason (the entry points that enqueue
- *     more than one kernel -- the host-buffer forms, sparq_gemm_s8_static,
- *     sparq_gemm_s8_sparse24 -- may have enqueued their earlier kernels when a later launch
- *     fails; their outputs are then undefined).  No entry point throws, aborts or traps the
+ *     enqueued and sparq_last_error() describes the reason (where a call takes more than one
+ *     kernel -- sparq_gemm_s8 and sparq_conv2d_nhwc_s8 on large problems, the host-buffer forms,
+ *     sparq_gemm_s8_static, sparq_gemm_s8_sparse24 -- its earlier kernels may have been enqueued
+ *     when a later LAUNCH fails; the outputs are then undefined).  No entry point throws, aborts or traps the
  *     device.
  *   - Consecutive launches on one stream overlap at their edges (programmatic dependent
  *     launch): a launch may set itself up while its predecessor, of this library or another,

@@ -250,6 +250,7 @@ static SmallForm pick_small(int64_t M, int64_t N, int64_t k_blocks, int sms, boo
 static bool transform_first(int64_t M, int64_t N, int64_t steps, size_t act_bytes, int sms, bool im2col)
 {
     if (pick_small(M, N, steps, sms, true).tile_rows) return false;
+    if ((M + kBM - 1) / kBM * ((N + 63) / 64) >= (int64_t)1 << 31) return false;      // near the refused sizes: refused, if at all, with nothing enqueued
     double fused, plain;
     pick_bn(M, N, steps, sms, true, im2col, &fused);
     pick_bn(M, N, steps, sms, false, im2col, &plain);
@@ -626,13 +627,11 @@ static int im2col_conv(const uint8_t *x_in, int n, int h, int w, int c, const in
 
 cudaError_t launch_x24(int bn, const CUtensorMap &ma, const CUtensorMap &mb, const GemmArgs &g, int n, int rnd, int grid, cudaStream_t st);
 
-// The 2:4 product with the expansion inside the kernel (sparq_gemm_sparse24_kernel).  Returns 1 if it
-// launched, 0 if expanding into the workspace first is expected to be faster, < 0 on error.
+// The 2:4 product with the expansion inside the kernel (sparq_gemm_sparse24_kernel), arguments checked by
+// the caller.  Returns 1 if it launched, 0 if expanding into the workspace first is expected to be faster, < 0 on error.
 int gemm_sparse24_fused(const uint8_t *A, const int8_t *w_exp, int64_t M, int64_t N, int64_t K, const XformArgs &x,
                         const sparq_epilogue *e, cudaStream_t st)
 {
-    if (K == 0 || K % 16 || 3 * K > 65536 || (((uintptr_t)A | (uintptr_t)w_exp) & 15u) || M > (int64_t)1 << 31 || N > (int64_t)1 << 31)
-        return 0;                                        // the two-kernel form reports it
     int sms = 0, rc = device_info(&sms);
     if (rc != SPARQ_OK) return rc;
     // A tile of 256 rows is expanded once per column tile, about 4200 cycles per 128 activations of its
@@ -662,6 +661,14 @@ int gemm_sparse24_fused(const uint8_t *A, const int8_t *w_exp, int64_t M, int64_
 
 int check_epilogue_args(const sparq_epilogue *e) { return check_epilogue(e); }
 
+// e->next_transform for N output columns: before anything is enqueued, for entry points of several kernels.
+int check_next_transform(const sparq_epilogue *e, int64_t N)
+{
+    int mode, rnd;
+    XformDev xf;
+    return next_transform_args(e, N, &mode, &rnd, &xf);
+}
+
 }  // namespace sparq
 
 using namespace sparq;
@@ -683,6 +690,7 @@ extern "C" int sparq_gemm_s8(const uint8_t *A, int64_t lda, const int8_t *B, int
         return set_error(SPARQ_ERR_UNSUPPORTED, "lda/ldb must be multiples of 16 and at least K");
     if (((uintptr_t)A | (uintptr_t)B) & 15u) return set_error(SPARQ_ERR_UNSUPPORTED, "A and B must be 16-byte aligned");
     if (M > (int64_t)1 << 31 || N > (int64_t)1 << 31) return set_error(SPARQ_ERR_UNSUPPORTED, "M or N too large");
+    if ((rc = check_next_transform(e, N)) != SPARQ_OK) return rc;
     return gemm_impl(A, lda, B, ldb, M, N, K, x, e, (cudaStream_t)stream);
 }
 
@@ -711,6 +719,7 @@ extern "C" int sparq_conv2d_nhwc_s8(const uint8_t *x_in, int n, int h, int w, in
     const int64_t M = (int64_t)n * ho * wo;
     const int64_t K = (int64_t)r * s * c;
     if (K > 65536) return set_error(SPARQ_ERR_UNSUPPORTED, "r*s*c = %lld exceeds 65536", (long long)K);
+    if ((rc = check_next_transform(e, cout)) != SPARQ_OK) return rc;
     cudaStream_t st = (cudaStream_t)stream;
 
     // A 1x1 filter with unit stride reads the NHWC tensor as the M x c matrix it already is.

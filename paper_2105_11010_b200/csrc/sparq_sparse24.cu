@@ -16,6 +16,7 @@
 namespace sparq {
 
 int check_epilogue_args(const sparq_epilogue *e);
+int check_next_transform(const sparq_epilogue *e, int64_t N);
 int gemm_sparse24_fused(const uint8_t *A, const int8_t *w_exp, int64_t M, int64_t N, int64_t K, const XformArgs &x,
                         const sparq_epilogue *e, cudaStream_t st);
 
@@ -182,6 +183,12 @@ extern "C" int sparq_gemm_s8_sparse24(const uint8_t *A, const int8_t *w_exp, int
     if (x.mode != SPARQ_MODE_VSPARQ)   // dense form of the weights, transform fused as usual
         return sparq_gemm_s8(A, K, w_exp, K, M, N, K, p, e, stream);
     if (!workspace) return set_error(SPARQ_ERR_INVALID_ARG, "workspace is NULL (M * 3K bytes are needed with vSPARQ)");
+    if ((uintptr_t)workspace & 15u) return set_error(SPARQ_ERR_UNSUPPORTED, "workspace must be 16-byte aligned");
+    if (!A || !w_exp) return set_error(SPARQ_ERR_INVALID_ARG, "A or w_exp is NULL");
+    if (((uintptr_t)A | (uintptr_t)w_exp) & 15u) return set_error(SPARQ_ERR_UNSUPPORTED, "A and w_exp must be 16-byte aligned");
+    if (K == 0 || K % 16 || 3 * K > 65536) return set_error(SPARQ_ERR_UNSUPPORTED, "K = %lld must be a multiple of 16 with 3K at most 65536", (long long)K);
+    if (M > (int64_t)1 << 31 || N > (int64_t)1 << 31) return set_error(SPARQ_ERR_UNSUPPORTED, "M or N too large");
+    if ((rc = check_next_transform(e, N)) != SPARQ_OK) return rc;
     if ((rc = gemm_sparse24_fused(A, w_exp, M, N, K, x, e, (cudaStream_t)stream)) != 0) return rc < 0 ? rc : SPARQ_OK;
     if ((rc = sparq_sparse24_expand_activations(A, (size_t)M, (size_t)K, p, workspace, stream)) != SPARQ_OK) return rc;
     const sparq_params none = {SPARQ_MODE_NONE, 4, 0x1Fu, 0};

@@ -9,6 +9,7 @@ namespace sparq {
 int gemm_with_status(const uint8_t *A, int64_t lda, const int8_t *B, int64_t ldb, int64_t M, int64_t N, int64_t K,
                      const XformArgs &x, const sparq_epilogue *e, unsigned int *status, cudaStream_t st);
 int check_epilogue_args(const sparq_epilogue *e);
+int check_next_transform(const sparq_epilogue *e, int64_t N);
 
 namespace {
 
@@ -81,6 +82,8 @@ extern "C" int sparq_gemm_s8_static(const uint8_t *A, int64_t lda, const int8_t 
         return set_error(SPARQ_ERR_UNSUPPORTED,
                          "M * K = %llu bytes of transformed activations exceed the %u-byte static scratch of sparq_gemm_s8_static",
                          (unsigned long long)((uint64_t)M * (uint64_t)K), (unsigned)SPARQ_STATIC_SCRATCH_BYTES);
+
+    if ((rc = check_next_transform(e, N)) != SPARQ_OK) return rc;
 
     unsigned char *base = nullptr;
     rc = scratch_base(&base);
