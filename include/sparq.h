@@ -26,8 +26,11 @@
  *     the stream has completed.  Nothing for the caller to do.
  *   - Where a fused call would transform the same activations many times (several column tiles,
  *     several filter taps), it runs as transform + plain contraction with the transformed
- *     activations in stream-ordered scratch memory from a pool of the library's own; without
- *     memory to be had it runs fused.  Same results.
+ *     activations (one byte each, up to 1 GiB a call) in stream-ordered scratch memory from a
+ *     pool of the library's own, which keeps at most 256 MiB of them between synchronizations.
+ *     It runs fused, slower by up to half, where the activations take more or have lda != K,
+ *     where there is no memory to be had, and while the stream is being captured: a captured
+ *     call is kernel nodes only.  Same results.
  *   - The library is thread-compatible: concurrent calls are allowed, the error string
  *     is per host thread.
  */
@@ -368,7 +371,8 @@ SPARQ_API int sparq_selftest_mma_rate(int bn, int iters, int64_t *cycles_out, vo
 SPARQ_API const char *sparq_last_error(void);
 
 /* Releases what the library itself holds on the current device (the status word, the
- * scratch pool, the host-buffer forms' staging buffers) and forgets the cached tensor-map encodings.  Safe to call more than once; later calls re-create what they need. */
+ * scratch pool, the host-buffer forms' staging buffers) and forgets the cached tensor-map
+ * encodings.  Safe to call more than once; later calls re-create what they need. */
 SPARQ_API int sparq_shutdown(void);
 
 #ifdef __cplusplus

@@ -36,8 +36,11 @@ int get_status_word(unsigned int **dptr);
 int quantize_rows(const uint8_t *in, uint8_t *out, size_t rows, size_t row_len, const XformArgs &a, cudaStream_t st);
 
 // Stream-ordered scratch memory (sparq_workspace.cu): valid for work enqueued on `st` after the call
-// and before the matching workspace_free.  Any thread, any stream, inside a stream capture too.
-// nullptr when there is none to be had (the caller then takes a path without it).
+// and before the matching workspace_free.  Any thread, any stream.  nullptr when there is none to be
+// had, and while the stream is being captured (the caller then takes a path without it).
+// A larger scratch tensor is not worth taking from the user's device: its caller has a path without.
+constexpr size_t kWorkspaceMaxBytes = (size_t)1 << 30;
+bool workspace_possible(size_t bytes, cudaStream_t st);     // whether it is worth asking
 void *workspace_alloc(size_t bytes, cudaStream_t st);
 void workspace_free(void *p, cudaStream_t st);
 

@@ -1,8 +1,10 @@
 // Scratch memory of the entry points that run as transform + plain contraction: a memory pool of
 // the library's own per device, allocated from and freed to in stream order, so that concurrent
-// calls on other threads and streams, and captured graphs, get memory of their own without any
-// bookkeeping here.  The pool keeps up to kKeepBytes between synchronizations (allocating from
-// the driver costs about a millisecond) and gives back the rest; sparq_shutdown releases it.
+// calls on other threads and streams get memory of their own without any bookkeeping here.  The
+// pool keeps up to kKeepBytes between synchronizations (allocating from the driver costs about a
+// millisecond) and gives back the rest; sparq_shutdown releases it.  A stream that is being
+// captured gets none: the allocation would become nodes of the user's graph, which then cannot be
+// cloned, be a child graph or be instantiated twice, and whose memory neither bound covers.
 #include <mutex>
 
 #include "sparq_common.cuh"
@@ -13,8 +15,6 @@ namespace {
 
 constexpr int kMaxDevices = 64;
 constexpr unsigned long long kKeepBytes = 256ull << 20;
-// A larger scratch tensor is not worth taking from the user's device: its caller has a path without.
-constexpr size_t kMaxBytes = (size_t)1 << 30;
 
 std::mutex g_mu;
 cudaMemPool_t g_pool[kMaxDevices] = {};
@@ -40,9 +40,18 @@ cudaMemPool_t pool_of_current_device()
 
 }  // namespace
 
+bool workspace_possible(size_t bytes, cudaStream_t st)
+{
+    if (bytes > kWorkspaceMaxBytes) return false;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &capture) == cudaSuccess) return capture == cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return false;
+}
+
 void *workspace_alloc(size_t bytes, cudaStream_t st)
 {
-    if (bytes > kMaxBytes) return nullptr;
+    if (!workspace_possible(bytes, st)) return nullptr;
     cudaMemPool_t pool = pool_of_current_device();
     void *p = nullptr;
     if (!pool || cudaMallocFromPoolAsync(&p, bytes, pool, st) != cudaSuccess) {

@@ -1,7 +1,12 @@
 """Calls that run as transform into scratch memory + plain contraction."""
+import ctypes
+
+import numpy as np
 import pytest
 import torch
 
+import oracle
+import sparq_synth as synth
 import paper_2105_11010_b200 as sparq
 
 pytestmark = pytest.mark.gpu
@@ -37,4 +42,46 @@ def test_a_refused_call_enqueues_nothing(entry, bad):
             call[entry](p, next_transform=nxt, **out)
         idle = torch.cuda.current_stream().query()
     assert idle, "the refused call has enqueued work"
+    sparq.sparq_check()
+
+
+def test_a_captured_call_is_kernels_only():
+    """Its graph can be cloned, added to another graph and instantiated more than once."""
+    m, n, k = 1024 + 33, 4096, 4096
+    A, B, p = synth.activations(5, (m, k), 0.5), synth.weights(5, (k, n)), sparq.SparqParams()
+    Ad, Bd = torch.from_numpy(A).cuda(), torch.from_numpy(np.ascontiguousarray(B.T)).cuda()
+    acc = torch.zeros((m, n), dtype=torch.int32, device="cuda")
+    sparq.sparq_gemm_s8(Ad, Bd, p, acc_out=acc)
+    sparq.sparq_check()
+    rows = np.arange(0, m, 61)
+    want = oracle.gemm(A[rows], B, p.mode, 4, 0x1F, 1)
+    assert np.array_equal(acc.cpu().numpy()[rows], want)
+    rt = ctypes.CDLL("libcudart.so.12")
+    vp = ctypes.c_void_p
+    stream = torch.cuda.Stream()
+    st = vp(stream.cuda_stream)
+
+    def ok(rc):
+        assert rc == 0, rc
+
+    graph, clone, parent, node = vp(), vp(), vp(), vp()
+    ok(rt.cudaStreamBeginCapture(st, 0))
+    sparq.sparq_gemm_s8(Ad, Bd, p, acc_out=acc, stream=stream)
+    ok(rt.cudaStreamEndCapture(st, ctypes.byref(graph)))
+    ok(rt.cudaGraphClone(ctypes.byref(clone), graph))
+    ok(rt.cudaGraphCreate(ctypes.byref(parent), 0))
+    ok(rt.cudaGraphAddChildGraphNode(ctypes.byref(node), parent, None, ctypes.c_size_t(0), graph))
+    execs = [vp() for _ in range(4)]
+    for e, g in zip(execs, (graph, graph, clone, parent)):
+        ok(rt.cudaGraphInstantiate(ctypes.byref(e), g, ctypes.c_ulonglong(0)))
+    for e in execs:
+        acc.zero_()
+        torch.cuda.synchronize()
+        ok(rt.cudaGraphLaunch(e, st))
+        stream.synchronize()
+        assert np.array_equal(acc.cpu().numpy()[rows], want)
+    for e in execs:
+        ok(rt.cudaGraphExecDestroy(e))
+    for g in (parent, clone, graph):
+        ok(rt.cudaGraphDestroy(g))
     sparq.sparq_check()
