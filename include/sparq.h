@@ -366,6 +366,21 @@ SPARQ_API int sparq_selftest_wait_timeout(int64_t limit_cycles, int use_static_w
  * launched (> 0) or a negative sparq_status.  The paper has no counterpart. */
 SPARQ_API int sparq_selftest_mma_rate(int bn, int iters, int64_t *cycles_out, void *stream);
 
+/* Diagnostic: the form that sparq_conv2d_nhwc_s8 takes for this layer (requantized output) on a
+ * device of `sms` multiprocessors, outside a stream capture; a 1x1 filter with unit strides is
+ * sparq_gemm_s8 with M = n*h*w, N = cout, K = c.  Host arithmetic only: needs no device.
+ * Returns one of the values below or a negative sparq_status.  The paper has no counterpart. */
+enum {
+    SPARQ_FORM_FULL = 0,            /* one persistent CTA per SM, transform per staged tile */
+    SPARQ_FORM_SMALL = 1,           /* few tiles: half an SM per CTA, clusters sharing a tile */
+    SPARQ_FORM_WINDOW_RESIDENT = 2, /* padded image rows in shared memory, all weights beside them */
+    SPARQ_FORM_WINDOW_STREAMED = 3, /* the same, weights through a ring */
+    SPARQ_FORM_TRANSFORM_FIRST = 4  /* transform into scratch memory, then a plain contraction */
+};
+SPARQ_API int sparq_selftest_form(int n, int h, int w, int c, int cout, int r, int s,
+                        int stride_h, int stride_w, int pad_h, int pad_w,
+                        const sparq_params *p, int sms);
+
 /* Text of the calling thread's most recent error ("" if none).  The pointer stays valid
  * until the thread's next failing call. */
 SPARQ_API const char *sparq_last_error(void);

@@ -19,5 +19,6 @@ from ._binding import (  # noqa: F401
     sparq_sparse24_expanded_k, sparq_sparse24_expand_weights, sparq_sparse24_expand_activations,
     sparq_gemm_s8_sparse24,
     sparq_absmax, sparq_quantize_act_u8, sparq_quantize_weight_s8, DTYPE_F32, DTYPE_BF16,
-    sparq_check, sparq_last_error, sparq_shutdown, sparq_selftest_wait_timeout, sparq_selftest_mma_rate,
+    sparq_check, sparq_last_error, sparq_shutdown, sparq_selftest_wait_timeout, sparq_selftest_mma_rate, sparq_selftest_form,
+    FORM_FULL, FORM_SMALL, FORM_WINDOW_RESIDENT, FORM_WINDOW_STREAMED, FORM_TRANSFORM_FIRST,
 )

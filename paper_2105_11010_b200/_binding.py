@@ -113,6 +113,8 @@ def load_library() -> ctypes.CDLL:
         L.sparq_selftest_wait_timeout.restype = i32
         L.sparq_selftest_mma_rate.argtypes = [i32, i32, vp, vp]
         L.sparq_selftest_mma_rate.restype = i32
+        L.sparq_selftest_form.argtypes = [i32] * 11 + [ctypes.POINTER(_CParams), i32]
+        L.sparq_selftest_form.restype = i32
         L.sparq_check.argtypes = [vp]
         L.sparq_check.restype = i32
         L.sparq_last_error.argtypes = []
@@ -194,6 +196,20 @@ def sparq_selftest_mma_rate(bn: int, iters: int, cycles_out: torch.Tensor, strea
     if cycles_out.dtype != torch.int64 or not cycles_out.is_cuda or cycles_out.numel() < 256:
         raise ValueError("cycles_out must be an int64 device tensor of at least 256 elements")
     rc = load_library().sparq_selftest_mma_rate(int(bn), int(iters), cycles_out.data_ptr(), _stream_ptr(stream))
+    if rc < 0:
+        _raise(rc)
+    return rc
+
+
+FORM_FULL, FORM_SMALL, FORM_WINDOW_RESIDENT, FORM_WINDOW_STREAMED, FORM_TRANSFORM_FIRST = range(5)
+
+
+def sparq_selftest_form(x_shape, w_shape, stride, pad, params: SparqParams, sms: int = 148) -> int:
+    """The form (``FORM_*``) that a convolution of this shape takes; host arithmetic only."""
+    n, h, w, c = x_shape
+    cout, r, s, _ = w_shape
+    p = params._c()
+    rc = load_library().sparq_selftest_form(n, h, w, c, cout, r, s, stride[0], stride[1], pad[0], pad[1], ctypes.byref(p), sms)
     if rc < 0:
         _raise(rc)
     return rc

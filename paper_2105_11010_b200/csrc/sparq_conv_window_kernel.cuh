@@ -48,6 +48,7 @@ struct WindowArgs {
     int plane_bytes;        // shared-memory bytes reserved per channel block (>= rows the MMA may touch)
     int win_bufs;           // window buffers in the ring
     int b_stages;           // weight stages (stream mode) or resident blocks (resident mode)
+    int team_copy;          // 256-wide tiles: room behind the weight stages for the second epilogue team's scale and bias
     int issuers;            // 2: the two issuer warps alternate (resident weights); 1: warp 1 issues every tile (streamed weights)
     uint32_t n_tiles;       // column tiles
     uint32_t units;         // n_img * tiles_per_img * n_tiles, column tile fastest
@@ -73,10 +74,13 @@ struct WindowArgs {
     float residual_scale;
 };
 
-// dynamic shared memory the kernel may ask for: 227 KB minus room for its static variables (with
-// streamed weights the epilogue teams keep scale and bias of their own column tiles)
+// dynamic shared memory the kernel may ask for: 227 KB minus room for its static variables
 constexpr int kWindowMaxDynSmem = 232448 - 4096;
-constexpr int kWindowMaxDynSmemStreamed = kWindowMaxDynSmem - 3072;
+// With streamed weights the epilogue teams keep scale and bias of their own column tiles.  On 256-wide
+// tiles the second team's lie in dynamic memory, where there is room (else one team): as static
+// variables they took a stage of the ring, or the whole kernel, from shapes that just fit
+// (64x35x35x384 -> 192 3x3 102 us, by the im2col kernel 150).
+constexpr int kTeamCopyBytes = 2 * 256 * 4;
 constexpr int kMaxWinBufs = 4;
 constexpr int kMaxG = 8;
 constexpr int kMaxBStages = 12;
@@ -174,12 +178,12 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
     // epilogue teams: as in sparq_gemm_kernel
     constexpr int kGroups = epi_warps(MODE) / 4;
     constexpr int kMaxTeams = kOneTeam ? 1 : kGroups < kAcc ? kGroups : kAcc;
-    const int teams = kMaxTeams > 1 && g.units > gridDim.x ? kMaxTeams : 1;
+    const int teams = kMaxTeams > 1 && g.units > gridDim.x && (BN != 256 || g.team_copy) ? kMaxTeams : 1;
     __shared__ __align__(8) uint64_t bar_acc_full[kAcc], bar_acc_empty[kAcc], bar_done;
     __shared__ uint32_t tmem_base_slot;
     __shared__ uint32_t abort_word;
     // one column tile (resident weights): the teams share one copy, all writing the same values
-    constexpr int kCopies = B_RESIDENT ? 1 : kMaxTeams;
+    constexpr int kCopies = B_RESIDENT || BN == 256 ? 1 : kMaxTeams;
     __shared__ __align__(16) float s_scale_all[kCopies][BN], s_bias_all[kCopies][BN];
 
     constexpr int kBBlock = BN * CB;                   // one (tap, channel block) of weights
@@ -537,7 +541,11 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
         const int parts = epi_parts(kGroups, teams, BN), part = group / teams;
         const int cols = BN / parts, cbase = part * cols;
         const int team_thread = (part * 4 + quarter) * 32 + lane, team_threads = parts * 128;
-        float *s_scale = s_scale_all[B_RESIDENT ? 0 : team], *s_bias = s_bias_all[B_RESIDENT ? 0 : team];
+        float *s_scale = s_scale_all[kCopies == 1 ? 0 : team], *s_bias = s_bias_all[kCopies == 1 ? 0 : team];
+        if (BN == 256 && team) {
+            s_scale = reinterpret_cast<float *>(smem_raw + (b_slot(g.b_stages) - smem_u32(smem_raw)));
+            s_bias = s_scale + BN;
+        }
         const EpiView ev = make_epi_view(g);
         uint32_t wt = 0;
         int64_t staged_nt = -1;
@@ -645,7 +653,7 @@ cudaError_t launch_window_kernel(const CUtensorMap &mx0, const CUtensorMap &mx1,
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-        e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, RES ? kWindowMaxDynSmem : kWindowMaxDynSmemStreamed);
+        e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, kWindowMaxDynSmem);
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) attr_set[dev] = true;
     }

@@ -403,26 +403,79 @@ static int encode_weights(CUtensorMap *map, const void *ptr, int c, int cout, in
 
 constexpr int kMaxDynSmem = kWindowMaxDynSmem;
 
-// Stride-1 filters larger than 1x1: the window kernel, when its tiling fits.  Returns
-// 1 if it launched, 0 if the shape should take the im2col kernel, < 0 on error.
-static int try_window_conv(const uint8_t *x_in, int n, int h, int w, int c, const int8_t *wgt, int cout, int r, int s,
-                           int pad_h, int pad_w, int ho, int wo, const XformArgs &x, const sparq_epilogue *e,
-                           int sms, unsigned int *status, cudaStream_t st)
+// ---- which form a stride-1 convolution takes ---------------------------------------------------------
+// Estimates in us, least-squares fits to 840 measured layers (1-128 images of 7..56 pixels, 16-512
+// channels and filters, 3x3 / 5x5 / 7x7, five transforms and none).  Root mean square error: window
+// with streamed weights on 128-wide tiles 7 %, on 256-wide ones 22 %, small form 10 %, im2col form
+// 11 %.  They are compared where either form can win by a factor: few tiles (over 493 layers the
+// choice costs 0.2 % against the faster form, at worst 20 %; always the window 48 %), half-empty channel
+// blocks (1.4 %; always the window 13 %) and rings of two stages.
+// The transform's work relative to the 4-bit form with all placements.
+static double xform_weight(const XformArgs &x)
+{
+    return x.mode == SPARQ_MODE_NONE ? 0.0 : x.n == 4 ? (x.widen_rounds ? 1.2 : 1.0) : (x.widen_rounds ? 2.0 : 1.35);
+}
+// Bytes per output element that the epilogue moves.
+static double out_weight(const sparq_epilogue *e)
+{
+    return (e->acc_out ? 4 : 0) + (e->f32_out ? 4 : 0) + (e->u8_out ? 1 : 0) + (e->residual ? 1 : 0);
+}
+static double small_us(const SmallForm &f, int64_t M, int64_t k_blocks, int bk, double xw)
+{
+    const double rows = (double)(M < f.tile_rows ? M : f.tile_rows) / kBM * bk / 128.0;
+    return 2.5 + (double)((k_blocks + f.split - 1) / f.split) * (0.21 + (0.09 + 0.60 * xw) * rows) + (f.split > 1 ? 1.3 : 0.0);
+}
+static double im2col_us(int64_t M, int64_t N, int taps, int c, double xw, double ow, int sms)
+{
+    const int bk = c % 128 == 0 ? 128 : 64;
+    const int bn = pick_bn(M, N, (int64_t)taps * ((c + 127) / 128), sms, xw > 0.0, true);
+    const double rounds = (double)(((M + kBM - 1) / kBM * ((N + bn - 1) / bn) + sms - 1) / sms), blocks = rounds * taps * ((c + bk - 1) / bk);
+    return 2.6 + blocks * bk / 128.0 * ((bn == 64 ? 0.05 : bn == 128 ? 0.10 : 0.13) + (bn == 256 ? 0.46 : 0.48) * xw) + 0.22 * blocks +
+           0.47 * rounds * bn / 128.0 * ow;
+}
+// The same layer by the im2col path, in the form that would be launched there.
+static double im2col_path_us(int64_t M, int64_t N, int taps, int c, double xw, double ow, int sms)
+{
+    const int bk = c % 128 == 0 ? 128 : 64;
+    const int64_t k_blocks = (int64_t)taps * ((c + bk - 1) / bk);
+    const SmallForm f = pick_small(M, N, k_blocks, sms, xw > 0.0);
+    return f.tile_rows ? small_us(f, M, k_blocks, bk, xw) : im2col_us(M, N, taps, c, xw, ow, sms);
+}
+
+// How the window kernel tiles a convolution.
+struct WindowPlan {
+    int wp, cb, tr, c_blocks, tiles_per_img, bn, n_tiles;
+    int64_t units;
+    bool resident;
+    int grp, win_bufs, b_stages, plane_bytes;
+    bool team_copy;
+    int smem_bytes;
+};
+
+// Stride-1 filters larger than 1x1: false where the window kernel's tiling does not fit, or another form
+// is expected to be faster.  ow: out_weight of the epilogue; scratch(bytes): whether T(x) may be
+// written to scratch memory.
+template <class Scratch>
+static bool plan_window(WindowPlan *q, int n, int h, int w, int c, int cout, int r, int s, int pad_w, int ho, int wo,
+                        const XformArgs &x, double ow, int sms, Scratch scratch)
 {
     int wp = w + 2 * pad_w;
-    if (wp > 128 || wo < 1) return 0;
+    if (wp > 128 || wo < 1) return false;
     // channel blocks; the last one's tail is zero fill.  Few channels and many filters: 128-wide blocks
     // that are half empty, because 64-channel blocks exist on 64-wide tiles only.
     const int cb = (c <= 64 && cout <= 64) ? 64 : 128;
     int tr = 128 / wp;
     if (tr > ho) tr = ho;
-    if (tr < 1 || tr * wo < 64) return 0;               // less than half of the MMA rows would be useful
+    if (tr < 1 || tr * wo < 64) return false;               // less than half of the MMA rows would be useful
     // Pieces land at multiples of tr * wp rows, which must be a multiple of 128 bytes: an even row
     // width makes it so for 64-byte rows.
     if (cb == 64 && (wp & 1) && wp + 1 <= 128 && (128 / (wp + 1) >= tr)) ++wp;
     const int c_blocks = (c + cb - 1) / cb;
     const int taps = r * s;
     const int kb_count = taps * c_blocks;
+    const bool half_empty = cb == 128 && c <= 64;
+    const int64_t M = (int64_t)n * ho * wo;
+    const double xw = xform_weight(x);
     const int tiles_per_img = (ho + tr - 1) / tr;
     const int64_t m_tiles = (int64_t)n * tiles_per_img;
 
@@ -435,8 +488,8 @@ static int try_window_conv(const uint8_t *x_in, int n, int h, int w, int c, cons
     const int b_block = bn * cb;
     const int n_tiles = (cout + bn - 1) / bn;
     const int64_t units = m_tiles * n_tiles;
-    if (units >= (int64_t)1 << 31) return 0;
-    int grid = (int)(units < sms ? units : sms);
+    if (units >= (int64_t)1 << 31) return false;
+    const int grid = (int)(units < sms ? units : sms);
 
     // Shared memory of one window buffer when up to `grp` tiles share it: a plane (one channel
     // block) holds every row the MMA of the group's last tile may touch.
@@ -466,43 +519,82 @@ static int try_window_conv(const uint8_t *x_in, int n, int h, int w, int c, cons
         while (win_bufs < kMaxWinBufs && win_bufs < groups_per_cta &&
                1024 + (win_bufs + 1) * plane_for(grp) * c_blocks + kb_count * b_block <= kMaxDynSmem) ++win_bufs;
     } else {
-        if (bn == 64) return 0;                          // only the resident form is built for 64-wide tiles
-        // Few tiles: the im2col form, whose long reduction a cluster can share (one image of
-        // 14x14x256 -> 256 3x3: 6.9 us against 14.6; with resident weights the window kernel wins).
-        if (pick_small((int64_t)n * ho * wo, cout, kb_count, sms, x.mode != SPARQ_MODE_NONE).split > 1) return 0;
+        if (bn == 64) return false;                          // only the resident form is built for 64-wide tiles
         // 128-wide tiles: up to two row tiles of one (image, column tile) are accumulated together
         // during ONE pass over the streamed weights (four accumulator stages: two groups in
         // flight), which halves the weight traffic out of L2 -- the bound of these layers.
         batched = bn == 128;
-        grp = batched ? (tiles_per_img < 2 ? tiles_per_img : 2) : gmax;
-        while (grp > 1 && kWindowMaxDynSmemStreamed - 1024 - 2 * plane_for(grp) * c_blocks < 4 * b_block) --grp;
-        const int win_bytes1 = plane_for(grp) * c_blocks;
-        // a CTA that owns a single group needs no second window buffer: the room goes to the
-        // weight ring, whose depth (bytes in flight) bounds how fast one SM can pull the weights
-        const int64_t groups_b = (int64_t)n * n_tiles * ((tiles_per_img + grp - 1) / grp);
-        if (batched && groups_b <= sms) win_bufs = 1;
-        const int left = kWindowMaxDynSmemStreamed - 1024 - win_bufs * win_bytes1;
-        b_stages = left / b_block;
-        if (b_stages > kMaxBStages) b_stages = kMaxBStages;
-        if (b_stages < 2) return 0;
-        // spare room beyond four weight stages goes to a third window buffer
-        if (win_bufs == 2 && b_stages > 4 && 1024 + 3 * win_bytes1 + 4 * b_block <= kWindowMaxDynSmemStreamed) {
-            win_bufs = 3;
-            b_stages = (kWindowMaxDynSmemStreamed - 1024 - 3 * win_bytes1) / b_block;
-            if (b_stages > kMaxBStages) b_stages = kMaxBStages;
+        double window_us = 0.0;
+        auto consider = [&](int g) {
+            const int bytes = plane_for(g) * c_blocks;
+            // a CTA that owns a single group needs no second window buffer: the room goes to the
+            // weight ring, whose depth (bytes in flight) bounds how fast one SM can pull the weights
+            const int64_t groups = (int64_t)n * n_tiles * ((tiles_per_img + g - 1) / g);
+            int bufs = batched && groups <= sms ? 1 : 2;
+            int stages = (kMaxDynSmem - 1024 - bufs * bytes) / b_block;
+            if (stages > kMaxBStages) stages = kMaxBStages;
+            if (stages < 2) return;
+            // spare room beyond four weight stages goes to a third window buffer
+            if (bufs == 2 && stages > 4 && 1024 + 3 * bytes + 4 * b_block <= kMaxDynSmem) {
+                bufs = 3;
+                stages = (kMaxDynSmem - 1024 - 3 * bytes) / b_block;
+                if (stages > kMaxBStages) stages = kMaxBStages;
+            }
+            const double rows = (double)((batched ? tr * g : tr) + r - 1) * wp / 128.0, ring = stages == 2 ? 0.09 : 0.0;
+            const double us =
+                batched ? 3.9 + (double)((groups + sms - 1) / sms) * (kb_count * (0.066 + 0.159 * g + ring) + c_blocks * rows * (0.73 * xw + 0.23))
+                        : 6.0 + (double)((units + sms - 1) / sms) * (kb_count * (0.373 + ring) + c_blocks * rows * (0.65 * xw + 0.46));
+            if (b_stages == 0 || us < window_us) { window_us = us; grp = g; win_bufs = bufs; b_stages = stages; }
+        };
+        if (batched) {
+            // one tile a group or two: two halve the weight traffic, one has more CTAs where they are few
+            // (8x28x28x256 -> 192: 10.9 us with one, 15.2 with two)
+            consider(1);
+            if (tiles_per_img > 1 && kMaxDynSmem - 1024 - 2 * plane_for(2) * c_blocks >= 4 * b_block) consider(2);
+        } else {
+            int g = gmax;
+            while (g > 1 && kMaxDynSmem - 1024 - 2 * plane_for(g) * c_blocks < 4 * b_block) --g;
+            consider(g);
+        }
+        if (b_stages == 0) return false;
+        // Few tiles: the small form, whose long reduction a cluster can share, may be faster (one image
+        // of 14x14x256 -> 256 3x3: 6.9 us against 14.6) or not (8x14x14x512 -> 512 5x5: 82 against 33).
+        // Half-empty channel blocks: the im2col form reads 64-channel ones, half the multiplications
+        // and operand bytes for one transform per tap (64x17x17x64 -> 256 3x3: 8.3 us against 12.7;
+        // 17x35x35x32 -> 160 7x7 at 2 bits 45 against 25).
+        if (half_empty || (batched && pick_small(M, cout, (int64_t)taps * ((c + 127) / 128), sms, xw > 0.0).tile_rows)) {
+            if (im2col_path_us(M, cout, taps, c, xw, ow, sms) < window_us) return false;
+        } else if (batched && b_stages == 2) {
+            // a ring this short leaves the tensor core waiting; transformed once, the im2col form may win
+            // (16x56x56x256 -> 64 5x5 at 3 bits, restricted: 56 us against 100)
+            const size_t act_bytes = (size_t)n * h * w * (size_t)c;
+            const double first = xw > 0.0 && scratch(act_bytes) ? 2.5 + (double)act_bytes / 2.9e6 + im2col_us(M, cout, taps, c, 0.0, ow, sms) : 1e30;
+            if (first < window_us || im2col_path_us(M, cout, taps, c, xw, ow, sms) < window_us) return false;
         }
     }
-    const int plane_bytes = plane_for(grp);
-    const int win_bytes = plane_bytes * c_blocks;
-    const int smem_bytes = 1024 + win_bufs * win_bytes + b_stages * b_block;
+    *q = {wp, cb, tr, c_blocks, tiles_per_img, bn, n_tiles, units, resident, grp, win_bufs, b_stages, plane_for(grp), false, 0};
+    q->smem_bytes = 1024 + win_bufs * q->plane_bytes * c_blocks + b_stages * b_block;
+    q->team_copy = bn == 256 && q->smem_bytes + kTeamCopyBytes <= kMaxDynSmem;
+    if (q->team_copy) q->smem_bytes += kTeamCopyBytes;
+    return true;
+}
 
+// Returns 1 if the window kernel was launched, 0 if the convolution should take another form, < 0 on error.
+static int try_window_conv(const uint8_t *x_in, int n, int h, int w, int c, const int8_t *wgt, int cout, int r, int s,
+                           int pad_h, int pad_w, int ho, int wo, const XformArgs &x, const sparq_epilogue *e,
+                           int sms, unsigned int *status, cudaStream_t st)
+{
+    WindowPlan q;
+    if (!plan_window(&q, n, h, w, c, cout, r, s, pad_w, ho, wo, x, out_weight(e), sms, [&](size_t bytes) { return workspace_possible(bytes, st); }))
+        return 0;
+    const int cb = q.cb, wp = q.wp, tr = q.tr, bn = q.bn;
     CUtensorMap mx, mx1, mw;
     int rc = encode_window(&mx, x_in, n, h, w, c, cb, wp, tr + r - 1);
     if (rc != SPARQ_OK) return rc;
     rc = encode_window(&mx1, x_in, n, h, w, c, cb, wp, tr);
     if (rc != SPARQ_OK) return rc;
     const int64_t K = (int64_t)r * s * c;
-    rc = encode_weights(&mw, wgt, c, cout, taps, cb, bn, !resident ? 1 : r == 3 && s == 3 ? taps : s);   // as the kernel copies them
+    rc = encode_weights(&mw, wgt, c, cout, r * s, cb, bn, !q.resident ? 1 : r == 3 && s == 3 ? r * s : s);   // as the kernel copies them
     if (rc != SPARQ_OK) return rc;
 
     WindowArgs g;
@@ -510,24 +602,26 @@ static int try_window_conv(const uint8_t *x_in, int n, int h, int w, int c, cons
     // Streamed weights pass through a ring that is shorter than one tile's blocks, in tile order:
     // two issuers on different tiles would wait on the same stage barriers several phases apart,
     // which a parity wait cannot tell apart.  One issuer then; two with resident weights.
-    g.issuers = resident ? 2 : 1;
+    g.issuers = q.resident ? 2 : 1;
     g.N = cout; g.K = K;
     g.n_img = n; g.H = h; g.W = w; g.C = c; g.R = r; g.S = s; g.pad_h = pad_h; g.pad_w = pad_w; g.Ho = ho; g.Wo = wo;
-    g.Wp = wp; g.TR = tr; g.tiles_per_img = tiles_per_img; g.c_blocks = c_blocks;
-    g.G = grp;
+    g.Wp = wp; g.TR = tr; g.tiles_per_img = q.tiles_per_img; g.c_blocks = q.c_blocks;
+    g.G = q.grp;
     g.piece0_bytes = cb * wp * (tr + r - 1);
     g.piece_bytes = cb * wp * tr;
-    g.n_tiles = (uint32_t)n_tiles;
-    g.units = (uint32_t)units;
-    if (batched) {
+    g.n_tiles = (uint32_t)q.n_tiles;
+    g.units = (uint32_t)q.units;
+    int grid = (int)(q.units < sms ? q.units : sms);
+    if (!q.resident && bn == 128) {
         // CTAs own whole groups, so that a group is never cut at a share boundary
-        const int64_t groups = (int64_t)n * n_tiles * ((tiles_per_img + grp - 1) / grp);
+        const int64_t groups = (int64_t)n * q.n_tiles * ((q.tiles_per_img + q.grp - 1) / q.grp);
         g.groups = (uint32_t)groups;
         grid = (int)(groups < sms ? groups : sms);
     }
-    g.plane_bytes = plane_bytes;
-    g.win_bufs = win_bufs;
-    g.b_stages = b_stages;
+    g.plane_bytes = q.plane_bytes;
+    g.win_bufs = q.win_bufs;
+    g.b_stages = q.b_stages;
+    g.team_copy = q.team_copy ? 1 : 0;
     g.xf = xform_dev(x);
     g.scale = e->scale; g.bias = e->bias; g.relu = e->relu ? 1 : 0; g.inv_out_scale = e->inv_out_scale;
     g.acc_out = e->acc_out; g.f32_out = e->f32_out; g.u8_out = e->u8_out;
@@ -538,10 +632,10 @@ static int try_window_conv(const uint8_t *x_in, int n, int h, int w, int c, cons
     rc = next_transform_args(e, g.N, &g.next_mode, &g.next_rnd, &g.next_xf);
     if (rc != SPARQ_OK) return rc;
     cudaError_t ce;
-    if (bn == 64) ce = launch_window_shape<64, 64, true>(mx, mx1, mw, g, x.mode, variant_n(x), x.rnd, grid, smem_bytes, st);
-    else if (bn == 128 && resident) ce = launch_window_shape<128, 128, true>(mx, mx1, mw, g, x.mode, variant_n(x), x.rnd, grid, smem_bytes, st);
-    else if (bn == 128) ce = launch_window_shape<128, 128, false>(mx, mx1, mw, g, x.mode, variant_n(x), x.rnd, grid, smem_bytes, st);
-    else ce = launch_window_shape<256, 128, false>(mx, mx1, mw, g, x.mode, variant_n(x), x.rnd, grid, smem_bytes, st);
+    if (bn == 64) ce = launch_window_shape<64, 64, true>(mx, mx1, mw, g, x.mode, variant_n(x), x.rnd, grid, q.smem_bytes, st);
+    else if (bn == 128 && q.resident) ce = launch_window_shape<128, 128, true>(mx, mx1, mw, g, x.mode, variant_n(x), x.rnd, grid, q.smem_bytes, st);
+    else if (bn == 128) ce = launch_window_shape<128, 128, false>(mx, mx1, mw, g, x.mode, variant_n(x), x.rnd, grid, q.smem_bytes, st);
+    else ce = launch_window_shape<256, 128, false>(mx, mx1, mw, g, x.mode, variant_n(x), x.rnd, grid, q.smem_bytes, st);
     if (ce != cudaSuccess) return cuda_error(ce, "sparq_conv_window_kernel launch");
     return 1;
 }
@@ -747,4 +841,26 @@ extern "C" int sparq_conv2d_nhwc_s8(const uint8_t *x_in, int n, int h, int w, in
         }
     }
     return im2col_conv(x_in, n, h, w, c, wgt, cout, r, s, stride_h, stride_w, pad_h, pad_w, ho, wo, x, e, sms, status, st);
+}
+
+extern "C" int sparq_selftest_form(int n, int h, int w, int c, int cout, int r, int s, int stride_h, int stride_w, int pad_h, int pad_w,
+                                   const sparq_params *p, int sms)
+{
+    XformArgs x;
+    const int rc = validate_params(p, &x);
+    if (rc != SPARQ_OK) return rc;
+    if (n < 1 || h < 1 || w < 1 || c < 16 || c % 16 || cout < 1 || r < 1 || s < 1 || r > 7 || s > 7 || stride_h < 1 || stride_w < 1 ||
+        pad_h < 0 || pad_w < 0 || pad_h >= r || pad_w >= s || h + 2 * pad_h < r || w + 2 * pad_w < s || sms < 1)
+        return set_error(SPARQ_ERR_INVALID_ARG, "bad convolution geometry");
+    const int ho = (h + 2 * pad_h - r) / stride_h + 1, wo = (w + 2 * pad_w - s) / stride_w + 1;
+    const int64_t M = (int64_t)n * ho * wo;
+    const bool matrix = r == 1 && s == 1 && stride_h == 1 && stride_w == 1;
+    WindowPlan q;
+    auto scratch = [](size_t bytes) { return bytes <= kWorkspaceMaxBytes; };
+    if (!matrix && stride_h == 1 && stride_w == 1 && plan_window(&q, n, h, w, c, cout, r, s, pad_w, ho, wo, x, 1.0, sms, scratch))
+        return q.resident ? SPARQ_FORM_WINDOW_RESIDENT : SPARQ_FORM_WINDOW_STREAMED;
+    const int64_t steps = (int64_t)r * s * ((c + 127) / 128);
+    const size_t act_bytes = (size_t)n * h * w * (size_t)c;
+    if (x.mode != SPARQ_MODE_NONE && transform_first(M, cout, steps, act_bytes, sms, !matrix) && scratch(act_bytes)) return SPARQ_FORM_TRANSFORM_FIRST;
+    return pick_small(M, cout, steps, sms, x.mode != SPARQ_MODE_NONE).tile_rows ? SPARQ_FORM_SMALL : SPARQ_FORM_FULL;
 }
