@@ -356,26 +356,45 @@ __device__ __forceinline__ uint32_t requant_pack4(float z0, float z1, float z2, 
     return w;
 }
 
+// The next layer's transform of one word, inline: one run-time form for every width, set and rounding.
+__device__ __forceinline__ uint32_t next_xform_word(uint32_t x, int mode, int rnd, const XformDev &xf)
+{
+    const uint32_t m = drop_mask<0, true>(x, xf.n, xf.widen_c);
+    const uint32_t q = rnd ? apply_mask<true>(x, m, xf.n) : apply_mask<false>(x, m, xf.n);
+    if (mode != SPARQ_MODE_VSPARQ) return q;
+    uint32_t lone = x;
+    if (xf.n < 4) {
+        const uint32_t ml = drop_mask<0, false>(x, 2 * xf.n, 0u);
+        lone = rnd ? apply_mask<true>(x, ml, 2 * xf.n) : apply_mask<false>(x, ml, 2 * xf.n);
+    }
+    const uint32_t nz = ((x & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | x;
+    const uint32_t partner_nz = prmt(nz, nz, 0xAB89u);
+    return (q & partner_nz) | (lone & ~partner_nz);
+}
+
 // The next layer's transform on requantized bytes (producer-side SPARQ): four adjacent output
 // channels per word, pairs (2j, 2j+1) inside it.  Kept out of line: the epilogue loops are hot
 // and every variant inlined at every use made the kernels several times larger than the
 // instruction caches, which the warp roles share.
-static __device__ __noinline__ void next_xform_words(uint32_t *w, int count, int mode, int rnd, XformDev xf)
+// (Words by value: through a pointer they went to local memory and back, 4-14 % of such a layer.)
+struct Words8 {
+    uint32_t w[8];
+};
+static __device__ __noinline__ Words8 next_xform_words(Words8 v, int mode, int rnd, XformDev xf)
 {
     const bool full = xf.rounds == 0 && xf.n != 4;   // 6opt / 7opt: the half-precision form
-    for (int q = 0; q < count; ++q) {
-        uint32_t x = w[q];
-        if (mode == SPARQ_MODE_VSPARQ) {
-            if (full) x = xform_word_fullset<SPARQ_MODE_VSPARQ>(x, xf);
-            else if (xf.rounds == 0) x = rnd ? xform_word<SPARQ_MODE_VSPARQ, 4, true, false>(x, xf) : xform_word<SPARQ_MODE_VSPARQ, 4, false, false>(x, xf);
-            else x = rnd ? xform_word<SPARQ_MODE_VSPARQ, 0, true, true>(x, xf) : xform_word<SPARQ_MODE_VSPARQ, 0, false, true>(x, xf);
-        } else {
-            if (full) x = xform_word_fullset<SPARQ_MODE_BSPARQ>(x, xf);
-            else if (xf.rounds == 0) x = rnd ? xform_word<SPARQ_MODE_BSPARQ, 4, true, false>(x, xf) : xform_word<SPARQ_MODE_BSPARQ, 4, false, false>(x, xf);
-            else x = rnd ? xform_word<SPARQ_MODE_BSPARQ, 0, true, true>(x, xf) : xform_word<SPARQ_MODE_BSPARQ, 0, false, true>(x, xf);
-        }
-        w[q] = x;
+    auto each = [&](auto f) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v.w[q] = f(v.w[q]);
+    };
+    if (mode == SPARQ_MODE_VSPARQ) {
+        if (full) each([&](uint32_t x) { return xform_word_fullset<SPARQ_MODE_VSPARQ>(x, xf); });
+        else if (xf.rounds == 0 && rnd) each([&](uint32_t x) { return xform_word<SPARQ_MODE_VSPARQ, 4, true, false>(x, xf); });
+        else each([&](uint32_t x) { return next_xform_word(x, mode, rnd, xf); });
+    } else {
+        each([&](uint32_t x) { return next_xform_word(x, mode, rnd, xf); });
     }
+    return v;
 }
 
 // Per-thread view of the epilogue's outputs and constants.
@@ -653,7 +672,14 @@ __device__ __forceinline__ void epi_general(const EpiView &e, uint32_t (&v)[32],
             f2_unpack(f2_mul(f2_pack(__uint_as_float(v[4 * q + 2]), __uint_as_float(v[4 * q + 3])), inv2), z[2], z[3]);
             w[q] = requant_pack4(z[0], z[1], z[2], z[3]);
         }
-        if (e.next_mode != SPARQ_MODE_NONE) next_xform_words(w, 8, e.next_mode, e.next_rnd, e.next_xf);
+        if (e.next_mode != SPARQ_MODE_NONE) {
+            Words8 t;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) t.w[q] = w[q];
+            t = next_xform_words(t, e.next_mode, e.next_rnd, e.next_xf);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) w[q] = t.w[q];
+        }
         if (ODD) store_bytes_unaligned(e.u8_out + off, w, cols);
         else store_bytes32(e.u8_out + off, w, cols, e.gran);
     }

@@ -84,7 +84,7 @@ __device__ __forceinline__ void epi_four(const EpiView &e, const int (&a)[4], co
     if (e.u8_out) {
         uint32_t w = requant_pack4(__fmul_rn(y[0], e.inv_out_scale), __fmul_rn(y[1], e.inv_out_scale),
                                    __fmul_rn(y[2], e.inv_out_scale), __fmul_rn(y[3], e.inv_out_scale));
-        if (e.next_mode != SPARQ_MODE_NONE) next_xform_words(&w, 1, e.next_mode, e.next_rnd, e.next_xf);
+        if (e.next_mode != SPARQ_MODE_NONE) w = next_xform_word(w, e.next_mode, e.next_rnd, e.next_xf);
         if (full) *reinterpret_cast<uint32_t *>(e.u8_out + off) = w;
         else for (int i = 0; i < cols; ++i) e.u8_out[off + i] = (uint8_t)(w >> (8 * i));
     }

@@ -3,10 +3,10 @@
 
 namespace sparq {
 
-template <int BN, int XN, bool RND>
-static cudaError_t launch_x24_kernel(const CUtensorMap &ma, const CUtensorMap &mb, const GemmArgs &g, int grid, cudaStream_t st)
+template <int BN, int XN, bool RND, int OUT>
+static cudaError_t launch_x24_out(const CUtensorMap &ma, const CUtensorMap &mb, const GemmArgs &g, int grid, cudaStream_t st)
 {
-    auto kfn = sparq_gemm_sparse24_kernel<BN, XN, RND>;
+    auto kfn = sparq_gemm_sparse24_kernel<BN, XN, RND, OUT>;
     static bool attr_set[64] = {};   // per device ordinal
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -17,6 +17,13 @@ static cudaError_t launch_x24_kernel(const CUtensorMap &ma, const CUtensorMap &m
         if (dev >= 0 && dev < 64) attr_set[dev] = true;
     }
     return launch_overlapped(kfn, grid, kX24Threads, X24Cfg<BN>::kSmemBytes, st, ma, mb, g);
+}
+
+template <int BN, int XN, bool RND>
+static cudaError_t launch_x24_kernel(const CUtensorMap &ma, const CUtensorMap &mb, const GemmArgs &g, int grid, cudaStream_t st)
+{
+    return make_epi_view(g).out == kOutBytes ? launch_x24_out<BN, XN, RND, kOutBytes>(ma, mb, g, grid, st)
+                                             : launch_x24_out<BN, XN, RND, kOutGeneral>(ma, mb, g, grid, st);
 }
 
 template <int BN>

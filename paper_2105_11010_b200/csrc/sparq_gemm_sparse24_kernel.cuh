@@ -39,7 +39,8 @@ struct X24Cfg {
     static constexpr int kTmemCols = 4 * BN;                          // two tiles of two accumulators
 };
 
-template <int BN, int XN, bool RND>
+// OUT: kOutBytes, or kOutGeneral for every other kind of output.
+template <int BN, int XN, bool RND, int OUT>
 __global__ void __launch_bounds__(kX24Threads, 1)
 sparq_gemm_sparse24_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, const GemmArgs g)
 {
@@ -183,8 +184,7 @@ sparq_gemm_sparse24_kernel(const __grid_constant__ CUtensorMap map_a, const __gr
                     tc_fence_after();
                 };
                 const uint32_t empty = smem_u32(&bar_acc_empty[acc]);
-                if (ev.out == kOutBytes) epi_warp_columns<kOutBytes>(ev, taddr0, 0, BN, row, row < g.M, nt * BN, s_scale, s_bias, empty, lane, wait_full);
-                else epi_warp_columns<kOutGeneral>(ev, taddr0, 0, BN, row, row < g.M, nt * BN, s_scale, s_bias, empty, lane, wait_full);
+                epi_warp_columns<OUT>(ev, taddr0, 0, BN, row, row < g.M, nt * BN, s_scale, s_bias, empty, lane, wait_full);
             }
         }
     } else {
