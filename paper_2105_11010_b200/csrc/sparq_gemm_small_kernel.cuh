@@ -66,8 +66,13 @@ __device__ __forceinline__ void epi_four(const EpiView &e, const int (&a)[4], co
     const int64_t off = row * e.N + col0;
     const int cols = (int)(e.N - col0 < 4 ? e.N - col0 : 4);
     if (e.acc_out) {
-        if (full) *reinterpret_cast<int4 *>(e.acc_out + off) = make_int4(a[0], a[1], a[2], a[3]);
-        else for (int i = 0; i < cols; ++i) e.acc_out[off + i] = a[i];
+        if (full) {
+            *reinterpret_cast<int4 *>(e.acc_out + off) = make_int4(a[0], a[1], a[2], a[3]);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (i < cols) e.acc_out[off + i] = a[i];
+        }
     }
     if (!e.need_f) return;
     float y[4];
@@ -78,15 +83,25 @@ __device__ __forceinline__ void epi_four(const EpiView &e, const int (&a)[4], co
         if (e.relu_op) y[i] = fmaxf(y[i], 0.0f);            // NaN -> 0, like (y > 0 ? y : 0)
     }
     if (e.f32_out) {
-        if (full) *reinterpret_cast<float4 *>(e.f32_out + off) = make_float4(y[0], y[1], y[2], y[3]);
-        else for (int i = 0; i < cols; ++i) e.f32_out[off + i] = y[i];
+        if (full) {
+            *reinterpret_cast<float4 *>(e.f32_out + off) = make_float4(y[0], y[1], y[2], y[3]);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (i < cols) e.f32_out[off + i] = y[i];
+        }
     }
     if (e.u8_out) {
         uint32_t w = requant_pack4(__fmul_rn(y[0], e.inv_out_scale), __fmul_rn(y[1], e.inv_out_scale),
                                    __fmul_rn(y[2], e.inv_out_scale), __fmul_rn(y[3], e.inv_out_scale));
         if (e.next_mode != SPARQ_MODE_NONE) w = next_xform_word(w, e.next_mode, e.next_rnd, e.next_xf);
-        if (full) *reinterpret_cast<uint32_t *>(e.u8_out + off) = w;
-        else for (int i = 0; i < cols; ++i) e.u8_out[off + i] = (uint8_t)(w >> (8 * i));
+        if (full) {
+            *reinterpret_cast<uint32_t *>(e.u8_out + off) = w;
+        } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (i < cols) e.u8_out[off + i] = (uint8_t)(w >> (8 * i));
+        }
     }
 }
 
@@ -229,7 +244,11 @@ sparq_gemm_small_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
         const int wt = threadIdx.x - 64;                  // 0 .. 255
         // scale and bias on their way while the operands are
         float c_scale[4], c_bias[4];                      // SHARED: of this thread's four columns
-        const int cg = wt & 15, fcol = n0 + cg * 4;
+        // Column groups of four that exist in this tile, and so rows that the workers write at a time: 512 x 10,
+        // K 144, took 6.2 us where only the first three of sixteen threads on a row had columns, 3.2 so.
+        const int groups = g.N - n0 < BN ? (int)(g.N - n0 + 3) / 4 : BN / 4;
+        const int first_row = wt / groups, row_step = kSmallWorkers * 32 / groups;
+        const int cg = wt - first_row * groups, fcol = n0 + cg * 4;
         const bool fvec = (g.N & 3) == 0 && (reinterpret_cast<uintptr_t>(g.residual) & 3u) == 0;
         if (ev.need_f) {
             if (SHARED) {
@@ -304,7 +323,7 @@ sparq_gemm_small_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
                 for (int q = 0; q < 4 && fcol + q < g.N; ++q) r |= (uint32_t)__ldg(src + q) << (8 * q);
                 return r;
             };
-            uint32_t r = residual_of(wt >> 4);
+            uint32_t r = residual_of(first_row);
             const uint32_t gbytes = (uint32_t)split_group_bytes(own_rows), rbytes = (uint32_t)split_rank_bytes(own_rows);
             wait_acc();
             uint32_t v[32];
@@ -333,8 +352,8 @@ sparq_gemm_small_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
                 }
                 mbar_wait(smem_u32(&bar_recv), 0, abort_flag, g.status, g.wait_limit);
             }
-            if (fcol < g.N) {
-                for (int lrow = wt >> 4; lrow < own_valid; lrow += 16) {
+            if (first_row < row_step) {        // the last threads have no place in a step
+                for (int lrow = first_row; lrow < own_valid; lrow += row_step) {
                     const uint32_t src = recv + (uint32_t)cg * gbytes + (uint32_t)lrow * 16u;
                     int p[kMaxSplit][4];
 #pragma unroll
@@ -344,7 +363,7 @@ sparq_gemm_small_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
                             asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(p[q][0]), "=r"(p[q][1]), "=r"(p[q][2]), "=r"(p[q][3])
                                          : "r"(src + (uint32_t)q * rbytes));
                     }
-                    const uint32_t r_next = residual_of(lrow + 16);
+                    const uint32_t r_next = residual_of(lrow + row_step);
                     int a[4];
 #pragma unroll
                     for (int k = 0; k < 4; ++k)

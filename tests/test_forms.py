@@ -93,3 +93,25 @@ def test_results_of_a_form(want, n, hw, c, cout, r, stride, p, kind):
     got = out.cpu().numpy()
     assert np.array_equal(got[:acc.size].reshape(acc.shape), want_out)
     assert (got[acc.size:] == fill).all()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n", [1, 3, 4, 7, 12, 20, 28, 36, 52, 60, 65, 76])
+@pytest.mark.parametrize("m,k", [(130, 48), (300, 1600)])
+def test_few_tiles_narrow_columns(n, m, k):
+    """Column counts whose groups of four do not divide the workers; one CTA a tile, and several."""
+    A, B = synth.activations(n, (m, k), 0.5), synth.weights(n, (k, n))
+    scale, bias, inv = synth.scales(n, n), synth.bias(n, n), synth.inv_out_scale(k)
+    res = synth.activations(n + 1, (m, n), 0.5)
+    acc = oracle.gemm(A, B, V5.mode, 4, 0x1F, 1)
+    f32, u8 = oracle.epilogue(acc, scale, bias, True, inv, residual=res, residual_scale=0.02)
+    d = lambda t: torch.from_numpy(t).cuda()  # noqa: E731
+    out = {q: torch.full((m * n + 64,), 3, dtype=t, device="cuda") for q, t in
+           (("acc_out", torch.int32), ("f32_out", torch.float32), ("u8_out", torch.uint8))}
+    sparq.sparq_gemm_s8(d(A), d(np.ascontiguousarray(B.T)), V5, scale=d(scale), bias=d(bias), relu=True, inv_out_scale=inv,
+                        residual=d(res), residual_scale=0.02, **out)
+    sparq.sparq_check()
+    for name, want in (("acc_out", acc), ("f32_out", f32), ("u8_out", u8)):
+        got = out[name].cpu().numpy()
+        assert np.array_equal(got[:m * n].reshape(m, n), want), name
+        assert (got[m * n:] == 3).all()
