@@ -217,7 +217,8 @@ static int pick_bn(int64_t M, int64_t N, int64_t steps, int sms, bool transform,
 // The small form (sparq_gemm_small_kernel): launches whose 64-wide tiles all run at once.  tile_rows = 0
 // where they do not.  Tiles of 64 or 128 rows, and 1 to 8 CTAs of a cluster on a tile, by the time
 // of the serial walk along K: a step takes such a launch about 0.25 us, and 0.35 us more for the
-// transform of 128 rows; sharing a tile costs about 1.6 us.  Measured (us, one image, 128-row
+// transform of 128 rows; sharing a tile costs about 1.6 us, and writing 128 rows out 0.4 (173 x 128 x 256,
+// fp32, without a transform: 4.3 us with 128 rows, 3.8 with 64).  Measured (us, one image, 128-row
 // tiles, 1 / 2 / 4 / 8 CTAs on each): 7x7x2048 -> 512 9.4 / 9.1 / 6.1 / 4.8, 14x14x1024 -> 256 6.9 /
 // 8.7 / 6.3 / 5.0, 28x28x512 -> 128 5.6 / 7.1 / 5.6, 7x7x512 -> 2048 4.7 / 6.3 / 5.1; chosen by this
 // rule, against the full kernel before: 7x7x512 -> 512 3x3 30.1 -> 6.7, 14x14x256 -> 256 3x3 14.9 ->
@@ -235,7 +236,7 @@ static SmallForm pick_small(int64_t M, int64_t N, int64_t k_blocks, int sms, boo
         const int64_t tiles = (M + rows - 1) / rows * n_tiles;
         const double step = 0.25 + (transform ? 0.35 * (double)(M < rows ? M : rows) / kBM : 0.0);
         for (int split = 1; split <= kMaxSplit && tiles * split <= sms && k_blocks >= split; split *= 2) {
-            const double cost = (double)((k_blocks + split - 1) / split) * step + (split > 1 ? 1.6 : 0.0) + (split == 2 ? 0.4 : 0.0);
+            const double cost = 0.4 * rows / kBM + (double)((k_blocks + split - 1) / split) * step + (split > 1 ? 1.6 : 0.0) + (split == 2 ? 0.4 : 0.0);
             if (!best.tile_rows || cost < best_cost - 0.05) { best = {rows, split}; best_cost = cost; }
         }
     }
