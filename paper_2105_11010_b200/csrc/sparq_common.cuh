@@ -32,8 +32,9 @@ int validate_params(const sparq_params *p, XformArgs *x);
 // Bit 0: a bounded wait expired.  Allocated on first use, freed by sparq_shutdown().
 int get_status_word(unsigned int **dptr);
 
-// The standalone transform (sparq_quantize) with validated parameters.
-int quantize_rows(const uint8_t *in, uint8_t *out, size_t rows, size_t row_len, const XformArgs &a, cudaStream_t st);
+// The standalone transform (sparq_quantize) with validated parameters.  feeds: the next launch is the
+// contraction that reads `out`.
+int quantize_rows(const uint8_t *in, uint8_t *out, size_t rows, size_t row_len, const XformArgs &a, bool feeds, cudaStream_t st);
 
 // Stream-ordered scratch memory (sparq_workspace.cu): valid for work enqueued on `st` after the call
 // and before the matching workspace_free.  Any thread, any stream.  nullptr when there is none to be

@@ -83,7 +83,6 @@ absmax_kernel(const void *__restrict__ x, size_t n, float *max_inout, size_t kee
 {
     __shared__ uint32_t s_red[kThreads / 32];
     dep_wait();
-    dep_launch();
     constexpr int kPer = BF16 ? 8 : 4;
     const size_t nvec = n / kPer;
     const uint4 *xv = reinterpret_cast<const uint4 *>(x);
@@ -91,12 +90,16 @@ absmax_kernel(const void *__restrict__ x, size_t n, float *max_inout, size_t kee
     const size_t tile = (size_t)kThreads * kVec;
     for (size_t base = (size_t)blockIdx.x * tile; base < nvec; base += (size_t)gridDim.x * tile) {
         uint4 v[kVec];
-        const bool keep = base >= keep_from;
+        auto fetch = [&](auto load) {
 #pragma unroll
-        for (int j = 0; j < kVec; ++j) {
-            const size_t i = base + (size_t)j * kThreads + threadIdx.x;
-            v[j] = i >= nvec ? make_uint4(0u, 0u, 0u, 0u) : keep ? ld16(xv + i) : ld_stream16(xv + i);
-        }
+            for (int j = 0; j < kVec; ++j) {
+                const size_t i = base + (size_t)j * kThreads + threadIdx.x;
+                v[j] = i < nvec ? load(xv + i) : make_uint4(0u, 0u, 0u, 0u);
+            }
+        };
+        // decided once for all loads, which then go out together
+        if (base >= keep_from) fetch([](const uint4 *p) { return ld16(p); });
+        else fetch([](const uint4 *p) { return ld_stream16(p); });
 #pragma unroll
         for (int j = 0; j < kVec; ++j) m = vec_absmax<BF16>(v[j], m);
     }
@@ -104,6 +107,7 @@ absmax_kernel(const void *__restrict__ x, size_t n, float *max_inout, size_t kee
         for (size_t i = nvec * kPer + threadIdx.x; i < n; i += kThreads) m = fmaxf(m, fabsf(elem<BF16>(x, i)));
     const uint32_t b = block_max_bits(m, s_red);
     if (threadIdx.x == 0 && b) atomicMax(reinterpret_cast<unsigned int *>(max_inout), b);
+    dep_launch();
 }
 
 // clamp(rint(z), 0, 255) as the low byte of a float: clamping first commutes with the
@@ -126,7 +130,6 @@ quantize_act_kernel(const void *__restrict__ x, size_t n, const float *__restric
 {
     constexpr int kPer = BF16 ? 8 : 4;
     dep_wait();
-    dep_launch();
     const float mx = *max_dev;
     const float inv = mx > 0.0f ? __fdiv_rn(255.0f, mx) : 0.0f;
     const size_t nvec = n / kPer;
@@ -161,6 +164,7 @@ quantize_act_kernel(const void *__restrict__ x, size_t n, const float *__restric
     if (blockIdx.x == 0)
         for (size_t i = nvec * kPer + threadIdx.x; i < n; i += kThreads)
             out[i] = (uint8_t)quant_u8_bits(elem<BF16>(x, i), inv);
+    dep_launch();
 }
 
 __device__ __forceinline__ int quant_s8(float w, float inv)

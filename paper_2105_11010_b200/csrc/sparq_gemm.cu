@@ -346,7 +346,7 @@ static int gemm_impl(const uint8_t *A, int64_t lda, const int8_t *B, int64_t ldb
     if (x.mode != SPARQ_MODE_NONE && lda == K && (rc = device_info(&sms)) == SPARQ_OK &&
         transform_first(M, N, (K + 127) / 128, (size_t)M * (size_t)K, sms, false)) {
         if (uint8_t *ta = (uint8_t *)workspace_alloc((size_t)M * (size_t)K, st)) {
-            rc = quantize_rows(A, ta, (size_t)M, (size_t)K, x, st);
+            rc = quantize_rows(A, ta, (size_t)M, (size_t)K, x, true, st);
             if (rc == SPARQ_OK) rc = gemm_with_status(ta, K, B, ldb, M, N, K, plain_a8w8(), e, status, st);
             workspace_free(ta, st);
             return rc;
@@ -835,7 +835,7 @@ extern "C" int sparq_conv2d_nhwc_s8(const uint8_t *x_in, int n, int h, int w, in
     const size_t act_bytes = (size_t)n * h * w * (size_t)c;
     if (x.mode != SPARQ_MODE_NONE && transform_first(M, cout, steps, act_bytes, sms, true)) {
         if (uint8_t *tx = (uint8_t *)workspace_alloc(act_bytes, st)) {
-            rc = quantize_rows(x_in, tx, (size_t)n * h * w, (size_t)c, x, st);
+            rc = quantize_rows(x_in, tx, (size_t)n * h * w, (size_t)c, x, true, st);
             if (rc == SPARQ_OK) rc = im2col_conv(tx, n, h, w, c, wgt, cout, r, s, stride_h, stride_w, pad_h, pad_w, ho, wo, plain_a8w8(), e, sms, status, st);
             workspace_free(tx, st);
             return rc;

@@ -35,15 +35,18 @@ __device__ __forceinline__ void st_stream(uint4 *p, uint4 v)
                  :: "l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 
+// release_first: the next launch starts while this one works, for a contraction that reads the result (one
+// CTA per SM, set up meanwhile).  Else it starts at the end: blocks of a streaming successor that take
+// the free places of the SMs early are spread over them unevenly (10 MB: 4.5 -> 5.4 us).
 // XN: the form of the transform, as in xform_fused.  The 3- and 2-bit full sets take the half-precision
 // one: with the packed-integer form at their compile-time width the kernel was bound by the integer
 // pipe (2^28 activations, vSPARQ: 6opt 105 -> 82 us, 7opt 119 -> 82 us, the measured copy rate).
 template <int MODE, int XN, bool RND>
 __global__ void __launch_bounds__(kThreads)
-quantize_vec_kernel(const uint4 *in, uint4 *out, size_t nvec, XformDev d)
+quantize_vec_kernel(const uint4 *in, uint4 *out, size_t nvec, XformDev d, int release_first)
 {
     dep_wait();
-    dep_launch();
+    if (release_first) dep_launch();
     const size_t tile = (size_t)kThreads * kVec;
     for (size_t base = (size_t)blockIdx.x * tile; base < nvec; base += (size_t)gridDim.x * tile) {
         uint4 v[kVec];
@@ -65,6 +68,7 @@ quantize_vec_kernel(const uint4 *in, uint4 *out, size_t nvec, XformDev d)
             }
         }
     }
+    if (!release_first) dep_launch();
 }
 
 // vSPARQ on rows of odd length (>= 16, so that a vector meets at most one row boundary).  Column parity is
@@ -74,12 +78,13 @@ quantize_vec_kernel(const uint4 *in, uint4 *out, size_t nvec, XformDev d)
 // beside a vector are read for its outer partners (in place too: the transform keeps zero zero and
 // everything else non-zero).
 constexpr int kOddVec = 2;
+// Below, a pair per thread spreads over more SMs (16 KB: 1.85 us against 2.45; 100 KB 2.0 against 2.1).
+constexpr size_t kOddVecMin = 128 << 10;
 template <int XN, bool RND>
 __global__ void __launch_bounds__(kThreads)
 quantize_odd_rows_kernel(const uint8_t *in, uint8_t *out, size_t bytes, size_t row_len, unsigned long long magic, XformDev d)
 {
     dep_wait();
-    dep_launch();
     const size_t nvec = (bytes + 15) / 16, tile = (size_t)kThreads * kOddVec;
     for (size_t base = (size_t)blockIdx.x * tile; base < nvec; base += (size_t)gridDim.x * tile) {
         uint4 v[kOddVec];
@@ -139,6 +144,7 @@ quantize_odd_rows_kernel(const uint8_t *in, uint8_t *out, size_t bytes, size_t r
             }
         }
     }
+    dep_launch();
 }
 
 // ---- scalar definitions (generic path) -----------------------------------------------
@@ -163,7 +169,6 @@ __global__ void quantize_pair_kernel(const uint8_t *in, uint8_t *out,
                                      size_t rows, size_t row_len, XformArgs a)
 {
     dep_wait();
-    dep_launch();
     const size_t pairs_per_row = (row_len + 1) / 2;
     const size_t total = rows * pairs_per_row;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
@@ -188,6 +193,7 @@ __global__ void quantize_pair_kernel(const uint8_t *in, uint8_t *out,
         out[k0] = (uint8_t)q0;
         if (has_b) out[k0 + 1] = (uint8_t)q1;
     }
+    dep_launch();
 }
 
 // Launches `kernel<XN, RND>` (given as a generic lambda over integral constants) for the parameters.
@@ -203,12 +209,12 @@ static cudaError_t by_variant(const XformArgs &a, F go)
 }
 
 template <int MODE>
-static cudaError_t launch_vec(const uint4 *in, uint4 *out, size_t nvec, const XformArgs &a, int blocks, cudaStream_t st)
+static cudaError_t launch_vec(const uint4 *in, uint4 *out, size_t nvec, const XformArgs &a, int blocks, bool feeds, cudaStream_t st)
 {
     XformDev d{a.widen_c, a.widen_rounds, a.n};
     fill_fullset(&d, a.n, a.rnd);
     return by_variant(a, [&](auto xn, auto rnd) {
-        return launch_overlapped(quantize_vec_kernel<MODE, decltype(xn)::value, decltype(rnd)::value>, blocks, kThreads, 0, st, in, out, nvec, d);
+        return launch_overlapped(quantize_vec_kernel<MODE, decltype(xn)::value, decltype(rnd)::value>, blocks, kThreads, 0, st, in, out, nvec, d, (int)feeds);
     });
 }
 
@@ -222,7 +228,7 @@ static cudaError_t launch_odd_rows(const uint8_t *in, uint8_t *out, size_t bytes
     });
 }
 
-int quantize_rows(const uint8_t *in, uint8_t *out, size_t rows, size_t row_len, const XformArgs &a, cudaStream_t st)
+int quantize_rows(const uint8_t *in, uint8_t *out, size_t rows, size_t row_len, const XformArgs &a, bool feeds, cudaStream_t st)
 {
     if (rows == 0 || row_len == 0) return SPARQ_OK;
     if (!in || !out) return set_error(SPARQ_ERR_INVALID_ARG, "in/out pointer is NULL");
@@ -249,14 +255,14 @@ int quantize_rows(const uint8_t *in, uint8_t *out, size_t rows, size_t row_len, 
         int blocks = (int)(want < cap ? want : cap);
         const uint4 *vi = (const uint4 *)in;
         uint4 *vo = (uint4 *)out;
-        if (a.mode == SPARQ_MODE_NONE) e = launch_vec<SPARQ_MODE_NONE>(vi, vo, nvec, a, blocks, st);
-        else if (a.mode == SPARQ_MODE_BSPARQ) e = launch_vec<SPARQ_MODE_BSPARQ>(vi, vo, nvec, a, blocks, st);
-        else e = launch_vec<SPARQ_MODE_VSPARQ>(vi, vo, nvec, a, blocks, st);
+        if (a.mode == SPARQ_MODE_NONE) e = launch_vec<SPARQ_MODE_NONE>(vi, vo, nvec, a, blocks, feeds, st);
+        else if (a.mode == SPARQ_MODE_BSPARQ) e = launch_vec<SPARQ_MODE_BSPARQ>(vi, vo, nvec, a, blocks, feeds, st);
+        else e = launch_vec<SPARQ_MODE_VSPARQ>(vi, vo, nvec, a, blocks, feeds, st);
         if (e != cudaSuccess) return cuda_error(e, "quantize_vec_kernel launch");
         done = nvec * 16;
         if (done == total) return SPARQ_OK;
     }
-    if (!pairs_flat && aligned && row_len >= 16) {
+    if (!pairs_flat && aligned && row_len >= 16 && total > kOddVecMin) {
         const size_t tile = (size_t)kThreads * kOddVec, want = ((total + 15) / 16 + tile - 1) / tile, cap = (size_t)sms * 64;
         e = launch_odd_rows(in, out, total, row_len, a, (int)(want < cap ? want : cap), st);
         if (e != cudaSuccess) return cuda_error(e, "quantize_odd_rows_kernel launch");
@@ -285,5 +291,5 @@ extern "C" int sparq_quantize(const uint8_t *in, uint8_t *out, size_t rows, size
 {
     XformArgs a;
     const int rc = validate_params(p, &a);
-    return rc != SPARQ_OK ? rc : quantize_rows(in, out, rows, row_len, a, (cudaStream_t)stream);
+    return rc != SPARQ_OK ? rc : quantize_rows(in, out, rows, row_len, a, false, (cudaStream_t)stream);
 }
