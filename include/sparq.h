@@ -158,7 +158,8 @@ SPARQ_API int sparq_gemm_s8(const uint8_t *A, int64_t lda, const int8_t *B, int6
  * Requirements (else SPARQ_ERR_UNSUPPORTED): x and wgt 16-byte aligned, c a multiple of
  * 16 (a count that is not a multiple of 64 is read in 64-channel blocks whose tail is zero
  * fill: correct, at the speed of the next multiple of 64), r, s in 1..7, strides in 1..8,
- * pads < filter size, r*s*c <= 65536. */
+ * pads < filter size, r*s*c <= 65536; at most 2^31 output pixels for a 1x1 filter with unit
+ * strides, below 2^32 else. */
 SPARQ_API int sparq_conv2d_nhwc_s8(const uint8_t *x, int n, int h, int w, int c,
                          const int8_t *wgt, int cout, int r, int s,
                          int stride_h, int stride_w, int pad_h, int pad_w,

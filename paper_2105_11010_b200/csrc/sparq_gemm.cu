@@ -814,12 +814,14 @@ extern "C" int sparq_conv2d_nhwc_s8(const uint8_t *x_in, int n, int h, int w, in
     const int64_t M = (int64_t)n * ho * wo;
     const int64_t K = (int64_t)r * s * c;
     if (K > 65536) return set_error(SPARQ_ERR_UNSUPPORTED, "r*s*c = %lld exceeds 65536", (long long)K);
+    // Beyond, the kernels' 32-bit coordinates (of a matrix row, of an output pixel) would wrap.
+    const bool matrix = r == 1 && s == 1 && stride_h == 1 && stride_w == 1 && pad_h == 0 && pad_w == 0;
+    if (M > (matrix ? (int64_t)1 << 31 : (int64_t)0xFFFFFFFF)) return set_error(SPARQ_ERR_UNSUPPORTED, "%lld output pixels are too many for one call", (long long)M);
     if ((rc = check_next_transform(e, cout)) != SPARQ_OK) return rc;
     cudaStream_t st = (cudaStream_t)stream;
 
     // A 1x1 filter with unit stride reads the NHWC tensor as the M x c matrix it already is.
-    if (r == 1 && s == 1 && stride_h == 1 && stride_w == 1 && pad_h == 0 && pad_w == 0)
-        return gemm_impl(x_in, c, wgt, c, M, cout, c, x, e, st);
+    if (matrix) return gemm_impl(x_in, c, wgt, c, M, cout, c, x, e, st);
 
     int sms = 0;
     rc = device_info(&sms);

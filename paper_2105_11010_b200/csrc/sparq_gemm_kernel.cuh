@@ -1053,7 +1053,7 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                     const int x = (int)nt * BN + cbase + c;
                     const int64_t y = (int64_t)mt32 * kBM + quarter * 32;
                     if (lane == 0) {
-                        if (x < (int)g.N && y < g.M) tma_store_2d(&map_out, buf, x, (int)y);
+                        if ((int64_t)x < g.N && y < g.M) tma_store_2d(&map_out, buf, x, (int)y);
                         tma_store_commit();
                     }
                 }

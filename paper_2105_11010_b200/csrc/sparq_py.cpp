@@ -233,7 +233,10 @@ PyObject *quantize_call(PyObject *const *args, Py_ssize_t nargs, bool host)
         Args a(args, nargs, 6);
         const Tensor &in = a.tensor("inp"), &out = a.tensor("out");
         const int64_t rows = a.integer(), len = a.integer();
-        if (in.numel() < rows * len || out.numel() < rows * len) fail("%s smaller than rows * row_len", "tensor");
+        int64_t count = 0;
+        if (rows < 0 || len < 0) fail("%s must not be negative", "rows and row_len");
+        if (__builtin_mul_overflow(rows, len, &count) || in.numel() < count || out.numel() < count)
+            fail("%s smaller than rows * row_len", "tensor");
         const sparq_params p = params_of(a.next());
         const uint8_t *src = data<uint8_t>(&in, at::kByte, "inp", host);
         uint8_t *dst = data<uint8_t>(&out, at::kByte, "out", host);
