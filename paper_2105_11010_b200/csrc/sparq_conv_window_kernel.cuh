@@ -49,7 +49,6 @@ struct WindowArgs {
     int win_bufs;           // window buffers in the ring
     int b_stages;           // weight stages (stream mode) or resident blocks (resident mode)
     int team_copy;          // 256-wide tiles: room behind the weight stages for the second epilogue team's scale and bias
-    int issuers;            // 2: the two issuer warps alternate (resident weights); 1: warp 1 issues every tile (streamed weights)
     uint32_t n_tiles;       // column tiles
     uint32_t units;         // n_img * tiles_per_img * n_tiles, column tile fastest
     uint32_t groups;        // streamed weights on 128-wide tiles: n_img * n_tiles * ceil(tiles_per_img / G) whole
@@ -170,6 +169,11 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
     // weights (kBatched), so a group holds up to two stages and four let the next group start
     // while the previous one is in its epilogue.
     constexpr bool kBatched = !B_RESIDENT && BN == 128;
+    // Streamed weights pass through a ring that is shorter than one tile's blocks, in tile order:
+    // two issuers on different tiles would wait on the same stage barriers several phases apart,
+    // which a parity wait cannot tell apart.  One issuer then; two take the tiles alternately with
+    // resident weights.
+    constexpr uint32_t kIssuers = B_RESIDENT ? 2 : 1;
     // 128-wide tiles without a transform keep one team of sixteen warps and, with resident weights, two
     // stages: nothing slows the issuers down there, so with four stages they finish tiles in pairs
     // and the epilogues run after them in a burst (128x28x28x128 -> 128 3x3: 16.5 -> 15.2 us).
@@ -419,7 +423,7 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
                     wt += (uint32_t)cnt;
                 } else
                 for (int j = 0; j < (int)walk.cnt; ++j, ++wt) {
-                    if (g.issuers == 2 ? (wt & 1u) != me : me != 0u) {
+                    if (kIssuers == 2 ? (wt & 1u) != me : me != 0u) {
                         if (!B_RESIDENT) {
                             // the other issuer consumes this tile's weight stages
                             s += kb_count;
@@ -443,7 +447,7 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
                     }
                     tc_fence_after();
                     pre_acc = pre_ops = 0;
-                    const uint32_t step = (uint32_t)g.issuers;          // this issuer's next tile is number wt + step
+                    constexpr uint32_t step = kIssuers;                 // this issuer's next tile is number wt + step
                     const bool look_ahead = j + (int)step < (int)walk.cnt;
                     auto look = [&]() {
                         if (!look_ahead) return;

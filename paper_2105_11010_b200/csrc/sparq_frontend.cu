@@ -175,7 +175,7 @@ __device__ __forceinline__ int quant_s8(float w, float inv)
 
 // One block per kernel (output channel): its largest magnitude, then its int8 row.  VEC: rows are whole
 // 16-byte vectors, and the first kWeightVecs per thread stay in registers between the two steps, which
-// is the whole row up to 4608 values (512 filters of 3x3); what lies beyond is read again.
+// is the whole row up to 5120 values (512 channels of 3x3 take 4608); what lies beyond is read again.
 constexpr int kWeightVecs = 5;
 template <bool VEC>
 __global__ void __launch_bounds__(kThreads)

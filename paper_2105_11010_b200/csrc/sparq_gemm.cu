@@ -600,10 +600,6 @@ static int try_window_conv(const uint8_t *x_in, int n, int h, int w, int c, cons
 
     WindowArgs g;
     memset(&g, 0, sizeof(g));
-    // Streamed weights pass through a ring that is shorter than one tile's blocks, in tile order:
-    // two issuers on different tiles would wait on the same stage barriers several phases apart,
-    // which a parity wait cannot tell apart.  One issuer then; two with resident weights.
-    g.issuers = q.resident ? 2 : 1;
     g.N = cout; g.K = K;
     g.n_img = n; g.H = h; g.W = w; g.C = c; g.R = r; g.S = s; g.pad_h = pad_h; g.pad_w = pad_w; g.Ho = ho; g.Wo = wo;
     g.Wp = wp; g.TR = tr; g.tiles_per_img = q.tiles_per_img; g.c_blocks = q.c_blocks;

@@ -8,8 +8,8 @@
 //   warp 1        allocates tensor memory; one lane issues tcgen05.mma kind::i8
 //                 (u8 x s8 -> s32) on each transformed stage
 //   warps 2..9    epilogue: tcgen05.ld of a finished accumulator, fp32 scale / bias /
-//                 ReLU / requantize, global stores (warp w reads lane quarter w % 4 and
-//                 one half of the tile's columns)
+//                 ReLU / requantize, global stores (warp w reads lane quarter w % 4 of its team's
+//                 tiles, and its share of their columns)
 //   warps 10..17  transform: rewrite the A stage in place with bSPARQ / vSPARQ
 //
 // A stage travels  TMA (async proxy) -> transform warps (generic proxy) -> MMA (async
@@ -221,23 +221,8 @@ __device__ __forceinline__ void fence_proxy_async_smem()
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-__device__ __forceinline__ void tc_commit(uint32_t bar)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(bar) : "memory");
-}
-
-// D[tmem] (+)= A[smem] * B[smem], 128 x N x 32, u8 x s8 -> s32.
-__device__ __forceinline__ void tc_mma_i8(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                          uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
-        :: "r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
-}
-
-// The same two instructions for a warp that runs its loop converged: every lane executes
+// D[tmem] (+)= A[smem] * B[smem], 128 x N x 32, u8 x s8 -> s32, and the commit that signals a barrier once the
+// MMAs before it have retired, for a warp that runs its loop converged: every lane executes
 // the surrounding code (so that descriptor arithmetic on warp-uniform values can stay in
 // the uniform datapath) and only the lane with `elected` != 0 issues.
 __device__ __forceinline__ void tc_mma_i8_if(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,

@@ -176,14 +176,11 @@ __host__ __device__ constexpr int stage_bytes() { return (kChunkUnits * PER + 4 
 template <int N>
 __host__ __device__ constexpr int data_stage_bytes() { return N == 3 ? stage_bytes<6>() : 0; }
 
-// Resident blocks per SM: the table and the staging areas of three fit in shared memory, of two
-// with the data plane staged too.
-template <int N>
-__host__ __device__ constexpr int pack_blocks() { return 2; }
-constexpr int kUnpackBlocks = 2;
+// Resident blocks per SM of both kernels: what 64 registers a thread allow.
+constexpr int kCodecBlocks = 2;
 
 template <int MODE, int N, int CB>
-__global__ void __launch_bounds__(kThreads, pack_blocks<N>())
+__global__ void __launch_bounds__(kThreads, kCodecBlocks)
 pack_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ data, uint8_t *__restrict__ ctrl,
             size_t units, const __grid_constant__ EncTable tab)
 {
@@ -300,7 +297,7 @@ __device__ __forceinline__ uint32_t digits_of(uint32_t dlo, uint32_t dhi)
 }
 
 template <int N, int CB>
-__global__ void __launch_bounds__(kThreads, kUnpackBlocks)
+__global__ void __launch_bounds__(kThreads, kCodecBlocks)
 unpack_kernel(const uint8_t *__restrict__ data, const uint8_t *__restrict__ ctrl, uint8_t *__restrict__ out,
               size_t units, const __grid_constant__ DecTable tab)
 {
@@ -491,14 +488,14 @@ int launch_codec(Kernel kernel, const char *what, int stage_per_warp, int blocks
 template <int MODE, int N, int CB>
 int launch_pack(const uint8_t *in, uint8_t *data, uint8_t *ctrl, size_t units, const XformArgs &x, cudaStream_t st)
 {
-    return launch_codec<kEncWords>(pack_kernel<MODE, N, CB>, "pack_kernel launch", stage_bytes<CB>() + data_stage_bytes<N>(), pack_blocks<N>(), units, st,
+    return launch_codec<kEncWords>(pack_kernel<MODE, N, CB>, "pack_kernel launch", stage_bytes<CB>() + data_stage_bytes<N>(), kCodecBlocks, units, st,
                                    in, data, ctrl, units, encoder_table(x));
 }
 
 template <int N, int CB>
 int launch_unpack(const uint8_t *data, const uint8_t *ctrl, uint8_t *out, size_t units, const XformArgs &x, cudaStream_t st)
 {
-    return launch_codec<kDecWords>(unpack_kernel<N, CB>, "unpack_kernel launch", stage_bytes<CB>() + data_stage_bytes<N>(), kUnpackBlocks, units, st,
+    return launch_codec<kDecWords>(unpack_kernel<N, CB>, "unpack_kernel launch", stage_bytes<CB>() + data_stage_bytes<N>(), kCodecBlocks, units, st,
                                    data, ctrl, out, units, decoder_table(x));
 }
 
