@@ -112,9 +112,10 @@ struct XformDev {
     int n;
     // Full placement sets only (every shift 0..8-n allowed; see xform_word_fullset): per 16-bit
     // half, twice in a word -- the rounding increment, the mask of the kept bits and the
-    // saturation value of the n-bit window (f_*) and of the 2n-bit window of a lone non-zero (l_*).
-    uint32_t f_add, f_mask, f_sat;
-    uint32_t l_add, l_mask, l_sat;
+    // largest sum that still trims to the top window, of the n-bit window (f_*) and of the 2n-bit
+    // window of a lone non-zero (l_*).
+    uint32_t f_add, f_mask, f_top;
+    uint32_t l_add, l_mask, l_top;
 };
 
 // binary16 bit pattern of an integer 0 < v < 2048 (exact)
@@ -128,19 +129,19 @@ inline uint32_t half_bits_of_int(uint32_t v)
 // Constants of xform_word_fullset for window width n and the rounding flag.
 inline void fill_fullset(XformDev *d, int n, int rnd)
 {
-    auto set = [&](int w, uint32_t *add, uint32_t *mask, uint32_t *sat) {
+    auto set = [&](int w, uint32_t *add, uint32_t *mask, uint32_t *top) {
         if (w >= 8) {                    // the window holds all 8 bits: nothing is dropped
-            *add = 0u; *mask = 0xFFFFFFFFu; *sat = half_bits_of_int(255u) * 0x00010001u;
+            *add = 0u; *mask = 0xFFFFFFFFu; *top = half_bits_of_int(255u) * 0x00010001u;
             return;
         }
         const uint32_t m16 = (0xFFFFu << (11 - w)) & 0xFFFFu;      // sign, exponent and the top w-1 fraction bits
         const uint32_t a16 = rnd ? (1u << (10 - w)) : 0u;          // half of the lowest kept bit
         *mask = m16 * 0x00010001u;
         *add = a16 * 0x00010001u;
-        *sat = half_bits_of_int(((1u << w) - 1u) << (8 - w)) * 0x00010001u;
+        *top = (half_bits_of_int(((1u << w) - 1u) << (8 - w)) | (~m16 & 0xFFFFu)) * 0x00010001u;
     };
-    set(n, &d->f_add, &d->f_mask, &d->f_sat);
-    set(2 * n, &d->l_add, &d->l_mask, &d->l_sat);
+    set(n, &d->f_add, &d->f_mask, &d->f_top);
+    set(2 * n, &d->l_add, &d->l_mask, &d->l_top);
 }
 
 // Mask of the bits BELOW the window for each of the four bytes of x (Section 3.1: the
@@ -214,16 +215,23 @@ SPARQ_HD uint32_t xform_word(uint32_t x, const XformDev &d)
 // one (Section 3.1) -- which is what a binary floating-point number with n - 1 fraction bits
 // holds.  A byte b is exact in binary16 (11 significant bits); as bit patterns, two bytes per
 // 32-bit register:
-//     0x6400 | b            = 1024 + b          (one byte permute per pair)
-//     (1024 + b) - 1024     = b, normalized: the subtraction finds the leading one
-//     (bits + half) & mask  = b rounded to n significant bits, ties up, a carry moving into the
-//                             exponent (31 -> 32); without the increment: trimmed
-//     min(., top window)    = the saturation at the top of the byte range (248.. -> 240)
-//     . + 1024              = the integer back in the low byte of each half
-// 13 instructions per four activations for any width and either rounding (17 with the pair
-// rule for n = 4, 26 for n < 4 with its second, 2n-bit window), where the packed integer form
-// with a run-time width needs about twice as many; for n = 4 the integer form specialized at
-// compile time (19 with the pair rule) measured a few per cent faster and is kept.
+//     0x6400 | b               = 1024 + b       (one byte permute per pair)
+//     (1024 + b) - 1024        = b, normalized: the subtraction finds the leading one
+//     min(bits + half, top)    the rounding increment, ties up, a carry moving into the exponent
+//                              (31 -> 32); top is the last pattern below 256, so that 248.. stay in
+//                              the top window (one fused add-and-minimum on 16-bit halves)
+//     . & mask                 = b rounded to n significant bits; without the increment: trimmed
+//     . + 1024                 = the integer back in the low byte of each half
+// 11 instructions per four activations for any width, 16 with the pair rule at n = 4 (25 at n < 4,
+// with its second, 2n-bit window).
+//
+// What the transform costs is the integer pipe: a logical operation, shift, permute or minimum takes it
+// two cycles a warp, an integer add one and a half, half-precision arithmetic two of another pipe.
+// The packed-integer form of n = 4 is 19 instructions, 17 of them logical or shifts: 32.2 cycles per
+// word and scheduler with two warps on it; this form 22.9.  56x56x256 -> 64 at batch 64 20.9 -> 17.6
+// us, 14x14x1024 -> 256 10.4 -> 9.5, the ResNet-50 pass 894 -> 841 us, one image 240 -> 229.
+// (Tried: choosing by the partner with multiplications in the half-precision pipe, 26.4 cycles with two
+// warps and 22.5 with four; zero masks per half, 25.0; halves of both kinds, 23.2 and 19.8.)
 __device__ __forceinline__ uint32_t h2_sub(uint32_t a, uint32_t b)
 {
     uint32_t d;
@@ -236,40 +244,48 @@ __device__ __forceinline__ uint32_t h2_add(uint32_t a, uint32_t b)
     asm("add.rn.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
     return d;
 }
-__device__ __forceinline__ uint32_t h2_min(uint32_t a, uint32_t b)
+
+constexpr uint32_t kHalf1024 = 0x64006400u;
+
+// Four bytes as normalized halves: bytes 0, 1 in lo, bytes 2, 3 in hi.
+__device__ __forceinline__ void bytes_to_halves(uint32_t x, uint32_t &lo, uint32_t &hi)
 {
-    uint32_t d;
-    asm("min.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
-    return d;
+    lo = h2_sub(prmt(x, 0x64646464u, 0x4140u), kHalf1024);
+    hi = h2_sub(prmt(x, 0x64646464u, 0x4342u), kHalf1024);
 }
 
-template <int MODE>
+// The window of four activations given as halves, back in bytes.
+template <bool ADD>
+__device__ __forceinline__ uint32_t window_of_halves(uint32_t lo, uint32_t hi, uint32_t add, uint32_t mask, uint32_t top)
+{
+    if (ADD) {
+        lo = __viaddmin_u16x2(lo, add, top);
+        hi = __viaddmin_u16x2(hi, add, top);
+    }
+    return prmt(h2_add(lo & mask, kHalf1024), h2_add(hi & mask, kHalf1024), 0x6420u);
+}
+
+// FIXED4: n = 4 with rounding RND, constants at compile time; otherwise width and rounding as in d.
+template <int MODE, bool FIXED4, bool RND>
 __device__ __forceinline__ uint32_t xform_word_fullset(uint32_t x, const XformDev &d)
 {
     if (MODE == SPARQ_MODE_NONE) return x;
-    const uint32_t k1024 = 0x64006400u;
-    // bytes 0,1 and bytes 2,3 as halves
-    const uint32_t lo = h2_sub(prmt(x, 0x64646464u, 0x4140u), k1024);
-    const uint32_t hi = h2_sub(prmt(x, 0x64646464u, 0x4342u), k1024);
-    const uint32_t qlo = h2_add(h2_min((lo + d.f_add) & d.f_mask, d.f_sat), k1024);
-    const uint32_t qhi = h2_add(h2_min((hi + d.f_add) & d.f_mask, d.f_sat), k1024);
-    const uint32_t q = prmt(qlo, qhi, 0x6420u);
+    uint32_t lo, hi;
+    bytes_to_halves(x, lo, hi);
+    const uint32_t q = FIXED4 ? window_of_halves<RND>(lo, hi, 0x00400040u, 0xFF80FF80u, 0x5BFF5BFFu)
+                              : window_of_halves<true>(lo, hi, d.f_add, d.f_mask, d.f_top);
     if (MODE == SPARQ_MODE_BSPARQ) return q;
     // vSPARQ: a byte whose partner is zero keeps the 2n-bit window (the whole byte for n = 4)
     uint32_t lone = x;
-    if (d.l_mask != 0xFFFFFFFFu) {       // uniform: a kernel argument
-        const uint32_t llo = h2_add(h2_min((lo + d.l_add) & d.l_mask, d.l_sat), k1024);
-        const uint32_t lhi = h2_add(h2_min((hi + d.l_add) & d.l_mask, d.l_sat), k1024);
-        lone = prmt(llo, lhi, 0x6420u);
-    }
+    if (!FIXED4 && d.l_mask != 0xFFFFFFFFu) lone = window_of_halves<true>(lo, hi, d.l_add, d.l_mask, d.l_top);   // uniform: a kernel argument
     const uint32_t nz = ((x & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | x;   // bit 7 of each byte: byte != 0
     const uint32_t partner_nz = prmt(nz, nz, 0xAB89u);           // swap within pairs, replicate bit 7
     return (q & partner_nz) | (lone & ~partner_nz);
 }
 
 // The transform of a fused kernel instantiated for (MODE, XN, RND): XN = 4 is n = 4 with all
-// five placements (packed-integer form, width fixed at compile time), XN = 5 the same with the
-// placement widening (any restricted set of n = 4: 3opt, 2opt), XN = 8 any other full placement set
+// five placements (half precision, constants at compile time), XN = 5 n = 4 with fewer (3opt, 2opt: the
+// packed-integer form with the width fixed and the placement widening), XN = 8 any other full placement set
 // (6opt, 7opt; either rounding, through the constants; RND unused), XN = 0 the general
 // packed-integer form with run-time width and the placement widening (restricted sets of n < 4); XN = 3
 // and 2 are that with the width fixed, in the standalone kernels only, which the integer pipe bounds
@@ -277,8 +293,7 @@ __device__ __forceinline__ uint32_t xform_word_fullset(uint32_t x, const XformDe
 template <int MODE, int XN, bool RND>
 __device__ __forceinline__ uint32_t xform_fused(uint32_t x, const XformDev &d)
 {
-    if (XN == 8) return xform_word_fullset<MODE>(x, d);
-    if (XN == 4) return xform_word<MODE, 4, RND, false>(x, d);
+    if (XN == 8 || XN == 4) return xform_word_fullset<MODE, XN == 4, RND>(x, d);
     if (XN == 5) return xform_word<MODE, 4, RND, true>(x, d);
     if (XN == 3) return xform_word<MODE, 3, RND, true>(x, d);
     if (XN == 2) return xform_word<MODE, 2, RND, true>(x, d);
@@ -294,10 +309,9 @@ __device__ __forceinline__ void window_and_lone(uint32_t x, const XformDev &d, u
     l = x;
     if (XN != 4 && XN != 5) {
         if (XN == 8) {
-            const uint32_t k1024 = 0x64006400u;
-            const uint32_t lo = h2_sub(prmt(x, 0x64646464u, 0x4140u), k1024), hi = h2_sub(prmt(x, 0x64646464u, 0x4342u), k1024);
-            l = prmt(h2_add(h2_min((lo + d.l_add) & d.l_mask, d.l_sat), k1024),
-                     h2_add(h2_min((hi + d.l_add) & d.l_mask, d.l_sat), k1024), 0x6420u);
+            uint32_t lo, hi;
+            bytes_to_halves(x, lo, hi);
+            l = window_of_halves<true>(lo, hi, d.l_add, d.l_mask, d.l_top);
         } else {
             l = apply_mask<RND>(x, drop_mask<0, false>(x, 2 * d.n, 0u), 2 * d.n);
         }

@@ -367,14 +367,14 @@ struct Words8 {
 };
 static __device__ __noinline__ Words8 next_xform_words(Words8 v, int mode, int rnd, XformDev xf)
 {
-    const bool full = xf.rounds == 0 && xf.n != 4;   // 6opt / 7opt: the half-precision form
     auto each = [&](auto f) {
 #pragma unroll
         for (int q = 0; q < 8; ++q) v.w[q] = f(v.w[q]);
     };
     if (mode == SPARQ_MODE_VSPARQ) {
-        if (full) each([&](uint32_t x) { return xform_word_fullset<SPARQ_MODE_VSPARQ>(x, xf); });
-        else if (xf.rounds == 0 && rnd) each([&](uint32_t x) { return xform_word<SPARQ_MODE_VSPARQ, 4, true, false>(x, xf); });
+        // full sets: the half-precision form
+        if (xf.rounds == 0 && xf.n != 4) each([&](uint32_t x) { return xform_word_fullset<SPARQ_MODE_VSPARQ, false, true>(x, xf); });
+        else if (xf.rounds == 0 && rnd) each([&](uint32_t x) { return xform_word_fullset<SPARQ_MODE_VSPARQ, true, true>(x, xf); });
         else each([&](uint32_t x) { return next_xform_word(x, mode, rnd, xf); });
     } else {
         each([&](uint32_t x) { return next_xform_word(x, mode, rnd, xf); });
