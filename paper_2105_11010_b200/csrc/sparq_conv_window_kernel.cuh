@@ -88,7 +88,7 @@ constexpr int kMaxBStages = 12;
 // queue behind the tensor core's own shared-memory traffic, descriptor set-up -- happens
 // while the other one's MMAs keep the tensor core busy.
 constexpr int kMmaBWarp = kFirstXfWarp + kNumXfWarps;      // the second issuer is the last warp
-constexpr int kWindowThreads = kGemmThreads + 32;
+constexpr int kWindowThreads = 32 * (kMmaBWarp + 1);
 
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *map, uint32_t bar, int c, int w, int h, int n)
 {

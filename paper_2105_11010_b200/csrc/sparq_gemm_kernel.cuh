@@ -4,7 +4,8 @@
 //
 // One persistent CTA per SM walks output tiles of 128 x BN.  Warp roles:
 //   warp 0        TMA producer: A tile (tiled 2-D box for the GEMM, im2col box for the
-//                 convolution) and B tile into a ring of shared-memory stages
+//                 convolution) and B tile into a ring of shared-memory stages; without a transform
+//                 warp 18 fetches B
 //   warp 1        allocates tensor memory; one lane issues tcgen05.mma kind::i8
 //                 (u8 x s8 -> s32) on each transformed stage
 //   warps 2..9    epilogue: tcgen05.ld of a finished accumulator, fp32 scale / bias /
@@ -41,7 +42,12 @@ constexpr int kXfTeams = 2;
 constexpr int kXfTeamWarps = kNumXfWarps / kXfTeams;
 constexpr int kFirstEpiWarp = 2;
 constexpr int kFirstXfWarp = kFirstEpiWarp + kNumEpiWarps;
-constexpr int kGemmThreads = 32 * (kFirstXfWarp + kNumXfWarps);
+// Without a transform sparq_gemm_kernel's last warp is a second producer: one thread's chain -- wait,
+// announce, two copies -- was the longest of a step where steps are short (batch 64, 7x7x512 -> 512
+// 3x3 transformed first 16.5 -> 14.4 us, 56x56x128 -> 128 3x3 stride 2 without a transform 12.8 -> 10.9).
+// With a transform a step is longer, and one producer as fast or faster (200704 x 64, K 256, 17.55 us against 17.75).
+constexpr int kWeightWarp = kFirstXfWarp + kNumXfWarps;
+__host__ __device__ constexpr int gemm_threads(int mode) { return 32 * (kWeightWarp + (mode == SPARQ_MODE_NONE ? 1 : 0)); }
 // Epilogue warps of a kernel instantiated for `mode`.
 __host__ __device__ constexpr int epi_warps(int mode) { return mode == SPARQ_MODE_NONE ? kNumEpiWarps + kNumXfWarps : kNumEpiWarps; }
 // Shares that a tile's columns are split into over the groups of one epilogue team.
@@ -304,7 +310,8 @@ struct TapWalk {
     int c, r, s, k, tap_k, bk, S;
     __device__ __forceinline__ TapWalk(const GemmArgs &g, int bk_, int first)
     {
-        tap_k = g.tap_k; bk = bk_; S = g.S;
+        tap_k = g.conv ? g.tap_k : 0x7FFFFFFF;      // a matrix: k only
+        bk = bk_; S = g.S;
         c = r = s = k = 0;
         if (g.conv && first) {
             const int tap = first / g.c_blocks;
@@ -815,11 +822,12 @@ struct TileCfg {
 };
 
 template <int BN, int BK, int MODE, int XN, bool RND, int OUT>
-__global__ void __launch_bounds__(kGemmThreads, 1)
+__global__ void __launch_bounds__(gemm_threads(MODE), 1)
 sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                   const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_res, const GemmArgs g)
 {
     using Cfg = TileCfg<BN, BK>;
+    constexpr bool kTwoProducers = MODE == SPARQ_MODE_NONE;
     const int S = g.stages;
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t bar_full[kMaxStages], bar_xf[kMaxStages], bar_empty[kMaxStages];
@@ -857,7 +865,7 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         prefetch_tensormap(&map_a);
         prefetch_tensormap(&map_b);
         for (int s = 0; s < S; ++s) {
-            mbar_init(smem_u32(&bar_full[s]), 1);
+            mbar_init(smem_u32(&bar_full[s]), kTwoProducers ? 2 : 1);
             mbar_init(smem_u32(&bar_xf[s]), kXfTeamWarps);
             mbar_init(smem_u32(&bar_empty[s]), 1);
         }
@@ -885,12 +893,13 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
 
     const int kb_count = g.k_blocks;
 
-    if (warp == 0) {
-        // ================= TMA producer =================
+    if (warp == 0 || (kTwoProducers && warp == kWeightWarp)) {
+        // ================= TMA producers =================
+        // A thread feeds the whole CTA, a few hundred cycles a step: positions are counters, not divisions,
+        // and the abort flag is read only where a wait has given up (every read of shared memory queues
+        // behind the tensor core's operand fetches).
         if (lane == 0) {
-            // One thread feeds the whole CTA, a few hundred cycles a step: positions are counters, not
-            // divisions, and the abort flag is read only where a wait has given up (every read of
-            // shared memory queues behind the tensor core's operand fetches).
+            constexpr uint32_t kBytes = kTwoProducers ? Cfg::kABytes : Cfg::kStageBytes;     // of the first producer
             uint32_t it = 0;   // running stage counter across tiles
             int s = 0;         // stage it % S
             uint32_t use = 0;  // it / S
@@ -899,31 +908,37 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                 const uint32_t mt = (n_tiles32 == 1) ? tile : tile / n_tiles32, nt = tile - mt * n_tiles32;
                 const int64_t m0 = (int64_t)mt * kBM;
                 const int n0 = (int)(nt * BN);
-                int base_w = 0, base_h = 0, base_n = 0;
-                if (g.conv) {
-                    const uint32_t hw = (uint32_t)(g.Ho * g.Wo), m032 = (uint32_t)m0;   // M of a convolution fits 31 bits
-                    base_n = (int)(m032 / hw);
-                    const int rem = (int)(m032 - (uint32_t)base_n * hw);
-                    base_h = (rem / g.Wo) * g.stride_h - g.pad_h;
-                    base_w = (rem % g.Wo) * g.stride_w - g.pad_w;
-                }
-                TapWalk tap(g, BK, 0);
-                for (int kb = 0; kb < kb_count; ++kb, ++it) {
-                    // stop issuing copies once the CTA has given up
-                    if (use > 0 && !mbar_wait(smem_u32(&bar_empty[s]), (use - 1) & 1, abort_flag, g.status, g.wait_limit)) { live = false; break; }
-                    const uint32_t full = smem_u32(&bar_full[s]);
-                    mbar_expect_tx(full, Cfg::kStageBytes);
-                    if (g.conv) {
-                        // Channels past C arrive as zeros, so whatever the weight block holds
-                        // there (the next tap's first bytes) adds nothing.
-                        tma_load_im2col_4d(a_stage(s), &map_a, full, tap.c, base_w, base_h, base_n, (uint16_t)tap.s, (uint16_t)tap.r);
-                        tma_load_2d(b_stage(s), &map_b, full, tap.k, n0);
+                // the tile's stages in turn, until the CTA has given up
+                auto stages = [&](uint32_t bytes, auto copy) {
+                    TapWalk tap(g, BK, 0);
+                    for (int kb = 0; kb < kb_count; ++kb, ++it) {
+                        if (use > 0 && !mbar_wait(smem_u32(&bar_empty[s]), (use - 1) & 1, abort_flag, g.status, g.wait_limit)) { live = false; break; }
+                        const uint32_t full = smem_u32(&bar_full[s]);
+                        mbar_expect_tx(full, bytes);
+                        copy(full, tap);
                         tap.next();
-                    } else {
-                        tma_load_2d(a_stage(s), &map_a, full, kb * BK, (int)m0);
-                        tma_load_2d(b_stage(s), &map_b, full, kb * BK, n0);
+                        if (++s == S) { s = 0; ++use; }
                     }
-                    if (++s == S) { s = 0; ++use; }
+                };
+                auto weights = [&](uint32_t full, const TapWalk &tap) { tma_load_2d(b_stage(s), &map_b, full, tap.k, n0); };
+                if (kTwoProducers && warp == kWeightWarp) {
+                    stages(Cfg::kBBytes, weights);
+                } else if (g.conv) {
+                    const uint32_t hw = (uint32_t)(g.Ho * g.Wo), m032 = (uint32_t)m0;   // M of a convolution fits 31 bits
+                    const int base_n = (int)(m032 / hw);
+                    const int rem = (int)(m032 - (uint32_t)base_n * hw);
+                    const int base_h = (rem / g.Wo) * g.stride_h - g.pad_h, base_w = (rem % g.Wo) * g.stride_w - g.pad_w;
+                    // Channels past C arrive as zeros, so whatever the weight block holds
+                    // there (the next tap's first bytes) adds nothing.
+                    stages(kBytes, [&](uint32_t full, const TapWalk &tap) {
+                        tma_load_im2col_4d(a_stage(s), &map_a, full, tap.c, base_w, base_h, base_n, (uint16_t)tap.s, (uint16_t)tap.r);
+                        if (!kTwoProducers) weights(full, tap);
+                    });
+                } else {
+                    stages(kBytes, [&](uint32_t full, const TapWalk &tap) {
+                        tma_load_2d(a_stage(s), &map_a, full, tap.k, (int)m0);
+                        if (!kTwoProducers) weights(full, tap);
+                    });
                 }
             }
             // After an abort: wait (bounded) for the copies this thread still has in
@@ -1150,7 +1165,7 @@ cudaError_t launch_gemm_kernel(const GemmMaps &m, GemmArgs &g, int grid, cudaStr
     const int staging = g.out_box ? epi_warps(MODE) * 2 * 32 * g.out_box : 0;
     g.stages = TileCfg<BN, BK>::stages(staging);
     const int smem = 1024 + g.stages * TileCfg<BN, BK>::kStageBytes + staging;
-    return launch_overlapped(kfn, grid, kGemmThreads, smem, st, m.a, m.b, m.out, m.res, g);
+    return launch_overlapped(kfn, grid, gemm_threads(MODE), smem, st, m.a, m.b, m.out, m.res, g);
 }
 
 template <int BN, int BK, int MODE, int XN, bool RND>
