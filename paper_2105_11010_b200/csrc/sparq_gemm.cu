@@ -100,6 +100,38 @@ static int encode_2d(CUtensorMap *map, const void *ptr, int64_t K, int64_t rows,
     return SPARQ_OK;
 }
 
+// The weight matrix [rows][K] in groups of 32 rows (rows a multiple of 32).  Row 8j + 2q + b of a group in
+// shared memory is matrix row 8q + 2j + b as epi_frag wants it (frag), else the same.  Dimensions (K, b, q, j, group).
+static int encode_row_groups(CUtensorMap *map, const void *ptr, int64_t K, int64_t rows, int64_t ld, int bk, int box_rows, bool frag)
+{
+    static EncodeTiledFn fn = nullptr;
+    if (!fn) {
+        int rc = driver_fn("cuTensorMapEncodeTiled", (void **)&fn);
+        if (rc != SPARQ_OK) return rc;
+    }
+    const MapKey key = {{5, (uint64_t)(uintptr_t)ptr, (uint64_t)K, (uint64_t)rows, (uint64_t)ld, (uint64_t)bk, (uint64_t)box_rows, (uint64_t)frag}};
+    if (map_lookup(key, map)) return SPARQ_OK;
+    const cuuint64_t pitch = (cuuint64_t)ld;
+    cuuint64_t dims[5] = {(cuuint64_t)K, 2, 4, 4, (cuuint64_t)rows / 32};
+    cuuint64_t strides[4] = {pitch, (frag ? 8 : 2) * pitch, (frag ? 2 : 8) * pitch, 32 * pitch};
+    cuuint32_t box[5] = {(cuuint32_t)bk, 2, 4, 4, (cuuint32_t)box_rows / 32};
+    cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 5, const_cast<void *>(ptr), dims, strides, box, estr,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_for(bk), CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return set_error(SPARQ_ERR_CUDA, "cuTensorMapEncodeTiled (weights) failed with CUresult %d", (int)r);
+    map_store(key, *map);
+    return SPARQ_OK;
+}
+
+// Weights as the GEMM kernels read them.
+static int encode_b(CUtensorMap *map, const void *ptr, int64_t K, int64_t rows, int64_t ld, int bk, int bn, const GemmArgs &g, bool small)
+{
+    const int out = make_epi_view(g).out;
+    if (small || out == kOutGeneral) return encode_2d(map, ptr, K, rows, ld, bk, bn);
+    return encode_row_groups(map, ptr, K, rows, ld, bk, bn, frag_rows(out, bn, g.out_box));
+}
+
 // NHWC activation tensor read as im2col columns of `rows` output pixels x bk channels.
 static int encode_im2col(CUtensorMap *map, const void *ptr, int n, int h, int w, int c, int r, int s,
                          int stride_h, int stride_w, int pad_h, int pad_w, int bk, int rows)
@@ -656,8 +688,6 @@ int gemm_with_status(const uint8_t *A, int64_t lda, const int8_t *B, int64_t ldb
     GemmMaps m = {};
     rc = encode_2d(&m.a, A, K, M, lda, bk, tile_rows);
     if (rc != SPARQ_OK) return rc;
-    rc = encode_2d(&m.b, B, K, N, ldb, bk, bn);
-    if (rc != SPARQ_OK) return rc;
     GemmArgs g;
     memset(&g, 0, sizeof(g));
     g.M = M; g.N = N; g.K = K;
@@ -670,6 +700,7 @@ int gemm_with_status(const uint8_t *A, int64_t lda, const int8_t *B, int64_t ldb
     g.split = small.split;
     const int grid = small.tile_rows ? (int)tiles * small.split : (int)(tiles < sms ? tiles : sms);
     if ((rc = output_maps(&m, &g, x.mode, bn, tiles, grid)) != SPARQ_OK) return rc;
+    if ((rc = encode_b(&m.b, B, K, N, ldb, bk, bn, g, small.tile_rows != 0)) != SPARQ_OK) return rc;
     cudaError_t ce = launch(bn, bk, small.tile_rows != 0, m, g, x, grid, st);
     if (ce != cudaSuccess) return cuda_error(ce, "sparq_gemm_kernel launch");
     return SPARQ_OK;
@@ -688,8 +719,6 @@ static int im2col_conv(const uint8_t *x_in, int n, int h, int w, int c, const in
     const int tile_rows = small.tile_rows ? small.tile_rows : kBM;
     GemmMaps m = {};
     rc = encode_im2col(&m.a, x_in, n, h, w, c, r, s, stride_h, stride_w, pad_h, pad_w, bk, tile_rows);
-    if (rc != SPARQ_OK) return rc;
-    rc = encode_2d(&m.b, wgt, K, cout, K, bk, bn);
     if (rc != SPARQ_OK) return rc;
     GemmArgs g;
     memset(&g, 0, sizeof(g));
@@ -711,6 +740,7 @@ static int im2col_conv(const uint8_t *x_in, int n, int h, int w, int c, const in
     g.split = small.split;
     const int grid = small.tile_rows ? (int)tiles * small.split : (int)(tiles < sms ? tiles : sms);
     if ((rc = output_maps(&m, &g, x.mode, bn, tiles, grid)) != SPARQ_OK) return rc;
+    if ((rc = encode_b(&m.b, wgt, K, cout, K, bk, bn, g, small.tile_rows != 0)) != SPARQ_OK) return rc;
     cudaError_t ce = launch(bn, bk, small.tile_rows != 0, m, g, x, grid, st);
     if (ce != cudaSuccess) return cuda_error(ce, "sparq_gemm_kernel (convolution) launch");
     return SPARQ_OK;

@@ -190,6 +190,15 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
         :: "r"(dst), "l"(map), "r"(bar), "r"(x), "r"(y) : "memory");
 }
 
+// Groups of 32 weight rows from row n0 (a multiple of 32), in the order that the map says (natural, or
+// that of epi_frag: one instruction for both, the loop that issues it has no time for a decision).
+__device__ __forceinline__ void tma_load_row_groups(uint32_t dst, const CUtensorMap *map, uint32_t bar, int k, int n0)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %4, %4, %5}], [%2];"
+        :: "r"(dst), "l"(map), "r"(bar), "r"(k), "r"(0), "r"(n0 >> 5) : "memory");
+}
+
 // im2col box: `pixels-per-column` output pixels starting at base pixel (w, h, n), channels
 // c .. c+box, filter tap offset (woff, hoff); out-of-image taps are filled with zeros.
 __device__ __forceinline__ void tma_load_im2col_4d(uint32_t dst, const CUtensorMap *map, uint32_t bar,
@@ -304,6 +313,25 @@ __device__ __forceinline__ void tmem_ld_32x32_issue(uint32_t taddr, uint32_t (&r
         : "r"(taddr) : "memory");
 }
 
+// 32 rows x 32 columns of an accumulator as matrix fragments: lane l gets, of each group j of eight
+// columns, columns 2 (l % 4) and + 1 of rows l / 4 (r[4j], r[4j + 1]), + 8 (r[4j + 2], r[4j + 3]) and, 16
+// places on in r, + 16 and + 24.
+__device__ __forceinline__ void tmem_ld_frag_issue(uint32_t taddr, uint32_t (&r)[32])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr) : "memory");
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(taddr + (16u << 16)) : "memory");
+}
+
 // Reduction steps of a convolution in order, from step `first`: filter tap (r, s), channel block
 // starting at c, and the block's first byte k of a filter.
 struct TapWalk {
@@ -415,6 +443,13 @@ struct EpiView {
 // 17.5 -> 16.9 us without the residual's code, 32x56x56x64 -> 64 10.75 -> 10.45.
 enum EpiOut { kOutGeneral, kOutBytes, kOutResidual };
 
+// Whether an epilogue of sparq_gemm_kernel works on matrix fragments (epi_frag), with the weight rows in fragment
+// order: boxes staged in shared memory, and 256-wide tiles.  Straight to global memory from narrower ones the
+// row form, a whole 32 bytes of a row per thread and store, is faster (200704 x 64, K 256, 17.5 us against
+// 17.9, without a transform 10.7 against 11.9), and in the window kernel (128x28x28x128 -> 128 3x3
+// 15.4 against 15.6, 256-wide tiles 35.6 against 36.4).
+__host__ __device__ constexpr bool frag_rows(int out, int bn, int out_box) { return out != kOutGeneral && (bn == 256 || out_box); }
+
 template <class Args>
 __host__ __device__ __forceinline__ EpiView make_epi_view(const Args &g)
 {
@@ -431,7 +466,8 @@ __host__ __device__ __forceinline__ EpiView make_epi_view(const Args &g)
     const bool aligned32 = ((reinterpret_cast<uintptr_t>(g.u8_out) | reinterpret_cast<uintptr_t>(g.f32_out) |
                              reinterpret_cast<uintptr_t>(g.acc_out) | reinterpret_cast<uintptr_t>(g.residual)) & 31u) == 0;
     e.gran = g.N % 32 == 0 && aligned32 ? 32 : g.N % 16 == 0 ? 16 : g.N % 8 == 0 ? 8 : g.N % 4 == 0 ? 4 : 1;
-    const bool bytes_only = e.u8_out && !g.acc_out && !g.f32_out && g.next_mode == SPARQ_MODE_NONE && !e.relu_op && e.gran == 32;
+    // (the fragment form keeps offsets over a tile's rows in 32 bits)
+    const bool bytes_only = e.u8_out && !g.acc_out && !g.f32_out && g.next_mode == SPARQ_MODE_NONE && !e.relu_op && e.gran == 32 && g.N < 1 << 24;
     e.out = !bytes_only ? kOutGeneral : g.residual ? kOutResidual : kOutBytes;
     e.next_mode = g.next_mode;
     e.next_rnd = g.next_rnd;
@@ -516,6 +552,43 @@ __device__ __forceinline__ void epi_lean(const uint32_t (&v)[32], const float *s
         f2_unpack(f2_mul(y0, inv2), z[0], z[1]);
         f2_unpack(f2_mul(y1, inv2), z[2], z[3]);
         w[q] = requant_pack4(z[0], z[1], z[2], z[3]);
+    }
+}
+
+// The same on matrix fragments (tmem_ld_frag_issue): a thread has four rows of eight columns, so that a
+// column's scale and bias are read once for four outputs, four 16-byte reads per 32 x 32 outputs where
+// a thread per row takes sixteen.  Those reads are broadcasts, but of more than one wavefront each, and shared
+// memory is what the epilogue shares with the tensor core's operands: they were 1200 of the 1600
+// wavefronts of the load / store pipe in a tile of an output-heavy layer.  16384 x 4096, K 512, 42.6 -> 38.7 us,
+// 50176 x 256, K 512, without a transform 9.95 -> 9.0, the ResNet-50 pass at batch 64 829 -> 799.
+// The eight columns are adjacent outputs because the weight rows lie in shared memory in fragment order:
+// row 8j + 2q + b of each group of 32 holds weight row 8q + 2j + b (a five-dimensional tensor map, no
+// extra copy), so accumulator columns 2q, 2q + 1 of the groups j = 0..3 are output columns 8q .. 8q + 7.
+// scale, bias: of this thread's eight columns.  res, w: bytes of row r in words 2r, 2r + 1.
+template <bool RES>
+__device__ __forceinline__ void epi_frag(const uint32_t (&v)[32], const float *scale, const float *bias, float inv, float res_scale,
+                                         const uint32_t (&res)[8], uint32_t (&w)[8])
+{
+    const uint64_t inv2 = f2_pack(inv, inv), rs2 = f2_pack(res_scale, res_scale);
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+        const float4 sc = *reinterpret_cast<const float4 *>(&scale[4 * p]);
+        const float4 bi = *reinterpret_cast<const float4 *>(&bias[4 * p]);
+        const uint64_t s0 = f2_pack(sc.x, sc.y), s1 = f2_pack(sc.z, sc.w), b0 = f2_pack(bi.x, bi.y), b1 = f2_pack(bi.z, bi.w);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int i = 16 * (r >> 1) + 8 * p + 2 * (r & 1);
+            uint64_t y0 = f2_fma(f2_pack(__int2float_rn((int)v[i]), __int2float_rn((int)v[i + 1])), s0, b0);
+            uint64_t y1 = f2_fma(f2_pack(__int2float_rn((int)v[i + 4]), __int2float_rn((int)v[i + 5])), s1, b1);
+            if (RES) {
+                y0 = f2_fma(bytes_to_f2<0>(res[2 * r + p]), rs2, y0);
+                y1 = f2_fma(bytes_to_f2<1>(res[2 * r + p]), rs2, y1);
+            }
+            float z[4];
+            f2_unpack(f2_mul(y0, inv2), z[0], z[1]);
+            f2_unpack(f2_mul(y1, inv2), z[2], z[3]);
+            w[2 * r + p] = requant_pack4(z[0], z[1], z[2], z[3]);
+        }
     }
 }
 
@@ -733,6 +806,59 @@ __device__ __forceinline__ void epi_warp_columns_as(const EpiView &e, uint32_t t
     }
 }
 
+// A warp's share of one accumulator in fragment form, straight to global memory: each row gets 32 bytes
+// of four adjacent threads.  pos: the tile's first output byte of these columns, off[r]: from there to this
+// thread's eight bytes in its row r, rows: bit r set where that row exists, left: columns up to N.
+// (All that is worked out once per tile, or launch: a 64-bit row position per store cost 4-6 %.)
+template <bool RES, class WaitFull>
+__device__ __forceinline__ void epi_frag_columns(const EpiView &e, uint32_t taddr0, int cols, int64_t pos, const uint32_t (&off)[4], uint32_t rows,
+                                                 int64_t left, const float *s_scale, const float *s_bias, uint32_t acc_empty_bar, int lane, WaitFull wait_full)
+{
+    s_scale += 8 * (lane & 3);
+    s_bias += 8 * (lane & 3);
+    const int valid = left < cols ? (int)left : cols;       // a multiple of 32, or none
+    uint8_t *out = e.u8_out + pos;
+    const uint8_t *residual = e.residual + pos;
+    uint32_t rn[8];
+    auto fetch_residual = [&](int c) {
+        if (c >= valid) return;
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+            if (rows >> r & 1u) {
+                const uint2 b = __ldg(reinterpret_cast<const uint2 *>(residual + c + off[r]));
+                rn[2 * r] = b.x;
+                rn[2 * r + 1] = b.y;
+            }
+    };
+    if (RES) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) rn[i] = 0u;
+        fetch_residual(0);
+    }
+    wait_full();
+#pragma unroll 1
+    for (int c = 0; c < cols; c += 32) {
+        uint32_t v[32], res[8], w[8];
+        tmem_ld_frag_issue(taddr0 + (uint32_t)c, v);
+        if (RES) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) res[i] = rn[i];
+            fetch_residual(c + 32);
+        }
+        tmem_ld_wait();
+        if (c + 32 == cols) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(acc_empty_bar);
+        }
+        if (c >= valid) continue;
+        epi_frag<RES>(v, s_scale + c, s_bias + c, e.inv_out_scale, e.residual_scale, res, w);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+            if (rows >> r & 1u) *reinterpret_cast<uint2 *>(out + c + off[r]) = make_uint2(w[2 * r], w[2 * r + 1]);
+    }
+}
+
 // OUT: the kind of output that the kernel is instantiated for (EpiOut).
 template <int OUT, class WaitFull>
 __device__ __forceinline__ void epi_warp_columns(const EpiView &e, uint32_t taddr0, int cbase, int cols, int64_t row, bool row_ok,
@@ -748,7 +874,7 @@ __device__ __forceinline__ void epi_warp_columns(const EpiView &e, uint32_t tadd
     }
 }
 
-// One box of the staged output: this thread's row of `box` (64 or 128) columns, from tensor memory to
+// One box of the staged output: 32 rows of `box` (64 or 128) columns, from tensor memory (in fragment form) to
 // the warp's shared-memory buffer `buf` (32 rows of `box` bytes, 16-byte pieces swizzled as the
 // tensor map says), which a TMA store then takes to global memory as whole 64- or 128-byte
 // pieces of a row.  With a residual the buffer holds the identity tensor's box, fetched by TMA,
@@ -758,22 +884,29 @@ __device__ __forceinline__ void epi_warp_columns(const EpiView &e, uint32_t tadd
 // into 32 different lines; a 51 MB output took 16.6 us that way against 10.5 in whole lines, and
 // its residual with it, with little L1 left beside the operand ring, 35 against 20.  (Fetching
 // the residual into L2 ahead of the boxes changed nothing: it is not HBM's latency.)  The whole
-// layer, M 200704 x K 64 -> N 256: 26.5 -> 23.3 us, with a residual 44.8 -> 33.2.
+// layer, M 200704 x K 64 -> N 256: 26.5 -> 23.3 us, with a residual 44.8 -> 33.2; and in fragment form 19.0 ->
+// 17.8 and 31.2 -> 28.1 (four buffers of 64 columns a warp, for more residual bytes in flight: 32.0).
 // next_residual() is called once the first 32 columns are done.
 template <bool RES, class Next>
 __device__ __forceinline__ void epi_staged_box(uint32_t taddr, int box, uint32_t buf, const float *s_scale, const float *s_bias,
                                                float inv, float res_scale, uint32_t acc_empty_bar, int lane, Next next_residual)
 {
-    const uint32_t row = buf + (uint32_t)(lane * box);
-    const uint32_t swz = box == 128 ? (uint32_t)(lane & 7) : (uint32_t)((lane >> 1) & 3);
+    // this thread's rows lane / 4 + 8r: the swizzle of all four is that of the first
+    const uint32_t row = (uint32_t)(lane >> 2), c8 = 8u * (uint32_t)(lane & 3);
+    const uint32_t row_buf = buf + row * (uint32_t)box, step = 8u * (uint32_t)box;
+    const uint32_t swz = box == 128 ? row & 7u : (row >> 1) & 3u;
+    s_scale += c8;
+    s_bias += c8;
 #pragma unroll 1
     for (int c = 0; c < box; c += 32) {
-        uint32_t v[32], r[8], w[8];
-        tmem_ld_32x32_issue(taddr + (uint32_t)c, v);
-        const uint32_t a0 = row + ((((uint32_t)c >> 4) ^ swz) << 4), a1 = row + (((((uint32_t)c >> 4) + 1u) ^ swz) << 4);
+        uint32_t v[32], res[8], w[8];
+        tmem_ld_frag_issue(taddr + (uint32_t)c, v);
+        const uint32_t col = (uint32_t)c + c8;
+        const uint32_t a = row_buf + (((col >> 4) ^ swz) << 4) + (col & 8u);
         if (RES) {
-            asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a0));
-            asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(a1));
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+                asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(res[2 * r]), "=r"(res[2 * r + 1]) : "r"(a + (uint32_t)r * step));
         }
         tmem_ld_wait();
         if (acc_empty_bar && c + 32 == box) {        // the accumulator's last columns are in registers
@@ -781,9 +914,10 @@ __device__ __forceinline__ void epi_staged_box(uint32_t taddr, int box, uint32_t
             __syncwarp();
             if (lane == 0) mbar_arrive(acc_empty_bar);
         }
-        epi_lean<RES>(v, s_scale + c, s_bias + c, inv, res_scale, r, w);
-        asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" :: "r"(a0), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]) : "memory");
-        asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" :: "r"(a1), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
+        epi_frag<RES>(v, s_scale + c, s_bias + c, inv, res_scale, res, w);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+            asm volatile("st.shared.v2.u32 [%0], {%1,%2};" :: "r"(a + (uint32_t)r * step), "r"(w[2 * r]), "r"(w[2 * r + 1]) : "memory");
         if (c == 0) next_residual();
     }
 }
@@ -920,7 +1054,10 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                         if (++s == S) { s = 0; ++use; }
                     }
                 };
-                auto weights = [&](uint32_t full, const TapWalk &tap) { tma_load_2d(b_stage(s), &map_b, full, tap.k, n0); };
+                auto weights = [&](uint32_t full, const TapWalk &tap) {
+                    if (OUT != kOutGeneral) tma_load_row_groups(b_stage(s), &map_b, full, tap.k, n0);
+                    else tma_load_2d(b_stage(s), &map_b, full, tap.k, n0);
+                };
                 if (kTwoProducers && warp == kWeightWarp) {
                     stages(Cfg::kBBytes, weights);
                 } else if (g.conv) {
@@ -998,6 +1135,9 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         const int cols = BN / parts, cbase = part * cols;    // this warp's share of the tile's columns
         const int team_thread = (part * 4 + quarter) * 32 + lane, team_threads = parts * 128;
         const EpiView ev = make_epi_view(g);
+        uint32_t off[4];                                     // epi_frag_columns
+#pragma unroll
+        for (int r = 0; r < 4; ++r) off[r] = (uint32_t)((lane >> 2) + 8 * r) * (uint32_t)g.N + 8u * (uint32_t)(lane & 3);
         int64_t staged_nt = -1;
         uint32_t local_tile = (uint32_t)team;
         if (OUT != kOutGeneral && g.out_box) {
@@ -1077,13 +1217,23 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                 staged_nt = nt;
                 epi_stage_scale_bias(g, nt * BN, BN, team_thread, team_threads, 1 + team, s_scale[team], s_bias[team]);
             }
-            const int64_t row = mt * kBM + quarter * 32 + lane;
             const uint32_t taddr0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * BN + cbase);
-            epi_warp_columns<OUT>(ev, taddr0, cbase, cols, row, row < g.M, nt * BN, s_scale[team], s_bias[team],
-                             smem_u32(&bar_acc_empty[acc]), lane, [&]() {
-                                 mbar_wait(smem_u32(&bar_acc_full[acc]), acc_use & 1, abort_flag, g.status, g.wait_limit);
-                                 tc_fence_after();
-                             });
+            auto wait_full = [&]() {
+                mbar_wait(smem_u32(&bar_acc_full[acc]), acc_use & 1, abort_flag, g.status, g.wait_limit);
+                tc_fence_after();
+            };
+            const int64_t row0 = mt * kBM + quarter * 32;
+            if constexpr (!frag_rows(OUT, BN, 0)) {
+                const int64_t row = row0 + lane;
+                epi_warp_columns<OUT>(ev, taddr0, cbase, cols, row, row < g.M, nt * BN, s_scale[team], s_bias[team],
+                                      smem_u32(&bar_acc_empty[acc]), lane, wait_full);
+            } else {
+                uint32_t rows = 0;
+#pragma unroll
+                for (int r = 0; r < 4; ++r) rows |= (row0 + (lane >> 2) + 8 * r < g.M ? 1u : 0u) << r;
+                epi_frag_columns<OUT == kOutResidual>(ev, taddr0, cols, row0 * g.N + nt * BN + cbase, off, rows, g.N - nt * BN - cbase, s_scale[team] + cbase,
+                                                      s_bias[team] + cbase, smem_u32(&bar_acc_empty[acc]), lane, wait_full);
+            }
         }
     } else if (MODE != SPARQ_MODE_NONE) {
         // ================= transform =================

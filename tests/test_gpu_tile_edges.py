@@ -60,6 +60,31 @@ def test_staged_output(mode, residual, n):
     assert (got[m * n:] == 0xA5).all()
 
 
+@pytest.mark.parametrize("mode", [sparq.MODE_NONE, sparq.MODE_VSPARQ])
+@pytest.mark.parametrize("residual", [False, True])
+@pytest.mark.parametrize("n,tail", [(160, 1), (224, 33), (256, 127), (480, 8)])
+def test_wide_tiles_straight_to_memory(mode, residual, n, tail):
+    """256-wide tiles of a long reduction (not staged): a warp's rows and 32-column groups at the tails of the
+    matrix, and tiles with columns past N; nothing written past the end."""
+    m, k = 148 * 128 + tail, 1024
+    A = synth.activations(n, (m, k), 0.5)
+    B = synth.weights(n, (k, n))
+    scale, bias, inv = synth.scales(n, n), synth.bias(n, n), synth.inv_out_scale(k)
+    res = synth.activations(n + 1, (m, n), 0.5) if residual else None
+    p = sparq.SparqParams(mode, 4, 0x1F, 1)
+    out = torch.full((m * n + 64,), 0xA5, dtype=torch.uint8, device="cuda")
+    sparq.sparq_gemm_s8(torch.from_numpy(A).cuda(), torch.from_numpy(np.ascontiguousarray(B.T)).cuda(), p,
+                        scale=torch.from_numpy(scale).cuda(), bias=torch.from_numpy(bias).cuda(), relu=True,
+                        inv_out_scale=inv, u8_out=out, residual=torch.from_numpy(res).cuda() if residual else None,
+                        residual_scale=0.02)
+    sparq.sparq_check()
+    acc = oracle.gemm(A, B, mode, 4, 0x1F, 1)
+    _, want = oracle.epilogue(acc, scale, bias, True, inv, residual=res, residual_scale=0.02)
+    got = out.cpu().numpy()
+    assert np.array_equal(got[:m * n].reshape(m, n), want)
+    assert (got[m * n:] == 0xA5).all()
+
+
 @pytest.mark.parametrize("mode,n", [(sparq.MODE_VSPARQ, 4), (sparq.MODE_BSPARQ, 3)])
 def test_transform_first_gemm(mode, n):
     """Long reductions with many column tiles run as transform + plain contraction: two streams at
