@@ -4,14 +4,14 @@
 //
 // One persistent CTA per SM walks output tiles of 128 x BN.  Warp roles:
 //   warp 0        TMA producer: A tile (tiled 2-D box for the GEMM, im2col box for the
-//                 convolution) and B tile into a ring of shared-memory stages; without a transform
-//                 warp 18 fetches B
+//                 convolution) and B tile into a ring of shared-memory stages; without a transform,
+//                 and with ATM, warp 18 fetches B
 //   warp 1        allocates tensor memory; one lane issues tcgen05.mma kind::i8
 //                 (u8 x s8 -> s32) on each transformed stage
 //   warps 2..9    epilogue: tcgen05.ld of a finished accumulator, fp32 scale / bias /
 //                 ReLU / requantize, global stores (warp w reads lane quarter w % 4 of its team's
 //                 tiles, and its share of their columns)
-//   warps 10..17  transform: rewrite the A stage in place with bSPARQ / vSPARQ
+//   warps 10..17  transform: rewrite the A stage in place with bSPARQ / vSPARQ (or, ATM, into tensor memory)
 //
 // A stage travels  TMA (async proxy) -> transform warps (generic proxy) -> MMA (async
 // proxy); the hand-offs are mbarriers, with fence.proxy.async after the in-place rewrite.
@@ -47,7 +47,7 @@ constexpr int kFirstXfWarp = kFirstEpiWarp + kNumEpiWarps;
 // 3x3 transformed first 16.5 -> 14.4 us, 56x56x128 -> 128 3x3 stride 2 without a transform 12.8 -> 10.9).
 // With a transform a step is longer, and one producer as fast or faster (200704 x 64, K 256, 17.55 us against 17.75).
 constexpr int kWeightWarp = kFirstXfWarp + kNumXfWarps;
-__host__ __device__ constexpr int gemm_threads(int mode) { return 32 * (kWeightWarp + (mode == SPARQ_MODE_NONE ? 1 : 0)); }
+__host__ __device__ constexpr int gemm_threads(int mode, bool in_tmem) { return 32 * (kWeightWarp + (mode == SPARQ_MODE_NONE || in_tmem ? 1 : 0)); }
 // Epilogue warps of a kernel instantiated for `mode`.
 __host__ __device__ constexpr int epi_warps(int mode) { return mode == SPARQ_MODE_NONE ? kNumEpiWarps + kNumXfWarps : kNumEpiWarps; }
 // Shares that a tile's columns are split into over the groups of one epilogue team.
@@ -89,6 +89,7 @@ struct GemmArgs {
     const uint8_t *residual;
     float residual_scale;
     int stages;             // of the operand ring
+    int raw_stages;         // of the ring of activations, where they have one of their own
     // staged output: bytes per row of the boxes that the epilogue warps store (and fetch the residual)
     // with through shared memory, 0 = straight from registers.  See epi_staged.
     int out_box;
@@ -251,6 +252,18 @@ __device__ __forceinline__ void tc_mma_i8_if(uint32_t d_tmem, uint64_t adesc, ui
         :: "r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(elected) : "memory");
 }
 
+// The same with A in tensor memory (row i in lane i, four bytes of K per column).
+__device__ __forceinline__ void tc_mma_i8_tmem_if(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
+                                                  uint32_t accumulate, uint32_t elected)
+{
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "setp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::i8 [%0], [%1], %2, %3, p;\n\t}"
+        :: "r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(elected) : "memory");
+}
+
 __device__ __forceinline__ void tc_commit_if(uint32_t bar, uint32_t elected)
 {
     asm volatile(
@@ -289,6 +302,15 @@ __device__ __forceinline__ constexpr uint32_t make_idesc_i8(int n, int m = kBM)
 {
     return (2u << 4) | (0u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
+
+// 16 words of each lane's row into 16 columns.
+__device__ __forceinline__ void tmem_st_32x16(uint32_t taddr, const uint4 (&v)[4])
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
+                 :: "r"(taddr), "r"(v[0].x), "r"(v[0].y), "r"(v[0].z), "r"(v[0].w), "r"(v[1].x), "r"(v[1].y), "r"(v[1].z), "r"(v[1].w),
+                    "r"(v[2].x), "r"(v[2].y), "r"(v[2].z), "r"(v[2].w), "r"(v[3].x), "r"(v[3].y), "r"(v[3].z), "r"(v[3].w) : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
@@ -955,18 +977,24 @@ struct TileCfg {
     static constexpr int kTmemCols = kAcc * BN;
 };
 
-template <int BN, int BK, int MODE, int XN, bool RND, int OUT>
-__global__ void __launch_bounds__(gemm_threads(MODE), 1)
+template <int BN, int BK, int MODE, int XN, bool RND, int OUT, bool ATM>
+__global__ void __launch_bounds__(gemm_threads(MODE, ATM), 1)
 sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                   const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_res, const GemmArgs g)
 {
     using Cfg = TileCfg<BN, BK>;
-    constexpr bool kTwoProducers = MODE == SPARQ_MODE_NONE;
+    constexpr bool kTwoProducers = MODE == SPARQ_MODE_NONE || ATM;
+    // ATM: the transform warps write their results to tensor memory, which the tensor core reads A from; the
+    // raw activations have a ring of their own.
+    static_assert(!ATM || (MODE != SPARQ_MODE_NONE && BK == 128 && BN == 256), "A in tensor memory: transformed steps of 128 bytes");
     const int S = g.stages;
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t bar_full[kMaxStages], bar_xf[kMaxStages], bar_empty[kMaxStages];
+    __shared__ __align__(8) uint64_t bar_raw[ATM ? kMaxStages : 1], bar_raw_empty[ATM ? kMaxStages : 1];
     __shared__ __align__(8) uint64_t bar_res[epi_warps(MODE)][2];       // residual boxes landed
-    constexpr int kAcc = Cfg::kAcc;
+    // tensor memory: accumulators, and with ATM four to eight stages of transformed activations
+    constexpr int kAcc = ATM ? 256 / BN : Cfg::kAcc;
+    constexpr int kTmemCols = ATM ? 512 : Cfg::kTmemCols;
     // The epilogue warps form groups of four (one warp per tensor-memory lane quarter) and the
     // groups teams: team t takes the CTA's tiles of number t modulo the number of teams, so that the
     // epilogues of consecutive tiles -- mostly latency -- overlap.  A CTA with a single tile puts
@@ -992,16 +1020,23 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     const int teams = total_tiles > gridDim.x ? kMaxTeams : 1;
 
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    auto a_stage = [&](int s) { return smem_base + (uint32_t)s * Cfg::kStageBytes; };
-    auto b_stage = [&](int s) { return smem_base + (uint32_t)s * Cfg::kStageBytes + Cfg::kABytes; };
+    const int SA = ATM ? g.raw_stages : S;
+    const uint32_t b_base = smem_base + (uint32_t)(ATM ? SA * Cfg::kABytes : Cfg::kABytes);
+    constexpr uint32_t kAStep = ATM ? Cfg::kABytes : Cfg::kStageBytes, kBStep = ATM ? Cfg::kBBytes : Cfg::kStageBytes;
+    auto a_stage = [&](int s) { return smem_base + (uint32_t)s * kAStep; };
+    auto b_stage = [&](int s) { return b_base + (uint32_t)s * kBStep; };
 
     if (threadIdx.x == 0) {
         prefetch_tensormap(&map_a);
         prefetch_tensormap(&map_b);
         for (int s = 0; s < S; ++s) {
-            mbar_init(smem_u32(&bar_full[s]), kTwoProducers ? 2 : 1);
+            mbar_init(smem_u32(&bar_full[s]), MODE == SPARQ_MODE_NONE ? 2 : 1);
             mbar_init(smem_u32(&bar_xf[s]), kXfTeamWarps);
             mbar_init(smem_u32(&bar_empty[s]), 1);
+        }
+        for (int s = 0; ATM && s < SA; ++s) {
+            mbar_init(smem_u32(&bar_raw[s]), 1);
+            mbar_init(smem_u32(&bar_raw_empty[s]), kXfTeamWarps);
         }
         for (int a = 0; a < kAcc; ++a) {
             mbar_init(smem_u32(&bar_acc_full[a]), 1);
@@ -1015,7 +1050,7 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     }
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     :: "r"(smem_u32(&tmem_base_slot)), "r"((uint32_t)Cfg::kTmemCols) : "memory");
+                     :: "r"(smem_u32(&tmem_base_slot)), "r"((uint32_t)kTmemCols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     tc_fence_before();
@@ -1034,9 +1069,13 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         // behind the tensor core's operand fetches).
         if (lane == 0) {
             constexpr uint32_t kBytes = kTwoProducers ? Cfg::kABytes : Cfg::kStageBytes;     // of the first producer
+            // the ring that this thread fills, and its barriers
+            const bool raw = ATM && warp == 0;
+            const int ring = raw ? SA : S;
+            const uint32_t bars_full = smem_u32(raw ? bar_raw : bar_full), bars_empty = smem_u32(raw ? bar_raw_empty : bar_empty);
             uint32_t it = 0;   // running stage counter across tiles
-            int s = 0;         // stage it % S
-            uint32_t use = 0;  // it / S
+            int s = 0;         // stage it % ring
+            uint32_t use = 0;  // it / ring
             bool live = true;
             for (uint32_t tile = blockIdx.x; tile < total_tiles && live; tile += gridDim.x) {
                 const uint32_t mt = (n_tiles32 == 1) ? tile : tile / n_tiles32, nt = tile - mt * n_tiles32;
@@ -1046,12 +1085,12 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                 auto stages = [&](uint32_t bytes, auto copy) {
                     TapWalk tap(g, BK, 0);
                     for (int kb = 0; kb < kb_count; ++kb, ++it) {
-                        if (use > 0 && !mbar_wait(smem_u32(&bar_empty[s]), (use - 1) & 1, abort_flag, g.status, g.wait_limit)) { live = false; break; }
-                        const uint32_t full = smem_u32(&bar_full[s]);
+                        if (use > 0 && !mbar_wait(bars_empty + 8u * (uint32_t)s, (use - 1) & 1, abort_flag, g.status, g.wait_limit)) { live = false; break; }
+                        const uint32_t full = bars_full + 8u * (uint32_t)s;
                         mbar_expect_tx(full, bytes);
                         copy(full, tap);
                         tap.next();
-                        if (++s == S) { s = 0; ++use; }
+                        if (++s == ring) { s = 0; ++use; }
                     }
                 };
                 auto weights = [&](uint32_t full, const TapWalk &tap) {
@@ -1081,9 +1120,9 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
             // After an abort: wait (bounded) for the copies this thread still has in
             // flight, so that none lands after the CTA has exited.
             if (*abort_flag) {
-                const uint32_t first = it > (uint32_t)S ? it - S : 0;
+                const uint32_t first = it > (uint32_t)ring ? it - ring : 0;
                 for (uint32_t j = first; j < it; ++j)
-                    mbar_wait(smem_u32(&bar_full[j % S]), (j / S) & 1, abort_flag, g.status, g.wait_limit, true);
+                    mbar_wait(bars_full + 8u * (j % ring), (j / ring) & 1, abort_flag, g.status, g.wait_limit, true);
             }
         }
         __syncwarp();
@@ -1096,7 +1135,7 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
             constexpr uint32_t idesc = make_idesc_i8(BN);
             // descriptors of stage 0; a stage adds its byte offset / 16 to the start-address field
             const uint64_t adesc0 = make_smem_desc<BK>(smem_base);
-            const uint64_t bdesc0 = make_smem_desc<BK>(smem_base + Cfg::kABytes);
+            const uint64_t bdesc0 = make_smem_desc<BK>(b_base);
             uint32_t local_tile = 0;
             int s = 0;             // stage
             uint32_t ph = 0;       // its phase parity
@@ -1109,13 +1148,16 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                 for (int kb = 0; kb < kb_count; ++kb) {
                     if (MODE == SPARQ_MODE_NONE) mbar_wait(smem_u32(&bar_full[s]), ph, abort_flag, g.status, g.wait_limit);
                     else mbar_wait(smem_u32(&bar_xf[s]), ph, abort_flag, g.status, g.wait_limit);
+                    if (ATM) mbar_wait(smem_u32(&bar_full[s]), ph, abort_flag, g.status, g.wait_limit);
                     tc_fence_after();
-                    const uint64_t st_off = (uint64_t)((uint32_t)s * (uint32_t)(Cfg::kStageBytes >> 4));
-                    const uint64_t adesc = adesc0 + st_off, bdesc = bdesc0 + st_off;
+                    const uint64_t adesc = adesc0 + (uint64_t)((uint32_t)s * (kAStep >> 4)), bdesc = bdesc0 + (uint64_t)((uint32_t)s * (kBStep >> 4));
+                    const uint32_t a_tmem = tmem_base + 256u + (uint32_t)s * 32u;
 #pragma unroll
-                    for (int k = 0; k < BK / 32; ++k)
-                        tc_mma_i8_if(d_tmem, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc,
+                    for (int k = 0; k < BK / 32; ++k) {
+                        if (ATM) tc_mma_i8_tmem_if(d_tmem, a_tmem + (uint32_t)(k * 8), bdesc + (uint64_t)(k * 2), idesc, (kb > 0 || k > 0) ? 1u : 0u, elected);
+                        else tc_mma_i8_if(d_tmem, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc,
                                      (kb > 0 || k > 0) ? 1u : 0u, elected);
+                    }
                     tc_commit_if(smem_u32(&bar_empty[s]), elected);       // stage reusable once these MMAs retire
                     if (++s == S) { s = 0; ph ^= 1u; }
                 }
@@ -1144,7 +1186,7 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
             // ---- through shared memory (see epi_staged_box) ----
             const int ew = warp - kFirstEpiWarp;
             const uint32_t box_bytes = 32u * (uint32_t)g.out_box;
-            const uint32_t stage0 = smem_base + (uint32_t)(S * Cfg::kStageBytes) + (uint32_t)ew * 2u * box_bytes;
+            const uint32_t stage0 = (ATM ? b_stage(S) : a_stage(S)) + (uint32_t)ew * 2u * box_bytes;
             constexpr bool res = OUT == kOutResidual;
             // boxes of this warp in order: the out_box-wide parts of its columns, tile after tile
             auto fetch = [&](uint32_t n, uint32_t tile, int c) {          // box n's residual, by lane 0
@@ -1242,42 +1284,110 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         constexpr int kXfThreads = kXfTeamWarps * 32;
         constexpr int kVecs = Cfg::kABytes / 16;
         constexpr int kPerThread = kVecs / kXfThreads;
-        constexpr int kBatch = kPerThread < 4 ? kPerThread : 4;     // vectors in flight per thread
-        static_assert(kVecs % kXfThreads == 0 && kPerThread % kBatch == 0, "A stage must split evenly over a team");
+        constexpr int kHalf = kPerThread / 2;                       // vectors that a thread works on at a time
+        static_assert(kVecs % kXfThreads == 0 && kPerThread % 2 == 0, "A stage must split evenly over a team, and in halves");
         const XformDev xf = g.xf;
-        uint32_t it = 0, ph = 0;
-        int sn = 0;
-        for (uint32_t tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
-            for (int kb = 0; kb < kb_count; ++kb, ++it) {
-                const int s = sn;
-                const uint32_t sph = ph;
-                if (++sn == S) { sn = 0; ph ^= 1u; }
-                if ((int)(it & 1u) != team) continue;      // the other team's stage
-                mbar_wait(smem_u32(&bar_full[s]), sph, abort_flag, g.status, g.wait_limit);
-                const uint32_t base = a_stage(s) + (uint32_t)xt * 16u;
+        // The team's stages in order: its number, the ring stage and its phase.  A stage's first half is
+        // loaded while the second half of the one before is worked on, if it has landed by then: with two
+        // warps to a scheduler, the barrier read and the loads' latency at the head of each stage were a
+        // tenth of its time: 200704 x 64, K 256, 17.7 -> 16.9 us, 50176 x 128, K 512, 11.4 -> 10.9.
+        const uint32_t my_tiles = blockIdx.x < total_tiles ? (total_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0u;
+        const uint32_t total = my_tiles * (uint32_t)kb_count;
+        auto load = [&](uint4 (&v)[kHalf], int s, int j0) {
 #pragma unroll
-                for (int j0 = 0; j0 < kPerThread; j0 += kBatch) {
-                    uint4 v[kBatch];
+            for (int j = 0; j < kHalf; ++j)
+                asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v[j].x), "=r"(v[j].y), "=r"(v[j].z), "=r"(v[j].w)
+                             : "r"(a_stage(s) + (uint32_t)((j0 + j) * kXfThreads + xt) * 16u));
+        };
+        auto work = [&](uint4 (&v)[kHalf], int s, int j0) {
 #pragma unroll
-                    for (int j = 0; j < kBatch; ++j)
-                        asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];"
-                                     : "=r"(v[j].x), "=r"(v[j].y), "=r"(v[j].z), "=r"(v[j].w)
-                                     : "r"(base + (uint32_t)((j0 + j) * kXfThreads * 16)));
+            for (int j = 0; j < kHalf; ++j) {
+                v[j].x = xform_fused<MODE, XN, RND>(v[j].x, xf);
+                v[j].y = xform_fused<MODE, XN, RND>(v[j].y, xf);
+                v[j].z = xform_fused<MODE, XN, RND>(v[j].z, xf);
+                v[j].w = xform_fused<MODE, XN, RND>(v[j].w, xf);
+                asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};"
+                             :: "r"(a_stage(s) + (uint32_t)((j0 + j) * kXfThreads + xt) * 16u),
+                                "r"(v[j].x), "r"(v[j].y), "r"(v[j].z), "r"(v[j].w) : "memory");
+            }
+        };
+        if constexpr (ATM) {
+            // A thread has one row (of its warp's tensor-memory lanes), half of its 128 bytes at a time; from the
+            // raw stage into the transformed one, which has the number of the weight stage beside it.
+            const int quarter = warp & 3;
+            const uint32_t row = (uint32_t)(quarter * 32 + lane), swz = row & 7u;
+            auto load_row = [&](uint4 (&v)[4], int sa, int c0) {
 #pragma unroll
-                    for (int j = 0; j < kBatch; ++j) {
-                        v[j].x = xform_fused<MODE, XN, RND>(v[j].x, xf);
-                        v[j].y = xform_fused<MODE, XN, RND>(v[j].y, xf);
-                        v[j].z = xform_fused<MODE, XN, RND>(v[j].z, xf);
-                        v[j].w = xform_fused<MODE, XN, RND>(v[j].w, xf);
-                        asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};"
-                                     :: "r"(base + (uint32_t)((j0 + j) * kXfThreads * 16)),
-                                        "r"(v[j].x), "r"(v[j].y), "r"(v[j].z), "r"(v[j].w) : "memory");
-                    }
+                for (int j = 0; j < 4; ++j)
+                    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v[j].x), "=r"(v[j].y), "=r"(v[j].z), "=r"(v[j].w)
+                                 : "r"(a_stage(sa) + row * 128u + (((uint32_t)(c0 + j) ^ swz) << 4)));
+            };
+            auto work_row = [&](uint4 (&v)[4]) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    v[j].x = xform_fused<MODE, XN, RND>(v[j].x, xf);
+                    v[j].y = xform_fused<MODE, XN, RND>(v[j].y, xf);
+                    v[j].z = xform_fused<MODE, XN, RND>(v[j].z, xf);
+                    v[j].w = xform_fused<MODE, XN, RND>(v[j].w, xf);
                 }
-                fence_proxy_async_smem();       // generic-proxy writes visible to the tensor core
+            };
+            uint4 va[4], vb[4];
+            int sa = team, s = team;
+            uint32_t pa = 0, use = 0;          // phase of the raw stage; uses of the transformed one before
+            bool loaded = false;
+            for (uint32_t it = (uint32_t)team; it < total; it += kXfTeams) {
+                if (!loaded) {
+                    mbar_wait(smem_u32(&bar_raw[sa]), pa, abort_flag, g.status, g.wait_limit);
+                    load_row(va, sa, 0);
+                }
+                load_row(vb, sa, 4);
+                work_row(va);
+                if (use > 0) mbar_wait(smem_u32(&bar_empty[s]), (use - 1u) & 1u, abort_flag, g.status, g.wait_limit);
+                tc_fence_after();
+                const uint32_t dst = tmem_base + ((uint32_t)(quarter * 32) << 16) + 256u + (uint32_t)s * 32u;
+                tmem_st_32x16(dst, va);
+                int na = sa + kXfTeams;
+                uint32_t npa = pa;
+                if (na >= SA) { na -= SA; npa ^= 1u; }
+                loaded = it + kXfTeams < total && __all_sync(0xFFFFFFFFu, mbar_test(smem_u32(&bar_raw[na]), npa));
+                if (loaded) load_row(va, na, 0);
+                work_row(vb);
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&bar_raw_empty[sa]));      // the whole stage is in registers
+                tmem_st_32x16(dst + 16u, vb);
+                tmem_st_wait();
+                tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&bar_xf[s]));
+                sa = na;
+                pa = npa;
+                s += kXfTeams;
+                if (s >= S) { s -= S; ++use; }
             }
+        } else {
+        uint4 va[kHalf], vb[kHalf];
+        int s = team;
+        uint32_t ph = 0;
+        bool loaded = false;
+        for (uint32_t it = (uint32_t)team; it < total; it += kXfTeams) {
+            if (!loaded) {
+                mbar_wait(smem_u32(&bar_full[s]), ph, abort_flag, g.status, g.wait_limit);
+                load(va, s, 0);
+            }
+            load(vb, s, kHalf);
+            work(va, s, 0);
+            int ns = s + kXfTeams;
+            uint32_t nph = ph;
+            if (ns >= S) { ns -= S; nph ^= 1u; }
+            loaded = it + kXfTeams < total && __all_sync(0xFFFFFFFFu, mbar_test(smem_u32(&bar_full[ns]), nph));
+            if (loaded) load(va, ns, 0);
+            work(vb, s, kHalf);
+            fence_proxy_async_smem();       // generic-proxy writes visible to the tensor core
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&bar_xf[s]));
+            s = ns;
+            ph = nph;
+        }
         }
     }
 
@@ -1286,7 +1396,7 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;"
-                     :: "r"(tmem_base), "r"((uint32_t)Cfg::kTmemCols) : "memory");
+                     :: "r"(tmem_base), "r"((uint32_t)kTmemCols) : "memory");
     }
 }
 
@@ -1299,10 +1409,10 @@ struct GemmMaps {
 template <int BN, int BK>
 cudaError_t launch_gemm_shape(const GemmMaps &m, GemmArgs &g, int mode, int n, int rnd, int grid, cudaStream_t st);
 
-template <int BN, int BK, int MODE, int XN, bool RND, int OUT>
+template <int BN, int BK, int MODE, int XN, bool RND, int OUT, bool ATM>
 cudaError_t launch_gemm_kernel(const GemmMaps &m, GemmArgs &g, int grid, cudaStream_t st)
 {
-    auto kfn = sparq_gemm_kernel<BN, BK, MODE, XN, RND, OUT>;
+    auto kfn = sparq_gemm_kernel<BN, BK, MODE, XN, RND, OUT, ATM>;
     static bool attr_set[64] = {};   // per device ordinal
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -1314,17 +1424,40 @@ cudaError_t launch_gemm_kernel(const GemmMaps &m, GemmArgs &g, int grid, cudaStr
     }
     const int staging = g.out_box ? epi_warps(MODE) * 2 * 32 * g.out_box : 0;
     g.stages = TileCfg<BN, BK>::stages(staging);
-    const int smem = 1024 + g.stages * TileCfg<BN, BK>::kStageBytes + staging;
-    return launch_overlapped(kfn, grid, gemm_threads(MODE), smem, st, m.a, m.b, m.out, m.res, g);
+    g.raw_stages = 0;
+    if (ATM) {       // what is left of the room goes to the raw ring
+        using Cfg = TileCfg<BN, BK>;
+        const int room = kMaxDynSmemGemm - 1024 - staging, n = room / Cfg::kStageBytes;
+        g.stages = n > kMaxStages ? kMaxStages : n;
+        const int left = (room - g.stages * Cfg::kBBytes) / Cfg::kABytes;
+        g.raw_stages = left > kMaxStages ? kMaxStages : left;
+    }
+    const int smem = 1024 + g.stages * TileCfg<BN, BK>::kStageBytes + (g.raw_stages > g.stages ? (g.raw_stages - g.stages) * TileCfg<BN, BK>::kABytes : 0) + staging;
+    return launch_overlapped(kfn, grid, gemm_threads(MODE, ATM), smem, st, m.a, m.b, m.out, m.res, g);
+}
+
+// Whether a fused launch of 256-wide tiles puts the transformed activations into tensor memory (ATM).  What a
+// step moves through shared memory falls from 1024 to 768 wavefronts, but the accumulator has to
+// do with one stage, and a launch starts and ends a little later: from a dozen steps a CTA.  us with / without:
+// 16384 x 512, K 4096 (64 steps) 42.1 / 46.7, 12544 x 512, K 1024 (16) 14.3 / 15.0, 28x28x512 -> 1024 stride 2 (12) 13.3 /
+// 13.7, 50176 x 256, K 512 (12) 13.04 / 12.97, 12544 x 256, K 1024 (8) 9.14 / 9.08, 6272 x 256, K 1024 (8) 8.4 / 8.05,
+// 50176 x 512, K 128 (6) 13.8 / 12.7.  On narrower tiles it gave nothing (50176 x 128, K 512, 11.3 / 10.9).
+inline bool a_in_tmem(const GemmArgs &g, int bn, int grid)
+{
+    const int64_t tiles = (g.M + kBM - 1) / kBM * ((g.N + bn - 1) / bn);
+    return g.k_blocks >= 4 && (tiles + grid - 1) / grid * g.k_blocks >= 12;
 }
 
 template <int BN, int BK, int MODE, int XN, bool RND>
 cudaError_t launch_gemm_variant(const GemmMaps &m, GemmArgs &g, int grid, cudaStream_t st)
 {
     const int out = make_epi_view(g).out;
-    if (out == kOutBytes) return launch_gemm_kernel<BN, BK, MODE, XN, RND, kOutBytes>(m, g, grid, st);
-    if (out == kOutResidual) return launch_gemm_kernel<BN, BK, MODE, XN, RND, kOutResidual>(m, g, grid, st);
-    return launch_gemm_kernel<BN, BK, MODE, XN, RND, kOutGeneral>(m, g, grid, st);
+    if constexpr (MODE != SPARQ_MODE_NONE && BK == 128 && BN == 256) {
+        if (out == kOutBytes && a_in_tmem(g, BN, grid)) return launch_gemm_kernel<BN, BK, MODE, XN, RND, kOutBytes, true>(m, g, grid, st);
+    }
+    if (out == kOutBytes) return launch_gemm_kernel<BN, BK, MODE, XN, RND, kOutBytes, false>(m, g, grid, st);
+    if (out == kOutResidual) return launch_gemm_kernel<BN, BK, MODE, XN, RND, kOutResidual, false>(m, g, grid, st);
+    return launch_gemm_kernel<BN, BK, MODE, XN, RND, kOutGeneral, false>(m, g, grid, st);
 }
 
 #define SPARQ_LAUNCH_VARIANT(MODE_, XN_, RND_) return launch_gemm_variant<BN, BK, MODE_, XN_, RND_>(m, g, grid, st)

@@ -85,6 +85,24 @@ def test_wide_tiles_straight_to_memory(mode, residual, n, tail):
     assert (got[m * n:] == 0xA5).all()
 
 
+@pytest.mark.parametrize("mode,n,mask", [(sparq.MODE_VSPARQ, 4, 0x1F), (sparq.MODE_VSPARQ, 4, 0x15), (sparq.MODE_BSPARQ, 3, 0x3F), (sparq.MODE_VSPARQ, 2, 0x55)])
+@pytest.mark.parametrize("m,cols,k", [(148 * 128 + 1, 160, 1040), (148 * 128 * 2 + 97, 256, 528), (148 * 128 - 31, 224, 1552)])
+def test_activations_in_tensor_memory(mode, n, mask, m, cols, k):
+    """256-wide tiles of long reductions: a last step that is mostly padding, more steps than either ring has
+    stages by an odd number, several tiles per CTA on one accumulator, a last tile of a few rows."""
+    A = synth.activations(k, (m, k), 0.5)
+    B = synth.weights(cols, (k, cols))
+    scale, bias, inv = synth.scales(cols, cols), synth.bias(cols, cols), synth.inv_out_scale(k)
+    out = torch.full((m * cols + 64,), 0xA5, dtype=torch.uint8, device="cuda")
+    sparq.sparq_gemm_s8(torch.from_numpy(A).cuda(), torch.from_numpy(np.ascontiguousarray(B.T)).cuda(), sparq.SparqParams(mode, n, mask, 1),
+                        scale=torch.from_numpy(scale).cuda(), bias=torch.from_numpy(bias).cuda(), relu=True, inv_out_scale=inv, u8_out=out)
+    sparq.sparq_check()
+    _, want = oracle.epilogue(oracle.gemm(A, B, mode, n, mask, 1), scale, bias, True, inv)
+    got = out.cpu().numpy()
+    assert np.array_equal(got[:m * cols].reshape(m, cols), want)
+    assert (got[m * cols:] == 0xA5).all()
+
+
 @pytest.mark.parametrize("mode,n", [(sparq.MODE_VSPARQ, 4), (sparq.MODE_BSPARQ, 3)])
 def test_transform_first_gemm(mode, n):
     """Long reductions with many column tiles run as transform + plain contraction: two streams at
