@@ -265,8 +265,6 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
             }
     };
     bool b_issued = false;
-    dep_wait();
-    dep_launch();
 
     if (warp == 0) {
         // ================= TMA producer =================
@@ -280,6 +278,9 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
                 const uint32_t use = ruse;
                 if (use > 0 && !mbar_wait(smem_u32(&bar_win_empty[b]), (use - 1) & 1, abort_flag, g.status, g.wait_limit)) break;
                 const int oh0 = (int)walk.tin * g.TR;
+                // the roles that touch the caller's memory wait for the kernel before (later waits return at once)
+                dep_wait();
+                dep_launch();
                 for (int j = 0; j < g.G; ++j) {
                     const uint32_t wfull = smem_u32(&bar_win_full[b * kMaxG + j]);
                     if (j < (int)walk.cnt) {
@@ -558,6 +559,7 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
         const int tr = slot / g.Wp;
         const int ow = slot - tr * g.Wp;
         const bool slot_ok = (tr < g.TR) && (ow < g.Wo);
+        dep_wait();
         for (; have && part < parts; have = walk.next()) {
             for (int j = 0; j < (int)walk.cnt; ++j, ++wt) {
                 if (wt % (uint32_t)teams != team) continue;

@@ -1057,9 +1057,6 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_slot;
-    dep_wait();
-    dep_launch();
-
     const int kb_count = g.k_blocks;
 
     if (warp == 0 || (kTwoProducers && warp == kWeightWarp)) {
@@ -1081,6 +1078,20 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                 const uint32_t mt = (n_tiles32 == 1) ? tile : tile / n_tiles32, nt = tile - mt * n_tiles32;
                 const int64_t m0 = (int64_t)mt * kBM;
                 const int n0 = (int)(nt * BN);
+                int base_n = 0, base_h = 0, base_w = 0;
+                if (g.conv) {
+                    const uint32_t hw = (uint32_t)(g.Ho * g.Wo), m032 = (uint32_t)m0;   // M of a convolution fits 31 bits
+                    base_n = (int)(m032 / hw);
+                    const int rem = (int)(m032 - (uint32_t)base_n * hw);
+                    base_h = (rem / g.Wo) * g.stride_h - g.pad_h;
+                    base_w = (rem % g.Wo) * g.stride_w - g.pad_w;
+                }
+                // The roles that touch the caller's memory wait for the kernel before, each behind what it can work
+                // out without it (later waits return at once); the others do not wait for it.  With one wait of all
+                // threads behind the set-up, its release was followed by every role's first index arithmetic
+                // and the fetch of its code: 0.2 to 0.6 us of each launch, the ResNet-50 pass 798 -> 763 us.
+                dep_wait();
+                dep_launch();
                 // the tile's stages in turn, until the CTA has given up
                 auto stages = [&](uint32_t bytes, auto copy) {
                     TapWalk tap(g, BK, 0);
@@ -1100,10 +1111,6 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                 if (kTwoProducers && warp == kWeightWarp) {
                     stages(Cfg::kBBytes, weights);
                 } else if (g.conv) {
-                    const uint32_t hw = (uint32_t)(g.Ho * g.Wo), m032 = (uint32_t)m0;   // M of a convolution fits 31 bits
-                    const int base_n = (int)(m032 / hw);
-                    const int rem = (int)(m032 - (uint32_t)base_n * hw);
-                    const int base_h = (rem / g.Wo) * g.stride_h - g.pad_h, base_w = (rem % g.Wo) * g.stride_w - g.pad_w;
                     // Channels past C arrive as zeros, so whatever the weight block holds
                     // there (the next tap's first bytes) adds nothing.
                     stages(kBytes, [&](uint32_t full, const TapWalk &tap) {
@@ -1182,6 +1189,7 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         for (int r = 0; r < 4; ++r) off[r] = (uint32_t)((lane >> 2) + 8 * r) * (uint32_t)g.N + 8u * (uint32_t)(lane & 3);
         int64_t staged_nt = -1;
         uint32_t local_tile = (uint32_t)team;
+        dep_wait();
         if (OUT != kOutGeneral && g.out_box) {
             // ---- through shared memory (see epi_staged_box) ----
             const int ew = warp - kFirstEpiWarp;

@@ -175,9 +175,8 @@ sparq_gemm_small_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
         __syncwarp();
         cluster_arrive();       // "barriers ready": waited for before the first remote store
     }
-    dep_wait();
-    dep_launch();
-
+    // Each role waits for the kernel before by itself, behind what it can work out without it (0.1 to 0.3 us of
+    // a launch without a transform: 49 x 512, K 2048, 4.1 -> 3.8 us).
     if (warp == 0) {
         // ================= TMA producer =================
         if (lane == 0) {
@@ -192,6 +191,8 @@ sparq_gemm_small_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
             int it = 0, s = 0;
             uint32_t ph = 1;       // phase parity of bar_empty to wait for (1: the ring's first round needs none)
             TapWalk tap(g, BK, kb_first);
+            dep_wait();
+            dep_launch();
             for (; it < steps; ++it) {
                 if (it >= S && !mbar_wait(smem_u32(&bar_empty[s]), ph, abort_flag, g.status, g.wait_limit)) break;
                 const uint32_t full = smem_u32(&bar_full[s]);
@@ -215,6 +216,7 @@ sparq_gemm_small_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
         // 0.1 us a stage to issue both, in front of the first MMA.
         if (elected) {
             TapWalk tap(g, BK, kb_first);
+            dep_wait();
             for (int it = 0; it < S && it < steps; ++it, tap.next())
                 tma_load_2d(b_stage(it), &map_b, smem_u32(&bar_full[it]), g.conv ? tap.k : (kb_first + it) * BK, n0);
         }
@@ -250,6 +252,7 @@ sparq_gemm_small_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
         const int first_row = wt / groups, row_step = kSmallWorkers * 32 / groups;
         const int cg = wt - first_row * groups, fcol = n0 + cg * 4;
         const bool fvec = (g.N & 3) == 0 && (reinterpret_cast<uintptr_t>(g.residual) & 3u) == 0;
+        dep_wait();
         if (ev.need_f) {
             if (SHARED) {
 #pragma unroll

@@ -95,9 +95,6 @@ sparq_gemm_sparse24_kernel(const __grid_constant__ CUtensorMap map_a, const __gr
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_slot;
-    dep_wait();
-    dep_launch();
-
     if (warp == 0) {
         // ================= TMA producer =================
         if (lane == 0) {
@@ -107,6 +104,9 @@ sparq_gemm_sparse24_kernel(const __grid_constant__ CUtensorMap map_a, const __gr
             for (uint32_t tile = blockIdx.x; tile < total_tiles && live; tile += gridDim.x) {
                 const uint32_t mt = n_tiles == 1 ? tile : tile / n_tiles;
                 const int n0 = (int)(tile - mt * n_tiles) * BN, m0 = (int)mt * kX24Rows;
+                // the roles that touch the caller's memory wait for the kernel before (later waits return at once)
+                dep_wait();
+                dep_launch();
                 for (int kb = 0; kb < steps && live; ++kb, ++use) {
                     const int s = (int)(use & 1u);
                     if (use >= 2 && !mbar_wait(smem_u32(&bar_raw_empty[s]), ((use >> 1) - 1u) & 1u, abort_flag, g.status, g.wait_limit)) { live = false; break; }
@@ -168,6 +168,7 @@ sparq_gemm_sparse24_kernel(const __grid_constant__ CUtensorMap map_a, const __gr
         const EpiView ev = make_epi_view(g);
         int64_t staged_nt = -1;
         uint32_t local_tile = 0;
+        dep_wait();
         for (uint32_t tile = blockIdx.x; tile < total_tiles; tile += gridDim.x, ++local_tile) {
             const uint32_t mt = n_tiles == 1 ? tile : tile / n_tiles;
             const int64_t nt = tile - mt * n_tiles;
