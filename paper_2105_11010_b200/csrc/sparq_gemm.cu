@@ -456,7 +456,7 @@ static double out_weight(const sparq_epilogue *e)
 static double small_us(const SmallForm &f, int64_t M, int64_t k_blocks, int bk, double xw)
 {
     const double rows = (double)(M < f.tile_rows ? M : f.tile_rows) / kBM * bk / 128.0;
-    return 2.5 + (double)((k_blocks + f.split - 1) / f.split) * (0.21 + (0.09 + 0.60 * xw) * rows) + (f.split > 1 ? 1.3 : 0.0);
+    return 1.9 + (double)((k_blocks + f.split - 1) / f.split) * (0.21 + (0.09 + 0.60 * xw) * rows) + (f.split > 1 ? 1.3 : 0.0);
 }
 static double im2col_us(int64_t M, int64_t N, int taps, int c, double xw, double ow, int sms)
 {
@@ -551,6 +551,11 @@ static bool plan_window(WindowPlan *q, int n, int h, int w, int c, int cout, int
         const int groups_per_cta = (int)((units + grid - 1) / grid + grp - 1) / grp + 1;
         while (win_bufs < kMaxWinBufs && win_bufs < groups_per_cta &&
                1024 + (win_bufs + 1) * plane_for(grp) * c_blocks + kb_count * b_block <= kMaxDynSmem) ++win_bufs;
+        // A tile per CTA at most: mostly the time of its weights, 3.35 us + 13 per MB (56x56x64 -> 64 3x3 3.8 us,
+        // 28x28x128 -> 128 5.3); the small form may share them out (one image of the latter 5.2 -> 4.6, of
+        // 20x20x96 -> 112 6.3 -> 4.3; 56x56x64 stays).
+        if (units <= sms && pick_small(M, cout, (int64_t)taps * ((c + 127) / 128), sms, xw > 0.0).tile_rows &&
+            im2col_path_us(M, cout, taps, c, xw, ow, sms) < 0.97 * (3.35 + 13.2e-6 * kb_count * b_block)) return false;
     } else {
         if (bn == 64) return false;                          // only the resident form is built for 64-wide tiles
         // 128-wide tiles: up to two row tiles of one (image, column tile) are accumulated together
