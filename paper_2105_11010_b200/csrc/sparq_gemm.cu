@@ -210,25 +210,27 @@ static int check_epilogue(const sparq_epilogue *e)
 
 // Cycles that one CTA spends on its reduction steps (128 bytes of K each) with 128 x bn tiles, the
 // estimate that tile width and form are chosen by.  A step takes the longest of
-//   transform of the A stage   1250 cycles when a SPARQ mode is on,
+//   transform of the A stage   1120 cycles when a SPARQ mode is on,
 //   MMA                        2 * bn cycles,
-//   operand fetch from L2      2.1 cycles per 128-byte row of A and B, 3.5 through an im2col map
+//   operand fetch from L2      1.9 cycles per 128-byte row of A and B, tiled or im2col
 // plus a hand-over, in ceil(tiles / SMs) passes; narrow tiles add CTAs but re-fetch and
-// re-transform A once per column tile.  (16384 x 4096 x 4096 at 128 x 256: 802 cycles a step
-// measured without a transform, 1473 with one; 7x7x512 -> 512 3x3: 917 and 1530.)
-static double tile_cycles(int64_t M, int64_t N, int64_t steps, int bn, int sms, bool transform, bool im2col)
+// re-transform A once per column tile.  wide: bytes of a step / 128.  (16384 x 512 x 4096 at 128 x 256: 680 cycles a step measured without
+// a transform, 1150 with one; 7x7x512 -> 512 3x3 at 128 x 128: 500 and 1120.  With the figures of a
+// slower transform and a fetch of 3.5 cycles through im2col maps, 3x56x56x448 -> 296 3x3 took 28.0 us, now 25.0, and
+// 117x28x28x64 -> 288, trimmed, 42.3, now 36.0; over 60 drawn layers one lost, 1.6 %.)
+static double tile_cycles(int64_t M, int64_t N, int64_t steps, int bn, int sms, bool transform, double wide)
 {
     const int64_t tiles = ((M + kBM - 1) / kBM) * ((N + bn - 1) / bn);
     const int64_t rounds = (tiles + sms - 1) / sms;
     double step = 2.0 * bn;
-    const double fetch = (im2col ? 3.5 : 2.1) * (kBM + bn);
+    const double fetch = 1.9 * (kBM + bn);
     if (fetch > step) step = fetch;
-    if (transform && step < 1250.0) step = 1250.0;
-    return (double)rounds * (double)steps * (step + 150.0) + 3.0 * bn;     // + the last tile's epilogue
+    if (transform && step < 1120.0) step = 1120.0;
+    return (double)rounds * (double)steps * (step * wide + 150.0) + 3.0 * bn;     // + the last tile's epilogue
 }
 
 // The tile width with the lowest estimate.
-static int pick_bn(int64_t M, int64_t N, int64_t steps, int sms, bool transform, bool im2col, double *cycles = nullptr)
+static int pick_bn(int64_t M, int64_t N, int64_t steps, int sms, bool transform, double *cycles = nullptr, double wide = 1.0)
 {
     const int cand[3] = {256, 128, 64};
     int best = 64;
@@ -236,7 +238,7 @@ static int pick_bn(int64_t M, int64_t N, int64_t steps, int sms, bool transform,
     for (int i = 0; i < 3; ++i) {
         const int bn = cand[i];
         if (bn > 64 && N <= bn / 2) continue;          // would be mostly padding
-        const double cost = tile_cycles(M, N, steps, bn, sms, transform, im2col);
+        const double cost = tile_cycles(M, N, steps, bn, sms, transform, wide);
         if (best_cost == 0.0 || cost < best_cost) {
             best_cost = cost;
             best = bn;
@@ -280,15 +282,22 @@ static SmallForm pick_small(int64_t M, int64_t N, int64_t k_blocks, int sms, boo
 // taps -- because the in-kernel transform is what such a step takes.  The extra pass costs about
 // 2.5 us and 2 bytes of traffic per activation (2.9 TB/s of activations).  A margin of 7 % keeps the
 // fused form, which needs no memory, where the two are close.
-static bool transform_first(int64_t M, int64_t N, int64_t steps, size_t act_bytes, int sms, bool im2col)
+static bool transform_first(int64_t M, int64_t N, int64_t steps, size_t act_bytes, int sms, double wide = 1.0)
 {
     if (pick_small(M, N, steps, sms, true).tile_rows) return false;
     if ((M + kBM - 1) / kBM * ((N + 63) / 64) >= (int64_t)1 << 31) return false;      // near the refused sizes: refused, if at all, with nothing enqueued
     double fused, plain;
-    pick_bn(M, N, steps, sms, true, im2col, &fused);
-    pick_bn(M, N, steps, sms, false, im2col, &plain);
+    pick_bn(M, N, steps, sms, true, &fused, wide);
+    pick_bn(M, N, steps, sms, false, &plain, wide);
     const double clk = 1900.0;      // cycles per us
     return plain + clk * (2.5 + (double)act_bytes / 2.9e6) < 0.93 * fused;
+}
+
+// The same for a convolution through an im2col map, in steps of its channel blocks.
+static bool transform_first_conv(int64_t M, int cout, int taps, int c, size_t act_bytes, int sms)
+{
+    const int bk = c % 128 == 0 ? 128 : 64;
+    return transform_first(M, cout, (int64_t)taps * ((c + bk - 1) / bk), act_bytes, sms, bk / 128.0);
 }
 
 // Variant argument of the launchers (XN of xform_fused): 4 = n = 4 with all five placements, 5 = n = 4
@@ -376,7 +385,7 @@ static int gemm_impl(const uint8_t *A, int64_t lda, const int8_t *B, int64_t ldb
     if (rc != SPARQ_OK) return rc;
     int sms = 0;
     if (x.mode != SPARQ_MODE_NONE && lda == K && (rc = device_info(&sms)) == SPARQ_OK &&
-        transform_first(M, N, (K + 127) / 128, (size_t)M * (size_t)K, sms, false)) {
+        transform_first(M, N, (K + 127) / 128, (size_t)M * (size_t)K, sms)) {
         if (uint8_t *ta = (uint8_t *)workspace_alloc((size_t)M * (size_t)K, st)) {
             rc = quantize_rows(A, ta, (size_t)M, (size_t)K, x, true, st);
             if (rc == SPARQ_OK) rc = gemm_with_status(ta, K, B, ldb, M, N, K, plain_a8w8(), e, status, st);
@@ -461,7 +470,7 @@ static double small_us(const SmallForm &f, int64_t M, int64_t k_blocks, int bk, 
 static double im2col_us(int64_t M, int64_t N, int taps, int c, double xw, double ow, int sms)
 {
     const int bk = c % 128 == 0 ? 128 : 64;
-    const int bn = pick_bn(M, N, (int64_t)taps * ((c + 127) / 128), sms, xw > 0.0, true);
+    const int bn = pick_bn(M, N, (int64_t)taps * ((c + 127) / 128), sms, xw > 0.0);
     const double rounds = (double)(((M + kBM - 1) / kBM * ((N + bn - 1) / bn) + sms - 1) / sms), blocks = rounds * taps * ((c + bk - 1) / bk);
     return 2.6 + blocks * bk / 128.0 * ((bn == 64 ? 0.05 : bn == 128 ? 0.10 : 0.13) + (bn == 256 ? 0.46 : 0.48) * xw) + 0.22 * blocks +
            0.47 * rounds * bn / 128.0 * ow;
@@ -688,7 +697,7 @@ int gemm_with_status(const uint8_t *A, int64_t lda, const int8_t *B, int64_t ldb
     // step is a hand-off between three warp roles, which is what a small launch is made of)
     const int bk = (pad64 < pad128 && !(pad64 >= 320 && pad128 * 8 <= pad64 * 9)) ? 64 : 128;
     const SmallForm small = pick_small(M, N, (K + bk - 1) / bk, sms, x.mode != SPARQ_MODE_NONE);
-    const int bn = small.tile_rows ? kSmallBN : pick_bn(M, N, (K + 127) / 128, sms, x.mode != SPARQ_MODE_NONE, false);
+    const int bn = small.tile_rows ? kSmallBN : pick_bn(M, N, (K + 127) / 128, sms, x.mode != SPARQ_MODE_NONE);
     const int tile_rows = small.tile_rows ? small.tile_rows : kBM;
     GemmMaps m = {};
     rc = encode_2d(&m.a, A, K, M, lda, bk, tile_rows);
@@ -719,7 +728,7 @@ static int im2col_conv(const uint8_t *x_in, int n, int h, int w, int c, const in
     const int64_t M = (int64_t)n * ho * wo, K = (int64_t)r * s * c;
     const int bk = (c % 128 == 0) ? 128 : 64;
     const SmallForm small = pick_small(M, cout, (int64_t)r * s * ((c + bk - 1) / bk), sms, x.mode != SPARQ_MODE_NONE);
-    const int bn = small.tile_rows ? kSmallBN : pick_bn(M, cout, (int64_t)r * s * ((c + 127) / 128), sms, x.mode != SPARQ_MODE_NONE, true);
+    const int bn = small.tile_rows ? kSmallBN : pick_bn(M, cout, (int64_t)r * s * ((c + 127) / 128), sms, x.mode != SPARQ_MODE_NONE);
     int rc;
     const int tile_rows = small.tile_rows ? small.tile_rows : kBM;
     GemmMaps m = {};
@@ -768,7 +777,7 @@ int gemm_sparse24_fused(const uint8_t *A, const int8_t *w_exp, int64_t M, int64_
     const int bn = N <= 64 ? 64 : 128;
     const int64_t tiles = (M + 255) / 256 * ((N + bn - 1) / bn);
     double plain;
-    pick_bn(M, N, steps3, sms, false, false, &plain);
+    pick_bn(M, N, steps3, sms, false, &plain);
     const double fused = (double)((tiles + sms - 1) / sms) * (double)steps * 4200.0;
     if (tiles >= (int64_t)1 << 31 || fused > plain + 1900.0 * (2.5 + (double)M * (double)K * 4.0 / 6.0e6)) return 0;
     CUtensorMap ma, mb;
@@ -864,9 +873,8 @@ extern "C" int sparq_conv2d_nhwc_s8(const uint8_t *x_in, int n, int h, int w, in
         rc = try_window_conv(x_in, n, h, w, c, wgt, cout, r, s, pad_h, pad_w, ho, wo, x, e, sms, status, st);
         if (rc != 0) return rc < 0 ? rc : SPARQ_OK;
     }
-    const int64_t steps = (int64_t)r * s * ((c + 127) / 128);
     const size_t act_bytes = (size_t)n * h * w * (size_t)c;
-    if (x.mode != SPARQ_MODE_NONE && transform_first(M, cout, steps, act_bytes, sms, true)) {
+    if (x.mode != SPARQ_MODE_NONE && transform_first_conv(M, cout, r * s, c, act_bytes, sms)) {
         if (uint8_t *tx = (uint8_t *)workspace_alloc(act_bytes, st)) {
             rc = quantize_rows(x_in, tx, (size_t)n * h * w, (size_t)c, x, true, st);
             if (rc == SPARQ_OK) rc = im2col_conv(tx, n, h, w, c, wgt, cout, r, s, stride_h, stride_w, pad_h, pad_w, ho, wo, plain_a8w8(), e, sms, status, st);
@@ -895,6 +903,7 @@ extern "C" int sparq_selftest_form(int n, int h, int w, int c, int cout, int r, 
         return q.resident ? SPARQ_FORM_WINDOW_RESIDENT : SPARQ_FORM_WINDOW_STREAMED;
     const int64_t steps = (int64_t)r * s * ((c + 127) / 128);
     const size_t act_bytes = (size_t)n * h * w * (size_t)c;
-    if (x.mode != SPARQ_MODE_NONE && transform_first(M, cout, steps, act_bytes, sms, !matrix) && scratch(act_bytes)) return SPARQ_FORM_TRANSFORM_FIRST;
+    if (x.mode != SPARQ_MODE_NONE && (matrix ? transform_first(M, cout, steps, act_bytes, sms) : transform_first_conv(M, cout, r * s, c, act_bytes, sms)) &&
+        scratch(act_bytes)) return SPARQ_FORM_TRANSFORM_FIRST;
     return pick_small(M, cout, steps, sms, x.mode != SPARQ_MODE_NONE).tile_rows ? SPARQ_FORM_SMALL : SPARQ_FORM_FULL;
 }
