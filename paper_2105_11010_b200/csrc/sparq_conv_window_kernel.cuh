@@ -587,7 +587,8 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
         // Vectors in flight per thread.  Two keep the loop shorter (instruction cache), four hide more of
         // the shared-memory latency behind the tensor core's operand fetches, which are denser on
         // 128-wide tiles: 32x56x56x64 -> 64 3x3 9.25 us with two, 9.4 with one, 9.6 with four;
-        // 128x28x28x128 -> 128 3x3 18.2, (three) 16.25, 15.95.
+        // 128x28x28x128 -> 128 3x3 18.2, (three) 16.25, 15.95.  (With the half-precision transform 8.6, 8.6, 8.75 and
+        // 15.1, 15.05, 15.05.)
         constexpr int kBatch = BN == 64 ? 2 : 4;
         const XformDev xf = g.xf;
         // Trimming pairs at n = 4 takes 12 packed-integer instructions and 14 in half precision; here, where the

@@ -11,13 +11,14 @@
 //   6..21    expansion: a thread owns one row and four of its eight 16-byte pieces; each piece (four
 //            groups) becomes 48 bytes, so a raw stage becomes exactly three expanded ones (threads of
 //            the first half fill stage 0 and the first half of stage 1, the others the rest)
-// The expansion is what bounds it: per four activations one bSPARQ transform (15 integer
+// The expansion is what bounds it: per four activations one bSPARQ transform (11
 // instructions at n = 4) and, for each of three output words, a permuted copy of the transformed and
-// of the raw bytes, a permuted mask of "partner is non-zero" and a select -- about 30 instructions
+// of the raw bytes, a permuted mask of "partner is non-zero" and a select -- 26 instructions
 // where transforming each of the six pairs took 57 -- and 256-row tiles halve the weight traffic
 // out of L2, which would bound it otherwise.  The two-kernel form moved 3 bytes per activation
-// to HBM and back.  M 100352, K 1152: N 128 164 -> 67 us, N 64 161 -> 66, N 256 176 -> 127;
-// N 128 with 3opt 219 -> 83, 6opt 253 -> 77.
+// to HBM and back.  M 100352, K 1152: N 128 164 -> 62 us, N 64 161 -> 60, N 256 176 -> 114;
+// N 128 with 3opt 219 -> 71, 6opt 253 -> 69.  (Expanded into tensor memory instead of shared memory: N 128 62, N 256
+// 117, K 512 N 512 107 in place of 99.)
 #pragma once
 
 #include "sparq_gemm_kernel.cuh"
