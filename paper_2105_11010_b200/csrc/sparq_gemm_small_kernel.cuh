@@ -270,27 +270,41 @@ sparq_gemm_small_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
         if (MODE != SPARQ_MODE_NONE) {
             const XformDev xf = g.xf;
             constexpr int kThreads = kSmallWorkers * 32, kPer = kBM * BK / 16 / kThreads;
+            // Vectors that a thread works on at a time.  A launch starts with cold instruction caches, and the
+            // transforms of 3- and 2-bit windows unrolled four times over are more code than the latency they hide is
+            // worth (6opt: 256 x 64 x 576 6.95 -> 6.25 us, 7x7x512 -> 512 3x3, one image, 7.2 -> 6.4, 100 x 1000 x 4096 10.3 ->
+            // 9.7); the shorter ones at n = 4 are better unrolled where the reduction is long (100 x 1000 x 4096 7.8 us, in
+            // twos 8.3; 3opt 9.9 and 10.2).
+            constexpr int kBatch = XN == 4 || XN == 5 ? kPer : 2;
             const int nvec = rows_left * (BK / 16);       // rows past M are padding: nothing to transform
             int s = 0;
             uint32_t ph = 0;
             for (int it = 0; it < steps; ++it) {
                 mbar_wait(smem_u32(&bar_full[s]), ph, abort_flag, g.status, g.wait_limit);
                 const uint32_t base = a_stage(s) + (uint32_t)wt * 16u;
-                uint4 v[kPer];
+                auto batch = [&](int j0) {
+                    uint4 v[kBatch];
 #pragma unroll
-                for (int j = 0; j < kPer; ++j)
-                    if (wt + j * kThreads < nvec)
-                        asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];"
-                                     : "=r"(v[j].x), "=r"(v[j].y), "=r"(v[j].z), "=r"(v[j].w) : "r"(base + (uint32_t)(j * kThreads * 16)));
+                    for (int j = 0; j < kBatch; ++j)
+                        if (wt + (j0 + j) * kThreads < nvec)
+                            asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v[j].x), "=r"(v[j].y), "=r"(v[j].z), "=r"(v[j].w)
+                                         : "r"(base + (uint32_t)((j0 + j) * kThreads * 16)));
 #pragma unroll
-                for (int j = 0; j < kPer; ++j) {
-                    if (wt + j * kThreads >= nvec) continue;
-                    v[j].x = xform_fused<MODE, XN, RND>(v[j].x, xf);
-                    v[j].y = xform_fused<MODE, XN, RND>(v[j].y, xf);
-                    v[j].z = xform_fused<MODE, XN, RND>(v[j].z, xf);
-                    v[j].w = xform_fused<MODE, XN, RND>(v[j].w, xf);
-                    asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};"
-                                 :: "r"(base + (uint32_t)(j * kThreads * 16)), "r"(v[j].x), "r"(v[j].y), "r"(v[j].z), "r"(v[j].w) : "memory");
+                    for (int j = 0; j < kBatch; ++j) {
+                        if (wt + (j0 + j) * kThreads >= nvec) continue;
+                        v[j].x = xform_fused<MODE, XN, RND>(v[j].x, xf);
+                        v[j].y = xform_fused<MODE, XN, RND>(v[j].y, xf);
+                        v[j].z = xform_fused<MODE, XN, RND>(v[j].z, xf);
+                        v[j].w = xform_fused<MODE, XN, RND>(v[j].w, xf);
+                        asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};"
+                                     :: "r"(base + (uint32_t)((j0 + j) * kThreads * 16)), "r"(v[j].x), "r"(v[j].y), "r"(v[j].z), "r"(v[j].w) : "memory");
+                    }
+                };
+                if constexpr (kBatch == kPer) {
+                    batch(0);
+                } else {
+#pragma unroll 1
+                    for (int j0 = 0; wt + j0 * kThreads < nvec; j0 += kBatch) batch(j0);
                 }
                 fence_proxy_async_smem();
                 __syncwarp();
