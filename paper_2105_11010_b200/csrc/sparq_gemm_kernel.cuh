@@ -989,8 +989,17 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     static_assert(!ATM || (MODE != SPARQ_MODE_NONE && BK == 128 && BN == 256), "A in tensor memory: transformed steps of 128 bytes");
     const int S = g.stages;
     extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) uint64_t bar_full[kMaxStages], bar_xf[kMaxStages], bar_empty[kMaxStages];
-    __shared__ __align__(8) uint64_t bar_raw[ATM ? kMaxStages : 1], bar_raw_empty[ATM ? kMaxStages : 1];
+    // The ring that the transform teams read has two sets of full barriers, for even and odd rounds.  A parity
+    // answers for every second phase, so a team may ask a barrier for a phase only once it knows that the one before
+    // has completed.  Of a single set, in a ring of an odd number of stages -- three beside the boxes of staged
+    // 256-wide tiles, seven of 64-wide ones, five raw ones with ATM -- that phase was the other team's, which
+    // nothing orders before the question; a barrier of two sets comes round after twice the stages, with the team
+    // that asked it before.  (Reading the stage's empty barrier first is as safe, but one more round trip per
+    // step: 200704 x 64, K 256, 16.85 -> 17.05 us, 12544 x 256, K 1024, 8.75 -> 9.05.  Two sets with the counters in
+    // every lane: 17.25 and 9.0; in the warp: 16.1 and 8.85.)
+    constexpr int kFullSets = MODE != SPARQ_MODE_NONE && !ATM ? 2 : 1, kRawSets = ATM ? 2 : 1;
+    __shared__ __align__(8) uint64_t bar_full[kFullSets * kMaxStages], bar_xf[kMaxStages], bar_empty[kMaxStages];
+    __shared__ __align__(8) uint64_t bar_raw[ATM ? kRawSets * kMaxStages : 1], bar_raw_empty[ATM ? kMaxStages : 1];
     __shared__ __align__(8) uint64_t bar_res[epi_warps(MODE)][2];       // residual boxes landed
     // tensor memory: accumulators, and with ATM four to eight stages of transformed activations
     constexpr int kAcc = ATM ? 256 / BN : Cfg::kAcc;
@@ -1007,7 +1016,8 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     __shared__ uint32_t abort_word;
     __shared__ __align__(16) float s_scale[kMaxTeams][BN], s_bias[kMaxTeams][BN];
 
-    const int warp = threadIdx.x >> 5;
+    // the same in all lanes, and so for the compiler: what a role keeps of its ring costs the lanes' integer pipe nothing
+    const int warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0);
     const int lane = threadIdx.x & 31;
     volatile uint32_t *abort_flag = &abort_word;
 
@@ -1029,15 +1039,13 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     if (threadIdx.x == 0) {
         prefetch_tensormap(&map_a);
         prefetch_tensormap(&map_b);
+        for (int q = 0; q < kFullSets * S; ++q) mbar_init(smem_u32(&bar_full[q]), MODE == SPARQ_MODE_NONE ? 2 : 1);
         for (int s = 0; s < S; ++s) {
-            mbar_init(smem_u32(&bar_full[s]), MODE == SPARQ_MODE_NONE ? 2 : 1);
             mbar_init(smem_u32(&bar_xf[s]), kXfTeamWarps);
             mbar_init(smem_u32(&bar_empty[s]), 1);
         }
-        for (int s = 0; ATM && s < SA; ++s) {
-            mbar_init(smem_u32(&bar_raw[s]), 1);
-            mbar_init(smem_u32(&bar_raw_empty[s]), kXfTeamWarps);
-        }
+        for (int q = 0; ATM && q < kRawSets * SA; ++q) mbar_init(smem_u32(&bar_raw[q]), 1);
+        for (int s = 0; ATM && s < SA; ++s) mbar_init(smem_u32(&bar_raw_empty[s]), kXfTeamWarps);
         for (int a = 0; a < kAcc; ++a) {
             mbar_init(smem_u32(&bar_acc_full[a]), 1);
             mbar_init(smem_u32(&bar_acc_empty[a]), 4 * epi_parts(kGroups, teams, BN));
@@ -1070,6 +1078,8 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
             const bool raw = ATM && warp == 0;
             const int ring = raw ? SA : S;
             const uint32_t bars_full = smem_u32(raw ? bar_raw : bar_full), bars_empty = smem_u32(raw ? bar_raw_empty : bar_empty);
+            const int sets = raw ? kRawSets : kFullSets;
+            const uint32_t set = sets == 2 ? 8u * (uint32_t)ring : 0u;       // bytes from one set of full barriers to the other
             uint32_t it = 0;   // running stage counter across tiles
             int s = 0;         // stage it % ring
             uint32_t use = 0;  // it / ring
@@ -1097,7 +1107,7 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                     TapWalk tap(g, BK, 0);
                     for (int kb = 0; kb < kb_count; ++kb, ++it) {
                         if (use > 0 && !mbar_wait(bars_empty + 8u * (uint32_t)s, (use - 1) & 1, abort_flag, g.status, g.wait_limit)) { live = false; break; }
-                        const uint32_t full = bars_full + 8u * (uint32_t)s;
+                        const uint32_t full = bars_full + 8u * (uint32_t)s + (use & 1u) * set;
                         mbar_expect_tx(full, bytes);
                         copy(full, tap);
                         tap.next();
@@ -1128,8 +1138,9 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
             // flight, so that none lands after the CTA has exited.
             if (*abort_flag) {
                 const uint32_t first = it > (uint32_t)ring ? it - ring : 0;
+                const uint32_t bars = (uint32_t)(sets * ring);
                 for (uint32_t j = first; j < it; ++j)
-                    mbar_wait(bars_full + 8u * (j % ring), (j / ring) & 1, abort_flag, g.status, g.wait_limit, true);
+                    mbar_wait(bars_full + 8u * (j % bars), j / bars & 1u, abort_flag, g.status, g.wait_limit, true);
             }
         }
         __syncwarp();
@@ -1341,11 +1352,12 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
             };
             uint4 va[4], vb[4];
             int sa = team, s = team;
-            uint32_t pa = 0, use = 0;          // phase of the raw stage; uses of the transformed one before
+            int qa = team;                     // full barrier of the raw stage,
+            uint32_t pa = 0, use = 0;          // its phase; uses of the transformed one before
             bool loaded = false;
             for (uint32_t it = (uint32_t)team; it < total; it += kXfTeams) {
                 if (!loaded) {
-                    mbar_wait(smem_u32(&bar_raw[sa]), pa, abort_flag, g.status, g.wait_limit);
+                    mbar_wait(smem_u32(&bar_raw[qa]), pa, abort_flag, g.status, g.wait_limit);
                     load_row(va, sa, 0);
                 }
                 load_row(vb, sa, 4);
@@ -1355,9 +1367,10 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                 const uint32_t dst = tmem_base + ((uint32_t)(quarter * 32) << 16) + 256u + (uint32_t)s * 32u;
                 tmem_st_32x16(dst, va);
                 int na = sa + kXfTeams;
-                uint32_t npa = pa;
-                if (na >= SA) { na -= SA; npa ^= 1u; }
-                loaded = it + kXfTeams < total && __all_sync(0xFFFFFFFFu, mbar_test(smem_u32(&bar_raw[na]), npa));
+                if (na >= SA) na -= SA;
+                qa += kXfTeams;
+                if (qa >= kRawSets * SA) { qa -= kRawSets * SA; pa ^= 1u; }
+                loaded = it + kXfTeams < total && __all_sync(0xFFFFFFFFu, mbar_test(smem_u32(&bar_raw[qa]), pa));
                 if (loaded) load_row(va, na, 0);
                 work_row(vb);
                 __syncwarp();
@@ -1368,33 +1381,33 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&bar_xf[s]));
                 sa = na;
-                pa = npa;
                 s += kXfTeams;
                 if (s >= S) { s -= S; ++use; }
             }
         } else {
         uint4 va[kHalf], vb[kHalf];
         int s = team;
-        uint32_t ph = 0;
+        int q = team;              // its full barrier,
+        uint32_t ph = 0;           // and that barrier's phase
         bool loaded = false;
         for (uint32_t it = (uint32_t)team; it < total; it += kXfTeams) {
             if (!loaded) {
-                mbar_wait(smem_u32(&bar_full[s]), ph, abort_flag, g.status, g.wait_limit);
+                mbar_wait(smem_u32(&bar_full[q]), ph, abort_flag, g.status, g.wait_limit);
                 load(va, s, 0);
             }
             load(vb, s, kHalf);
             work(va, s, 0);
             int ns = s + kXfTeams;
-            uint32_t nph = ph;
-            if (ns >= S) { ns -= S; nph ^= 1u; }
-            loaded = it + kXfTeams < total && __all_sync(0xFFFFFFFFu, mbar_test(smem_u32(&bar_full[ns]), nph));
+            if (ns >= S) ns -= S;
+            q += kXfTeams;
+            if (q >= kFullSets * S) { q -= kFullSets * S; ph ^= 1u; }
+            loaded = it + kXfTeams < total && __all_sync(0xFFFFFFFFu, mbar_test(smem_u32(&bar_full[q]), ph));
             if (loaded) load(va, ns, 0);
             work(vb, s, kHalf);
             fence_proxy_async_smem();       // generic-proxy writes visible to the tensor core
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&bar_xf[s]));
             s = ns;
-            ph = nph;
         }
         }
     }
