@@ -278,7 +278,8 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
                 const uint32_t use = ruse;
                 if (use > 0 && !mbar_wait(smem_u32(&bar_win_empty[b]), (use - 1) & 1, abort_flag, g.status, g.wait_limit)) break;
                 const int oh0 = (int)walk.tin * g.TR;
-                // the roles that touch the caller's memory wait for the kernel before (later waits return at once)
+                // the roles that touch the caller's memory wait for the kernel before (later waits return at once), the
+                // others do not (EARLY waits)
                 dep_wait();
                 dep_launch();
                 for (int j = 0; j < g.G; ++j) {
@@ -361,7 +362,7 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
             const uint32_t row16 = (uint32_t)(g.Wp * CB) >> 4;
             const uint32_t plane16 = (uint32_t)g.plane_bytes >> 4;
             const uint32_t tile16 = (uint32_t)(g.TR * g.Wp * CB) >> 4;
-            if (B_RESIDENT) mbar_wait(smem_u32(&bar_b_full[0]), 0, abort_flag, g.status, g.wait_limit);
+            if (B_RESIDENT) mbar_wait<true>(smem_u32(&bar_b_full[0]), 0, abort_flag, g.status, g.wait_limit);
             bool weights_there = !by_row;      // else waited for row by row, during this issuer's first tile
             for (; have; have = walk.next()) {
                 const int b = rb;
@@ -390,9 +391,9 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
                         // transform the copies land in any order
                         if (MODE == SPARQ_MODE_NONE) {
                             for (int j = 0; j < cnt; ++j)
-                                mbar_wait(smem_u32(&bar_win_full[b * kMaxG + j]), wph, abort_flag, g.status, g.wait_limit);
+                                mbar_wait<true>(smem_u32(&bar_win_full[b * kMaxG + j]), wph, abort_flag, g.status, g.wait_limit);
                         } else {
-                            mbar_wait(smem_u32(&bar_win_xf[b * kMaxG + cnt - 1]), wph, abort_flag, g.status, g.wait_limit);
+                            mbar_wait<true>(smem_u32(&bar_win_xf[b * kMaxG + cnt - 1]), wph, abort_flag, g.status, g.wait_limit);
                         }
                         tc_fence_after();
                         uint64_t a_cb = a_grp;
@@ -443,8 +444,8 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
                     // of the group, j-2, waited for the two before).
                     const uint32_t ops_bar = smem_u32(MODE == SPARQ_MODE_NONE ? &bar_win_full[b * kMaxG + j] : &bar_win_xf[b * kMaxG + j]);
                     if (!pre_ops) {
-                        if (MODE == SPARQ_MODE_NONE && j > 0) mbar_wait(ops_bar - 8u, wph, abort_flag, g.status, g.wait_limit);
-                        mbar_wait(ops_bar, wph, abort_flag, g.status, g.wait_limit);
+                        if (MODE == SPARQ_MODE_NONE && j > 0) mbar_wait<!B_RESIDENT>(ops_bar - 8u, wph, abort_flag, g.status, g.wait_limit);
+                        mbar_wait<!B_RESIDENT>(ops_bar, wph, abort_flag, g.status, g.wait_limit);
                     }
                     tc_fence_after();
                     pre_acc = pre_ops = 0;
@@ -520,14 +521,14 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
                 // last), so that none of them can still be waiting on a phase when the producer
                 // starts the next.
                 if (MODE != SPARQ_MODE_NONE && (int)walk.cnt < g.G)
-                    mbar_wait(smem_u32(&bar_win_xf[b * kMaxG + g.G - 1]), wph, abort_flag, g.status, g.wait_limit);
+                    mbar_wait<!B_RESIDENT>(smem_u32(&bar_win_xf[b * kMaxG + g.G - 1]), wph, abort_flag, g.status, g.wait_limit);
                 if (issued) {
                     tc_commit_if(smem_u32(&bar_win_empty[b]), elected);
                 } else {
                     // No tile of this group was this issuer's.  It arrives only once the producer has
                     // started this use of the buffer (its first piece has landed), i.e. after the
                     // previous use's phase of the barrier has completed.
-                    mbar_wait(smem_u32(&bar_win_full[b * kMaxG]), wph, abort_flag, g.status, g.wait_limit);
+                    mbar_wait<!B_RESIDENT>(smem_u32(&bar_win_full[b * kMaxG]), wph, abort_flag, g.status, g.wait_limit);
                     if (elected) mbar_arrive(smem_u32(&bar_win_empty[b]));
                 }
                 ++gi;
@@ -603,7 +604,7 @@ sparq_conv_window_kernel(const __grid_constant__ CUtensorMap map_x0, const __gri
             const int b = rb;
             const uint32_t wph = ruse & 1u;
             for (int j = 0; j < g.G; ++j) {
-                mbar_wait(smem_u32(&bar_win_full[b * kMaxG + j]), wph, abort_flag, g.status, g.wait_limit);
+                mbar_wait<true>(smem_u32(&bar_win_full[b * kMaxG + j]), wph, abort_flag, g.status, g.wait_limit);
                 if (j < (int)walk.cnt) {
                     const uint32_t nvec = piece_len(j) >> 4;
                     uint32_t pbase = win_buf(b) + piece_off(j);

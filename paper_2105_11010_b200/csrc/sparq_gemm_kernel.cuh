@@ -165,17 +165,31 @@ __device__ __forceinline__ uint32_t mbar_test3(uint32_t bar0, uint32_t parity0, 
 
 // Bounded wait.  Returns false (after flagging) if the phase did not complete in time or
 // if another thread of the CTA already gave up.
+//
+// EARLY: for a role that touches on-chip memory only and so does not wait for the kernel before, on the barriers of the
+// operands that it starts with.  That kernel may release this one early and then take long, which must not count
+// against the limit: the first expiry waits for it (at once if it has finished) and starts the clock again.
+// (Every role waiting for it in front of its first barrier instead: 32x56x56x64 -> 64 3x3 8.44 -> 8.63 us, the
+// ResNet-50 pass at batch 64 744 -> 755; every wait EARLY: 256 x 64 x 576 5.42 -> 5.54.)
+template <bool EARLY = false>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile uint32_t *abort_flag,
                                           unsigned int *status, long long limit_cycles, bool ignore_abort = false)
 {
     if (mbar_try_wait(bar, parity)) return true;
     if (!ignore_abort && *abort_flag) return false;
-    const long long t0 = clock64();
+    long long t0 = clock64();
+    bool alone = !EARLY;            // the kernel before has finished
     for (uint32_t it = 1;; ++it) {
         if (mbar_try_wait(bar, parity)) return true;
         if ((it & 0x3Fu) == 0) {
             if (!ignore_abort && *abort_flag) return false;
             if (clock64() - t0 > limit_cycles) {
+                if (!alone) {
+                    dep_wait();
+                    alone = true;
+                    t0 = clock64();
+                    continue;
+                }
                 *abort_flag = 1u;
                 atomicOr(status, 1u);
                 return false;
@@ -1097,7 +1111,7 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                     base_w = (rem % g.Wo) * g.stride_w - g.pad_w;
                 }
                 // The roles that touch the caller's memory wait for the kernel before, each behind what it can work
-                // out without it (later waits return at once); the others do not wait for it.  With one wait of all
+                // out without it (later waits return at once); the others do not (EARLY waits).  With one wait of all
                 // threads behind the set-up, its release was followed by every role's first index arithmetic
                 // and the fetch of its code: 0.2 to 0.6 us of each launch, the ResNet-50 pass 798 -> 763 us.
                 dep_wait();
@@ -1164,8 +1178,8 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
                 for (int kb = 0; kb < kb_count; ++kb) {
-                    if (MODE == SPARQ_MODE_NONE) mbar_wait(smem_u32(&bar_full[s]), ph, abort_flag, g.status, g.wait_limit);
-                    else mbar_wait(smem_u32(&bar_xf[s]), ph, abort_flag, g.status, g.wait_limit);
+                    if (MODE == SPARQ_MODE_NONE) mbar_wait<true>(smem_u32(&bar_full[s]), ph, abort_flag, g.status, g.wait_limit);
+                    else mbar_wait<true>(smem_u32(&bar_xf[s]), ph, abort_flag, g.status, g.wait_limit);
                     if (ATM) mbar_wait(smem_u32(&bar_full[s]), ph, abort_flag, g.status, g.wait_limit);
                     tc_fence_after();
                     const uint64_t adesc = adesc0 + (uint64_t)((uint32_t)s * (kAStep >> 4)), bdesc = bdesc0 + (uint64_t)((uint32_t)s * (kBStep >> 4));
@@ -1357,7 +1371,7 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
             bool loaded = false;
             for (uint32_t it = (uint32_t)team; it < total; it += kXfTeams) {
                 if (!loaded) {
-                    mbar_wait(smem_u32(&bar_raw[qa]), pa, abort_flag, g.status, g.wait_limit);
+                    mbar_wait<true>(smem_u32(&bar_raw[qa]), pa, abort_flag, g.status, g.wait_limit);
                     load_row(va, sa, 0);
                 }
                 load_row(vb, sa, 4);
@@ -1392,7 +1406,7 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         bool loaded = false;
         for (uint32_t it = (uint32_t)team; it < total; it += kXfTeams) {
             if (!loaded) {
-                mbar_wait(smem_u32(&bar_full[q]), ph, abort_flag, g.status, g.wait_limit);
+                mbar_wait<true>(smem_u32(&bar_full[q]), ph, abort_flag, g.status, g.wait_limit);
                 load(va, s, 0);
             }
             load(vb, s, kHalf);

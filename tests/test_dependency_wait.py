@@ -30,15 +30,76 @@ def without_lambdas(text):
     return out + text[i:]
 
 
+def block_end(text, i):
+    """Index behind the block whose opening brace is at text[i]."""
+    depth, j = 1, i + 1
+    while depth:
+        depth += {"{": 1, "}": -1}.get(text[j], 0)
+        j += 1
+    return j
+
+
 def kernels():
     for f in sorted(os.listdir(CSRC)):
         if not f.endswith((".cu", ".cuh")):
             continue
         text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, f)).read())
-        for m in re.finditer(r"__global__[^;{]*?(\w+)\s*\([^;{]*\)\s*\{", text):
-            body = text[m.end():text.find("__global__", m.end()) if "__global__" in text[m.end():] else len(text)]
+        for m in re.finditer(r"__global__\s+void\s+(?:__launch_bounds__\s*\((?:[^()]|\([^()]*\))*\)\s*)?(\w+)\s*\([^;{]*\)\s*\{", text):
+            body = text[m.end():block_end(text, m.end() - 1)]
             if "dep_wait();" in body:
                 yield f, m.group(1), body
+
+
+def roles(body):
+    """(set-up, branches): the branches of the if / else-if chain over the warp's number that a kernel with several
+    roles consists of (its longest such chain), and the text before it.  A kernel without one is all set-up."""
+    best = (body, [])
+    for m in re.finditer(r"\n    if (?=\([^{]*\bwarp\b)", body):
+        chain, i = [], m.end()
+        while True:
+            a = body.index("{", i)
+            i = block_end(body, a)
+            chain.append(body[a:i])
+            more = re.match(r"\s*else(?: if (?=\()| (?=\{))", body[i:])
+            if not more:
+                break
+            i += more.end()
+        if len(chain) > max(2, len(best[1])):
+            best = (body[:m.start()], chain)
+    return best
+
+
+def test_bounded_waits_do_not_count_the_kernel_before():
+    """A wait for a barrier gives up after about a second.  Where a role has not waited for the kernel before, one that
+    releases its successor early and then takes long would use that time up: an expired EARLY wait first waits for
+    that kernel and starts its clock again, once."""
+    text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "sparq_gemm_kernel.cuh")).read())
+    wait = text[text.index("bool mbar_wait("):]
+    wait = wait[:block_end(wait, wait.index("{"))]
+    a = wait.index("{", wait.index("if (clock64() - t0 > limit_cycles)"))
+    expired = wait[a + 1:block_end(wait, a) - 1]
+    again = re.match(r"\s*if \(!alone\) \{(.*?)\}", expired, re.S)
+    assert again and [s.strip() for s in again.group(1).split(";")] == ["dep_wait()", "alone = true", "t0 = clock64()", "continue", ""]
+    assert "*abort_flag = 1u;" in expired[again.end():] and "bool alone = !EARLY;" in wait
+    # Waits of the roles that have not waited for the kernel before, in order: what their first operands land on or
+    # come from is EARLY.  (Barriers that start free are waited for from a stage's second use on.)
+    early = {}
+    for f, name, body in kernels():
+        setup, branches = roles(body)
+        assert "mbar_wait" not in setup, name
+        for i, role in enumerate(branches):
+            waits = [m for m in re.finditer(r"mbar_wait(?:<([^>]*)>)?\((?:smem_u32\(&)?(\w+)", role) if not re.search("empty|done", m.group(2))]
+            if "dep_wait();" not in role[:waits[0].start()]:
+                early[name, i] = [(m.group(2), m.group(1)) for m in waits]
+    streamed = "!B_RESIDENT"
+    assert early == {
+        ("sparq_gemm_kernel", 1): [("bar_full", "true"), ("bar_xf", "true"), ("bar_full", None)],
+        ("sparq_gemm_kernel", 3): [("bar_raw", "true"), ("bar_full", "true")],
+        # resident weights are the first thing waited for; streamed ones are behind the window's pieces
+        ("sparq_conv_window_kernel", 1): [("bar_b_full", "true"), ("bar_win_full", "true"), ("bar_win_xf", "true"), ("bar_b_full", None),
+                                          ("ops_bar", streamed), ("ops_bar", streamed), ("bar_b_full", None), ("bar_b_full", None),
+                                          ("bar_win_xf", streamed), ("bar_win_full", streamed)],
+        ("sparq_conv_window_kernel", 3): [("bar_win_full", "true")]}
 
 
 def test_no_access_before_the_wait():
