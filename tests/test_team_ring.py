@@ -36,7 +36,7 @@ def test_teams_ask_two_sets_of_full_barriers():
     assert "bars_full + 8u * (uint32_t)s + (use & 1u) * set;" in src
     # and the teams ask for it there, nowhere else: every other barrier of both sets in turn
     for ring, sets, stages, q, ph in (("bar_full", "kFullSets", "S", "q", "ph"), ("bar_raw", "kRawSets", "SA", "qa", "pa")):
-        asked = re.findall(r"(\w+)\(smem_u32\(&%s\[(\w+)\]\), (\w+)" % ring, role)
+        asked = re.findall(r"(\w+)(?:<true>)?\(smem_u32\(&%s\[(\w+)\]\), (\w+)" % ring, role)
         assert sorted(asked) == [("mbar_test", q, ph), ("mbar_wait", q, ph)] and len(re.findall(r"\b%s\b" % ring, role)) == 2
         assert f"int {q} = team;" in role and f"{q} += kXfTeams;" in role
         assert f"if ({q} >= {sets} * {stages}) {{ {q} -= {sets} * {stages}; {ph} ^= 1u; }}" in role
