@@ -1028,6 +1028,9 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     __shared__ __align__(8) uint64_t bar_acc_full[kAcc], bar_acc_empty[kAcc], bar_done;
     __shared__ uint32_t tmem_base_slot;
     __shared__ uint32_t abort_word;
+    constexpr bool kSharedFull = MODE == SPARQ_MODE_NONE;        // both producers announce on bar_full
+    constexpr uint32_t kStillIssuing = 0xFFFFFFFFu;
+    __shared__ volatile uint32_t announced[kSharedFull ? 2 : 1];        // stages that each of them announced, once it has stopped
     __shared__ __align__(16) float s_scale[kMaxTeams][BN], s_bias[kMaxTeams][BN];
 
     // the same in all lanes, and so for the compiler: what a role keeps of its ring costs the lanes' integer pipe nothing
@@ -1053,7 +1056,7 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     if (threadIdx.x == 0) {
         prefetch_tensormap(&map_a);
         prefetch_tensormap(&map_b);
-        for (int q = 0; q < kFullSets * S; ++q) mbar_init(smem_u32(&bar_full[q]), MODE == SPARQ_MODE_NONE ? 2 : 1);
+        for (int q = 0; q < kFullSets * S; ++q) mbar_init(smem_u32(&bar_full[q]), kSharedFull ? 2 : 1);
         for (int s = 0; s < S; ++s) {
             mbar_init(smem_u32(&bar_xf[s]), kXfTeamWarps);
             mbar_init(smem_u32(&bar_empty[s]), 1);
@@ -1068,6 +1071,7 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
             for (int b = 0; b < 2; ++b) mbar_init(smem_u32(&bar_res[w][b]), 1);
         mbar_init(smem_u32(&bar_done), 1);
         abort_word = 0;
+        if (kSharedFull) announced[0] = announced[1] = kStillIssuing;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
@@ -1148,12 +1152,24 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                     });
                 }
             }
-            // After an abort: wait (bounded) for the copies this thread still has in
-            // flight, so that none lands after the CTA has exited.
+            const int me = warp == 0 ? 0 : 1;
+            if (kSharedFull) announced[me] = it;
+            // After an abort: wait (bounded) for the copies still in flight, so that none
+            // lands after the CTA has exited.
             if (*abort_flag) {
-                const uint32_t first = it > (uint32_t)ring ? it - ring : 0;
+                uint32_t last = it;
+                if (kSharedFull) {
+                    // The two may have stopped at different stages, at most a ring apart: no stage is released that
+                    // both have not announced.  The one behind arrives for the other one's, which complete with
+                    // that one's copies then, and waits for them, too.
+                    const long long t0 = clock64();
+                    uint32_t other;
+                    while ((other = announced[me ^ 1]) == kStillIssuing && clock64() - t0 <= g.wait_limit) {}
+                    for (uint32_t j = it; other != kStillIssuing && j < other; ++j, ++last) mbar_arrive(bars_full + 8u * (j % (uint32_t)ring));
+                }
+                const uint32_t first = last > (uint32_t)ring ? last - ring : 0;
                 const uint32_t bars = (uint32_t)(sets * ring);
-                for (uint32_t j = first; j < it; ++j)
+                for (uint32_t j = first; j < last; ++j)
                     mbar_wait(bars_full + 8u * (j % bars), j / bars & 1u, abort_flag, g.status, g.wait_limit, true);
             }
         }
@@ -1171,15 +1187,18 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
             uint32_t local_tile = 0;
             int s = 0;             // stage
             uint32_t ph = 0;       // its phase parity
-            for (uint32_t tile = blockIdx.x; tile < total_tiles; tile += gridDim.x, ++local_tile) {
+            bool live = true;
+            for (uint32_t tile = blockIdx.x; tile < total_tiles && live; tile += gridDim.x, ++local_tile) {
                 const int acc = local_tile % kAcc;
                 const uint32_t acc_use = local_tile / kAcc;
                 if (acc_use > 0) mbar_wait(smem_u32(&bar_acc_empty[acc]), (acc_use - 1) & 1, abort_flag, g.status, g.wait_limit);
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
                 for (int kb = 0; kb < kb_count; ++kb) {
-                    if (MODE == SPARQ_MODE_NONE) mbar_wait<true>(smem_u32(&bar_full[s]), ph, abort_flag, g.status, g.wait_limit);
-                    else mbar_wait<true>(smem_u32(&bar_xf[s]), ph, abort_flag, g.status, g.wait_limit);
+                    if (kSharedFull) {
+                        // (a stage that is not there is not released, see the producers)
+                        if (!mbar_wait<true>(smem_u32(&bar_full[s]), ph, abort_flag, g.status, g.wait_limit)) { live = false; break; }
+                    } else mbar_wait<true>(smem_u32(&bar_xf[s]), ph, abort_flag, g.status, g.wait_limit);
                     if (ATM) mbar_wait(smem_u32(&bar_full[s]), ph, abort_flag, g.status, g.wait_limit);
                     tc_fence_after();
                     const uint64_t adesc = adesc0 + (uint64_t)((uint32_t)s * (kAStep >> 4)), bdesc = bdesc0 + (uint64_t)((uint32_t)s * (kBStep >> 4));
