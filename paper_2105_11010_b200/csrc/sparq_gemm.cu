@@ -229,8 +229,8 @@ static double tile_cycles(int64_t M, int64_t N, int64_t steps, int bn, int sms, 
     return (double)rounds * (double)steps * (step * wide + 150.0) + 3.0 * bn;     // + the last tile's epilogue
 }
 
-// The tile width with the lowest estimate.
-static int pick_bn(int64_t M, int64_t N, int64_t steps, int sms, bool transform, double *cycles = nullptr, double wide = 1.0)
+// The tile width with the lowest estimate in 128-byte steps.
+static int pick_bn(int64_t M, int64_t N, int64_t steps, int sms, bool transform, double *cycles = nullptr)
 {
     const int cand[3] = {256, 128, 64};
     int best = 64;
@@ -238,7 +238,7 @@ static int pick_bn(int64_t M, int64_t N, int64_t steps, int sms, bool transform,
     for (int i = 0; i < 3; ++i) {
         const int bn = cand[i];
         if (bn > 64 && N <= bn / 2) continue;          // would be mostly padding
-        const double cost = tile_cycles(M, N, steps, bn, sms, transform, wide);
+        const double cost = tile_cycles(M, N, steps, bn, sms, transform, 1.0);
         if (best_cost == 0.0 || cost < best_cost) {
             best_cost = cost;
             best = bn;
@@ -277,27 +277,35 @@ static SmallForm pick_small(int64_t M, int64_t N, int64_t k_blocks, int sms, boo
     return best;
 }
 
+// The 128-byte steps that a convolution's tile width is chosen by.
+static int64_t conv_steps(int64_t taps, int c) { return taps * ((c + 127) / 128); }
+
 // Whether to write T(A) to scratch memory once and contract that, instead of transforming every
 // staged tile: worth it when A is staged several times -- several column tiles, several filter
 // taps -- because the in-kernel transform is what such a step takes.  The extra pass costs about
 // 2.5 us and 2 bytes of traffic per activation (2.9 TB/s of activations).  A margin of 7 % keeps the
-// fused form, which needs no memory, where the two are close.
-static bool transform_first(int64_t M, int64_t N, int64_t steps, size_t act_bytes, int sms, double wide = 1.0)
+// fused form, which needs no memory, where the two are close.  `blocks`: the launch's own reduction steps, of
+// wide * 128 bytes; `steps`: the 128-byte ones that both launches choose their tile width by.  (Judged by the width
+// with the lowest estimate in its own steps, which is not launched, 64x56x56x80 -> 320 3x3 stride 2 was transformed
+// first: 91.5 us, fused 70.7.)
+static bool transform_first(int64_t M, int64_t N, int64_t steps, int64_t blocks, double wide, size_t act_bytes, int sms)
 {
-    if (pick_small(M, N, steps, sms, true).tile_rows) return false;
+    if (pick_small(M, N, blocks, sms, true).tile_rows) return false;
     if ((M + kBM - 1) / kBM * ((N + 63) / 64) >= (int64_t)1 << 31) return false;      // near the refused sizes: refused, if at all, with nothing enqueued
-    double fused, plain;
-    pick_bn(M, N, steps, sms, true, &fused, wide);
-    pick_bn(M, N, steps, sms, false, &plain, wide);
+    const double fused = tile_cycles(M, N, blocks, pick_bn(M, N, steps, sms, true), sms, true, wide);
+    const double plain = tile_cycles(M, N, blocks, pick_bn(M, N, steps, sms, false), sms, false, wide);
     const double clk = 1900.0;      // cycles per us
     return plain + clk * (2.5 + (double)act_bytes / 2.9e6) < 0.93 * fused;
 }
-
-// The same for a convolution through an im2col map, in steps of its channel blocks.
+static bool transform_first_gemm(int64_t M, int64_t N, int64_t K, size_t act_bytes, int sms)
+{
+    return transform_first(M, N, (K + 127) / 128, (K + 127) / 128, 1.0, act_bytes, sms);
+}
+// A convolution through an im2col map: steps of its channel blocks.
 static bool transform_first_conv(int64_t M, int cout, int taps, int c, size_t act_bytes, int sms)
 {
     const int bk = c % 128 == 0 ? 128 : 64;
-    return transform_first(M, cout, (int64_t)taps * ((c + bk - 1) / bk), act_bytes, sms, bk / 128.0);
+    return transform_first(M, cout, conv_steps(taps, c), (int64_t)taps * ((c + bk - 1) / bk), bk / 128.0, act_bytes, sms);
 }
 
 // Variant argument of the launchers (XN of xform_fused): 4 = n = 4 with all five placements, 5 = n = 4
@@ -385,7 +393,7 @@ static int gemm_impl(const uint8_t *A, int64_t lda, const int8_t *B, int64_t ldb
     if (rc != SPARQ_OK) return rc;
     int sms = 0;
     if (x.mode != SPARQ_MODE_NONE && lda == K && (rc = device_info(&sms)) == SPARQ_OK &&
-        transform_first(M, N, (K + 127) / 128, (size_t)M * (size_t)K, sms)) {
+        transform_first_gemm(M, N, K, (size_t)M * (size_t)K, sms)) {
         if (uint8_t *ta = (uint8_t *)workspace_alloc((size_t)M * (size_t)K, st)) {
             rc = quantize_rows(A, ta, (size_t)M, (size_t)K, x, true, st);
             if (rc == SPARQ_OK) rc = gemm_with_status(ta, K, B, ldb, M, N, K, plain_a8w8(), e, status, st);
@@ -470,7 +478,7 @@ static double small_us(const SmallForm &f, int64_t M, int64_t k_blocks, int bk, 
 static double im2col_us(int64_t M, int64_t N, int taps, int c, double xw, double ow, int sms)
 {
     const int bk = c % 128 == 0 ? 128 : 64;
-    const int bn = pick_bn(M, N, (int64_t)taps * ((c + 127) / 128), sms, xw > 0.0);
+    const int bn = pick_bn(M, N, conv_steps(taps, c), sms, xw > 0.0);
     const double rounds = (double)(((M + kBM - 1) / kBM * ((N + bn - 1) / bn) + sms - 1) / sms), blocks = rounds * taps * ((c + bk - 1) / bk);
     return 2.6 + blocks * bk / 128.0 * ((bn == 64 ? 0.05 : bn == 128 ? 0.10 : 0.13) + (bn == 256 ? 0.46 : 0.48) * xw) + 0.22 * blocks +
            0.47 * rounds * bn / 128.0 * ow;
@@ -728,7 +736,7 @@ static int im2col_conv(const uint8_t *x_in, int n, int h, int w, int c, const in
     const int64_t M = (int64_t)n * ho * wo, K = (int64_t)r * s * c;
     const int bk = (c % 128 == 0) ? 128 : 64;
     const SmallForm small = pick_small(M, cout, (int64_t)r * s * ((c + bk - 1) / bk), sms, x.mode != SPARQ_MODE_NONE);
-    const int bn = small.tile_rows ? kSmallBN : pick_bn(M, cout, (int64_t)r * s * ((c + 127) / 128), sms, x.mode != SPARQ_MODE_NONE);
+    const int bn = small.tile_rows ? kSmallBN : pick_bn(M, cout, conv_steps((int64_t)r * s, c), sms, x.mode != SPARQ_MODE_NONE);
     int rc;
     const int tile_rows = small.tile_rows ? small.tile_rows : kBM;
     GemmMaps m = {};
@@ -903,7 +911,7 @@ extern "C" int sparq_selftest_form(int n, int h, int w, int c, int cout, int r, 
         return q.resident ? SPARQ_FORM_WINDOW_RESIDENT : SPARQ_FORM_WINDOW_STREAMED;
     const int64_t steps = (int64_t)r * s * ((c + 127) / 128);
     const size_t act_bytes = (size_t)n * h * w * (size_t)c;
-    if (x.mode != SPARQ_MODE_NONE && (matrix ? transform_first(M, cout, steps, act_bytes, sms) : transform_first_conv(M, cout, r * s, c, act_bytes, sms)) &&
+    if (x.mode != SPARQ_MODE_NONE && (matrix ? transform_first_gemm(M, cout, c, act_bytes, sms) : transform_first_conv(M, cout, r * s, c, act_bytes, sms)) &&
         scratch(act_bytes)) return SPARQ_FORM_TRANSFORM_FIRST;
     return pick_small(M, cout, steps, sms, x.mode != SPARQ_MODE_NONE).tile_rows ? SPARQ_FORM_SMALL : SPARQ_FORM_FULL;
 }

@@ -47,6 +47,14 @@ def test_form(n, hw, c, cout, r, stride, p, want):
     assert form(n, hw, c, cout, r, stride, p) == want
 
 
+@pytest.mark.parametrize("n,hw", [(64, 56), (16, 112)])
+@pytest.mark.parametrize("cout", [264, 320, 384])
+def test_form_is_judged_by_the_tiles_it_is_launched_with(n, hw, cout):
+    """80 channels: the launch chooses its tile width by one 128-byte step per tap, where two 64-byte ones would choose
+    another.  Judged by that other one these layers were transformed first and took up to a quarter longer."""
+    assert form(n, hw, 80, cout, 3, 2, V5) == sparq.FORM_FULL
+
+
 def test_form_refuses_bad_geometry():
     with pytest.raises(sparq.SparqError):
         sparq.sparq_selftest_form((1, 8, 8, 24), (16, 3, 3, 24), (1, 1), (1, 1), V5)
