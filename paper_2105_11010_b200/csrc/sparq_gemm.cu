@@ -208,29 +208,63 @@ static int check_epilogue(const sparq_epilogue *e)
     return SPARQ_OK;
 }
 
-// Cycles that one CTA spends on its reduction steps (128 bytes of K each) with 128 x bn tiles, the
-// estimate that tile width and form are chosen by.  A step takes the longest of
-//   transform of the A stage   1120 cycles when a SPARQ mode is on,
-//   MMA                        2 * bn cycles,
-//   operand fetch from L2      1.9 cycles per 128-byte row of A and B, tiled or im2col
-// plus a hand-over, in ceil(tiles / SMs) passes; narrow tiles add CTAs but re-fetch and
-// re-transform A once per column tile.  wide: bytes of a step / 128.  (16384 x 512 x 4096 at 128 x 256: 680 cycles a step measured without
-// a transform, 1150 with one; 7x7x512 -> 512 3x3 at 128 x 128: 500 and 1120.  With the figures of a
-// slower transform and a fetch of 3.5 cycles through im2col maps, 3x56x56x448 -> 296 3x3 took 28.0 us, now 25.0, and
-// 117x28x28x64 -> 288, trimmed, 42.3, now 36.0; over 60 drawn layers one lost, 1.6 %.)
-static double tile_cycles(int64_t M, int64_t N, int64_t steps, int bn, int sms, bool transform, double wide)
+// Bytes per output element that the epilogue writes.
+static double out_bytes(const sparq_epilogue *e) { return (e->acc_out ? 4 : 0) + (e->f32_out ? 4 : 0) + (e->u8_out ? 1 : 0); }
+
+// A contraction as its tiles are estimated: `blocks` reduction steps of wide * 128 bytes, `fetch` cycles per row of A
+// and B in each, `ow` bytes of output per element (without a residual's, which the staged form hides: counted, 50176 x
+// 512, K 128, with one took 128-wide tiles, 16.6 us against 15.8).
+struct Steps {
+    int64_t blocks;
+    double wide, fetch, ow;
+};
+static Steps gemm_steps(int64_t K, double ow) { return {(K + 127) / 128, 1.0, 2.2, ow}; }
+static int conv_bk(int c) { return c % 128 == 0 ? 128 : 64; }
+static Steps conv_steps(int64_t taps, int c, double ow)
+{
+    if (conv_bk(c) == 128) return {taps * (c / 128), 1.0, 1.3, ow};
+    // 64-byte rows cost nearly as much as 128-byte ones, and the last block's that reach past C two to three
+    // times that (128-wide tiles, 3x3: 500 cycles a step with 64 channels, 925 with 32, 1700 with 16)
+    const int full = c / 64, rest = c % 64, per_tap = full + (rest ? 1 : 0);
+    const double last = rest == 0 ? 0.0 : rest == 32 ? 2.1 : rest == 48 ? 3.05 : 3.5;
+    return {taps * per_tap, 0.5, (1.15 * full + last) / per_tap, ow};
+}
+
+// Cycles that the transform takes of a 128-byte step.  (Measured, 128-wide tiles, pairs: n = 4 with all
+// placements 1090, with fewer 1450, 3 and 2 bits 1945, restricted 2720; without the pair rule the 3- and 2-bit
+// sets are as quick as n = 4.)
+static double xform_cycles(const XformArgs &x)
+{
+    if (x.mode == SPARQ_MODE_NONE) return 0.0;
+    if (x.n == 4) return x.widen_rounds ? 1450.0 : 1150.0;
+    return x.widen_rounds || x.mode == SPARQ_MODE_VSPARQ ? 2000.0 : 1150.0;
+}
+
+// Cycles that one CTA spends with 128 x bn tiles, the estimate that tile width and form are chosen by.  A step
+// takes the longest of
+//   transform of the A stage   xform_cycles per 128 bytes (xf; 0 without one),
+//   MMA                        2 * bn cycles per 128 bytes,
+//   operand fetch from L2      Steps::fetch per row of A and B
+// plus a hand-over; a tile its steps or its epilogue, in ceil(tiles / SMs) passes.  Narrow tiles add CTAs but re-fetch
+// and re-transform A once per column tile.  A fit of the choices (not the times) to 1700 layers measured in every
+// form.  Over 2400 others that are too large for the small form it costs 2.3 % against the fastest form, 2.5 % of them
+// lose more than 20 %.  The estimate before (one cost for all transforms, 64-byte rows at half price): 4.7 % and 6.8 %,
+// and 5.5 % of the layers lost against the one before that, up to 1.9 times: 5151 x 1680, K 2608, at 2 bits 50.7 us fused,
+// 36.6 transformed first; 8x44x44x48 -> 488 5x5 49.6 transformed first, 39.4 fused.
+static double tile_cycles(int64_t M, int64_t N, const Steps &k, int bn, int sms, double xf)
 {
     const int64_t tiles = ((M + kBM - 1) / kBM) * ((N + bn - 1) / bn);
     const int64_t rounds = (tiles + sms - 1) / sms;
-    double step = 2.0 * bn;
-    const double fetch = 1.9 * (kBM + bn);
+    double step = 2.0 * bn * k.wide;
+    const double fetch = k.fetch * (kBM + bn);
     if (fetch > step) step = fetch;
-    if (transform && step < 1120.0) step = 1120.0;
-    return (double)rounds * (double)steps * (step * wide + 150.0) + 3.0 * bn;     // + the last tile's epilogue
+    if (xf * k.wide > step) step = xf * k.wide;
+    const double epi = bn * (2.6 + 2.1 * k.ow), walk = (double)k.blocks * (step + 105.0);
+    return (double)rounds * (walk > 1.35 * epi ? walk : 1.35 * epi) + epi;     // + the last tile's epilogue
 }
 
-// The tile width with the lowest estimate in 128-byte steps.
-static int pick_bn(int64_t M, int64_t N, int64_t steps, int sms, bool transform, double *cycles = nullptr)
+// The tile width with the lowest estimate.
+static int pick_bn(int64_t M, int64_t N, const Steps &k, int sms, double xf, double *cycles = nullptr)
 {
     const int cand[3] = {256, 128, 64};
     int best = 64;
@@ -238,7 +272,7 @@ static int pick_bn(int64_t M, int64_t N, int64_t steps, int sms, bool transform,
     for (int i = 0; i < 3; ++i) {
         const int bn = cand[i];
         if (bn > 64 && N <= bn / 2) continue;          // would be mostly padding
-        const double cost = tile_cycles(M, N, steps, bn, sms, transform, 1.0);
+        const double cost = tile_cycles(M, N, k, bn, sms, xf);
         if (best_cost == 0.0 || cost < best_cost) {
             best_cost = cost;
             best = bn;
@@ -277,35 +311,21 @@ static SmallForm pick_small(int64_t M, int64_t N, int64_t k_blocks, int sms, boo
     return best;
 }
 
-// The 128-byte steps that a convolution's tile width is chosen by.
-static int64_t conv_steps(int64_t taps, int c) { return taps * ((c + 127) / 128); }
-
 // Whether to write T(A) to scratch memory once and contract that, instead of transforming every
 // staged tile: worth it when A is staged several times -- several column tiles, several filter
 // taps -- because the in-kernel transform is what such a step takes.  The extra pass costs about
-// 2.5 us and 2 bytes of traffic per activation (2.9 TB/s of activations).  A margin of 7 % keeps the
-// fused form, which needs no memory, where the two are close.  `blocks`: the launch's own reduction steps, of
-// wide * 128 bytes; `steps`: the 128-byte ones that both launches choose their tile width by.  (Judged by the width
-// with the lowest estimate in its own steps, which is not launched, 64x56x56x80 -> 320 3x3 stride 2 was transformed
-// first: 91.5 us, fused 70.7.)
-static bool transform_first(int64_t M, int64_t N, int64_t steps, int64_t blocks, double wide, size_t act_bytes, int sms)
+// 3.7 us and 2 bytes of traffic per activation (2.8 TB/s of activations), and the contraction reads them again
+// (89x56x56x352 -> 24 at 2 bits: 53.2 us fused, 65.5 transformed first).
+static bool transform_first(int64_t M, int64_t N, const Steps &k, const XformArgs &x, size_t act_bytes, int sms)
 {
-    if (pick_small(M, N, blocks, sms, true).tile_rows) return false;
+    if (pick_small(M, N, k.blocks, sms, true).tile_rows) return false;
     if ((M + kBM - 1) / kBM * ((N + 63) / 64) >= (int64_t)1 << 31) return false;      // near the refused sizes: refused, if at all, with nothing enqueued
-    const double fused = tile_cycles(M, N, blocks, pick_bn(M, N, steps, sms, true), sms, true, wide);
-    const double plain = tile_cycles(M, N, blocks, pick_bn(M, N, steps, sms, false), sms, false, wide);
+    double fused, plain;
+    pick_bn(M, N, k, sms, xform_cycles(x), &fused);
+    pick_bn(M, N, k, sms, 0.0, &plain);
     const double clk = 1900.0;      // cycles per us
-    return plain + clk * (2.5 + (double)act_bytes / 2.9e6) < 0.93 * fused;
-}
-static bool transform_first_gemm(int64_t M, int64_t N, int64_t K, size_t act_bytes, int sms)
-{
-    return transform_first(M, N, (K + 127) / 128, (K + 127) / 128, 1.0, act_bytes, sms);
-}
-// A convolution through an im2col map: steps of its channel blocks.
-static bool transform_first_conv(int64_t M, int cout, int taps, int c, size_t act_bytes, int sms)
-{
-    const int bk = c % 128 == 0 ? 128 : 64;
-    return transform_first(M, cout, conv_steps(taps, c), (int64_t)taps * ((c + bk - 1) / bk), bk / 128.0, act_bytes, sms);
+    const double read = clk * (double)act_bytes / 6.0e6;
+    return (plain > read ? plain : read) + clk * (3.7 + (double)act_bytes / 2.8e6) < 0.99 * fused;
 }
 
 // Variant argument of the launchers (XN of xform_fused): 4 = n = 4 with all five placements, 5 = n = 4
@@ -393,7 +413,7 @@ static int gemm_impl(const uint8_t *A, int64_t lda, const int8_t *B, int64_t ldb
     if (rc != SPARQ_OK) return rc;
     int sms = 0;
     if (x.mode != SPARQ_MODE_NONE && lda == K && (rc = device_info(&sms)) == SPARQ_OK &&
-        transform_first_gemm(M, N, K, (size_t)M * (size_t)K, sms)) {
+        transform_first(M, N, gemm_steps(K, out_bytes(e)), x, (size_t)M * (size_t)K, sms)) {
         if (uint8_t *ta = (uint8_t *)workspace_alloc((size_t)M * (size_t)K, st)) {
             rc = quantize_rows(A, ta, (size_t)M, (size_t)K, x, true, st);
             if (rc == SPARQ_OK) rc = gemm_with_status(ta, K, B, ldb, M, N, K, plain_a8w8(), e, status, st);
@@ -466,30 +486,28 @@ static double xform_weight(const XformArgs &x)
     return x.mode == SPARQ_MODE_NONE ? 0.0 : x.n == 4 ? (x.widen_rounds ? 1.2 : 1.0) : (x.widen_rounds ? 2.0 : 1.35);
 }
 // Bytes per output element that the epilogue moves.
-static double out_weight(const sparq_epilogue *e)
-{
-    return (e->acc_out ? 4 : 0) + (e->f32_out ? 4 : 0) + (e->u8_out ? 1 : 0) + (e->residual ? 1 : 0);
-}
+static double out_weight(const sparq_epilogue *e) { return out_bytes(e) + (e->residual ? 1 : 0); }
 static double small_us(const SmallForm &f, int64_t M, int64_t k_blocks, int bk, double xw)
 {
     const double rows = (double)(M < f.tile_rows ? M : f.tile_rows) / kBM * bk / 128.0;
     return 1.9 + (double)((k_blocks + f.split - 1) / f.split) * (0.21 + (0.09 + 0.60 * xw) * rows) + (f.split > 1 ? 1.3 : 0.0);
 }
-static double im2col_us(int64_t M, int64_t N, int taps, int c, double xw, double ow, int sms)
+static double im2col_us(int64_t M, int64_t N, int taps, int c, const XformArgs &x, double ow, int sms)
 {
-    const int bk = c % 128 == 0 ? 128 : 64;
-    const int bn = pick_bn(M, N, conv_steps(taps, c), sms, xw > 0.0);
-    const double rounds = (double)(((M + kBM - 1) / kBM * ((N + bn - 1) / bn) + sms - 1) / sms), blocks = rounds * taps * ((c + bk - 1) / bk);
+    const int bk = conv_bk(c);
+    const double xw = xform_weight(x);
+    const Steps k = conv_steps(taps, c, ow);
+    const int bn = pick_bn(M, N, k, sms, xform_cycles(x));
+    const double rounds = (double)(((M + kBM - 1) / kBM * ((N + bn - 1) / bn) + sms - 1) / sms), blocks = rounds * k.blocks;
     return 2.6 + blocks * bk / 128.0 * ((bn == 64 ? 0.05 : bn == 128 ? 0.10 : 0.13) + (bn == 256 ? 0.46 : 0.48) * xw) + 0.22 * blocks +
            0.47 * rounds * bn / 128.0 * ow;
 }
 // The same layer by the im2col path, in the form that would be launched there.
-static double im2col_path_us(int64_t M, int64_t N, int taps, int c, double xw, double ow, int sms)
+static double im2col_path_us(int64_t M, int64_t N, int taps, int c, const XformArgs &x, double ow, int sms)
 {
-    const int bk = c % 128 == 0 ? 128 : 64;
-    const int64_t k_blocks = (int64_t)taps * ((c + bk - 1) / bk);
-    const SmallForm f = pick_small(M, N, k_blocks, sms, xw > 0.0);
-    return f.tile_rows ? small_us(f, M, k_blocks, bk, xw) : im2col_us(M, N, taps, c, xw, ow, sms);
+    const int64_t k_blocks = conv_steps(taps, c, ow).blocks;
+    const SmallForm f = pick_small(M, N, k_blocks, sms, x.mode != SPARQ_MODE_NONE);
+    return f.tile_rows ? small_us(f, M, k_blocks, conv_bk(c), xform_weight(x)) : im2col_us(M, N, taps, c, x, ow, sms);
 }
 
 // How the window kernel tiles a convolution.
@@ -572,7 +590,7 @@ static bool plan_window(WindowPlan *q, int n, int h, int w, int c, int cout, int
         // 28x28x128 -> 128 5.3); the small form may share them out (one image of the latter 5.2 -> 4.6, of
         // 20x20x96 -> 112 6.3 -> 4.3; 56x56x64 stays).
         if (units <= sms && pick_small(M, cout, (int64_t)taps * ((c + 127) / 128), sms, xw > 0.0).tile_rows &&
-            im2col_path_us(M, cout, taps, c, xw, ow, sms) < 0.97 * (3.35 + 13.2e-6 * kb_count * b_block)) return false;
+            im2col_path_us(M, cout, taps, c, x, ow, sms) < 0.97 * (3.35 + 13.2e-6 * kb_count * b_block)) return false;
     } else {
         if (bn == 64) return false;                          // only the resident form is built for 64-wide tiles
         // 128-wide tiles: up to two row tiles of one (image, column tile) are accumulated together
@@ -618,13 +636,13 @@ static bool plan_window(WindowPlan *q, int n, int h, int w, int c, int cout, int
         // and operand bytes for one transform per tap (64x17x17x64 -> 256 3x3: 8.3 us against 12.7;
         // 17x35x35x32 -> 160 7x7 at 2 bits 45 against 25).
         if (half_empty || (batched && pick_small(M, cout, (int64_t)taps * ((c + 127) / 128), sms, xw > 0.0).tile_rows)) {
-            if (im2col_path_us(M, cout, taps, c, xw, ow, sms) < window_us) return false;
+            if (im2col_path_us(M, cout, taps, c, x, ow, sms) < window_us) return false;
         } else if (batched && b_stages == 2) {
             // a ring this short leaves the tensor core waiting; transformed once, the im2col form may win
             // (16x56x56x256 -> 64 5x5 at 3 bits, restricted: 56 us against 100)
             const size_t act_bytes = (size_t)n * h * w * (size_t)c;
-            const double first = xw > 0.0 && scratch(act_bytes) ? 2.5 + (double)act_bytes / 2.9e6 + im2col_us(M, cout, taps, c, 0.0, ow, sms) : 1e30;
-            if (first < window_us || im2col_path_us(M, cout, taps, c, xw, ow, sms) < window_us) return false;
+            const double first = xw > 0.0 && scratch(act_bytes) ? 2.5 + (double)act_bytes / 2.9e6 + im2col_us(M, cout, taps, c, plain_a8w8(), ow, sms) : 1e30;
+            if (first < window_us || im2col_path_us(M, cout, taps, c, x, ow, sms) < window_us) return false;
         }
     }
     *q = {wp, cb, tr, c_blocks, tiles_per_img, bn, n_tiles, units, resident, grp, win_bufs, b_stages, plane_for(grp), false, 0};
@@ -705,7 +723,7 @@ int gemm_with_status(const uint8_t *A, int64_t lda, const int8_t *B, int64_t ldb
     // step is a hand-off between three warp roles, which is what a small launch is made of)
     const int bk = (pad64 < pad128 && !(pad64 >= 320 && pad128 * 8 <= pad64 * 9)) ? 64 : 128;
     const SmallForm small = pick_small(M, N, (K + bk - 1) / bk, sms, x.mode != SPARQ_MODE_NONE);
-    const int bn = small.tile_rows ? kSmallBN : pick_bn(M, N, (K + 127) / 128, sms, x.mode != SPARQ_MODE_NONE);
+    const int bn = small.tile_rows ? kSmallBN : pick_bn(M, N, gemm_steps(K, out_bytes(e)), sms, xform_cycles(x));
     const int tile_rows = small.tile_rows ? small.tile_rows : kBM;
     GemmMaps m = {};
     rc = encode_2d(&m.a, A, K, M, lda, bk, tile_rows);
@@ -734,9 +752,10 @@ static int im2col_conv(const uint8_t *x_in, int n, int h, int w, int c, const in
                        int sms, unsigned int *status, cudaStream_t st)
 {
     const int64_t M = (int64_t)n * ho * wo, K = (int64_t)r * s * c;
-    const int bk = (c % 128 == 0) ? 128 : 64;
-    const SmallForm small = pick_small(M, cout, (int64_t)r * s * ((c + bk - 1) / bk), sms, x.mode != SPARQ_MODE_NONE);
-    const int bn = small.tile_rows ? kSmallBN : pick_bn(M, cout, conv_steps((int64_t)r * s, c), sms, x.mode != SPARQ_MODE_NONE);
+    const int bk = conv_bk(c);
+    const Steps k = conv_steps((int64_t)r * s, c, out_bytes(e));
+    const SmallForm small = pick_small(M, cout, k.blocks, sms, x.mode != SPARQ_MODE_NONE);
+    const int bn = small.tile_rows ? kSmallBN : pick_bn(M, cout, k, sms, xform_cycles(x));
     int rc;
     const int tile_rows = small.tile_rows ? small.tile_rows : kBM;
     GemmMaps m = {};
@@ -785,7 +804,7 @@ int gemm_sparse24_fused(const uint8_t *A, const int8_t *w_exp, int64_t M, int64_
     const int bn = N <= 64 ? 64 : 128;
     const int64_t tiles = (M + 255) / 256 * ((N + bn - 1) / bn);
     double plain;
-    pick_bn(M, N, steps3, sms, false, &plain);
+    pick_bn(M, N, gemm_steps(3 * K, out_bytes(e)), sms, 0.0, &plain);
     const double fused = (double)((tiles + sms - 1) / sms) * (double)steps * 4200.0;
     if (tiles >= (int64_t)1 << 31 || fused > plain + 1900.0 * (2.5 + (double)M * (double)K * 4.0 / 6.0e6)) return 0;
     CUtensorMap ma, mb;
@@ -882,7 +901,7 @@ extern "C" int sparq_conv2d_nhwc_s8(const uint8_t *x_in, int n, int h, int w, in
         if (rc != 0) return rc < 0 ? rc : SPARQ_OK;
     }
     const size_t act_bytes = (size_t)n * h * w * (size_t)c;
-    if (x.mode != SPARQ_MODE_NONE && transform_first_conv(M, cout, r * s, c, act_bytes, sms)) {
+    if (x.mode != SPARQ_MODE_NONE && transform_first(M, cout, conv_steps((int64_t)r * s, c, out_bytes(e)), x, act_bytes, sms)) {
         if (uint8_t *tx = (uint8_t *)workspace_alloc(act_bytes, st)) {
             rc = quantize_rows(x_in, tx, (size_t)n * h * w, (size_t)c, x, true, st);
             if (rc == SPARQ_OK) rc = im2col_conv(tx, n, h, w, c, wgt, cout, r, s, stride_h, stride_w, pad_h, pad_w, ho, wo, plain_a8w8(), e, sms, status, st);
@@ -909,9 +928,8 @@ extern "C" int sparq_selftest_form(int n, int h, int w, int c, int cout, int r, 
     auto scratch = [](size_t bytes) { return bytes <= kWorkspaceMaxBytes; };
     if (!matrix && stride_h == 1 && stride_w == 1 && plan_window(&q, n, h, w, c, cout, r, s, pad_w, ho, wo, x, 1.0, sms, scratch))
         return q.resident ? SPARQ_FORM_WINDOW_RESIDENT : SPARQ_FORM_WINDOW_STREAMED;
-    const int64_t steps = (int64_t)r * s * ((c + 127) / 128);
+    const Steps k = matrix ? gemm_steps(c, 1.0) : conv_steps((int64_t)r * s, c, 1.0);
     const size_t act_bytes = (size_t)n * h * w * (size_t)c;
-    if (x.mode != SPARQ_MODE_NONE && (matrix ? transform_first_gemm(M, cout, c, act_bytes, sms) : transform_first_conv(M, cout, r * s, c, act_bytes, sms)) &&
-        scratch(act_bytes)) return SPARQ_FORM_TRANSFORM_FIRST;
-    return pick_small(M, cout, steps, sms, x.mode != SPARQ_MODE_NONE).tile_rows ? SPARQ_FORM_SMALL : SPARQ_FORM_FULL;
+    if (x.mode != SPARQ_MODE_NONE && transform_first(M, cout, k, x, act_bytes, sms) && scratch(act_bytes)) return SPARQ_FORM_TRANSFORM_FIRST;
+    return pick_small(M, cout, k.blocks, sms, x.mode != SPARQ_MODE_NONE).tile_rows ? SPARQ_FORM_SMALL : SPARQ_FORM_FULL;
 }

@@ -9,6 +9,7 @@ import paper_2105_11010_b200 as sparq
 
 V5 = sparq.SparqParams()
 V6 = sparq.SparqParams(sparq.MODE_VSPARQ, 3, sparq.SET_6OPT, sparq.ROUND_NEAREST)
+V7 = sparq.SparqParams(sparq.MODE_VSPARQ, 2, sparq.SET_7OPT, sparq.ROUND_NEAREST)
 R35 = sparq.SparqParams(sparq.MODE_VSPARQ, 3, 0x35, sparq.ROUND_NEAREST)
 R55 = sparq.SparqParams(sparq.MODE_VSPARQ, 2, 0x55, sparq.ROUND_NEAREST)
 NONE = sparq.SparqParams(sparq.MODE_NONE)
@@ -50,9 +51,21 @@ def test_form(n, hw, c, cout, r, stride, p, want):
 @pytest.mark.parametrize("n,hw", [(64, 56), (16, 112)])
 @pytest.mark.parametrize("cout", [264, 320, 384])
 def test_form_is_judged_by_the_tiles_it_is_launched_with(n, hw, cout):
-    """80 channels: the launch chooses its tile width by one 128-byte step per tap, where two 64-byte ones would choose
+    """80 channels: the launch chose its tile width by one 128-byte step per tap, where two 64-byte ones choose
     another.  Judged by that other one these layers were transformed first and took up to a quarter longer."""
     assert form(n, hw, 80, cout, 3, 2, V5) == sparq.FORM_FULL
+
+
+@pytest.mark.parametrize("n,hw,c,cout,r,p,want", [
+    # what a transform costs: 3- and 2-bit windows with the pair rule nearly twice that of 4-bit ones
+    (5151, 1, 2608, 1680, 1, V7, sparq.FORM_TRANSFORM_FIRST), (4335, 1, 2160, 1352, 1, V6, sparq.FORM_TRANSFORM_FIRST),
+    (1433, 1, 2944, 1896, 1, V7, sparq.FORM_TRANSFORM_FIRST), (12172, 1, 544, 1840, 1, V6, sparq.FORM_TRANSFORM_FIRST),
+    # what a row costs through an im2col map: no less in 64-byte blocks, more where the last block is not full
+    (8, 44, 48, 488, 5, V5, sparq.FORM_FULL), (6, 56, 432, 288, 3, V5, sparq.FORM_FULL), (3, 56, 272, 488, 3, V5, sparq.FORM_FULL),
+    (10, 48, 336, 256, 3, V5, sparq.FORM_FULL)])
+def test_form_follows_the_costs_of_transform_and_fetch(n, hw, c, cout, r, p, want):
+    """Layers that took 10 to 40 % longer in the other form."""
+    assert form(n, hw, c, cout, r, 1, p) == want
 
 
 def test_form_refuses_bad_geometry():
