@@ -30,6 +30,17 @@ def without_lambdas(text):
     return out + text[i:]
 
 
+def kernels():
+    for f in sorted(os.listdir(CSRC)):
+        if not f.endswith((".cu", ".cuh")):
+            continue
+        text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, f)).read())
+        for m in re.finditer(r"__global__[^;{]*?(\w+)\s*\([^;{]*\)\s*\{", text):
+            body = text[m.end():text.find("__global__", m.end()) if "__global__" in text[m.end():] else len(text)]
+            if "dep_wait();" in body:
+                yield f, m.group(1), body
+
+
 def block_end(text, i):
     """Index behind the block whose opening brace is at text[i]."""
     depth, j = 1, i + 1
@@ -39,7 +50,8 @@ def block_end(text, i):
     return j
 
 
-def kernels():
+def kernel_bodies():
+    """kernels() with each body ending where it does."""
     for f in sorted(os.listdir(CSRC)):
         if not f.endswith((".cu", ".cuh")):
             continue
@@ -84,7 +96,7 @@ def test_bounded_waits_do_not_count_the_kernel_before():
     # Waits of the roles that have not waited for the kernel before, in order: what their first operands land on or
     # come from is EARLY.  (Barriers that start free are waited for from a stage's second use on.)
     early = {}
-    for f, name, body in kernels():
+    for f, name, body in kernel_bodies():
         setup, branches = roles(body)
         assert "mbar_wait" not in setup, name
         for i, role in enumerate(branches):
