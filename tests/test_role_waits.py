@@ -181,12 +181,12 @@ def test_scale_and_bias_of_the_24_product_written_by_the_operation_before():
     sparq.sparq_sparse24_expand_weights(*[torch.from_numpy(t).cuda() for t in sparse], p, w)
     Ad, dev = torch.from_numpy(A).cuda(), [[torch.from_numpy(t).cuda() for t in s] for s in sets]
     scale, bias = [torch.empty_like(t) for t in dev[0]]
-    out = torch.empty((m, n), dtype=torch.uint8, device="cuda")
+    out, work = torch.empty((m, n), dtype=torch.uint8, device="cuda"), torch.empty((m, 3 * k), dtype=torch.uint8, device="cuda")
     kept = [torch.empty_like(out) for _ in range(20)]
     for i, q in enumerate(kept):
         scale.copy_(dev[i & 1][0])
         bias.copy_(dev[i & 1][1])
-        sparq.sparq_gemm_s8_sparse24(Ad, w, p, scale=scale, bias=bias, relu=True, inv_out_scale=inv, u8_out=out)
+        sparq.sparq_gemm_s8_sparse24(Ad, w, p, workspace=work, scale=scale, bias=bias, relu=True, inv_out_scale=inv, u8_out=out)
         sparq.sparq_quantize(out, q, m, n, none)
     sparq.sparq_check()
     for i, q in enumerate(kept):
