@@ -126,14 +126,11 @@ inline uint32_t half_bits_of_int(uint32_t v)
     return ((uint32_t)(p + 15) << 10) | ((v << (10 - p)) & 0x3FFu);
 }
 
-// Constants of xform_word_fullset for window width n and the rounding flag.
+// Constants of xform_word_fullset for window width n and the rounding flag (at n = 4 it has its own, and a lone
+// non-zero keeps all bits).
 inline void fill_fullset(XformDev *d, int n, int rnd)
 {
     auto set = [&](int w, uint32_t *add, uint32_t *mask, uint32_t *top) {
-        if (w >= 8) {                    // the window holds all 8 bits: nothing is dropped
-            *add = 0u; *mask = 0xFFFFFFFFu; *top = half_bits_of_int(255u) * 0x00010001u;
-            return;
-        }
         const uint32_t m16 = (0xFFFFu << (11 - w)) & 0xFFFFu;      // sign, exponent and the top w-1 fraction bits
         const uint32_t a16 = rnd ? (1u << (10 - w)) : 0u;          // half of the lowest kept bit
         *mask = m16 * 0x00010001u;
@@ -141,7 +138,7 @@ inline void fill_fullset(XformDev *d, int n, int rnd)
         *top = (half_bits_of_int(((1u << w) - 1u) << (8 - w)) | (~m16 & 0xFFFFu)) * 0x00010001u;
     };
     set(n, &d->f_add, &d->f_mask, &d->f_top);
-    set(2 * n, &d->l_add, &d->l_mask, &d->l_top);
+    if (n < 4) set(2 * n, &d->l_add, &d->l_mask, &d->l_top);
 }
 
 // Mask of the bits BELOW the window for each of the four bytes of x (Section 3.1: the
@@ -265,7 +262,7 @@ __device__ __forceinline__ uint32_t window_of_halves(uint32_t lo, uint32_t hi, u
     return prmt(h2_add(lo & mask, kHalf1024), h2_add(hi & mask, kHalf1024), 0x6420u);
 }
 
-// FIXED4: n = 4 with rounding RND, constants at compile time; otherwise width and rounding as in d.
+// FIXED4: n = 4 with rounding RND, constants at compile time; otherwise n < 4, width and rounding as in d.
 template <int MODE, bool FIXED4, bool RND>
 __device__ __forceinline__ uint32_t xform_word_fullset(uint32_t x, const XformDev &d)
 {
@@ -277,7 +274,7 @@ __device__ __forceinline__ uint32_t xform_word_fullset(uint32_t x, const XformDe
     if (MODE == SPARQ_MODE_BSPARQ) return q;
     // vSPARQ: a byte whose partner is zero keeps the 2n-bit window (the whole byte for n = 4)
     uint32_t lone = x;
-    if (!FIXED4 && d.l_mask != 0xFFFFFFFFu) lone = window_of_halves<true>(lo, hi, d.l_add, d.l_mask, d.l_top);   // uniform: a kernel argument
+    if (!FIXED4) lone = window_of_halves<true>(lo, hi, d.l_add, d.l_mask, d.l_top);
     const uint32_t nz = ((x & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | x;   // bit 7 of each byte: byte != 0
     const uint32_t partner_nz = prmt(nz, nz, 0xAB89u);           // swap within pairs, replicate bit 7
     return (q & partner_nz) | (lone & ~partner_nz);

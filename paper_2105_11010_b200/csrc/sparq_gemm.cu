@@ -285,7 +285,7 @@ static int pick_bn(int64_t M, int64_t N, const Steps &k, int sms, double xf, dou
 // The small form (sparq_gemm_small_kernel): launches whose 64-wide tiles all run at once.  tile_rows = 0
 // where they do not.  Tiles of 64 or 128 rows, and 1 to 8 CTAs of a cluster on a tile, by the time
 // of the serial walk along K: a step takes such a launch about 0.25 us, and 0.35 us more for the
-// transform of 128 rows; sharing a tile costs about 1.6 us, and writing 128 rows out 0.4 (173 x 128 x 256,
+// transform of 128 rows (packed integers; the half-precision one at n = 4 takes less); sharing a tile costs about 1.6 us, and writing 128 rows out 0.4 (173 x 128 x 256,
 // fp32, without a transform: 4.3 us with 128 rows, 3.8 with 64).  Measured (us, one image, 128-row
 // tiles, 1 / 2 / 4 / 8 CTAs on each): 7x7x2048 -> 512 9.4 / 9.1 / 6.1 / 4.8, 14x14x1024 -> 256 6.9 /
 // 8.7 / 6.3 / 5.0, 28x28x512 -> 128 5.6 / 7.1 / 5.6, 7x7x512 -> 2048 4.7 / 6.3 / 5.1; chosen by this
@@ -475,11 +475,13 @@ constexpr int kMaxDynSmem = kWindowMaxDynSmem;
 
 // ---- which form a stride-1 convolution takes ---------------------------------------------------------
 // Estimates in us, least-squares fits to 840 measured layers (1-128 images of 7..56 pixels, 16-512
-// channels and filters, 3x3 / 5x5 / 7x7, five transforms and none).  Root mean square error: window
-// with streamed weights on 128-wide tiles 7 %, on 256-wide ones 22 %, small form 10 %, im2col form
-// 11 %.  They are compared where either form can win by a factor: few tiles (over 493 layers the
-// choice costs 0.2 % against the faster form, at worst 20 %; always the window 48 %), half-empty channel
-// blocks (1.4 %; always the window 13 %) and rings of two stages.
+// channels and filters, 3x3 / 5x5 / 7x7, five transforms and none), with the packed-integer transform at n = 4 and one wait
+// of all roles for the kernel before.  Root mean square error then: window with streamed weights on
+// 128-wide tiles 7 %, on 256-wide ones 22 %, small form 10 %, im2col form 11 %.  Both forms have become faster since;
+// only the start of the small one was measured again (2.5 -> 1.9 us).  They are compared where either
+// form can win by a factor: few tiles (over 493 layers the choice cost 0.2 % against the faster form, at
+// worst 20 %; always the window 48 %), half-empty channel blocks (1.4 %; always the window 13 %) and
+// rings of two stages.
 // The transform's work relative to the 4-bit form with all placements.
 static double xform_weight(const XformArgs &x)
 {

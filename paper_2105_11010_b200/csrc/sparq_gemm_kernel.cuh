@@ -89,7 +89,6 @@ struct GemmArgs {
     const uint8_t *residual;
     float residual_scale;
     int stages;             // of the operand ring
-    int raw_stages;         // of the ring of activations, where they have one of their own
     // staged output: bytes per row of the boxes that the epilogue warps store (and fetch the residual)
     // with through shared memory, 0 = straight from registers.  See epi_staged.
     int out_box;
@@ -989,6 +988,10 @@ struct TileCfg {
     }
     static constexpr int kAcc = BN == 256 ? 2 : 4;                  // accumulator stages in tensor memory
     static constexpr int kTmemCols = kAcc * BN;
+    // With the activations in tensor memory (ATM): stages of weights, and of raw activations in what room is left
+    static constexpr int kAtmRoom = kMaxDynSmemGemm - 1024, kAtmStages = 4;
+    static constexpr int kAtmRawStages = (kAtmRoom - kAtmStages * kBBytes) / kABytes;
+    static constexpr int kAtmSmem = 1024 + kAtmStages * kBBytes + kAtmRawStages * kABytes;
 };
 
 template <int BN, int BK, int MODE, int XN, bool RND, int OUT, bool ATM>
@@ -1000,8 +1003,9 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     constexpr bool kTwoProducers = MODE == SPARQ_MODE_NONE || ATM;
     // ATM: the transform warps write their results to tensor memory, which the tensor core reads A from; the
     // raw activations have a ring of their own.
-    static_assert(!ATM || (MODE != SPARQ_MODE_NONE && BK == 128 && BN == 256), "A in tensor memory: transformed steps of 128 bytes");
-    const int S = g.stages;
+    static_assert(!ATM || (MODE != SPARQ_MODE_NONE && BK == 128 && BN == 256 && OUT == kOutBytes), "A in tensor memory: transformed steps of 128 bytes");
+    static_assert(!ATM || (Cfg::kAtmRawStages == 5 && Cfg::kAtmStages * 32 + BN <= 512), "rings with A in tensor memory");
+    const int S = ATM ? Cfg::kAtmStages : g.stages;
     extern __shared__ uint8_t smem_raw[];
     // The ring that the transform teams read has two sets of full barriers, for even and odd rounds.  A parity
     // answers for every second phase, so a team may ask a barrier for a phase only once it knows that the one before
@@ -1015,8 +1019,8 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     __shared__ __align__(8) uint64_t bar_full[kFullSets * kMaxStages], bar_xf[kMaxStages], bar_empty[kMaxStages];
     __shared__ __align__(8) uint64_t bar_raw[ATM ? kRawSets * kMaxStages : 1], bar_raw_empty[ATM ? kMaxStages : 1];
     __shared__ __align__(8) uint64_t bar_res[epi_warps(MODE)][2];       // residual boxes landed
-    // tensor memory: accumulators, and with ATM four to eight stages of transformed activations
-    constexpr int kAcc = ATM ? 256 / BN : Cfg::kAcc;
+    // tensor memory: accumulators; with ATM one, and four stages of transformed activations
+    constexpr int kAcc = ATM ? 1 : Cfg::kAcc;
     constexpr int kTmemCols = ATM ? 512 : Cfg::kTmemCols;
     // The epilogue warps form groups of four (one warp per tensor-memory lane quarter) and the
     // groups teams: team t takes the CTA's tiles of number t modulo the number of teams, so that the
@@ -1047,7 +1051,7 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     const int teams = total_tiles > gridDim.x ? kMaxTeams : 1;
 
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    const int SA = ATM ? g.raw_stages : S;
+    const int SA = ATM ? Cfg::kAtmRawStages : S;
     const uint32_t b_base = smem_base + (uint32_t)(ATM ? SA * Cfg::kABytes : Cfg::kABytes);
     constexpr uint32_t kAStep = ATM ? Cfg::kABytes : Cfg::kStageBytes, kBStep = ATM ? Cfg::kBBytes : Cfg::kStageBytes;
     auto a_stage = [&](int s) { return smem_base + (uint32_t)s * kAStep; };
@@ -1234,11 +1238,11 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         int64_t staged_nt = -1;
         uint32_t local_tile = (uint32_t)team;
         dep_wait();
-        if (OUT != kOutGeneral && g.out_box) {
-            // ---- through shared memory (see epi_staged_box) ----
+        if (!ATM && OUT != kOutGeneral && g.out_box) {
+            // ---- through shared memory (see epi_staged_box); a reduction long enough for ATM outweighs its output ----
             const int ew = warp - kFirstEpiWarp;
             const uint32_t box_bytes = 32u * (uint32_t)g.out_box;
-            const uint32_t stage0 = (ATM ? b_stage(S) : a_stage(S)) + (uint32_t)ew * 2u * box_bytes;
+            const uint32_t stage0 = a_stage(S) + (uint32_t)ew * 2u * box_bytes;
             constexpr bool res = OUT == kOutResidual;
             // boxes of this warp in order: the out_box-wide parts of its columns, tile after tile
             auto fetch = [&](uint32_t n, uint32_t tile, int c) {          // box n's residual, by lane 0
@@ -1478,15 +1482,7 @@ cudaError_t launch_gemm_kernel(const GemmMaps &m, GemmArgs &g, int grid, cudaStr
     }
     const int staging = g.out_box ? epi_warps(MODE) * 2 * 32 * g.out_box : 0;
     g.stages = TileCfg<BN, BK>::stages(staging);
-    g.raw_stages = 0;
-    if (ATM) {       // what is left of the room goes to the raw ring
-        using Cfg = TileCfg<BN, BK>;
-        const int room = kMaxDynSmemGemm - 1024 - staging, n = room / Cfg::kStageBytes;
-        g.stages = n > kMaxStages ? kMaxStages : n;
-        const int left = (room - g.stages * Cfg::kBBytes) / Cfg::kABytes;
-        g.raw_stages = left > kMaxStages ? kMaxStages : left;
-    }
-    const int smem = 1024 + g.stages * TileCfg<BN, BK>::kStageBytes + (g.raw_stages > g.stages ? (g.raw_stages - g.stages) * TileCfg<BN, BK>::kABytes : 0) + staging;
+    const int smem = ATM ? TileCfg<BN, BK>::kAtmSmem : 1024 + g.stages * TileCfg<BN, BK>::kStageBytes + staging;
     return launch_overlapped(kfn, grid, gemm_threads(MODE, ATM), smem, st, m.a, m.b, m.out, m.res, g);
 }
 
