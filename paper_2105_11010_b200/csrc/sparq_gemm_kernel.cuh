@@ -1422,30 +1422,30 @@ sparq_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                 if (s >= S) { s -= S; ++use; }
             }
         } else {
-        uint4 va[kHalf], vb[kHalf];
-        int s = team;
-        int q = team;              // its full barrier,
-        uint32_t ph = 0;           // and that barrier's phase
-        bool loaded = false;
-        for (uint32_t it = (uint32_t)team; it < total; it += kXfTeams) {
-            if (!loaded) {
-                mbar_wait<true>(smem_u32(&bar_full[q]), ph, abort_flag, g.status, g.wait_limit);
-                load(va, s, 0);
+            uint4 va[kHalf], vb[kHalf];
+            int s = team;
+            int q = team;              // its full barrier,
+            uint32_t ph = 0;           // and that barrier's phase
+            bool loaded = false;
+            for (uint32_t it = (uint32_t)team; it < total; it += kXfTeams) {
+                if (!loaded) {
+                    mbar_wait<true>(smem_u32(&bar_full[q]), ph, abort_flag, g.status, g.wait_limit);
+                    load(va, s, 0);
+                }
+                load(vb, s, kHalf);
+                work(va, s, 0);
+                int ns = s + kXfTeams;
+                if (ns >= S) ns -= S;
+                q += kXfTeams;
+                if (q >= kFullSets * S) { q -= kFullSets * S; ph ^= 1u; }
+                loaded = it + kXfTeams < total && __all_sync(0xFFFFFFFFu, mbar_test(smem_u32(&bar_full[q]), ph));
+                if (loaded) load(va, ns, 0);
+                work(vb, s, kHalf);
+                fence_proxy_async_smem();       // generic-proxy writes visible to the tensor core
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&bar_xf[s]));
+                s = ns;
             }
-            load(vb, s, kHalf);
-            work(va, s, 0);
-            int ns = s + kXfTeams;
-            if (ns >= S) ns -= S;
-            q += kXfTeams;
-            if (q >= kFullSets * S) { q -= kFullSets * S; ph ^= 1u; }
-            loaded = it + kXfTeams < total && __all_sync(0xFFFFFFFFu, mbar_test(smem_u32(&bar_full[q]), ph));
-            if (loaded) load(va, ns, 0);
-            work(vb, s, kHalf);
-            fence_proxy_async_smem();       // generic-proxy writes visible to the tensor core
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&bar_xf[s]));
-            s = ns;
-        }
         }
     }
 
