@@ -19,7 +19,7 @@ B5_TRIM = sparq.SparqParams(sparq.MODE_BSPARQ, 4, 0x1F, sparq.ROUND_TRUNCATE)
 
 CASES = [
     # 256-wide tiles, a dozen and more steps: activations in tensor memory
-    (25, 39, 1536, 256, 1, 2, V5, False), (25, 39, 1536, 224, 1, 2, V5_TRIM, False), (25, 39, 1408, 256, 1, 2, B5_TRIM, False),
+    (25, 39, 1536, 256, 1, 2, V5, False), (25, 39, 1536, 224, 1, 2, V5_TRIM, False), (25, 39, 1792, 256, 1, 2, B5_TRIM, False),
     (25, 39, 1664, 256, 1, 2, V7_TRIM, False), (26, 39, 768, 480, 1, 2, V3OPT, False), (25, 39, 256, 256, 3, 2, B6, False),
     # 256-wide tiles, fragments straight to memory, with and without a residual
     (25, 39, 512, 256, 1, 2, V5, True), (25, 39, 512, 256, 1, 2, NONE, False), (25, 39, 384, 224, 1, 2, NONE, True), (25, 39, 128, 256, 3, 2, NONE, False), (25, 39, 1552, 256, 1, 2, B5_TRIM, False),
