@@ -49,9 +49,9 @@ MIN_TIMED_MS = 50.0                 # device time every reported figure is the m
 
 # dram__bytes_read.sum + dram__bytes_write.sum per launch from the ncu captures summarized under
 # profiles/; None whenever the kernel has changed since its capture.
-TRAFFIC = {"head": 13051648 + 0,                # profiles/sparq_conv_window_kernel_cfg5.txt (output still dirty in L2)
-           "rn18": 6509312 + 0,                  # profiles/sparq_conv_window_kernel_cfg2.txt
-           "layer1x1": 12900608 + 914176,        # profiles/sparq_gemm_kernel_layer1x1.txt (mean of the two launches)
+TRAFFIC = {"head": 13051904 + 0,                # profiles/sparq_conv_window_kernel_cfg5.txt (output still dirty in L2)
+           "rn18": 6509824 + 0,                  # profiles/sparq_conv_window_kernel_cfg2.txt
+           "layer1x1": 12901504 + 775936,        # profiles/sparq_gemm_kernel_layer1x1.txt (mean of the two launches)
            "transform_per_2p28": 268445184 + 214811392}   # profiles/quantize_vec_kernel_2p28.txt
 
 

@@ -593,8 +593,8 @@ __device__ __forceinline__ void epi_lean(const uint32_t (&v)[32], const float *s
 // The same on matrix fragments (tmem_ld_frag_issue): a thread has four rows of eight columns, so that a
 // column's scale and bias are read once for four outputs, four 16-byte reads per 32 x 32 outputs where
 // a thread per row takes sixteen.  Those reads are broadcasts, but of more than one wavefront each, and shared
-// memory is what the epilogue shares with the tensor core's operands: they were 1200 of the 1600
-// wavefronts of the load / store pipe in a tile of an output-heavy layer.  16384 x 4096, K 512, 42.6 -> 38.7 us,
+// memory is what the epilogue shares with the tensor core's operands: 200704 x 256, K 64, 1600 -> 1370 wavefronts of
+// the load / store pipe a tile (425 of them now bank conflicts of the staged boxes).  16384 x 4096, K 512, 42.6 -> 38.7 us,
 // 50176 x 256, K 512, without a transform 9.95 -> 9.0, the ResNet-50 pass at batch 64 829 -> 799.
 // The eight columns are adjacent outputs because the weight rows lie in shared memory in fragment order:
 // row 8j + 2q + b of each group of 32 holds weight row 8q + 2j + b (a five-dimensional tensor map, no
@@ -1487,7 +1487,7 @@ cudaError_t launch_gemm_kernel(const GemmMaps &m, GemmArgs &g, int grid, cudaStr
 }
 
 // Whether a fused launch of 256-wide tiles puts the transformed activations into tensor memory (ATM).  What a
-// step moves through shared memory falls from 1024 to 768 wavefronts, but the accumulator has to
+// step moves through shared memory falls from 1024 to 768 wavefronts (counted, with copies and operand reads), but the accumulator has to
 // do with one stage, and a launch starts and ends a little later: from a dozen steps a CTA.  us with / without:
 // 16384 x 512, K 4096 (64 steps) 42.1 / 46.7, 12544 x 512, K 1024 (16) 14.3 / 15.0, 28x28x512 -> 1024 stride 2 (12) 13.3 /
 // 13.7, 50176 x 256, K 512 (12) 13.04 / 12.97, 12544 x 256, K 1024 (8) 9.14 / 9.08, 6272 x 256, K 1024 (8) 8.4 / 8.05,
